@@ -79,7 +79,7 @@ struct dc_ctx {
   void* v = nullptr;         // [M, nkv*hd]
   void* o = nullptr;         // attention output [M, nq*hd]
   void* act = nullptr;       // SwiGLU output [M, F]
-  float* tmp = nullptr;      // fp32 GEMM outputs of the CUDA-core path
+  float* tmp = nullptr;      // q / k / v projections of the CUDA-core path before the rotation (head_dim % 32 != 0)
   void* h = nullptr;         // LM-head input [M_lm, d]
   float* logits = nullptr;   // [M_lm, V] fp32, CUDA-core LM head only
   float* cos_sin = nullptr;  // RoPE table [max_batch * R_cap_max + 1, hd] (last row: angle step)
@@ -200,11 +200,13 @@ int run_step(dc_ctx* c, const dc_step_in* in, const dc_step_out* out, const SeqM
   T* act = (T*)c->act; T* h = (T*)c->h;
   const size_t k_layer = (size_t)g.max_batch * nkv * g.max_ctx * hd;
 
-  cudaMemsetAsync(out->status, 0, sizeof(int32_t) * m.batch, s);
   pf.begin(DC_STAGE_EMBED, 2);
+  unsigned int* words = nullptr;
+  int n_words = 0;
+  if (c->use_tc) tc_step_begin(c->tc, &words, &n_words);
+  launch_step_begin(m, hd, g.rope_theta, c->cos_sin, out->status, words, n_words, s);
   launch_embed<T>((const T*)c->embed, in->last_ids, in->win_ids, g.max_last, g.max_window,
                   g.mask_id, g.vocab, d, m, c->x, out->status, s);
-  launch_rope_table(m, hd, g.rope_theta, c->cos_sin, s);
   pf.end();
   DC_CHECK_LAUNCH(c);
 
@@ -215,7 +217,6 @@ int run_step(dc_ctx* c, const dc_step_in* in, const dc_step_out* out, const SeqM
 
   const bool export_kv = (in->flags & DC_STEP_EXPORT_KV) != 0;
   const bool chain = c->use_tc && tc_chain_ok(c->tc, m);
-  if (c->use_tc) tc_step_begin(c->tc);
   if (chain) {
     // persistent dense chain: norm1 + QKV of layer 0, then per layer attention and one launch
     // that runs O projection .. QKV of the next layer
@@ -260,36 +261,51 @@ int run_step(dc_ctx* c, const dc_step_in* in, const dc_step_out* out, const SeqM
       if (rc != DC_OK) return fail(c, rc, "tensor-core layer %d failed: %s", l, tc_error(c->tc));
       continue;
     }
-    pf.begin(DC_STAGE_QKV, 4);
-    launch_gemm_simt<T>(a, (const T*)c->wq[l], c->tmp, M, nq * hd, d, nqkv, EPI_STORE_F32, s);
-    launch_gemm_simt<T>(a, (const T*)c->wk[l], c->tmp + nq * hd, M, nkv * hd, d, nqkv,
-                        EPI_STORE_F32, s);
-    launch_gemm_simt<T>(a, (const T*)c->wv[l], c->tmp + (nq + nkv) * hd, M, nkv * hd, d, nqkv,
-                        EPI_STORE_F32, s);
-    launch_rope_store<T>(c->tmp, c->cos_sin, m, nq, nkv, hd,
-                         c->bq.empty() ? nullptr : (const T*)c->bq[l], c->bq.empty() ? nullptr : (const T*)c->bk[l],
-                         c->bq.empty() ? nullptr : (const T*)c->bv[l], q, k, v, s);
+    SimtGemm<T> ga;
+    ga.A = a; ga.M = M; ga.K = d; ga.m = m;
+    ga.nq = nq; ga.nkv = nkv; ga.hd = hd; ga.cos_sin = c->cos_sin; ga.q = q; ga.k = k; ga.v = v;
+    if (!c->bq.empty()) { ga.bq = (const T*)c->bq[l]; ga.bk = (const T*)c->bk[l]; ga.bv = (const T*)c->bv[l]; }
+    if (export_kv) {
+      ga.max_ctx = g.max_ctx;
+      ga.k_cache = (T*)in->k_cache + (size_t)l * k_layer;
+      ga.v_cache = (T*)in->v_cache + (size_t)l * k_layer;
+    }
+    if (hd % 32 == 0) {
+      pf.begin(DC_STAGE_QKV, 1);
+      ga.w0 = (const T*)c->wq[l]; ga.w1 = (const T*)c->wk[l]; ga.w2 = (const T*)c->wv[l];
+      launch_gemm_simt<T>(ga, EPI_QKV, s);
+    } else {
+      pf.begin(DC_STAGE_QKV, 4);
+      ga.ldc = nqkv;
+      const void* w[3] = {c->wq[l], c->wk[l], c->wv[l]};
+      int col = 0;
+      for (int i = 0; i < 3; ++i) {
+        ga.w0 = (const T*)w[i]; ga.N = (i == 0 ? nq : nkv) * hd; ga.C = c->tmp + col;
+        launch_gemm_simt<T>(ga, EPI_STORE_F32, s);
+        col += ga.N;
+      }
+      launch_rope_store<T>(c->tmp, ga, s);
+    }
     pf.end();
-    if (export_kv)
-      launch_export_kv<T>(k, v, 0, m, nkv, hd, g.max_ctx, (T*)in->k_cache + (size_t)l * k_layer,
-                          (T*)in->v_cache + (size_t)l * k_layer, s);
     if (kv_only && l + 1 == g.n_layers) break;
     pf.begin(DC_STAGE_ATTN, 1);
     launch_attn_simt<T>(q, k, v, kc, vc, g.max_ctx, m, nq, nkv, hd, o, s);
     pf.end();
+    SimtGemm<T> gb;
+    gb.M = M; gb.A = o; gb.w0 = (const T*)c->wo[l]; gb.N = d; gb.K = nq * hd; gb.C = c->x; gb.ldc = d;
     pf.begin(DC_STAGE_OPROJ, 1);
-    launch_gemm_simt<T>(o, (const T*)c->wo[l], c->x, M, d, nq * hd, d, EPI_ADD_F32, s);
+    launch_gemm_simt<T>(gb, EPI_ADD_F32, s);
     pf.end();
     pf.begin(DC_STAGE_NORM, 1);
     launch_rmsnorm<T>(c->x, nullptr, 0, 0, (const T*)c->norm2[l], g.rms_eps, M, d, a, s);
     pf.end();
-    pf.begin(DC_STAGE_GATEUP, 3);
-    launch_gemm_simt<T>(a, (const T*)c->w_gate[l], c->tmp, M, F, d, 2 * F, EPI_STORE_F32, s);
-    launch_gemm_simt<T>(a, (const T*)c->w_up[l], c->tmp + F, M, F, d, 2 * F, EPI_STORE_F32, s);
-    launch_swiglu<T>(c->tmp, M, F, act, s);
+    pf.begin(DC_STAGE_GATEUP, 1);
+    gb.A = a; gb.w0 = (const T*)c->w_gate[l]; gb.w1 = (const T*)c->w_up[l]; gb.N = F; gb.K = d; gb.act = act;
+    launch_gemm_simt<T>(gb, EPI_SWIGLU, s);
     pf.end();
     pf.begin(DC_STAGE_DOWN, 1);
-    launch_gemm_simt<T>(act, (const T*)c->w_down[l], c->x, M, d, F, d, EPI_ADD_F32, s);
+    gb.A = act; gb.w0 = (const T*)c->w_down[l]; gb.w1 = nullptr; gb.N = d; gb.K = F;
+    launch_gemm_simt<T>(gb, EPI_ADD_F32, s);
     pf.end();
     DC_CHECK_LAUNCH(c);
   }
@@ -299,16 +315,14 @@ int run_step(dc_ctx* c, const dc_step_in* in, const dc_step_out* out, const SeqM
     DC_CHECK_LAUNCH(c);
     return DC_OK;
   }
-  pf.begin(DC_STAGE_NORM, in->h_final_in ? 2 : 1);
-  launch_final_norm<T>(c->x, part, nsplit, part_stride, (const T*)c->final_norm, g.rms_eps, d, ml,
-                       h, s, m.nv);
-  if (carried || out->h_out) {
-    PrevLen pl{};
-    if (carried) for (int b = 0; b < m.batch; ++b) pl.n[b] = in->prev_len[b];
-    launch_carry<T>(carried ? (const T*)in->h_prev_in : nullptr, pl, (T*)out->h_out, g.max_window, d,
-                    ml, h, s);
+  pf.begin(DC_STAGE_NORM, 1);
+  LmRowsIo<T> io;
+  io.h_in = (const T*)in->h_final_in; io.h_out = (T*)out->h_out; io.max_window = g.max_window;
+  if (carried) {
+    io.h_prev_in = (const T*)in->h_prev_in;
+    for (int b = 0; b < m.batch; ++b) io.prev.n[b] = in->prev_len[b];
   }
-  if (in->h_final_in) launch_h_override<T>((const T*)in->h_final_in, g.max_window, d, ml, h, s);
+  launch_lm_rows<T>(c->x, part, nsplit, part_stride, (const T*)c->final_norm, g.rms_eps, d, ml, m.nv, io, h, s);
   pf.end();
 
   SignalOut so{out->pred_id, out->conf, out->entropy, out->influence, out->lse, g.max_window};
@@ -321,8 +335,9 @@ int run_step(dc_ctx* c, const dc_step_in* in, const dc_step_out* out, const SeqM
     c->have_logits = false;
   } else {
     pf.begin(DC_STAGE_LMHEAD, 2);
-    launch_gemm_simt<T>(h, (const T*)c->lm_head, c->logits, Mlm, g.vocab, d, g.vocab,
-                        EPI_STORE_F32, s);
+    SimtGemm<T> gl;
+    gl.A = h; gl.w0 = (const T*)c->lm_head; gl.M = Mlm; gl.N = g.vocab; gl.K = d; gl.C = c->logits; gl.ldc = g.vocab;
+    launch_gemm_simt<T>(gl, EPI_STORE_F32, s);
     launch_signals_from_logits(c->logits, g.vocab, g.mask_id, g.forbid_mask_pred, ml, c->ws_pred,
                                c->ws_conf, c->ws_ent, c->ws_infl, c->ws_lse, so, out->status, s);
     pf.end();
@@ -541,9 +556,11 @@ int dc_create(const dc_config* cfg, const dc_weights* w, void* cuda_stream, dc_c
     c->v = ws_alloc<char>(c, M * nkv * hd * es, &ok);
     c->o = ws_alloc<char>(c, M * nq * hd * es, &ok);
     c->act = ws_alloc<char>(c, M * g.d_ff * es, &ok);
-    const size_t tmp_cols = (size_t)((nq + 2 * nkv) * hd > 2 * g.d_ff ? (nq + 2 * nkv) * hd
-                                                                      : 2 * g.d_ff);
-    c->tmp = ws_alloc<float>(c, M * tmp_cols, &ok);
+    if (hd % 32) c->tmp = ws_alloc<float>(c, M * (nq + 2 * nkv) * hd, &ok);
+  }
+  if ((!c->use_tc || !c->tc_lm) && !simt_init(c->bf16, hd)) {
+    dc_destroy(c);
+    return fail(nullptr, DC_ERR_UNSUPPORTED, "head_dim %d needs more shared memory than the CUDA-core kernels have", hd);
   }
   if (!c->tc_lm) c->logits = ws_alloc<float>(c, (size_t)c->Mlm_max * g.vocab, &ok);
   if (!ok) {

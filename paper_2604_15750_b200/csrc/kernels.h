@@ -55,45 +55,62 @@ template <typename T>
 void launch_rmsnorm(float* x, const float* part, int nsplit, size_t part_stride, const T* g,
                     float eps, int M, int d, T* out, cudaStream_t s);
 
-// final norm of the window rows into the LM-head row order (pad rows are zeroed)
-template <typename T>
-void launch_final_norm(float* x, const float* part, int nsplit, size_t part_stride, const T* g,
-                       float eps, int d, const SeqMeta& m, T* h, cudaStream_t s, int nv_x = -1);
-// LM rows carried between steps: h_out[b][k] <- curr row (if h_out); prev rows <- h_prev_in[b][k]
-// for k < prev_len.n[b], else the curr row of the same position (if h_prev_in); m.nv must be 2 then
+// LM-head input rows (k_lm_rows): the final norm of the window's rows, and what may stand in for them
 struct PrevLen { int n[DC_MAX_BATCH]; };
 template <typename T>
-void launch_carry(const T* h_prev_in, const PrevLen& pl, T* h_out, int max_window, int d,
-                  const SeqMeta& m, T* h, cudaStream_t s);
-
-// copy caller-supplied LM-head input [B][2][max_window][d] into the LM-head row order
+struct LmRowsIo {
+  const T* h_in = nullptr;       // [B][2][max_window][d]: replaces every row
+  const T* h_prev_in = nullptr;  // [B][max_window][d]: prev row k of sequence b for k < prev.n[b]
+  T* h_out = nullptr;            // [B][max_window][d]: gets the curr rows
+  int max_window = 0;
+  PrevLen prev{};
+};
+// x holds nv_x variants; with nv_x < m.nv the prev rows are carried in.  Pad rows are zeroed.
 template <typename T>
-void launch_h_override(const T* h_in, int max_window, int d, const SeqMeta& m, T* h,
-                       cudaStream_t s);
+void launch_lm_rows(const float* x, const float* part, int nsplit, size_t part_stride, const T* g, float eps, int d,
+                    const SeqMeta& m, int nv_x, const LmRowsIo<T>& io, T* h, cudaStream_t s);
 
-enum { EPI_STORE_F32 = 0, EPI_ADD_F32 = 1 };
-// C[M,N] (fp32, ldc) (=|+=) A[M,K] * W[N,K]^T
+// One CUDA-core GEMM over A [M, K] with the epilogue of its place in a layer.  w0 .. w2: weight
+// matrices [rows, K] (QKV: q, k, v;  SWIGLU: gate, up;  otherwise w0 [N, K]).
+enum { EPI_STORE_F32 = 0,  // C = acc                                             (fp32, row pitch ldc)
+       EPI_ADD_F32 = 1,    // C += acc
+       EPI_SWIGLU = 2,     // act [M, N] = silu(gate) * up
+       EPI_QKV = 3 };      // q, k: + bias, rotated;  v: + bias; and into the cache (head_dim % 32 == 0)
 template <typename T>
-void launch_gemm_simt(const T* A, const T* W, float* C, int M, int N, int K, int ldc, int epi,
-                      cudaStream_t s);
-
-void launch_rope_table(const SeqMeta& m, int head_dim, float theta, float* cos_sin,
-                       cudaStream_t s);
-
-// q,k: (+ bias) rotate + store as T; v: (+ bias) store as T.  tmp layout [M, (nq + 2 nkv) * hd]
-// fp32; bq / bk / bv: projection biases or null.
+struct SimtGemm {
+  const T* A = nullptr;
+  const T *w0 = nullptr, *w1 = nullptr, *w2 = nullptr;
+  int M = 0, N = 0, K = 0, ldc = 0;
+  int vec = 0;              // set by the launcher: rows start on 16-byte boundaries
+  float* C = nullptr;
+  T* act = nullptr;
+  // QKV
+  int nq = 0, nkv = 0, hd = 0, max_ctx = 0;
+  const float* cos_sin = nullptr;
+  const T *bq = nullptr, *bk = nullptr, *bv = nullptr;   // projection biases or null
+  T *q = nullptr, *k = nullptr, *v = nullptr;            // [M, heads * hd]
+  T *k_cache = nullptr, *v_cache = nullptr;              // one layer's context cache to append the last block's rows to, or null
+  SeqMeta m{};
+};
 template <typename T>
-void launch_rope_store(const float* tmp, const float* cos_sin, const SeqMeta& m, int nq, int nkv,
-                       int hd, const T* bq, const T* bk, const T* bv, T* q, T* k, T* v, cudaStream_t s);
+void launch_gemm_simt(const SimtGemm<T>& g, int epi, cudaStream_t s);
 
+// RoPE table of the step's rows; clears status[batch] and words[n_words]
+void launch_step_begin(const SeqMeta& m, int head_dim, float theta, float* cos_sin, int32_t* status,
+                       unsigned int* words, int n_words, cudaStream_t s);
+
+// the QKV epilogue over projections in `tmp` [M, (nq + 2 nkv) * hd], for any head_dim
 template <typename T>
-void launch_swiglu(const float* gate_up, int M, int F, T* act, cudaStream_t s);
+void launch_rope_store(const float* tmp, const SimtGemm<T>& g, cudaStream_t s);
 
 // k_cache [.. max_ctx][hd], v_cache [.. hd][max_ctx] of one layer: [max_batch][nkv][...]
 template <typename T>
 void launch_attn_simt(const T* q, const T* k, const T* v, const T* k_cache, const T* v_cache,
                       int max_ctx, const SeqMeta& m, int nq, int nkv, int hd, T* o,
                       cudaStream_t s);
+
+// once per context: shared-memory opt-in of the CUDA-core kernels on the current device
+bool simt_init(bool bf16, int head_dim);
 
 struct SignalOut {
   int32_t* pred_id;

@@ -4,9 +4,13 @@
 // of the tensor-core path.
 #include <math.h>
 
+#include <type_traits>
+
 #include "kernels.h"
 
 namespace dc {
+
+constexpr size_t kSimtSmemMax = 220 * 1024;   // dynamic shared memory a kernel of this file may ask for
 
 template <typename T> __device__ __forceinline__ float to_f(T v);
 template <> __device__ __forceinline__ float to_f<float>(float v) { return v; }
@@ -151,157 +155,334 @@ void launch_rmsnorm(float* x, const float* part, int nsplit, size_t part_stride,
   k_rmsnorm<T><<<M, 256, 0, s>>>(x, part, nsplit, part_stride, g, eps, d, out);
 }
 
+// LM-head input rows, one block per row of the LM head's order (groups of G positions: curr rows, then
+// prev rows): the final norm of the window's rows (nothing reads x after it, so the folded row stays
+// on chip); rows of p_prev carried in from an earlier step, or - no earlier prediction for the
+// position - a copy of the curr row, which makes the two distributions equal and I_k = 0; the
+// caller's shaped rows in place of either; and the copy of the curr rows that a later step carries.
+// (One launch: as three the second and third cost 3 us each of a step for a few hundred KB.)
 template <typename T>
-__global__ void k_final_norm(float* __restrict__ x, const float* __restrict__ part, int nsplit,
-                             size_t part_stride, const T* __restrict__ g, float eps, int d,
-                             SeqMeta m, T* __restrict__ h, int nv_x) {
+__global__ void __launch_bounds__(256) k_lm_rows(const float* __restrict__ x, const float* __restrict__ part, int nsplit,
+                                                 size_t part_stride, const T* __restrict__ g, float eps, int d,
+                                                 const SeqMeta m, int nv_x, const LmRowsIo<T> io, T* __restrict__ h) {
+  extern __shared__ __align__(16) float lm_row_s[];   // the row with the partial sums folded in
   __shared__ float red[32];
-  // grid: nv * npos_pad LM rows
   const int lrow = blockIdx.x;
   const int grp = lrow / (m.nv * m.G), in = lrow % (m.nv * m.G);
   const int v = in / m.G, p = grp * m.G + in % m.G;
-  if (v >= nv_x) return;   // x holds fewer variants than the LM head sees: those rows are carried in
+  const int b = p / m.W_cap, k = p % m.W_cap;
   T* hr = h + (size_t)lrow * d;
-  const int b = p / m.W_cap, k = p % m.W_cap;
+  const T* src = nullptr;        // copied instead of normed
+  bool norm = true;
   if (b >= m.batch || k >= m.win_len[b]) {
-    for (int i = threadIdx.x; i < d; i += blockDim.x) hr[i] = from_f<T>(0.f);
-    return;
+    norm = false;                // pad row: zero
+  } else if (io.h_in != nullptr) {
+    src = io.h_in + (((size_t)b * 2 + v) * io.max_window + k) * d;
+    norm = v == 0 && io.h_out != nullptr;
+  } else if (v >= nv_x && k < io.prev.n[b]) {
+    src = io.h_prev_in + ((size_t)b * io.max_window + k) * d;
+    norm = false;
   }
-  const size_t off = (size_t)act_row(m, v, b, m.last_len[b] + k) * d;
-  rmsnorm_row<T>(x + off, part ? part + off : nullptr, nsplit, part_stride, g, eps, d, hr, red);
-}
-
-template <typename T>
-void launch_final_norm(float* x, const float* part, int nsplit, size_t part_stride, const T* g,
-                       float eps, int d, const SeqMeta& m, T* h, cudaStream_t s, int nv_x) {
-  k_final_norm<T><<<m.nv * m.npos_pad, 256, 0, s>>>(x, part, nsplit, part_stride, g, eps, d, m, h,
-                                                    nv_x < 0 ? m.nv : nv_x);
-}
-
-template <typename T>
-__global__ void k_carry(const T* __restrict__ h_prev_in, PrevLen pl, T* __restrict__ h_out,
-                        int max_window, int d, SeqMeta m, T* __restrict__ h) {
-  const int lrow = blockIdx.x;
-  const int grp = lrow / (m.nv * m.G), in = lrow % (m.nv * m.G);
-  const int v = in / m.G, p = grp * m.G + in % m.G;
-  const int b = p / m.W_cap, k = p % m.W_cap;
-  const bool live = b < m.batch && k < m.win_len[b];
-  T* row = h + (size_t)lrow * d;
-  if (v == 0) {
-    if (!live || !h_out) return;
-    T* dst = h_out + ((size_t)b * max_window + k) * d;
+  if (src != nullptr || !norm) {
     for (int i = threadIdx.x * 4; i < d; i += blockDim.x * 4) {
-      float v4[4];
-      load4<T>(row + i, v4);
-      store4<T>(dst + i, v4);
+      float o[4] = {0.f, 0.f, 0.f, 0.f};
+      if (src != nullptr) load4<T>(src + i, o);
+      store4<T>(hr + i, o);
     }
-    return;
+    if (!norm) return;
   }
-  if (!h_prev_in) return;
-  // prev row: the carried row, or (no earlier prediction for this position) the curr row itself,
-  // which makes the two distributions equal and I_k = 0; pad rows are zero
-  const T* src = !live ? nullptr
-               : (k < pl.n[b]) ? h_prev_in + ((size_t)b * max_window + k) * d
-                               : h + (size_t)lm_row(m, 0, p) * d;
+  const size_t off = (size_t)act_row(m, v < nv_x ? v : 0, b, m.last_len[b] + k) * d;
+  T* dst0 = src == nullptr ? hr : nullptr;
+  T* dst1 = (v == 0 && io.h_out != nullptr) ? io.h_out + ((size_t)b * io.max_window + k) * d : nullptr;
+  float ss = 0.f;
   for (int i = threadIdx.x * 4; i < d; i += blockDim.x * 4) {
-    float v4[4] = {0.f, 0.f, 0.f, 0.f};
-    if (src) load4<T>(src + i, v4);
-    store4<T>(row + i, v4);
+    float4 w = *reinterpret_cast<const float4*>(x + off + i);
+    if (part)
+      for (int sidx = 0; sidx < nsplit; ++sidx) {
+        const float4 pv = *reinterpret_cast<const float4*>(part + sidx * part_stride + off + i);
+        w.x += pv.x; w.y += pv.y; w.z += pv.z; w.w += pv.w;
+      }
+    *reinterpret_cast<float4*>(lm_row_s + i) = w;
+    ss += w.x * w.x + w.y * w.y + w.z * w.z + w.w * w.w;
   }
-}
-
-template <typename T>
-void launch_carry(const T* h_prev_in, const PrevLen& pl, T* h_out, int max_window, int d,
-                  const SeqMeta& m, T* h, cudaStream_t s) {
-  k_carry<T><<<m.nv * m.npos_pad, 128, 0, s>>>(h_prev_in, pl, h_out, max_window, d, m, h);
-}
-template void launch_carry<float>(const float*, const PrevLen&, float*, int, int, const SeqMeta&, float*, cudaStream_t);
-template void launch_carry<__nv_bfloat16>(const __nv_bfloat16*, const PrevLen&, __nv_bfloat16*, int, int,
-                                          const SeqMeta&, __nv_bfloat16*, cudaStream_t);
-
-template <typename T>
-__global__ void k_h_override(const T* __restrict__ h_in, int max_window, int d, SeqMeta m,
-                             T* __restrict__ h) {
-  const int lrow = blockIdx.x;
-  const int grp = lrow / (m.nv * m.G), in = lrow % (m.nv * m.G);
-  const int v = in / m.G, p = grp * m.G + in % m.G;
-  const int b = p / m.W_cap, k = p % m.W_cap;
-  if (b >= m.batch || k >= m.win_len[b]) return;  // pad rows were zeroed by the final norm
-  const T* src = h_in + (((size_t)b * 2 + v) * max_window + k) * d;
-  T* dst = h + (size_t)lrow * d;
+  ss = block_sum(ss, red);
+  const float inv = rsqrtf(ss / (float)d + eps);
   for (int i = threadIdx.x * 4; i < d; i += blockDim.x * 4) {
-    float v4[4];
-    load4<T>(src + i, v4);
-    store4<T>(dst + i, v4);
+    const float4 w = *reinterpret_cast<const float4*>(lm_row_s + i);
+    float gv[4];
+    load4<T>(g + i, gv);
+    const float o[4] = {w.x * inv * gv[0], w.y * inv * gv[1], w.z * inv * gv[2], w.w * inv * gv[3]};
+    if (dst0) store4<T>(dst0 + i, o);
+    if (dst1) store4<T>(dst1 + i, o);
   }
 }
 
 template <typename T>
-void launch_h_override(const T* h_in, int max_window, int d, const SeqMeta& m, T* h,
-                       cudaStream_t s) {
-  k_h_override<T><<<m.nv * m.npos_pad, 128, 0, s>>>(h_in, max_window, d, m, h);
+void launch_lm_rows(const float* x, const float* part, int nsplit, size_t part_stride, const T* g, float eps, int d,
+                    const SeqMeta& m, int nv_x, const LmRowsIo<T>& io, T* h, cudaStream_t s) {
+  k_lm_rows<T><<<m.nv * m.npos_pad, 256, d * sizeof(float), s>>>(x, part, nsplit, part_stride, g, eps, d, m, nv_x, io, h);
 }
 
-// ---- plain tiled GEMM: C[M,N] (=|+=) A[M,K] W[N,K]^T, fp32 accumulate -------------------------
+// ---- CUDA-core GEMM: acc[m, n] = sum_k A[m, k] W[n, k], fp32 FMAs, with the epilogues of a layer ----
+//
+// These run for models of a few million parameters (fp32, or shapes the tensor cores do not take),
+// where a GEMM is 10..400 M FMAs and its time is the latency of one pass: load, multiply, reduce,
+// store.  So the tile is small (16 x 32: 48..512 CTAs at d 256 instead of 4..64 with 64 x 64), the
+// eight warps of a CTA split K among them (a chunk of 128 k is 16 per warp), chunks arrive through
+// a three-stage cp.async ring, and a lane's 4 x 4 outputs are fed by 16-byte shared-memory reads of
+// four k at a time, multiplied as packed fp32 pairs.  Measured with d 256, d_ff 1024, M 96 (a 64 x 64
+// tile with element-wise loads before): QKV with its rotation 3 launches of 38 us + 2.3 -> 4.9 us,
+// gate / up with SwiGLU 2 x 41 + 2 -> 7.3 us, O and down projection 41 -> 7.4 us on average.  Above
+// kSmallTiles tiles (eight per SM) the 64 x 64 tile takes over: the same inner loop (bound by
+// shared-memory reads either way) with a third of the L2 traffic per output, which binds once every
+// SM holds several small tiles.
+//
+// A tile's 32 columns are either 32 consecutive rows of W, or - for the epilogues that combine two
+// output features - 16 features and their partners: i and i + head_dim / 2 of a head (RoPE), or
+// gate and up of an MLP feature.
+template <typename T> struct GemmIo {
+  static constexpr int kPiece = 16 / (int)sizeof(T);   // elements of a 16-byte copy
+  static constexpr int kPad = kPiece;                  // row padding: no bank conflicts between 8 rows
+};
+__device__ __forceinline__ void cp_async16(void* dst, const void* src, int bytes) {   // the rest of the 16 bytes is zeroed
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;"
+               ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src), "r"(bytes) : "memory");
+}
+typedef unsigned long long f2;
+__device__ __forceinline__ f2 pack2(float lo, float hi) {
+  f2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ void fma2(f2& d, f2 a, f2 b) {
+  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
+}
+__device__ __forceinline__ float sum2(f2 v) {
+  float lo, hi;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+  return lo + hi;
+}
+
 template <typename T>
-__global__ void __launch_bounds__(256) k_gemm_simt(const T* __restrict__ A,
-                                                   const T* __restrict__ W, float* __restrict__ C,
-                                                   int M, int N, int K, int ldc, int epi) {
-  constexpr int BM = 64, BN = 64, BK = 16;
-  __shared__ float As[BK][BM + 4];
-  __shared__ float Ws[BK][BN + 4];
-  const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-  const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
-  float acc[4][4] = {};
-  for (int k0 = 0; k0 < K; k0 += BK) {
-    for (int i = threadIdx.x; i < BM * BK; i += 256) {
-      const int r = i / BK, c = i % BK;
-      const int gm = m0 + r, gk = k0 + c;
-      As[c][r] = (gm < M && gk < K) ? to_f<T>(A[(size_t)gm * K + gk]) : 0.f;
-      const int gn = n0 + r;
-      Ws[c][r] = (gn < N && gk < K) ? to_f<T>(W[(size_t)gn * K + gk]) : 0.f;
+__device__ __forceinline__ void simt_store_qkv(const SimtGemm<T>& g, int m, int head, int e, float y1, float y2);
+
+template <typename T, int WM, int WN, int WK, int KC, int STAGES, int EPI>
+__global__ void __launch_bounds__(256) k_gemm_simt(const SimtGemm<T> g) {
+  constexpr int BM = 16 * WM, BN = 32 * WN, PITCH = KC + GemmIo<T>::kPad, PIECE = GemmIo<T>::kPiece;
+  constexpr int ROWS = BM + BN, STAGE = ROWS * PITCH, CP = BN + 1;
+  static_assert(WM * WN * WK == 8 && KC % (4 * WK) == 0 && KC % PIECE == 0, "eight warps");
+  extern __shared__ __align__(16) unsigned char simt_smem[];
+  T* ring = reinterpret_cast<T*>(simt_smem);
+  float* cs = reinterpret_cast<float*>(simt_smem);     // [WK][BM][CP], over the ring once it is drained
+  __shared__ const T* rowp[ROWS];                      // source rows of the tile; null: beyond the matrix
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int m0 = blockIdx.y * BM, u0 = blockIdx.x * WN;   // u: unit of 32 columns
+  for (int r = tid; r < ROWS; r += 256) {
+    const T* src = nullptr;
+    if (r < BM) {
+      if (m0 + r < g.M) src = g.A + (size_t)(m0 + r) * g.K;
+    } else {
+      const int j = r - BM, u = u0 + (j >> 5), jj = j & 31;
+      if (EPI == EPI_QKV) {
+        const int half = g.hd >> 1, per_head = g.hd >> 5, head = u / per_head;
+        const int e = (u - head * per_head) * 16 + (jj & 15) + (jj >> 4) * half;
+        if (head < g.nq) src = g.w0 + (size_t)(head * g.hd + e) * g.K;
+        else if (head < g.nq + g.nkv) src = g.w1 + (size_t)((head - g.nq) * g.hd + e) * g.K;
+        else if (head < g.nq + 2 * g.nkv) src = g.w2 + (size_t)((head - g.nq - g.nkv) * g.hd + e) * g.K;
+      } else if (EPI == EPI_SWIGLU) {
+        const int f = u * 16 + (jj & 15);
+        if (f < g.N) src = (jj < 16 ? g.w0 : g.w1) + (size_t)f * g.K;
+      } else {
+        const int n = u * 32 + jj;
+        if (n < g.N) src = g.w0 + (size_t)n * g.K;
+      }
     }
-    __syncthreads();
+    rowp[r] = src;
+  }
+  __syncthreads();
+
+  const int chunks = (g.K + KC - 1) / KC;
+  auto load = [&](int c) {
+    T* dst = ring + (size_t)(c % STAGES) * STAGE;
+    const int k0 = c * KC;
+    if (g.vec) {
+      for (int p = tid; p < ROWS * (KC / PIECE); p += 256) {
+        const int r = p / (KC / PIECE), k = (p - r * (KC / PIECE)) * PIECE;
+        const T* src = rowp[r];
+        const int bytes = src == nullptr ? 0 : max(0, min(16, (g.K - k0 - k) * (int)sizeof(T)));
+        cp_async16(dst + r * PITCH + k, bytes ? src + k0 + k : g.A, bytes);
+      }
+    } else {   // rows that are not 16-byte aligned
+      for (int p = tid; p < ROWS * KC; p += 256) {
+        const int r = p / KC, k = p - r * KC;
+        const T* src = rowp[r];
+        dst[r * PITCH + k] = (src != nullptr && k0 + k < g.K) ? src[k0 + k] : from_f<T>(0.f);
+      }
+    }
+  };
+  for (int c = 0; c < STAGES - 1; ++c) {
+    if (c < chunks) load(c);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  }
+  const int wk = warp % WK, wn = (warp / WK) % WN, wm = warp / (WK * WN);
+  const int ty = lane >> 3, tx = lane & 7;
+  f2 acc[4][4];
 #pragma unroll
-    for (int kk = 0; kk < BK; ++kk) {
-      float a[4], w[4];
+  for (int i = 0; i < 4; ++i)
 #pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = As[kk][ty * 4 + i];
+    for (int j = 0; j < 4; ++j) acc[i][j] = 0ull;
+  for (int c = 0; c < chunks; ++c) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(STAGES - 2) : "memory");
+    __syncthreads();     // chunk c has landed for every thread; the stage of chunk c - 1 is free
+    if (c + STAGES - 1 < chunks) load(c + STAGES - 1);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    const T* st = ring + (size_t)(c % STAGES) * STAGE + wk * (KC / WK);
+    const T* ap = st + (wm * 16 + ty * 4) * PITCH;
+    const T* wp = st + (BM + wn * 32 + tx) * PITCH;
 #pragma unroll
-      for (int j = 0; j < 4; ++j) w[j] = Ws[kk][tx * 4 + j];
+    for (int k = 0; k < KC / WK; k += 4) {
+      f2 av[4][2], wv[4][2];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        float v[4];
+        load4<T>(ap + i * PITCH + k, v);
+        av[i][0] = pack2(v[0], v[1]); av[i][1] = pack2(v[2], v[3]);
+        load4<T>(wp + i * 8 * PITCH + k, v);
+        wv[i][0] = pack2(v[0], v[1]); wv[i][1] = pack2(v[2], v[3]);
+      }
 #pragma unroll
       for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], w[j], acc[i][j]);
+        for (int j = 0; j < 4; ++j) {
+          fma2(acc[i][j], av[i][0], wv[j][0]);
+          fma2(acc[i][j], av[i][1], wv[j][1]);
+        }
     }
-    __syncthreads();
   }
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  __syncthreads();       // the ring is read; the sums go over it
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int gm = m0 + ty * 4 + i;
-    if (gm >= M) continue;
+  for (int i = 0; i < 4; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int gn = n0 + tx * 4 + j;
-      if (gn >= N) continue;
-      float* c = C + (size_t)gm * ldc + gn;
-      *c = (epi == EPI_ADD_F32) ? (*c + acc[i][j]) : acc[i][j];
+    for (int j = 0; j < 4; ++j)
+      cs[(wk * BM + wm * 16 + ty * 4 + i) * CP + wn * 32 + tx + 8 * j] = sum2(acc[i][j]);
+  __syncthreads();
+  auto value = [&](int r, int c) {
+    float v = cs[r * CP + c];
+#pragma unroll
+    for (int w = 1; w < WK; ++w) v += cs[(w * BM + r) * CP + c];
+    return v;
+  };
+  if (EPI == EPI_STORE_F32 || EPI == EPI_ADD_F32) {
+    for (int p = tid; p < BM * BN; p += 256) {
+      const int r = p / BN, c = p - r * BN, m = m0 + r, n = u0 * 32 + c;
+      if (m >= g.M || n >= g.N) continue;
+      float* dst = g.C + (size_t)m * g.ldc + n;
+      const float v = value(r, c);
+      *dst = EPI == EPI_ADD_F32 ? *dst + v : v;
     }
+  } else {
+    for (int p = tid; p < BM * BN / 2; p += 256) {
+      const int r = p / (BN / 2), c = p - r * (BN / 2), m = m0 + r;
+      const int u = u0 + (c >> 4), i = c & 15;
+      if (m >= g.M) continue;
+      const float y1 = value(r, (c >> 4) * 32 + i), y2 = value(r, (c >> 4) * 32 + 16 + i);
+      if (EPI == EPI_SWIGLU) {
+        const int f = u * 16 + i;
+        if (f < g.N) g.act[(size_t)m * g.N + f] = from_f<T>(y1 / (1.f + expf(-y1)) * y2);
+      } else {
+        const int half = g.hd >> 1, per_head = g.hd >> 5, head = u / per_head;
+        if (head >= g.nq + 2 * g.nkv) continue;
+        const int e = (u - head * per_head) * 16 + i;
+        simt_store_qkv<T>(g, m, head, e, y1, y2);
+      }
+    }
+  }
+}
+
+// One rotated pair (features e and e + head_dim / 2 of a head) of activation row m: bias, rotation,
+// store, and the copy into the context cache when the row belongs to an exported last block.
+template <typename T>
+__device__ __forceinline__ void simt_store_qkv(const SimtGemm<T>& g, int m, int head, int e, float y1, float y2) {
+  const int hd = g.hd, half = hd >> 1;
+  const int rv = g.m.batch * g.m.R_cap, br = m % rv;   // (b, r): the RoPE table is shared by both variants
+  if (g.bq != nullptr) {   // projection bias, before the rotation
+    const T* bb = head < g.nq ? g.bq + head * hd : head < g.nq + g.nkv ? g.bk + (head - g.nq) * hd
+                                                                       : g.bv + (head - g.nq - g.nkv) * hd;
+    y1 += to_f<T>(bb[e]); y2 += to_f<T>(bb[half + e]);
+  }
+  const bool is_v = head >= g.nq + g.nkv;
+  if (!is_v) {
+    const float c = g.cos_sin[(size_t)br * hd + e], sn = g.cos_sin[(size_t)br * hd + half + e];
+    const float t = y1 * c - y2 * sn;
+    y2 = y2 * c + y1 * sn;
+    y1 = t;
+  }
+  const T o1 = from_f<T>(y1), o2 = from_f<T>(y2);
+  if (head < g.nq) {
+    T* dst = g.q + (size_t)m * g.nq * hd + head * hd + e;
+    dst[0] = o1; dst[half] = o2;
+    return;
+  }
+  const int hk = is_v ? head - g.nq - g.nkv : head - g.nq;
+  T* dst = (is_v ? g.v : g.k) + (size_t)m * g.nkv * hd + hk * hd + e;
+  dst[0] = o1; dst[half] = o2;
+  if (g.k_cache != nullptr && m < rv) {
+    const int b = br / g.m.R_cap, r = br - b * g.m.R_cap;
+    if (r < g.m.last_len[b]) {
+      const size_t kv = (size_t)b * g.nkv + hk;
+      const int key = g.m.ctx_len[b] + r;
+      if (is_v) {
+        g.v_cache[(kv * hd + e) * g.max_ctx + key] = o1;
+        g.v_cache[(kv * hd + half + e) * g.max_ctx + key] = o2;
+      } else {
+        g.k_cache[(kv * g.max_ctx + key) * hd + e] = o1;
+        g.k_cache[(kv * g.max_ctx + key) * hd + half + e] = o2;
+      }
+    }
+  }
+}
+
+constexpr long long kSmallTiles = 148 * 8;
+
+template <typename T, int EPI>
+static void launch_gemm_epi(SimtGemm<T> g, int units, cudaStream_t s) {
+  auto aligned = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
+  g.vec = g.K % GemmIo<T>::kPiece == 0 && aligned(g.A) && aligned(g.w0) &&
+          (g.w1 == nullptr || aligned(g.w1)) && (g.w2 == nullptr || aligned(g.w2));
+  const long long tiles = (long long)((g.M + 15) / 16) * units;
+  if (tiles <= kSmallTiles) {
+    constexpr int KC = 128, STAGES = 3;
+    const size_t ring = (size_t)STAGES * 48 * (KC + GemmIo<T>::kPad) * sizeof(T), sums = 8 * 16 * 33 * sizeof(float);
+    k_gemm_simt<T, 1, 1, 8, KC, STAGES, EPI><<<dim3(units, (g.M + 15) / 16), 256, ring > sums ? ring : sums, s>>>(g);
+  } else {
+    constexpr int KC = 32, STAGES = 3;
+    const size_t ring = (size_t)STAGES * 128 * (KC + GemmIo<T>::kPad) * sizeof(T), sums = 64 * 65 * sizeof(float);
+    k_gemm_simt<T, 4, 2, 1, KC, STAGES, EPI><<<dim3((units + 1) / 2, (g.M + 63) / 64), 256, ring > sums ? ring : sums, s>>>(g);
   }
 }
 
 template <typename T>
-void launch_gemm_simt(const T* A, const T* W, float* C, int M, int N, int K, int ldc, int epi,
-                      cudaStream_t s) {
-  dim3 grid((N + 63) / 64, (M + 63) / 64);
-  k_gemm_simt<T><<<grid, 256, 0, s>>>(A, W, C, M, N, K, ldc, epi);
+void launch_gemm_simt(const SimtGemm<T>& g, int epi, cudaStream_t s) {
+  switch (epi) {
+    case EPI_STORE_F32: launch_gemm_epi<T, EPI_STORE_F32>(g, (g.N + 31) / 32, s); break;
+    case EPI_ADD_F32: launch_gemm_epi<T, EPI_ADD_F32>(g, (g.N + 31) / 32, s); break;
+    case EPI_SWIGLU: launch_gemm_epi<T, EPI_SWIGLU>(g, (g.N + 15) / 16, s); break;
+    default: launch_gemm_epi<T, EPI_QKV>(g, (g.nq + 2 * g.nkv) * (g.hd / 32), s);
+  }
 }
 
-// ---- RoPE ----------------------------------------------------------------------------------------
+// ---- start of a step: RoPE table, cleared words --------------------------------------------------
 // cos_sin[(b * R_cap + r) * hd + i] = cos(angle), [.. + hd/2 + i] = sin(angle),
 // angle = (pos0[b] + r) * theta^(-2i/hd), evaluated in double precision.  Row batch * R_cap
 // holds cos / sin of theta^(-2i/hd) itself, the angle step between consecutive rows.
-__global__ void k_rope_table(SeqMeta m, int hd, float theta, float* __restrict__ cos_sin) {
+// The first block also clears status[batch] and the synchronisation words of the dense chain.
+__global__ void k_step_begin(const SeqMeta m, int hd, float theta, float* __restrict__ cos_sin,
+                             int32_t* __restrict__ status, unsigned int* __restrict__ words, int n_words) {
+  if (blockIdx.x == 0) {
+    for (int i = threadIdx.x; i < m.batch; i += blockDim.x) status[i] = 0;
+    for (int i = threadIdx.x; i < n_words; i += blockDim.x) words[i] = 0u;
+  }
   const int half = hd / 2;
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
   const int rows = m.batch * m.R_cap;
@@ -317,126 +498,189 @@ __global__ void k_rope_table(SeqMeta m, int hd, float theta, float* __restrict__
   cos_sin[(size_t)br * hd + half + i] = (float)sn;
 }
 
-void launch_rope_table(const SeqMeta& m, int head_dim, float theta, float* cos_sin,
-                       cudaStream_t s) {
+void launch_step_begin(const SeqMeta& m, int head_dim, float theta, float* cos_sin, int32_t* status,
+                       unsigned int* words, int n_words, cudaStream_t s) {
   const int total = (m.batch * m.R_cap + 1) * (head_dim / 2);
-  k_rope_table<<<(total + 255) / 256, 256, 0, s>>>(m, head_dim, theta, cos_sin);
+  k_step_begin<<<(total + 255) / 256, 256, 0, s>>>(m, head_dim, theta, cos_sin, status, words, n_words);
 }
 
+// head_dim not a multiple of 32: the projections go through `tmp` [M, (nq + 2 nkv) hd] and this
+// kernel, everything else has the rotation in the GEMM's epilogue.
 template <typename T>
-__global__ void k_rope_store(const float* __restrict__ tmp, const float* __restrict__ cos_sin,
-                             SeqMeta m, int nq, int nkv, int hd, const T* __restrict__ bq,
-                             const T* __restrict__ bk, const T* __restrict__ bv, T* __restrict__ q,
-                             T* __restrict__ k, T* __restrict__ v) {
-  const int row = blockIdx.x;
-  const int br = row % (m.batch * m.R_cap);  // (b, r): the table is shared by both variants
-  const int half = hd / 2;
-  const int ntot = (nq + 2 * nkv) * hd;
-  const float* t = tmp + (size_t)row * ntot;
-  const float* cs = cos_sin + (size_t)br * hd;
-  // rotated heads: q then k; one thread per (head, i < half)
-  for (int idx = threadIdx.x; idx < (nq + nkv) * half; idx += blockDim.x) {
-    const int h = idx / half, i = idx % half;
-    float x1 = t[h * hd + i], x2 = t[h * hd + half + i];
-    if (bq != nullptr) {   // projection bias, before the rotation
-      const T* bb = h < nq ? bq + h * hd : bk + (h - nq) * hd;
-      x1 += to_f<T>(bb[i]); x2 += to_f<T>(bb[half + i]);
-    }
-    const float c = cs[i], sn = cs[half + i];
-    const float y1 = x1 * c - x2 * sn, y2 = x2 * c + x1 * sn;
-    if (h < nq) {
-      q[(size_t)row * nq * hd + h * hd + i] = from_f<T>(y1);
-      q[(size_t)row * nq * hd + h * hd + half + i] = from_f<T>(y2);
-    } else {
-      const int hk = h - nq;
-      k[(size_t)row * nkv * hd + hk * hd + i] = from_f<T>(y1);
-      k[(size_t)row * nkv * hd + hk * hd + half + i] = from_f<T>(y2);
-    }
+__global__ void k_rope_store(const float* __restrict__ tmp, const SimtGemm<T> g) {
+  const int m = blockIdx.x, half = g.hd / 2, heads = g.nq + 2 * g.nkv;
+  const float* t = tmp + (size_t)m * heads * g.hd;
+  for (int idx = threadIdx.x; idx < heads * half; idx += blockDim.x) {
+    const int head = idx / half, e = idx % half;
+    simt_store_qkv<T>(g, m, head, e, t[head * g.hd + e], t[head * g.hd + half + e]);
   }
-  for (int idx = threadIdx.x; idx < nkv * hd; idx += blockDim.x)
-    v[(size_t)row * nkv * hd + idx] = from_f<T>(t[(nq + nkv) * hd + idx] + (bv != nullptr ? to_f<T>(bv[idx]) : 0.f));
 }
 
 template <typename T>
-void launch_rope_store(const float* tmp, const float* cos_sin, const SeqMeta& m, int nq, int nkv,
-                       int hd, const T* bq, const T* bk, const T* bv, T* q, T* k, T* v, cudaStream_t s) {
-  const int M = m.nv * m.batch * m.R_cap;
-  k_rope_store<T><<<M, 256, 0, s>>>(tmp, cos_sin, m, nq, nkv, hd, bq, bk, bv, q, k, v);
+void launch_rope_store(const float* tmp, const SimtGemm<T>& g, cudaStream_t s) {
+  k_rope_store<T><<<g.M, 256, 0, s>>>(tmp, g);
 }
 
-// ---- SwiGLU: act = silu(gate) * up; gate_up is [M, 2F] (gate columns first) ----------------------
-template <typename T>
-__global__ void k_swiglu(const float* __restrict__ gate_up, int M, int F, T* __restrict__ act) {
-  const size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= (size_t)M * F) return;
-  const size_t r = idx / F, c = idx % F;
-  const float g = gate_up[r * 2 * F + c], u = gate_up[r * 2 * F + F + c];
-  act[idx] = from_f<T>(g / (1.f + expf(-g)) * u);
-}
-
-template <typename T>
-void launch_swiglu(const float* gate_up, int M, int F, T* act, cudaStream_t s) {
-  const size_t n = (size_t)M * F;
-  k_swiglu<T><<<(unsigned)((n + 255) / 256), 256, 0, s>>>(gate_up, M, F, act);
-}
-
-// ---- bidirectional attention, one warp per query row -----------------------------------------
+// ---- bidirectional attention on CUDA cores ------------------------------------------------------
 // Keys of query (v, b, r): the ctx_len[b] cached rows, then the last_len[b] + win_len[b] active
 // rows of the same variant.  No causal mask.
+//
+// A CTA takes 16 query rows of one head (two per warp) and streams tiles of `kt` keys through
+// shared memory with a running softmax: K rows and V columns are staged with padded pitches, so that
+// a lane scores one key and accumulates one output feature with conflict-free 16-byte reads.  The
+// work is tiny (a few MFMAs per head); what it took the time on was serial: one warp per row read
+// every K row element by element from global memory (112 keys, head_dim 64: 44 -> 14 us).
+constexpr int kAttnSimtRows = 16;
 template <typename T>
-__global__ void __launch_bounds__(128) k_attn_simt(
+__global__ void __launch_bounds__(256) k_attn_simt(
     const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ v,
-    const T* __restrict__ k_cache, const T* __restrict__ v_cache, int max_ctx, SeqMeta m, int nq,
-    int nkv, int hd, T* __restrict__ o, int score_stride) {
-  extern __shared__ float smem[];
+    const T* __restrict__ k_cache, const T* __restrict__ v_cache, int max_ctx, const SeqMeta m, int nq,
+    int nkv, int hd, T* __restrict__ o, int kt, int rows, int vec) {
+  extern __shared__ __align__(16) float attn_smem[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int h = blockIdx.y;
-  const int vb = blockIdx.z;
+  const int h = blockIdx.y, vb = blockIdx.z;
   const int b = vb % m.batch, vv = vb / m.batch;
   const int g = h / (nq / nkv);
   const int P = m.ctx_len[b], R = m.last_len[b] + m.win_len[b];
-  const int nkeys = P + R;
-  float* sc = smem + (size_t)warp * score_stride;  // scores of this warp's row
-  float* qs = sc + (score_stride - hd);            // the query row, tail of the warp's slice
+  const int r0 = blockIdx.x * rows;
+  if (r0 >= R) return;
+  const int hp = (hd + 3) / 4 * 4, kp = hp + 4, vp = kt + 4;   // padded head_dim; pitches of K and V^T rows
+  float* Ks = attn_smem;                        // [kt][kp]
+  float* Vs = Ks + (size_t)kt * kp;             // [hd][vp]
+  float* qs = Vs + (size_t)hd * vp;             // [rows][kp]
+  float* ps = qs + rows * kp;                   // [rows][vp]
+  float* os = ps + rows * vp;                   // [rows][hp]
   const float scale = rsqrtf((float)hd);
-  const T* kc = k_cache ? k_cache + ((size_t)b * nkv + g) * (size_t)max_ctx * hd : nullptr;
-  const T* vc = v_cache ? v_cache + ((size_t)b * nkv + g) * (size_t)hd * max_ctx : nullptr;
-  const int row0 = act_row(m, vv, b, 0);
-  for (int r = blockIdx.x * 4 + warp; r < R; r += gridDim.x * 4) {
-    const size_t qoff = (size_t)(row0 + r) * nq * hd + (size_t)h * hd;
-    for (int e = lane; e < hd; e += 32) qs[e] = to_f<T>(q[qoff + e]);
-    __syncwarp();
-    float mx = -INFINITY;
-    for (int j = lane; j < nkeys; j += 32) {
-      const T* kr = (j < P) ? kc + (size_t)j * hd
-                            : k + (size_t)(row0 + j - P) * nkv * hd + (size_t)g * hd;
-      float acc = 0.f;
-      for (int e = 0; e < hd; ++e) acc = fmaf(qs[e], to_f<T>(kr[e]), acc);
-      acc *= scale;
-      sc[j] = acc;
-      mx = fmaxf(mx, acc);
-    }
-    mx = warp_max(mx);
-    float sum = 0.f;
-    for (int j = lane; j < nkeys; j += 32) {
-      const float p = expf(sc[j] - mx);
-      sc[j] = p;
-      sum += p;
-    }
-    sum = warp_sum(sum);
-    __syncwarp();
-    const float inv = 1.f / sum;
-    for (int e = lane; e < hd; e += 32) {
-      float acc = 0.f;
-      if (P > 0) {
-        const T* vr = vc + (size_t)e * max_ctx;
-        for (int j = 0; j < P; ++j) acc = fmaf(sc[j], to_f<T>(vr[j]), acc);
+  const size_t kvh = (size_t)b * nkv + g;
+  const T* kc = k_cache ? k_cache + kvh * (size_t)max_ctx * hd : nullptr;
+  const T* vc = v_cache ? v_cache + kvh * (size_t)hd * max_ctx : nullptr;
+  const int row0 = act_row(m, vv, b, 0), ld = nkv * hd;
+  for (int i = threadIdx.x; i < rows * kp; i += 256) {
+    const int r = i / kp, e = i - r * kp;
+    qs[i] = (r0 + r < R && e < hd) ? to_f<T>(q[(size_t)(row0 + r0 + r) * nq * hd + (size_t)h * hd + e]) : 0.f;
+  }
+  const int ra = warp * 2;                      // this warp's rows: ra, ra + 1
+  const bool live = ra < rows && r0 + ra < R;
+  float* oa = os + ra * hp;
+  if (live)
+    for (int e = lane; e < 2 * hp; e += 32) oa[e] = 0.f;
+  float mx[2] = {-INFINITY, -INFINITY}, sum[2] = {0.f, 0.f};
+
+  const int tc = (P + kt - 1) / kt, ta = (R + kt - 1) / kt;
+  for (int t = 0; t < tc + ta; ++t) {
+    const bool ctx = t < tc;
+    const int j0 = (ctx ? t : t - tc) * kt, n = min(kt, (ctx ? P : R) - j0);
+    __syncthreads();                            // the last tile has been read
+    // K rows; rows and elements beyond the valid ones are zero
+    if (vec) {
+      const int q4 = hp / 4;
+      for (int i = threadIdx.x; i < kt * q4; i += 256) {
+        const int j = i / q4, e = (i - j * q4) * 4;
+        float x[4] = {0.f, 0.f, 0.f, 0.f};
+        if (j < n) load4<T>((ctx ? kc + (size_t)(j0 + j) * hd : k + (size_t)(row0 + j0 + j) * ld + (size_t)g * hd) + e, x);
+        *reinterpret_cast<float4*>(Ks + j * kp + e) = make_float4(x[0], x[1], x[2], x[3]);
       }
-      for (int j = 0; j < R; ++j)
-        acc = fmaf(sc[P + j], to_f<T>(v[(size_t)(row0 + j) * nkv * hd + (size_t)g * hd + e]), acc);
-      o[qoff + e] = from_f<T>(acc * inv);
+    } else {
+      for (int i = threadIdx.x; i < kt * hp; i += 256) {
+        const int j = i / hp, e = i - j * hp;
+        Ks[j * kp + e] = (j < n && e < hd) ? to_f<T>(ctx ? kc[(size_t)(j0 + j) * hd + e]
+                                                         : k[(size_t)(row0 + j0 + j) * ld + (size_t)g * hd + e]) : 0.f;
+      }
     }
+    // V with the keys contiguous; the cache may hold anything beyond ctx_len
+    if (ctx && !vec) {
+      for (int i = threadIdx.x; i < hd * kt; i += 256) {
+        const int e = i / kt, j = i - e * kt;
+        Vs[e * vp + j] = j < n ? to_f<T>(vc[(size_t)e * max_ctx + j0 + j]) : 0.f;
+      }
+    } else if (ctx) {
+      for (int i = threadIdx.x; i < hd * (kt / 4); i += 256) {
+        const int e = i / (kt / 4), j = (i - e * (kt / 4)) * 4;
+        float x[4] = {0.f, 0.f, 0.f, 0.f};
+        if (j < n) load4<T>(vc + (size_t)e * max_ctx + j0 + j, x);
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (j + u >= n) x[u] = 0.f;
+        *reinterpret_cast<float4*>(Vs + e * vp + j) = make_float4(x[0], x[1], x[2], x[3]);
+      }
+    } else {
+      const int steps = vec ? hd / 4 : hd;
+      for (int i = threadIdx.x; i < kt * steps; i += 256) {
+        const int e = i / kt, j = i - e * kt;   // lanes along the keys: conflict-free stores
+        const T* src = v + (size_t)(row0 + j0 + j) * ld + (size_t)g * hd;
+        if (vec) {
+          float x[4] = {0.f, 0.f, 0.f, 0.f};
+          if (j < n) load4<T>(src + e * 4, x);
+#pragma unroll
+          for (int u = 0; u < 4; ++u) Vs[(e * 4 + u) * vp + j] = x[u];
+        } else {
+          Vs[e * vp + j] = j < n ? to_f<T>(src[e]) : 0.f;
+        }
+      }
+    }
+    __syncthreads();
+    if (!live) continue;
+    // scores of the warp's two rows: one key per lane and step
+    const float *q0 = qs + ra * kp, *q1 = q0 + kp;
+    float *p0 = ps + ra * vp, *p1 = p0 + vp;
+    float tm0 = -INFINITY, tm1 = -INFINITY;
+    for (int j = lane; j < kt; j += 32) {
+      float s0 = -INFINITY, s1 = -INFINITY;
+      if (j < n) {
+        float a0 = 0.f, a1 = 0.f, b0 = 0.f, b1 = 0.f;
+        const float* kr = Ks + j * kp;
+        for (int e = 0; e < hp; e += 4) {
+          const float4 kv = *reinterpret_cast<const float4*>(kr + e);
+          const float4 x = *reinterpret_cast<const float4*>(q0 + e), y = *reinterpret_cast<const float4*>(q1 + e);
+          a0 = fmaf(x.x, kv.x, a0); b0 = fmaf(x.y, kv.y, b0); a0 = fmaf(x.z, kv.z, a0); b0 = fmaf(x.w, kv.w, b0);
+          a1 = fmaf(y.x, kv.x, a1); b1 = fmaf(y.y, kv.y, b1); a1 = fmaf(y.z, kv.z, a1); b1 = fmaf(y.w, kv.w, b1);
+        }
+        s0 = (a0 + b0) * scale; s1 = (a1 + b1) * scale;
+      }
+      p0[j] = s0; p1[j] = s1;
+      tm0 = fmaxf(tm0, s0); tm1 = fmaxf(tm1, s1);
+    }
+    const float n0 = fmaxf(mx[0], warp_max(tm0)), n1 = fmaxf(mx[1], warp_max(tm1));
+    const float c0 = expf(mx[0] - n0), c1 = expf(mx[1] - n1);   // 0 on the first tile
+    float t0 = 0.f, t1 = 0.f;
+    for (int j = lane; j < kt; j += 32) {
+      const float e0 = expf(p0[j] - n0), e1 = expf(p1[j] - n1);
+      p0[j] = e0; p1[j] = e1;
+      t0 += e0; t1 += e1;
+    }
+    sum[0] = sum[0] * c0 + warp_sum(t0); sum[1] = sum[1] * c1 + warp_sum(t1);
+    mx[0] = n0; mx[1] = n1;
     __syncwarp();
+    for (int e = lane; e < hd; e += 32) {
+      const float* vr = Vs + e * vp;
+      float x0 = 0.f, x1 = 0.f, y0 = 0.f, y1 = 0.f;
+      for (int j = 0; j < kt; j += 4) {
+        const float4 w = *reinterpret_cast<const float4*>(vr + j);
+        const float4 x = *reinterpret_cast<const float4*>(p0 + j), y = *reinterpret_cast<const float4*>(p1 + j);
+        x0 = fmaf(x.x, w.x, x0); x1 = fmaf(x.y, w.y, x1); x0 = fmaf(x.z, w.z, x0); x1 = fmaf(x.w, w.w, x1);
+        y0 = fmaf(y.x, w.x, y0); y1 = fmaf(y.y, w.y, y1); y0 = fmaf(y.z, w.z, y0); y1 = fmaf(y.w, w.w, y1);
+      }
+      oa[e] = oa[e] * c0 + (x0 + x1);
+      oa[hp + e] = oa[hp + e] * c1 + (y0 + y1);
+    }
+  }
+  for (int i = 0; i < 2; ++i) {
+    if (!live || r0 + ra + i >= R) break;
+    const float inv = 1.f / sum[i];
+    T* dst = o + (size_t)(row0 + r0 + ra + i) * nq * hd + (size_t)h * hd;
+    for (int e = lane; e < hd; e += 32) dst[e] = from_f<T>(oa[i * hp + e] * inv);
+  }
+}
+
+// keys per tile, query rows per CTA (two per warp) and shared memory: as many as fit
+struct AttnSimtShape { int kt, rows; size_t smem; };
+static AttnSimtShape attn_simt_shape(int hd) {
+  const size_t hp = (hd + 3) / 4 * 4;
+  AttnSimtShape a{64, kAttnSimtRows, 0};
+  while (true) {
+    a.smem = sizeof(float) * (a.kt * (hp + 4) + (size_t)hd * (a.kt + 4) + a.rows * ((hp + 4) + (a.kt + 4) + hp));
+    if (a.smem <= kSimtSmemMax || (a.kt == 4 && a.rows == 2)) return a;
+    if (a.kt > 8 || a.rows == 2) a.kt >>= 1; else a.rows >>= 1;
   }
 }
 
@@ -444,25 +688,38 @@ template <typename T>
 void launch_attn_simt(const T* q, const T* k, const T* v, const T* k_cache, const T* v_cache,
                       int max_ctx, const SeqMeta& m, int nq, int nkv, int hd, T* o,
                       cudaStream_t s) {
-  int max_keys = 0;
-  for (int b = 0; b < m.batch; ++b)
-    max_keys = max(max_keys, m.ctx_len[b] + m.last_len[b] + m.win_len[b]);
-  const int score_stride = ((max_keys + 31) / 32) * 32 + hd;
-  const size_t smem = (size_t)4 * score_stride * sizeof(float);
-  static size_t configured = 0;
-  if (smem > 48 * 1024 && smem > configured) {
-    cudaFuncSetAttribute(k_attn_simt<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    configured = smem;
-  }
-  dim3 grid((m.R_cap + 3) / 4, nq, m.nv * m.batch);
-  k_attn_simt<T><<<grid, 128, smem, s>>>(q, k, v, k_cache, v_cache, max_ctx, m, nq, nkv, hd, o,
-                                          score_stride);
+  const AttnSimtShape a = attn_simt_shape(hd);
+  auto aligned = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
+  const int vec = hd % 4 == 0 && aligned(k_cache) && aligned(v_cache);
+  dim3 grid((m.R_cap + a.rows - 1) / a.rows, nq, m.nv * m.batch);
+  k_attn_simt<T><<<grid, 256, a.smem, s>>>(q, k, v, k_cache, v_cache, max_ctx, m, nq, nkv, hd, o, a.kt, a.rows, vec);
+}
+
+// Opts the kernels of this file in to the shared memory they may ask for, on the current device;
+// false when head_dim is too large for the attention kernel's buffers.
+template <typename T>
+static bool simt_init_t() {
+  auto opt = [](auto* f) { return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSimtSmemMax) == cudaSuccess; };
+  auto gemm = [&](auto epi) {
+    constexpr int E = decltype(epi)::value;
+    return opt(k_gemm_simt<T, 1, 1, 8, 128, 3, E>) && opt(k_gemm_simt<T, 4, 2, 1, 32, 3, E>);
+  };
+  return opt(k_attn_simt<T>) && opt(k_lm_rows<T>) && gemm(std::integral_constant<int, EPI_STORE_F32>{}) &&
+         gemm(std::integral_constant<int, EPI_ADD_F32>{}) && gemm(std::integral_constant<int, EPI_SWIGLU>{}) &&
+         gemm(std::integral_constant<int, EPI_QKV>{});
+}
+bool simt_init(bool bf16, int head_dim) {
+  const bool ok = (bf16 ? simt_init_t<__nv_bfloat16>() : simt_init_t<float>()) &&
+                  attn_simt_shape(head_dim).smem <= kSimtSmemMax;
+  cudaGetLastError();
+  return ok;
 }
 
 // ---- per-position signals from full logits (CUDA-core LM head only) ------------------------------
 // One block per window position.  c = max_v p(v), yhat = argmax (lowest id on ties),
 // H = lse - sum p z, I = sum p [(z - lse) - (z' - lse')] clamped at 0 (Eq. 3).
-__global__ void __launch_bounds__(256) k_signals(const float* __restrict__ logits, int V,
+constexpr int kSigThreads = 512;
+__global__ void __launch_bounds__(kSigThreads) k_signals(const float* __restrict__ logits, int V,
                                                  int mask_id, int forbid, SeqMeta m,
                                                  int32_t* __restrict__ ws_pred,
                                                  float* __restrict__ ws_conf,
@@ -471,8 +728,8 @@ __global__ void __launch_bounds__(256) k_signals(const float* __restrict__ logit
                                                  float* __restrict__ ws_lse, SignalOut out,
                                                  int32_t* __restrict__ status) {
   __shared__ float red[32];
-  __shared__ float s_m[8], s_m2[8];
-  __shared__ int s_i[8];
+  __shared__ float s_m[kSigThreads / 32], s_m2[kSigThreads / 32];
+  __shared__ int s_i[kSigThreads / 32];
   const int p = blockIdx.x;
   const int b = p / m.W_cap, k = p % m.W_cap;
   if (b >= m.batch || k >= m.win_len[b]) return;
@@ -482,12 +739,23 @@ __global__ void __launch_bounds__(256) k_signals(const float* __restrict__ logit
   const int skip = forbid ? mask_id : -1;
   float mx = -INFINITY, mx2 = -INFINITY;
   int am = 0x7fffffff;
-  for (int v = threadIdx.x; v < V; v += blockDim.x) {
-    if (v == skip) continue;
-    const float a = z[v];
+  // four logits at a time where the rows are 16-byte aligned
+  auto each = [&](auto&& f) {
+    if (V % 4 == 0) {
+      for (int v = threadIdx.x * 4; v < V; v += kSigThreads * 4) {
+        const float4 a = *reinterpret_cast<const float4*>(z + v);
+        const float4 p4 = prev ? *reinterpret_cast<const float4*>(z2 + v) : make_float4(0.f, 0.f, 0.f, 0.f);
+        f(v, a.x, p4.x); f(v + 1, a.y, p4.y); f(v + 2, a.z, p4.z); f(v + 3, a.w, p4.w);
+      }
+    } else {
+      for (int v = threadIdx.x; v < V; v += kSigThreads) f(v, z[v], prev ? z2[v] : 0.f);
+    }
+  };
+  each([&](int v, float a, float a2) {
+    if (v == skip) return;
     if (a > mx) { mx = a; am = v; }  // strided ascending: the first maximum kept per thread
-    if (prev) mx2 = fmaxf(mx2, z2[v]);
-  }
+    if (prev) mx2 = fmaxf(mx2, a2);
+  });
   // reduce (max, lowest index) across the block
   for (int o = 16; o > 0; o >>= 1) {
     const float om = __shfl_xor_sync(0xffffffffu, mx, o);
@@ -499,22 +767,21 @@ __global__ void __launch_bounds__(256) k_signals(const float* __restrict__ logit
   if (l == 0) { s_m[w] = mx; s_i[w] = am; s_m2[w] = mx2; }
   __syncthreads();
   mx = s_m[0]; am = s_i[0]; mx2 = s_m2[0];
-  for (int i = 1; i < 8; ++i) {
+  for (int i = 1; i < kSigThreads / 32; ++i) {
     if (s_m[i] > mx || (s_m[i] == mx && s_i[i] < am)) { mx = s_m[i]; am = s_i[i]; }
     mx2 = fmaxf(mx2, s_m2[i]);
   }
   float S = 0.f, Az = 0.f, Ad = 0.f, S2 = 0.f;
-  for (int v = threadIdx.x; v < V; v += blockDim.x) {
-    if (v == skip) continue;
-    const float a = z[v];
+  each([&](int v, float a, float a2) {
+    if (v == skip) return;
     const float e = expf(a - mx);
     S += e;
     if (e > 0.f) {
       Az = fmaf(e, a, Az);
-      if (prev) Ad = fmaf(e, a - z2[v], Ad);
+      if (prev) Ad = fmaf(e, a - a2, Ad);
     }
-    if (prev) S2 += expf(z2[v] - mx2);
-  }
+    if (prev) S2 += expf(a2 - mx2);
+  });
   S = block_sum(S, red);
   Az = block_sum(Az, red);
   Ad = block_sum(Ad, red);
@@ -549,7 +816,7 @@ void launch_signals_from_logits(const float* logits, int V, int mask_id, int for
                                 const SeqMeta& m, int32_t* ws_pred, float* ws_conf,
                                 float* ws_ent, float* ws_infl, float* ws_lse, SignalOut out,
                                 int32_t* status, cudaStream_t s) {
-  k_signals<<<m.batch * m.W_cap, 256, 0, s>>>(logits, V, mask_id, forbid, m, ws_pred, ws_conf,
+  k_signals<<<m.batch * m.W_cap, kSigThreads, 0, s>>>(logits, V, mask_id, forbid, m, ws_pred, ws_conf,
                                               ws_ent, ws_infl, ws_lse, out, status);
 }
 
@@ -645,8 +912,6 @@ void launch_export_kv(const T* k, const T* v, int v_ld, const SeqMeta& m, int nk
   dim3 grid(maxl, m.batch);
   k_export_kv<T><<<grid, 256, 0, s>>>(k, v, v_ld, m, nkv, hd, max_ctx, k_cache, v_cache);
 }
-template void launch_export_kv<float>(const float*, const float*, int, const SeqMeta&, int, int, int,
-                                      float*, float*, cudaStream_t);
 template void launch_export_kv<__nv_bfloat16>(const __nv_bfloat16*, const __nv_bfloat16*, int,
                                               const SeqMeta&, int, int, int, __nv_bfloat16*,
                                               __nv_bfloat16*, cudaStream_t);
@@ -657,14 +922,10 @@ template void launch_export_kv<__nv_bfloat16>(const __nv_bfloat16*, const __nv_b
                                 int, const SeqMeta&, float*, int32_t*, cudaStream_t);           \
   template void launch_rmsnorm<T>(float*, const float*, int, size_t, const T*, float, int, int, \
                                   T*, cudaStream_t);                                            \
-  template void launch_final_norm<T>(float*, const float*, int, size_t, const T*, float, int,   \
-                                     const SeqMeta&, T*, cudaStream_t, int);                         \
-  template void launch_h_override<T>(const T*, int, int, const SeqMeta&, T*, cudaStream_t);     \
-  template void launch_gemm_simt<T>(const T*, const T*, float*, int, int, int, int, int,        \
-                                    cudaStream_t);                                              \
-  template void launch_rope_store<T>(const float*, const float*, const SeqMeta&, int, int, int, \
-                                     const T*, const T*, const T*, T*, T*, T*, cudaStream_t);                                 \
-  template void launch_swiglu<T>(const float*, int, int, T*, cudaStream_t);                     \
+  template void launch_lm_rows<T>(const float*, const float*, int, size_t, const T*, float, int,  \
+                                  const SeqMeta&, int, const LmRowsIo<T>&, T*, cudaStream_t);    \
+  template void launch_gemm_simt<T>(const SimtGemm<T>&, int, cudaStream_t);                     \
+  template void launch_rope_store<T>(const float*, const SimtGemm<T>&, cudaStream_t);           \
   template void launch_attn_simt<T>(const T*, const T*, const T*, const T*, const T*, int,      \
                                     const SeqMeta&, int, int, int, T*, cudaStream_t);           \
   template void launch_xlogp<T>(const T*, const T*, const int32_t*, const float*, int, int,     \

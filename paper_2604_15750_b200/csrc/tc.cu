@@ -442,9 +442,9 @@ bool tc_chain_ok(const TcState* t, const SeqMeta& m) {
          units_d <= t->chain_grid && norm_bytes <= (size_t)kChainRing;
 }
 
-void tc_step_begin(TcState* t) {
+void tc_step_begin(TcState* t, unsigned int** words, int* n_words) {
   // a step that gave up inside a grid barrier leaves the arrival count behind
-  cudaMemsetAsync(t->grid_bar, 0, (2 + kFlagWords) * sizeof(unsigned int), t->s);
+  *words = t->grid_bar; *n_words = 2 + kFlagWords;
   t->bar_count = 0;
   t->qkv_launches = 0;
 }

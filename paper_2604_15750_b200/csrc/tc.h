@@ -58,8 +58,8 @@ int tc_set_wait_limit_us(TcState* t, long long us);
 void tc_set_stall_lmhead(TcState* t, bool on);
 // true if the persistent dense chain takes this step (all activation rows in one column block)
 bool tc_chain_ok(const TcState* t, const SeqMeta& m);
-// resets the chain's grid barrier; call once at the start of a step
-void tc_step_begin(TcState* t);
+// once at the start of a step: the words of the chain's grid barrier that must be cleared before it
+void tc_step_begin(TcState* t, unsigned int** words, int* n_words);
 // Phases [phase_begin, phase_end) of the dense chain (CH_* in tc_chain.cuh): O projection,
 // residual + norm2 (gain g2), gate/up, down projection of `layer`; residual + norm1 (gain g1,
 // folding fold_norm1 partial sums) and the rotated QKV of `qkv_layer`.  The partial sums of the
