@@ -4,6 +4,7 @@
 // of the tensor-core path.
 #include <math.h>
 
+#include <atomic>
 #include <type_traits>
 
 #include "kernels.h"
@@ -709,10 +710,19 @@ static bool simt_init_t() {
          gemm(std::integral_constant<int, EPI_QKV>{});
 }
 bool simt_init(bool bf16, int head_dim) {
-  const bool ok = (bf16 ? simt_init_t<__nv_bfloat16>() : simt_init_t<float>()) &&
-                  attn_simt_shape(head_dim).smem <= kSimtSmemMax;
-  cudaGetLastError();
-  return ok;
+  // the attributes belong to the functions on a device, not to a context: setting them costs 2 ms,
+  // so it is done by the first context of a type on a device (again by a racing one: same values)
+  static std::atomic<unsigned long long> done[2];
+  int dev = 0;
+  cudaGetDevice(&dev);
+  const unsigned long long bit = dev < 64 ? 1ull << dev : 0ull;
+  bool ok = (done[bf16].load(std::memory_order_acquire) & bit) != 0;
+  if (!ok) {
+    ok = bf16 ? simt_init_t<__nv_bfloat16>() : simt_init_t<float>();
+    if (ok) done[bf16].fetch_or(bit, std::memory_order_release);
+    cudaGetLastError();
+  }
+  return ok && attn_simt_shape(head_dim).smem <= kSimtSmemMax;
 }
 
 // ---- per-position signals from full logits (CUDA-core LM head only) ------------------------------

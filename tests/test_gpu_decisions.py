@@ -165,3 +165,44 @@ def test_batched_decisions_8192_sequences_bit_exact_on_a_sample():
         picked += cnt
     assert picked > 96
     eng.close()
+
+
+@pytest.mark.parametrize("W,B,cap_mode", [(16, 3, 1), (64, 700, 0), (80, 593, 1), (256, 601, 0), (256, 2, 1)])
+def test_decisions_one_warp_per_sequence_bit_exact(W, B, cap_mode):
+    """Two, four and eight positions per lane; one sequence per CTA (up to 592) and eight."""
+    hp = Hyper(cap_mode=cap_mode, L_max=256, smooth_radius=2)
+    eng = _engine(hp, max_batch=1, max_window=W)
+    r = np.random.default_rng(W + B)
+    mask_id = WL.mask_id
+    win = r.integers(1, W + 1, B).astype(np.int32)
+    win[:2] = W
+    remain = r.integers(1, 300, B).astype(np.int32)
+    I = (np.abs(r.standard_normal((B, W))) * np.exp(-np.arange(W) / 16.0)).astype(np.float32)
+    H = (r.random((B, W)) * 8).astype(np.float32)
+    blk = np.array([r.integers(0, w + 1) for w in win]).astype(np.int32)
+    conf = np.where(r.random((B, W)) < 0.5, 0.9 + 0.1 * r.random((B, W)), r.random((B, W))).astype(np.float32)
+    x = (r.standard_normal((B, W, W)) * 6 - 12).astype(np.float32)
+    ids = np.where(r.random((B, W)) < 0.8, mask_id, 5).astype(np.int32)
+    dev = eng.device
+    t = lambda a: torch.from_numpy(a).to(dev)
+    f = lambda: torch.zeros((B, W), device=dev)
+    bo = dict(score=f(), cum_influence=f(), cum_score=f(), block_len=torch.zeros((B,), dtype=torch.int32, device=dev))
+    so = dict(sel_mask=torch.zeros((B, W), dtype=torch.uint8, device=dev),
+              sel_idx=torch.zeros((B, W), dtype=torch.int32, device=dev),
+              sel_count=torch.zeros((B,), dtype=torch.int32, device=dev))
+    eng.boundary_batched(t(I), t(H), t(win), t(remain), bo)
+    eng.select_batched(t(conf), t(ids), t(x), t(blk), t(win), so)
+    eng.synchronize()
+    g = {k: v.cpu().numpy() for k, v in {**bo, **so}.items()}
+    for b in sorted({0, 1, B - 1} | set(r.integers(0, B, 20).tolist())):
+        L, score, ci, cs = O.boundary(I[b], H[b], int(win[b]), int(remain[b]), True, _ocfg(hp))
+        n = len(score)
+        assert int(g["block_len"][b]) == L, b
+        for name, want in (("score", score), ("cum_influence", ci), ("cum_score", cs)):
+            assert np.array_equal(g[name][b, :n].view(np.uint32), want.view(np.uint32)), (b, name)
+        w = int(win[b])
+        want = O.cap_select(conf[b, :w], ids[b, :w] == mask_id, x[b, :w, :w], int(blk[b]), hp.tau_low, hp.tau_high,
+                            hp.gamma, cap_mode)
+        assert list(g["sel_idx"][b, :int(g["sel_count"][b])]) == want, b
+        assert [i for i in range(w) if g["sel_mask"][b, i]] == want, b
+    eng.close()
