@@ -227,14 +227,13 @@ int run_step(dc_ctx* c, const dc_step_in* in, const dc_step_out* out, const SeqM
     pf.end();
     if (rc != DC_OK) return fail(c, rc, "dense chain failed: %s", tc_error(c->tc));
     for (int l = 0; l < L; ++l) {
-      if (export_kv) tc_export_kv(c->tc, l, m, (__nv_bfloat16*)in->k_cache, (__nv_bfloat16*)in->v_cache);
-      if (kv_only && l + 1 == L) break;   // prefill: nothing after the last layer's K / V is used
+      const bool last = l + 1 == L;
       pf.begin(DC_STAGE_ATTN, 1);
       rc = tc_attention(c->tc, l, m, (const __nv_bfloat16*)in->k_cache,
-                        (const __nv_bfloat16*)in->v_cache);
+                        (const __nv_bfloat16*)in->v_cache, export_kv, kv_only && last);
       pf.end();
       if (rc != DC_OK) return fail(c, rc, "attention failed: %s", tc_error(c->tc));
-      const bool last = l + 1 == L;
+      if (kv_only && last) break;   // prefill: nothing after the last layer's K / V is used
       pf.begin(DC_STAGE_DENSE, 1);
       rc = tc_chain(c->tc, l, l + 1, CH_OPROJ, last ? CH_NORM1 : CH_END, m, c->x,
                     (const __nv_bfloat16*)a, c->cos_sin, (const __nv_bfloat16*)c->norm2[l],

@@ -128,12 +128,6 @@ template <typename T>
 void launch_xlogp(const T* h, const T* lm_head, const int32_t* ws_pred, const float* ws_lse,
                   int d, int V, const SeqMeta& m, int max_window, float* xlogp, cudaStream_t s);
 
-// appends the curr variant's K / V of the last-block rows to one layer's context cache
-// (k_cache / v_cache: that layer's slice); v_ld != 0: v is transposed with that row pitch
-template <typename T>
-void launch_export_kv(const T* k, const T* v, int v_ld, const SeqMeta& m, int nkv, int hd,
-                      int max_ctx, T* k_cache, T* v_cache, cudaStream_t s);
-
 // ---- decision kernels --------------------------------------------------------------------------
 // per-sequence lengths in device memory (all null: the lengths inside SeqMeta are used)
 struct DevLens {

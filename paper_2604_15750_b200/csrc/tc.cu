@@ -374,7 +374,7 @@ static int pick_split_rounds(const TcState* t, int tiles, int M, int BN, int N, 
 }
 
 int tc_attention(TcState* t, int layer, const SeqMeta& m, const __nv_bfloat16* k_cache,
-                 const __nv_bfloat16* v_cache) {
+                 const __nv_bfloat16* v_cache, bool export_kv, bool export_only) {
   const dc_config& g = t->g;
   const int nq = g.n_q_heads, nkv = g.n_kv_heads, hd = g.head_dim;
   bool any_ctx = false;
@@ -390,22 +390,28 @@ int tc_attention(TcState* t, int layer, const SeqMeta& m, const __nv_bfloat16* k
   ap.m = m; ap.nq = nq; ap.nkv = nkv; ap.max_ctx = g.max_ctx; ap.layer = layer;
   ap.scale_log2 = 1.4426950408889634f / sqrtf((float)hd);
   ap.o = t->o; ap.status = t->status;
+  ap.k = t->k; ap.v = t->v; ap.ldv = t->ldv; ap.k_cache = ap.v_cache = nullptr;
+  int export_tiles = 0;   // tiles of 128 last-block rows to append to the caches
+  if (export_kv) {
+    const size_t per_layer = (size_t)g.max_batch * nkv * g.max_ctx * hd;
+    ap.k_cache = const_cast<__nv_bfloat16*>(k_cache) + (size_t)layer * per_layer;
+    ap.v_cache = const_cast<__nv_bfloat16*>(v_cache) + (size_t)layer * per_layer;
+    for (int b = 0; b < m.batch; ++b) {
+      const int n = (m.last_len[b] + kBK - 1) / kBK;
+      export_tiles = n > export_tiles ? n : export_tiles;
+    }
+  }
   const int nqt = (m.R_cap + 127) / 128;
   // one CTA per query tile: (row tile, variant) with two variants in the pass (a row tile with 64
   // rows or fewer packs both variants into the curr CTA, the prev CTA returns at once)
-  dim3 grid(m.nv == 2 ? 2 * nqt : nqt, nq, m.batch);
+  ap.units = export_only ? 0 : m.nv == 2 ? 2 * nqt : nqt;
+  if (ap.units + export_tiles == 0) return DC_OK;
+  dim3 grid(ap.units + export_tiles, nq, m.batch);
   k_attn_tc<<<grid, kAttnThreads, kAttnSmem, t->s>>>(t->map_q, t->map_k, t->map_vt, t->map_kc,
                                                      t->map_vc, ap);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return tfail(t, DC_ERR_CUDA, "attention launch failed: %s", cudaGetErrorString(e));
   return DC_OK;
-}
-
-void tc_export_kv(TcState* t, int layer, const SeqMeta& m, __nv_bfloat16* k_cache, __nv_bfloat16* v_cache) {
-  const dc_config& g = t->g;
-  const size_t per_layer = (size_t)g.max_batch * g.n_kv_heads * g.max_ctx * g.head_dim;
-  launch_export_kv<__nv_bfloat16>(t->k, t->v, t->ldv, m, g.n_kv_heads, g.head_dim, g.max_ctx,
-                                  k_cache + (size_t)layer * per_layer, v_cache + (size_t)layer * per_layer, t->s);
 }
 
 void tc_set_qkv_bias(TcState* t, const std::vector<const void*>& bq, const std::vector<const void*>& bk,
@@ -560,13 +566,10 @@ int tc_layer(TcState* t, int layer, const SeqMeta& m, float* x, const __nv_bfloa
   hook.end();
   if (rc != DC_OK) return rc;
 
-  if (export_kv)
-    tc_export_kv(t, layer, m, const_cast<__nv_bfloat16*>(k_cache), const_cast<__nv_bfloat16*>(v_cache));
-  if (kv_only) return DC_OK;   // prefill, last layer: only its K / V were wanted
   hook.begin(DC_STAGE_ATTN, 1);
-  rc = tc_attention(t, layer, m, k_cache, v_cache);
+  rc = tc_attention(t, layer, m, k_cache, v_cache, export_kv, kv_only);
   hook.end();
-  if (rc != DC_OK) return rc;
+  if (rc != DC_OK || kv_only) return rc;   // prefill, last layer: only its K / V were wanted
 
   hook.begin(DC_STAGE_OPROJ, 1);
   p.N = d; p.K = nq * hd; p.nsplit = pick_split_rounds(t, d / kTileN, M, BN, p.N, p.K, t->max_split);

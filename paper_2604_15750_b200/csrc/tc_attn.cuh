@@ -47,6 +47,11 @@ struct AttnParams {
   float scale_log2;        // log2(e) / sqrt(head_dim)
   __nv_bfloat16* o;        // [M, nq * 128]
   int32_t* status;
+  // CTAs blockIdx.x >= units append the last block's K / V to the context cache instead
+  int units;
+  const __nv_bfloat16 *k, *v;        // active K [M, nkv * 128], V transposed [nkv * 128, ldv]
+  int ldv;
+  __nv_bfloat16 *k_cache, *v_cache;  // this layer's caches
 };
 
 constexpr int kAttnThreads = 512;
@@ -123,6 +128,59 @@ __device__ __forceinline__ AttnTile attn_tile(const AttnUnit& a, int j) {
 }
 
 
+// Appends rows r0 .. r0 + 127 of the last decoded block (curr variant) of one sequence and kv head to
+// the context cache, behind its ctx_len keys.  Attention reads keys below ctx_len only (what a tile
+// holds beyond them is masked), so these CTAs run beside the attention CTAs of the same launch, on
+// SMs that a small batch leaves idle.  As a kernel of its own, with a row per CTA and element-wise
+// stores of V at a stride of max_ctx, this took 11 us of each layer of a one-sequence step and 59 us
+// of a 1024-token prefill, plus a launch.
+__device__ __forceinline__ void attn_export_tile(const AttnParams& p, int b, int g, int r0) {
+  const int n = min(kBK, p.m.last_len[b] - r0);
+  const int row = act_row(p.m, 0, b, r0), key = p.m.ctx_len[b] + r0;
+  const size_t kv = (size_t)b * p.nkv + g;
+  const __nv_bfloat16* ks = p.k + (size_t)row * p.nkv * kHd + g * kHd;
+  __nv_bfloat16* kd = p.k_cache + (kv * p.max_ctx + key) * kHd;
+#pragma unroll 4
+  for (int i = threadIdx.x; i < n * (kHd / 8); i += kAttnThreads) {
+    const int r = i / (kHd / 8), c = i % (kHd / 8) * 8;
+    *reinterpret_cast<uint4*>(kd + (size_t)r * kHd + c) =
+        *reinterpret_cast<const uint4*>(ks + (size_t)r * p.nkv * kHd + c);
+  }
+  // V: keys are contiguous on both sides, but the cache position has any alignment: eight keys at a
+  // time where it allows that (a prefill from position 0), else pairs of keys, aligned in the cache
+  if ((key & 7) == 0 && (n & 7) == 0) {
+    const __nv_bfloat16* vs = p.v + (size_t)g * kHd * p.ldv + row;
+    __nv_bfloat16* vd = p.v_cache + kv * kHd * p.max_ctx + key;
+#pragma unroll 4
+    for (int i = threadIdx.x; i < kHd * (kBK / 8); i += kAttnThreads) {
+      const int e = i / (kBK / 8), c = i % (kBK / 8) * 8;
+      if (c < n)
+        *reinterpret_cast<uint4*>(vd + (size_t)e * p.max_ctx + c) = *reinterpret_cast<const uint4*>(vs + (size_t)e * p.ldv + c);
+    }
+    return;
+  }
+  const int odd = key & 1, pairs = (n + odd + 1) >> 1, lane = threadIdx.x & 31;
+#pragma unroll 2
+  for (int e = threadIdx.x >> 5; e < kHd; e += kAttnThreads / 32) {
+    const __nv_bfloat16* vs = p.v + (size_t)(g * kHd + e) * p.ldv + row;
+    __nv_bfloat16* vd = p.v_cache + (kv * kHd + e) * p.max_ctx + key;
+#pragma unroll 3
+    for (int w = lane; w < pairs; w += 32) {
+      const int j = 2 * w - odd;
+      if (j >= 0 && j + 1 < n) {
+        __nv_bfloat162 two;
+        if (odd) { two.x = vs[j]; two.y = vs[j + 1]; }
+        else two = *reinterpret_cast<const __nv_bfloat162*>(vs + j);
+        *reinterpret_cast<__nv_bfloat162*>(vd + j) = two;
+      } else if (j >= 0) {
+        vd[j] = vs[j];
+      } else {
+        vd[0] = vs[0];
+      }
+    }
+  }
+}
+
 __global__ void __launch_bounds__(kAttnThreads, 1)
 k_attn_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
           const __grid_constant__ CUtensorMap map_vt, const __grid_constant__ CUtensorMap map_kc,
@@ -137,6 +195,11 @@ k_attn_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
   __shared__ float xm[3][128];     // [slot][row]: maximum raw score of the slot's tiles
 
   const int b = blockIdx.z, h = blockIdx.y;
+  if ((int)blockIdx.x >= p.units) {
+    const int r0 = ((int)blockIdx.x - p.units) * kBK;
+    if (h < p.nkv && r0 < p.m.last_len[b]) attn_export_tile(p, b, h, r0);
+    return;
+  }
   AttnUnit un;
   if (!attn_unit(p.m, b, blockIdx.x, un)) return;   // nothing of this sequence in this unit (uniform)
 
