@@ -436,7 +436,10 @@ void tc_set_cooperative(TcState* t, bool on) { t->chain_coop = on && t->coop_sup
 bool tc_chain_ok(const TcState* t, const SeqMeta& m) {
   const dc_config& g = t->g;
   const int M = m.nv * m.batch * m.R_cap;
-  // One column block of at most 256 activation rows.  The norm phases reuse the TMA ring as
+  // One column block of 16 to 256 activation rows (N of a pair MMA is any multiple of 16 there).  A
+  // LLaDA-8B denoising step over a block of up to 16 positions takes 4640 us on the per-op kernels
+  // (7 launches per layer, 2 us of gap each, no weight stream across them) and 4006 us here.  The
+  // norm phases reuse the TMA ring as
   // staging space, which needs at most one GEMM unit per CTA and phase, and both rows of a norm
   // step (x plus the split-K partial sums) inside the ring.
   const int units_qkv = g.n_q_heads + 2 * g.n_kv_heads, units_f = g.d_ff / kChainTile;
@@ -444,7 +447,7 @@ bool tc_chain_ok(const TcState* t, const SeqMeta& m) {
   const size_t norm_bytes = (size_t)2 * (1 + t->max_split) * g.d_model * sizeof(float) + g.d_model * 2;
   const bool even = g.n_q_heads % 2 == 0 && g.n_kv_heads % 2 == 0 && (g.d_model / kChainTile) % 2 == 0 &&
                     (g.d_ff / kChainTile) % 2 == 0;   // a CTA pair takes two adjacent tiles of one matrix
-  return t->chain_grid > 0 && even && M >= 32 && M <= 256 && units_qkv <= t->chain_grid && units_f <= t->chain_grid &&
+  return t->chain_grid > 0 && even && M <= 256 && units_qkv <= t->chain_grid && units_f <= t->chain_grid &&
          units_d <= t->chain_grid && norm_bytes <= (size_t)kChainRing;
 }
 

@@ -121,9 +121,10 @@ def test_fused_dense_chain_is_the_path_taken_when_the_rows_fit_one_block():
         eng.close()
 
 
-@pytest.mark.parametrize("last,win,influence,rows", [(32, 96, True, 256), (0, 16, True, 32), (0, 32, False, 32)])
+@pytest.mark.parametrize("last,win,influence,rows", [(32, 96, True, 256), (0, 16, True, 32), (0, 32, False, 32),
+                                                     (0, 7, False, 16), (0, 16, False, 16), (0, 40, False, 48)])
 def test_fused_chain_at_its_row_limits(last, win, influence, rows):
-    """The fused chain takes 32 .. 256 activation rows: both ends, against the oracle."""
+    """The fused chain takes 16 .. 256 activation rows: both ends, against the oracle."""
     wl = _wl(1, last=max(last, 1), win=win)
     lengths = dict(ctx_len=[100], last_len=[last], win_len=[win], remain_len=[128])
     case = Case(wl, lengths=lengths)
