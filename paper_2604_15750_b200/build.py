@@ -8,7 +8,7 @@ import sys
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libdepcap.so")
-SOURCES = ["depcap.cu", "kernels_simt.cu", "decisions.cu", "tc.cu"]
+SOURCES = ["depcap.cu", "kernels_simt.cu", "decisions.cu", "simt_step.cu", "tc.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "--cudart", "static", "-Xcompiler", "-fPIC", "-Xcompiler", "-fvisibility=hidden",
               "--expt-relaxed-constexpr"]

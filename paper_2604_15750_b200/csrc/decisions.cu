@@ -8,201 +8,19 @@
 
 #include <type_traits>
 
-#include "kernels.h"
+#include "decisions.cuh"
 
 namespace dc {
 
-constexpr int kMaxW = DC_MAX_WINDOW;  // 256
 constexpr int kThreads = 256;         // one thread per window position (k_commit)
-constexpr float kFxScale = 1099511627776.f;           // 2^40
-constexpr unsigned kAll = 0xffffffffu;
-
-// 2^40 fixed point.  Scaling by a power of two is exact, so one conversion rounds (to nearest) either
-// way; a sum of 2^53 or more goes through a double first, as it always did, and may round twice.
-__device__ __forceinline__ long long to_fixed(float v) { return __float2ll_rn(__fmul_rn(v, kFxScale)); }
-__device__ __forceinline__ float from_fixed(long long v) {
-  if (v > -(1ll << 53) && v < (1ll << 53)) return __fmul_rn(__ll2float_rn(v), 1.f / kFxScale);
-  return __double2float_rn(__ll2double_rn(v) * (1.0 / 1099511627776.0));
-}
-
-// Both decisions are a few hundred dependent operations per sequence, so a sequence is one warp with
-// NQ positions per lane, every reduction and scan is a shuffle, and nothing waits on a block-wide
-// barrier.  A call over many sequences is
-// then bound by its memory traffic: all 8192 sequences of a large call are resident at once and
-// their load latencies overlap (8192 x 128: k_boundary 26 -> 13 us, k_select 222 -> 39 us against
-// one block with a thread per position).  With few sequences - a step - every warp is a CTA of its
-// own, so that they spread over the SMs.
-constexpr int kSeqWarps = 8;          // sequences per CTA of a call with more sequences than kSpread
-constexpr int kSpread = 4 * 148;
-
-// NQ consecutive values of a row from position k0 on; positions >= n are 0 / not written
-template <int NQ>
-__device__ __forceinline__ void load_run(const float* __restrict__ row, int k0, int n, int vec, float (&v)[NQ]) {
-  constexpr int V = NQ >= 4 ? 4 : 2;
-#pragma unroll
-  for (int q = 0; q < NQ; q += V) {
-    if (vec && k0 + q + V <= n) {
-      if (V == 4) {
-        const float4 t = *reinterpret_cast<const float4*>(row + k0 + q);
-        v[q] = t.x; v[q + 1] = t.y; v[q + V / 2] = t.z; v[q + V - 1] = t.w;
-      } else {
-        const float2 t = *reinterpret_cast<const float2*>(row + k0 + q);
-        v[q] = t.x; v[q + 1] = t.y;
-      }
-    } else {
-#pragma unroll
-      for (int u = 0; u < V; ++u) v[q + u] = k0 + q + u < n ? row[k0 + q + u] : 0.f;
-    }
-  }
-}
-template <int NQ>
-__device__ __forceinline__ void store_run(float* __restrict__ row, int k0, int n, int vec, const float (&v)[NQ]) {
-  constexpr int V = NQ >= 4 ? 4 : 2;
-#pragma unroll
-  for (int q = 0; q < NQ; q += V) {
-    if (vec && k0 + q + V <= n) {
-      if (V == 4) *reinterpret_cast<float4*>(row + k0 + q) = make_float4(v[q], v[q + 1], v[q + V / 2], v[q + V - 1]);
-      else *reinterpret_cast<float2*>(row + k0 + q) = make_float2(v[q], v[q + 1]);
-    } else {
-#pragma unroll
-      for (int u = 0; u < V; ++u)
-        if (k0 + q + u < n) row[k0 + q + u] = v[q + u];
-    }
-  }
-}
-__device__ __forceinline__ float warp_max(float v) {   // exact, order-free
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(kAll, v, o));
-  return v;
-}
-// inclusive prefix sum over the lanes
-__device__ __forceinline__ long long warp_scan(long long v) {
-  const int lane = threadIdx.x & 31;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const long long t = __shfl_up_sync(kAll, v, o);
-    if (lane >= o) v += t;
-  }
-  return v;
-}
-
-__device__ __forceinline__ float normalise(float x, float hi, float lo, int mode) {
-  if (mode == DC_NORM_NONE) return x;
-  if (mode == DC_NORM_MAX) return __fdiv_rn(x, fmaxf(hi, 1e-8f));
-  return __fdiv_rn(__fsub_rn(x, lo), fmaxf(__fsub_rn(hi, lo), 1e-8f));
-}
-
-// Lengths of the sequences of a call: by value inside SeqMeta (a step: at most DC_MAX_BATCH
-// sequences), or - when the pointers are set - arrays in device memory, for calls over any number
-// of sequences.
-__device__ __forceinline__ int len_of(const int32_t* dev, const int* by_value, int b) {
-  return dev != nullptr ? dev[b] : by_value[b];
-}
 
 template <int NQ>
-__global__ void __launch_bounds__(32 * kSeqWarps) k_boundary(
-    const float* __restrict__ influence, const float* __restrict__ entropy, int ld, int batch,
-    const __grid_constant__ SeqMeta m, DevLens dl, Hyper hp, int max_window, float* __restrict__ score,
-    float* __restrict__ cum_i, float* __restrict__ cum_s, int32_t* __restrict__ block_len, int vec) {
+__global__ void __launch_bounds__(32 * kSeqWarps) k_boundary(const float* influence, const float* entropy, int batch,
+                                                             const __grid_constant__ SeqMeta m, DevLens dl, Hyper hp,
+                                                             BoundaryIo io) {
   __shared__ float sI[kSeqWarps][33 * NQ], sH[kSeqWarps][33 * NQ];
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int b = blockIdx.x * (blockDim.x >> 5) + w;
-  if (b >= batch) return;
-  const int Lw = max(0, min(min(hp.L_max, len_of(dl.remain, m.remain, b)), len_of(dl.win_len, m.win_len, b)));
-  const size_t o = (size_t)b * max_window;
-  if (!len_of(dl.have_prev, m.have_prev, b)) {  // cold start: the first block uses L_min
-    for (int k = lane; k < Lw; k += 32) {
-      if (score) score[o + k] = 0.f;
-      if (cum_i) cum_i[o + k] = 0.f;
-      if (cum_s) cum_s[o + k] = 0.f;
-    }
-    if (lane == 0) block_len[b] = min(hp.L_min, Lw);
-    return;
-  }
-  // lane l holds the NQ consecutive positions NQ l ..: 16-byte accesses where the rows allow it, and
-  // one scan over the lanes' totals instead of NQ scans (the kernel is bound by instruction issue)
-  const int k0 = NQ * lane;
-  float rawI[NQ], Is[NQ], Hs[NQ];
-  load_run<NQ>(influence + (size_t)b * ld, k0, Lw, vec, rawI);
-  load_run<NQ>(entropy + (size_t)b * ld, k0, Lw, vec, Hs);
-  // centred moving average over the in-range taps, added left to right
-  if (hp.smooth_radius == 1) {   // the default: the neighbours are in this lane or the next ones
-    const float lI = __shfl_up_sync(kAll, rawI[NQ - 1], 1), rI = __shfl_down_sync(kAll, rawI[0], 1);
-    const float lH = __shfl_up_sync(kAll, Hs[NQ - 1], 1), rH = __shfl_down_sync(kAll, Hs[0], 1);
-    float hPrev = lH;
-#pragma unroll
-    for (int q = 0; q < NQ; ++q) {
-      const int k = k0 + q;
-      const bool l = k > 0, r = k + 1 < Lw;
-      const float iL = q ? rawI[q ? q - 1 : 0] : lI, iR = q + 1 < NQ ? rawI[q + 1 < NQ ? q + 1 : q] : rI;
-      const float hR = q + 1 < NQ ? Hs[q + 1 < NQ ? q + 1 : q] : rH;
-      float aI = l ? __fadd_rn(iL, rawI[q]) : rawI[q], aH = l ? __fadd_rn(hPrev, Hs[q]) : Hs[q];
-      if (r) { aI = __fadd_rn(aI, iR); aH = __fadd_rn(aH, hR); }
-      hPrev = Hs[q];
-      const float n = (float)(1 + (l ? 1 : 0) + (r ? 1 : 0));
-      Is[q] = k < Lw ? __fdiv_rn(aI, n) : 0.f;
-      Hs[q] = k < Lw ? __fdiv_rn(aH, n) : 0.f;
-    }
-  } else {
-    // (one word of padding per 32: lanes read at a stride of NQ words)
-    auto at = [](int k) { return k + (k >> 5); };
-#pragma unroll
-    for (int q = 0; q < NQ; ++q) { sI[w][at(k0 + q)] = rawI[q]; sH[w][at(k0 + q)] = Hs[q]; }
-    __syncwarp();
-#pragma unroll
-    for (int q = 0; q < NQ; ++q) {
-      const int k = k0 + q;
-      Is[q] = 0.f; Hs[q] = 0.f;
-      if (k < Lw) {
-        const int lo = max(0, k - hp.smooth_radius), hi = min(Lw - 1, k + hp.smooth_radius);
-        float aI = sI[w][at(lo)], aH = sH[w][at(lo)];
-        for (int j = lo + 1; j <= hi; ++j) { aI = __fadd_rn(aI, sI[w][at(j)]); aH = __fadd_rn(aH, sH[w][at(j)]); }
-        const float n = (float)(hi - lo + 1);
-        Is[q] = __fdiv_rn(aI, n); Hs[q] = __fdiv_rn(aH, n);
-      }
-    }
-  }
-  float hiI = -INFINITY, hiH = -INFINITY, nlI = -INFINITY, nlH = -INFINITY;   // maxima, and of the negated values
-#pragma unroll
-  for (int q = 0; q < NQ; ++q)
-    if (k0 + q < Lw) {
-      hiI = fmaxf(hiI, Is[q]); hiH = fmaxf(hiH, Hs[q]);
-      nlI = fmaxf(nlI, -Is[q]); nlH = fmaxf(nlH, -Hs[q]);
-    }
-  if (hp.norm_mode != DC_NORM_NONE) {
-    hiI = warp_max(hiI); hiH = warp_max(hiH);
-    if (hp.norm_mode == DC_NORM_MINMAX) { nlI = -warp_max(nlI); nlH = -warp_max(nlH); }
-#pragma unroll
-    for (int q = 0; q < NQ; ++q) {
-      Is[q] = normalise(Is[q], hiI, nlI, hp.norm_mode);
-      Hs[q] = normalise(Hs[q], hiH, nlH, hp.norm_mode);
-    }
-  }
-  float S[NQ];
-  long long accS[NQ], accI[NQ];
-#pragma unroll
-  for (int q = 0; q < NQ; ++q) {
-    const bool in = k0 + q < Lw;
-    S[q] = in ? __fsub_rn(Is[q], __fmul_rn(hp.lambda, Hs[q])) : 0.f;
-    const long long fS = in ? to_fixed(S[q]) : 0, fI = in ? to_fixed(rawI[q]) : 0;
-    accS[q] = (q ? accS[q ? q - 1 : 0] : 0) + fS;
-    accI[q] = (q ? accI[q ? q - 1 : 0] : 0) + fI;
-  }
-  const long long baseS = warp_scan(accS[NQ - 1]) - accS[NQ - 1], baseI = warp_scan(accI[NQ - 1]) - accI[NQ - 1];
-  int first = Lw;
-  float ci[NQ], cs[NQ];
-#pragma unroll
-  for (int q = NQ - 1; q >= 0; --q) {
-    const long long tS = baseS + accS[q], tI = baseI + accI[q];
-    if (k0 + q < Lw && ((hp.boundary_mode == DC_BOUNDARY_CUMULATIVE) ? (tS < 0) : (S[q] < 0.f))) first = k0 + q;
-    ci[q] = from_fixed(tI);
-    cs[q] = from_fixed(tS);
-  }
-  const int kstar = __reduce_min_sync(kAll, first);
-  if (score) store_run<NQ>(score + o, k0, Lw, vec, S);
-  if (cum_i) store_run<NQ>(cum_i + o, k0, Lw, vec, ci);
-  if (cum_s) store_run<NQ>(cum_s + o, k0, Lw, vec, cs);
-  if (lane == 0) block_len[b] = min(max(kstar, hp.L_min), Lw);
+  const int w = threadIdx.x >> 5, b = blockIdx.x * (blockDim.x >> 5) + w;
+  if (b < batch) boundary_seq<NQ>(influence, entropy, b, m, dl, hp, io, sI[w], sH[w]);
 }
 
 // f(NQ as a constant): positions per lane for a window of max_window, warps per CTA for a batch
@@ -218,12 +36,9 @@ static void decide_launch(int batch, int max_window, F&& f) {
 static void boundary(const float* influence, const float* entropy, int ld, int batch, const SeqMeta& m,
                      const DevLens& dl, const Hyper& hp, int max_window, float* score, float* cum_i, float* cum_s,
                      int32_t* block_len, cudaStream_t s) {
-  auto aligned = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
-  const int vec = ld % 4 == 0 && max_window % 4 == 0 && aligned(influence) && aligned(entropy) && aligned(score) &&
-                  aligned(cum_i) && aligned(cum_s);
+  const BoundaryIo io = make_boundary_io(influence, entropy, ld, max_window, score, cum_i, cum_s, block_len);
   decide_launch(batch, max_window, [&](auto nq, dim3 grid, int threads) {
-    k_boundary<decltype(nq)::value><<<grid, threads, 0, s>>>(influence, entropy, ld, batch, m, dl, hp, max_window, score,
-                                                             cum_i, cum_s, block_len, vec);
+    k_boundary<decltype(nq)::value><<<grid, threads, 0, s>>>(influence, entropy, batch, m, dl, hp, io);
   });
 }
 
@@ -318,17 +133,20 @@ __device__ __forceinline__ unsigned greedy(const float* __restrict__ xb, unsigne
 
 template <int NQ>
 __global__ void __launch_bounds__(32 * kSeqWarps, 5) k_select(
-    const float* __restrict__ conf, const int32_t* __restrict__ win_ids,
+    const float* __restrict__ conf, const int32_t* win_ids,
     const float* __restrict__ xlogp, const int32_t* __restrict__ block_len, int batch,
     const __grid_constant__ SeqMeta m, DevLens dl, Hyper hp, int mask_id, int max_window,
-    uint8_t* __restrict__ sel_mask, int32_t* __restrict__ sel_idx, int32_t* __restrict__ sel_count) {
+    uint8_t* __restrict__ sel_mask, int32_t* __restrict__ sel_idx, int32_t* __restrict__ sel_count,
+    const __grid_constant__ SelectCommit cm) {
   constexpr int NA = 4;
   __shared__ __align__(16) int members[kSeqWarps][32 * NQ + NA];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int b = blockIdx.x * (blockDim.x >> 5) + w;
   if (b >= batch) return;
   const int W = len_of(dl.win_len, m.win_len, b);
-  const int L = min(max(block_len[b], 0), W);
+  const int kept = cm.win_ids != nullptr ? cm.keep.n[b] : -1;   // the length of a block that a generation is in the middle of
+  const int blk = kept >= 0 ? kept : block_len[b];
+  const int L = min(max(blk, 0), W);
   const size_t o = (size_t)b * max_window;
   const float* xb = xlogp + o * max_window;
   unsigned key[NQ];                           // M^t ∩ B^t
@@ -389,14 +207,29 @@ __global__ void __launch_bounds__(32 * kSeqWarps, 5) k_select(
     total += __popc(word);
   }
   if (lane == 0 && sel_count) sel_count[b] = total;
+  if (cm.win_ids == nullptr) return;
+  // Eq. (2) and what the host loop of a generation reads, straight into its pinned buffer
+  int left = 0;
+#pragma unroll
+  for (int q = 0; q < NQ; ++q) {
+    const int k = 32 * q + lane;
+    left += __popc(__ballot_sync(kAll, key[q] != 0u && !((sel >> q) & 1u)));
+    if (k < W) {
+      int id = win_ids[o + k];
+      if ((sel >> q) & 1u) { id = cm.pred_id[o + k]; cm.win_ids[o + k] = id; }
+      cm.host_ids[o + k] = id;
+    }
+  }
+  if (lane == 0) { cm.host_blk[b] = blk; cm.host_left[b] = left; cm.host_status[b] = cm.status[b]; }
 }
 
 static void select(const float* conf, const int32_t* win_ids, const float* xlogp, const int32_t* block_len, int batch,
                    const SeqMeta& m, const DevLens& dl, const Hyper& hp, int mask_id, int max_window,
-                   uint8_t* sel_mask, int32_t* sel_idx, int32_t* sel_count, cudaStream_t s) {
+                   uint8_t* sel_mask, int32_t* sel_idx, int32_t* sel_count, cudaStream_t s,
+                   const SelectCommit& cm = SelectCommit{}) {
   decide_launch(batch, max_window, [&](auto nq, dim3 grid, int threads) {
     k_select<decltype(nq)::value><<<grid, threads, 0, s>>>(conf, win_ids, xlogp, block_len, batch, m, dl, hp, mask_id,
-                                                           max_window, sel_mask, sel_idx, sel_count);
+                                                           max_window, sel_mask, sel_idx, sel_count, cm);
   });
 }
 
@@ -442,13 +275,9 @@ __global__ void __launch_bounds__(kThreads) k_commit(int32_t* __restrict__ win_i
   }
 }
 
-__global__ void k_keep_block_len(int32_t* block_len, const PrevLen keep, int batch) {
-  const int b = threadIdx.x;
-  if (b < batch && keep.n[b] >= 0) block_len[b] = keep.n[b];
-}
-
-void launch_keep_block_len(int32_t* block_len, const PrevLen& keep, int batch, cudaStream_t s) {
-  k_keep_block_len<<<1, DC_MAX_BATCH, 0, s>>>(block_len, keep, batch);
+void launch_select_commit(const float* conf, const float* xlogp, const int32_t* block_len, const SeqMeta& m,
+                          const Hyper& hp, int mask_id, int max_window, const SelectCommit& cm, cudaStream_t s) {
+  select(conf, cm.win_ids, xlogp, block_len, m.batch, m, DevLens{}, hp, mask_id, max_window, nullptr, nullptr, nullptr, s, cm);
 }
 
 void launch_commit(int32_t* win_ids, const int32_t* pred_id, const uint8_t* sel_mask,

@@ -11,6 +11,7 @@
 #include <vector>
 
 #include "kernels.h"
+#include "simt_step.h"
 #include "tc.h"
 
 using namespace dc;
@@ -86,12 +87,14 @@ struct dc_ctx {
   int32_t* ws_pred = nullptr;
   float *ws_conf = nullptr, *ws_ent = nullptr, *ws_infl = nullptr, *ws_lse = nullptr;
   TcState* tc = nullptr;
+  SimtFuse fuse;                    // the CUDA-core step in one launch, where the shape allows it
+  void* simt_layers = nullptr;      // device [n_layers] SimtLayer
+  unsigned int* simt_bar = nullptr; // its grid-barrier words
+  bool coop = true;                 // DC_OPT_COOPERATIVE
   // workspace of dc_generate: window / last-block ids, step and selection outputs, counters
-  int32_t *g_win = nullptr, *g_last = nullptr, *g_pred = nullptr, *g_blk = nullptr, *g_cnt = nullptr,
-          *g_idx = nullptr, *g_rem = nullptr, *g_status = nullptr;
+  int32_t *g_win = nullptr, *g_last = nullptr, *g_pred = nullptr, *g_blk = nullptr, *g_status = nullptr;
   float *g_conf = nullptr, *g_xlogp = nullptr;
   char *g_hout = nullptr, *g_carry = nullptr;   // LM-head rows of a boundary step / kept for the next one
-  uint8_t* g_mask = nullptr;
   int32_t* g_host = nullptr;   // pinned: what a generation step reads back (block_len, remaining, status, window ids)
   SeqMeta last_meta{};
   bool have_logits = false;
@@ -200,15 +203,51 @@ int run_step(dc_ctx* c, const dc_step_in* in, const dc_step_out* out, const SeqM
   T* act = (T*)c->act; T* h = (T*)c->h;
   const size_t k_layer = (size_t)g.max_batch * nkv * g.max_ctx * hd;
 
-  pf.begin(DC_STAGE_EMBED, 2);
+  pf.begin(DC_STAGE_EMBED, 1);
   unsigned int* words = nullptr;
   int n_words = 0;
   if (c->use_tc) tc_step_begin(c->tc, &words, &n_words);
-  launch_step_begin(m, hd, g.rope_theta, c->cos_sin, out->status, words, n_words, s);
-  launch_embed<T>((const T*)c->embed, in->last_ids, in->win_ids, g.max_last, g.max_window,
-                  g.mask_id, g.vocab, d, m, c->x, out->status, s);
+  else if (c->simt_bar) { words = c->simt_bar; n_words = 2; }
+  launch_step_begin<T>((const T*)c->embed, in->last_ids, in->win_ids, g.max_last, g.max_window, g.mask_id, g.vocab, d, m,
+                       c->x, out->status, hd, g.rope_theta, c->cos_sin, words, n_words, s);
   pf.end();
   DC_CHECK_LAUNCH(c);
+
+  LmRowsIo<T> io;
+  io.h_in = (const T*)in->h_final_in; io.h_out = (T*)out->h_out; io.max_window = g.max_window;
+  if (carried) {
+    io.h_prev_in = (const T*)in->h_prev_in;
+    for (int b = 0; b < m.batch; ++b) io.prev.n[b] = in->prev_len[b];
+  }
+  const SignalOut so{out->pred_id, out->conf, out->entropy, out->influence, out->lse, g.max_window};
+  const SimtSignals sg{c->logits, g.vocab, g.mask_id, g.forbid_mask_pred, c->ws_pred, c->ws_conf, c->ws_ent,
+                       c->ws_infl, c->ws_lse, so, out->status};
+
+  if (!c->use_tc && c->fuse.grid > 0 && c->coop && !pf.on) {   // (profiling wants the stages apart)
+    SimtStep<T> st{};
+    st.layers = (const SimtLayer<T>*)c->simt_layers; st.n_layers = g.n_layers; st.kv_only = kv_only;
+    st.export_kv = (in->flags & DC_STEP_EXPORT_KV) != 0;
+    st.m = m; st.ml = ml; st.d = d; st.F = F; st.nq = nq; st.nkv = nkv; st.hd = hd; st.V = g.vocab;
+    st.max_ctx = g.max_ctx; st.max_window = g.max_window; st.cache_layer = k_layer; st.eps = g.rms_eps;
+    st.x = c->x; st.q = q; st.k = k; st.v = v; st.o = o; st.act = act; st.h = h; st.cos_sin = c->cos_sin;
+    st.k_cache = (T*)in->k_cache; st.v_cache = (T*)in->v_cache;
+    st.final_norm = (const T*)c->final_norm; st.lm_head = (const T*)c->lm_head; st.io = io; st.logits = c->logits;
+    st.sig = sg; st.xlogp = out->xlogp; st.hp = c->hp; st.bar = c->simt_bar;
+    if ((in->flags & DC_STEP_BOUNDARY) && out->block_len)
+      st.bnd = make_boundary_io(c->ws_infl, c->ws_ent, ml.W_cap, g.max_window, out->score, out->cum_influence,
+                                out->cum_score, out->block_len);
+    auto aligned = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
+    if (simt_step_ok<T>(c->fuse, st) && aligned(in->k_cache) && aligned(in->v_cache) && aligned(io.h_in) &&
+        aligned(io.h_prev_in) && aligned(io.h_out)) {
+      const cudaError_t e = (cudaError_t)launch_simt_step<T>(c->fuse, st, s);
+      if (e != cudaSuccess) {
+        cudaGetLastError();
+        return fail(c, DC_ERR_CUDA, "fused step launch failed: %s", cudaGetErrorString(e));
+      }
+      if (!kv_only) { c->have_logits = true; c->last_meta = ml; }
+      return DC_OK;
+    }
+  }
 
   // split-K partial sums produced by the previous residual GEMM, folded in by the next norm
   const float* part = nullptr;
@@ -315,16 +354,9 @@ int run_step(dc_ctx* c, const dc_step_in* in, const dc_step_out* out, const SeqM
     return DC_OK;
   }
   pf.begin(DC_STAGE_NORM, 1);
-  LmRowsIo<T> io;
-  io.h_in = (const T*)in->h_final_in; io.h_out = (T*)out->h_out; io.max_window = g.max_window;
-  if (carried) {
-    io.h_prev_in = (const T*)in->h_prev_in;
-    for (int b = 0; b < m.batch; ++b) io.prev.n[b] = in->prev_len[b];
-  }
   launch_lm_rows<T>(c->x, part, nsplit, part_stride, (const T*)c->final_norm, g.rms_eps, d, ml, m.nv, io, h, s);
   pf.end();
 
-  SignalOut so{out->pred_id, out->conf, out->entropy, out->influence, out->lse, g.max_window};
   if (c->tc_lm) {
     pf.begin(DC_STAGE_LMHEAD, 2);
     int rc = tc_lmhead(c->tc, ml, (const __nv_bfloat16*)h, g.mask_id, g.forbid_mask_pred,
@@ -337,8 +369,7 @@ int run_step(dc_ctx* c, const dc_step_in* in, const dc_step_out* out, const SeqM
     SimtGemm<T> gl;
     gl.A = h; gl.w0 = (const T*)c->lm_head; gl.M = Mlm; gl.N = g.vocab; gl.K = d; gl.C = c->logits; gl.ldc = g.vocab;
     launch_gemm_simt<T>(gl, EPI_STORE_F32, s);
-    launch_signals_from_logits(c->logits, g.vocab, g.mask_id, g.forbid_mask_pred, ml, c->ws_pred,
-                               c->ws_conf, c->ws_ent, c->ws_infl, c->ws_lse, so, out->status, s);
+    launch_signals_from_logits(sg, ml, s);
     pf.end();
     c->have_logits = true;
   }
@@ -530,11 +561,7 @@ int dc_create(const dc_config* cfg, const dc_weights* w, void* cuda_stream, dc_c
     c->g_pred = ws_alloc<int32_t>(c, nw, &ok);
     c->g_conf = ws_alloc<float>(c, nw, &ok);
     c->g_xlogp = ws_alloc<float>(c, nww, &ok);
-    c->g_mask = ws_alloc<uint8_t>(c, nw, &ok);
-    c->g_idx = ws_alloc<int32_t>(c, nw, &ok);
     c->g_blk = ws_alloc<int32_t>(c, g.max_batch, &ok);
-    c->g_cnt = ws_alloc<int32_t>(c, g.max_batch, &ok);
-    c->g_rem = ws_alloc<int32_t>(c, g.max_batch, &ok);
     c->g_status = ws_alloc<int32_t>(c, g.max_batch, &ok);
     const size_t hbytes = nw * g.d_model * (g.dtype == DC_BF16 ? 2 : 4);
     c->g_hout = ws_alloc<char>(c, hbytes, &ok);
@@ -560,6 +587,34 @@ int dc_create(const dc_config* cfg, const dc_weights* w, void* cuda_stream, dc_c
   if ((!c->use_tc || !c->tc_lm) && !simt_init(c->bf16, hd)) {
     dc_destroy(c);
     return fail(nullptr, DC_ERR_UNSUPPORTED, "head_dim %d needs more shared memory than the CUDA-core kernels have", hd);
+  }
+  if (!c->use_tc) {
+    auto init = [&](auto t) {
+      using T = decltype(t);
+      if (!simt_step_init<T>(&c->fuse, g.d_model, g.d_ff, nq, nkv, hd, g.vocab, g.max_ctx)) return false;
+      auto aligned = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
+      bool all = aligned(w->lm_head) && aligned(w->final_norm);
+      std::vector<SimtLayer<T>> ls(g.n_layers);
+      for (int l = 0; l < g.n_layers; ++l) {
+        SimtLayer<T>& L = ls[l];
+        const void* src[9] = {w->wq[l], w->wk[l], w->wv[l], w->wo[l], w->w_gate[l], w->w_up[l], w->w_down[l], w->norm1[l], w->norm2[l]};
+        const T** dst[9] = {&L.wq, &L.wk, &L.wv, &L.wo, &L.wg, &L.wu, &L.wd, &L.n1, &L.n2};
+        for (int i = 0; i < 9; ++i) { *dst[i] = (const T*)src[i]; all = all && aligned(src[i]); }
+        L.bq = g.qkv_bias ? (const T*)w->bq[l] : nullptr;
+        L.bk = g.qkv_bias ? (const T*)w->bk[l] : nullptr;
+        L.bv = g.qkv_bias ? (const T*)w->bv[l] : nullptr;
+      }
+      if (!all) c->fuse.grid = 0;
+      if (c->fuse.grid == 0) return true;
+      c->simt_bar = ws_alloc<unsigned int>(c, 2, &ok);
+      c->simt_layers = ws_alloc<SimtLayer<T>>(c, g.n_layers, &ok);
+      return ok && (g.n_layers == 0 || cudaMemcpy(c->simt_layers, ls.data(), ls.size() * sizeof(ls[0]), cudaMemcpyHostToDevice) == cudaSuccess);
+    };
+    if (!(c->bf16 ? init(__nv_bfloat16{}) : init(0.f)) && ok) {
+      cudaGetLastError();
+      dc_destroy(c);
+      return fail(nullptr, DC_ERR_CUDA, "setting up the fused CUDA-core step failed");
+    }
   }
   if (!c->tc_lm) c->logits = ws_alloc<float>(c, (size_t)c->Mlm_max * g.vocab, &ok);
   if (!ok) {
@@ -724,7 +779,7 @@ int dc_generate(dc_ctx* c, const dc_generate_in* in, const dc_generate_out* out)
     c->g_host = nullptr;
     return fail(c, DC_ERR_NOMEM, "pinned staging buffer of dc_generate");
   }
-  // one read-back per forward: [block_len | remaining | status | window ids], then one wait
+  // what a forward hands back, written by its last kernel: [block_len | remaining | status | window ids]
   int32_t *h_blk = c->g_host, *h_rem = h_blk + g.max_batch, *h_status = h_rem + g.max_batch,
           *h_ids = h_status + g.max_batch;
   for (int b = 0; b < B; ++b) sq[b] = Seq{in->ctx_len[b], 0, 0, 0, 0, 0};
@@ -790,30 +845,18 @@ int dc_generate(dc_ctx* c, const dc_generate_in* in, const dc_generate_out* out)
     if (rc != DC_OK) return rc;
     ++nfe;
     // sequences inside a block keep their block length; the boundary rule wrote the others'
-    {
-      PrevLen keep{};
-      bool any_keep = false;
-      for (int b = 0; b < B; ++b) {
-        const bool at_boundary = sq[b].done < N && sq[b].blk == 0;
-        keep.n[b] = at_boundary ? -1 : (sq[b].done >= N ? 1 : sq[b].blk);
-        any_keep |= !at_boundary;
-      }
-      if (any_keep) launch_keep_block_len(c->g_blk, keep, B, s);
+    SeqMeta ms;
+    rc = build_meta(c, B, 0, nullptr, nullptr, h_winlen.data(), nullptr, &ms);
+    if (rc != DC_OK) return rc;
+    SelectCommit cm;
+    cm.win_ids = c->g_win; cm.pred_id = c->g_pred; cm.status = c->g_status;
+    for (int b = 0; b < B; ++b) {
+      const bool at_boundary = sq[b].done < N && sq[b].blk == 0;
+      cm.keep.n[b] = at_boundary ? -1 : (sq[b].done >= N ? 1 : sq[b].blk);
     }
-    dc_select_in se{};
-    se.batch = B; se.conf = c->g_conf; se.win_ids = c->g_win; se.xlogp = c->g_xlogp;
-    se.block_len = c->g_blk; se.win_len = h_winlen.data();
-    dc_select_out seo{c->g_mask, c->g_idx, c->g_cnt};
-    rc = dc_select(c, &se, &seo);
-    if (rc != DC_OK) return rc;
-    dc_commit_in ci{B, c->g_win, c->g_pred, c->g_mask, c->g_blk, h_winlen.data()};
-    dc_commit_out co{c->g_rem};
-    rc = dc_commit(c, &ci, &co);
-    if (rc != DC_OK) return rc;
-    cudaMemcpyAsync(h_blk, c->g_blk, sizeof(int32_t) * B, cudaMemcpyDeviceToHost, s);
-    cudaMemcpyAsync(h_rem, c->g_rem, sizeof(int32_t) * B, cudaMemcpyDeviceToHost, s);
-    cudaMemcpyAsync(h_status, c->g_status, sizeof(int32_t) * B, cudaMemcpyDeviceToHost, s);
-    cudaMemcpyAsync(h_ids, c->g_win, sizeof(int32_t) * (size_t)B * MW, cudaMemcpyDeviceToHost, s);
+    cm.host_blk = h_blk; cm.host_left = h_rem; cm.host_status = h_status; cm.host_ids = h_ids;
+    launch_select_commit(c->g_conf, c->g_xlogp, c->g_blk, ms, c->hp, g.mask_id, MW, cm, s);
+    DC_CHECK_LAUNCH(c);
     if (ev1) cudaEventRecord(ev1, s);
     if (cudaStreamSynchronize(s) != cudaSuccess) return fail(c, DC_ERR_CUDA, "stream sync failed in dc_generate");
     if (ev1) {
@@ -857,12 +900,14 @@ int dc_generate(dc_ctx* c, const dc_generate_in* in, const dc_generate_out* out)
 int dc_set_option(dc_ctx* c, int32_t option, int32_t value) {
   if (!c) return DC_ERR_INVALID_ARG;
   if (option == DC_OPT_COOPERATIVE) {
+    c->coop = value != 0;
     if (c->tc) tc_set_cooperative(c->tc, value != 0);
     return DC_OK;
   }
   if (option == DC_OPT_WAIT_LIMIT_US) {
     if (value < 1000 || value > 60000000) return fail(c, DC_ERR_INVALID_ARG, "wait limit outside [1000, 60000000] us");
-    if (!c->tc) return DC_OK;   // the CUDA-core kernels have no device-side waits
+    if (!c->tc)
+      return simt_set_wait_limit_us(value, c->stream) == 0 ? DC_OK : fail(c, DC_ERR_CUDA, "setting the wait limit failed");
     const int rc = tc_set_wait_limit_us(c->tc, value);
     return rc == DC_OK ? DC_OK : fail(c, rc, "%s", tc_error(c->tc));
   }

@@ -45,10 +45,11 @@ struct Hyper {
 };
 
 // ---- CUDA-core kernels (any shape, fp32 or bf16 storage) -------------------------------------
+// start of a step: x[row] = E[token], status[batch], RoPE table; clears words[n_words]
 template <typename T>
-void launch_embed(const T* embed, const int32_t* last_ids, const int32_t* win_ids, int max_last,
-                  int max_window, int mask_id, int vocab, int d, const SeqMeta& m, float* x,
-                  int32_t* status, cudaStream_t s);
+void launch_step_begin(const T* embed, const int32_t* last_ids, const int32_t* win_ids, int max_last, int max_window,
+                       int mask_id, int vocab, int d, const SeqMeta& m, float* x, int32_t* status, int head_dim,
+                       float theta, float* cos_sin, unsigned int* words, int n_words, cudaStream_t s);
 
 // x += sum of nsplit partials (if part != null), then out = T(rmsnorm(x) * g).  rows of x: M.
 template <typename T>
@@ -95,10 +96,6 @@ struct SimtGemm {
 template <typename T>
 void launch_gemm_simt(const SimtGemm<T>& g, int epi, cudaStream_t s);
 
-// RoPE table of the step's rows; clears status[batch] and words[n_words]
-void launch_step_begin(const SeqMeta& m, int head_dim, float theta, float* cos_sin, int32_t* status,
-                       unsigned int* words, int n_words, cudaStream_t s);
-
 // the QKV epilogue over projections in `tmp` [M, (nq + 2 nkv) * hd], for any head_dim
 template <typename T>
 void launch_rope_store(const float* tmp, const SimtGemm<T>& g, cudaStream_t s);
@@ -119,10 +116,15 @@ struct SignalOut {
 };
 // logits [M_lm, V] fp32 in LM-head row order -> per-position signals (into ws arrays, always
 // non-null, laid out [B][W_cap]) and optionally the caller's arrays.
-void launch_signals_from_logits(const float* logits, int V, int mask_id, int forbid,
-                                const SeqMeta& m, int32_t* ws_pred, float* ws_conf,
-                                float* ws_ent, float* ws_infl, float* ws_lse, SignalOut out,
-                                int32_t* status, cudaStream_t s);
+struct SimtSignals {
+  const float* logits;
+  int V, mask_id, forbid;
+  int32_t* ws_pred;
+  float *ws_conf, *ws_ent, *ws_infl, *ws_lse;
+  SignalOut out;
+  int32_t* status;
+};
+void launch_signals_from_logits(const SimtSignals& sg, const SeqMeta& m, cudaStream_t s);
 
 template <typename T>
 void launch_xlogp(const T* h, const T* lm_head, const int32_t* ws_pred, const float* ws_lse,
@@ -135,7 +137,20 @@ struct DevLens {
   const int32_t* remain = nullptr;
   const int32_t* have_prev = nullptr;
 };
-// influence/entropy rows have stride `ld`; outputs have stride max_window.
+// influence / entropy rows have stride ld, outputs stride max_window (and may be null but block_len);
+// vec: every row starts on a 16-byte boundary
+struct BoundaryIo {
+  int ld, max_window, vec;
+  float *score, *cum_i, *cum_s;
+  int32_t* block_len;
+};
+inline BoundaryIo make_boundary_io(const float* influence, const float* entropy, int ld, int max_window, float* score,
+                                   float* cum_i, float* cum_s, int32_t* block_len) {
+  auto aligned = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
+  const int vec = ld % 4 == 0 && max_window % 4 == 0 && aligned(influence) && aligned(entropy) && aligned(score) &&
+                  aligned(cum_i) && aligned(cum_s);
+  return BoundaryIo{ld, max_window, vec, score, cum_i, cum_s, block_len};
+}
 void launch_boundary(const float* influence, const float* entropy, int ld, const SeqMeta& m,
                      const Hyper& hp, int max_window, float* score, float* cum_i, float* cum_s,
                      int32_t* block_len, cudaStream_t s);
@@ -160,8 +175,16 @@ void launch_commit(int32_t* win_ids, const int32_t* pred_id, const uint8_t* sel_
                    const int32_t* block_len, const SeqMeta& m, int mask_id, int max_window,
                    int32_t* remaining, cudaStream_t s);
 
-// block_len[b] = keep.n[b] for every sequence with keep.n[b] >= 0 (the others keep what the
-// boundary rule wrote)
-void launch_keep_block_len(int32_t* block_len, const PrevLen& keep, int batch, cudaStream_t s);
+// CAP-Decoding and the commit in one launch, for the decoding loop: sequences with keep.n[b] >= 0 are inside a
+// block of that length (block_len[b] is not read); win_ids is updated as by launch_commit, and the host's
+// copies (pinned memory: block length, masked positions left, status, window ids) are written
+struct SelectCommit {
+  int32_t* win_ids = nullptr;         // null: select only
+  const int32_t *pred_id = nullptr, *status = nullptr;
+  PrevLen keep{};
+  int32_t *host_blk = nullptr, *host_left = nullptr, *host_status = nullptr, *host_ids = nullptr;
+};
+void launch_select_commit(const float* conf, const float* xlogp, const int32_t* block_len, const SeqMeta& m,
+                          const Hyper& hp, int mask_id, int max_window, const SelectCommit& cm, cudaStream_t s);
 
 }  // namespace dc

@@ -7,33 +7,12 @@
 #include <atomic>
 #include <type_traits>
 
-#include "kernels.h"
+#include "simt_dev.cuh"
 
 namespace dc {
 
 constexpr size_t kSimtSmemMax = 220 * 1024;   // dynamic shared memory a kernel of this file may ask for
 
-template <typename T> __device__ __forceinline__ float to_f(T v);
-template <> __device__ __forceinline__ float to_f<float>(float v) { return v; }
-template <> __device__ __forceinline__ float to_f<__nv_bfloat16>(__nv_bfloat16 v) {
-  return __bfloat162float(v);
-}
-template <typename T> __device__ __forceinline__ T from_f(float v);
-template <> __device__ __forceinline__ float from_f<float>(float v) { return v; }
-template <> __device__ __forceinline__ __nv_bfloat16 from_f<__nv_bfloat16>(float v) {
-  return __float2bfloat16_rn(v);
-}
-
-__device__ __forceinline__ float warp_sum(float v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-__device__ __forceinline__ float warp_max(float v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
-  return v;
-}
 // block-wide sum for blockDim.x <= 1024 (multiple of 32); red: >= 32 floats of shared memory
 __device__ __forceinline__ float block_sum(float v, float* red) {
   v = warp_sum(v);
@@ -46,67 +25,74 @@ __device__ __forceinline__ float block_sum(float v, float* red) {
   return t;
 }
 
-// ---- 4-element vector loads / stores ------------------------------------------------------------
-template <typename T> __device__ __forceinline__ void store4(T* dst, const float (&v)[4]);
-template <> __device__ __forceinline__ void store4<float>(float* dst, const float (&v)[4]) {
-  *reinterpret_cast<float4*>(dst) = make_float4(v[0], v[1], v[2], v[3]);
-}
-template <> __device__ __forceinline__ void store4<__nv_bfloat16>(__nv_bfloat16* dst,
-                                                                   const float (&v)[4]) {
-  __nv_bfloat162 a = __floats2bfloat162_rn(v[0], v[1]), b = __floats2bfloat162_rn(v[2], v[3]);
-  *reinterpret_cast<uint2*>(dst) =
-      make_uint2(*reinterpret_cast<uint32_t*>(&a), *reinterpret_cast<uint32_t*>(&b));
-}
-template <typename T> __device__ __forceinline__ void load4(const T* src, float (&v)[4]);
-template <> __device__ __forceinline__ void load4<float>(const float* src, float (&v)[4]) {
-  const float4 t = *reinterpret_cast<const float4*>(src);
-  v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
-}
-template <> __device__ __forceinline__ void load4<__nv_bfloat16>(const __nv_bfloat16* src,
-                                                                  float (&v)[4]) {
-  const uint2 t = *reinterpret_cast<const uint2*>(src);
-  const __nv_bfloat162 a = *reinterpret_cast<const __nv_bfloat162*>(&t.x);
-  const __nv_bfloat162 b = *reinterpret_cast<const __nv_bfloat162*>(&t.y);
-  v[0] = __low2float(a); v[1] = __high2float(a); v[2] = __low2float(b); v[3] = __high2float(b);
+// ---- start of a step: embedding gather, RoPE table, cleared words -----------------------------------
+// Blocks [0, M): x[row] = E[token of row].  Variant 0 (curr): [last block ; window]; variant 1 (prev):
+// the last block's ids replaced by the mask id, everything else fixed, which makes p_prev =
+// p(Z_k | c) (Section 4.4).  The block of a sequence's first curr row checks all of its ids and writes
+// status[b] (so that nothing has to clear it first).
+// The other blocks: cos_sin[(b * R_cap + r) * hd + i] = cos(angle), [.. + hd/2 + i] = sin(angle), angle =
+// (pos0[b] + r) * theta^(-2i/hd), evaluated in double precision; row batch * R_cap holds cos / sin of
+// theta^(-2i/hd) itself, the angle step between consecutive rows.  The first of them also clears the
+// grid-barrier words of the kernels that follow.
+// (One launch: as a memset and two kernels the start of a step took 8 us, most of it launch latency.)
+template <typename T>
+__global__ void __launch_bounds__(128) k_step_begin(const T* __restrict__ embed, const int32_t* __restrict__ last_ids,
+                                                    const int32_t* __restrict__ win_ids, int max_last, int max_window,
+                                                    int mask_id, int vocab, int d, const __grid_constant__ SeqMeta m,
+                                                    float* __restrict__ x, int32_t* __restrict__ status, int hd, float theta,
+                                                    float* __restrict__ cos_sin, unsigned int* __restrict__ words, int n_words) {
+  const int M = m.nv * m.batch * m.R_cap, row = blockIdx.x;
+  if (row < M) {
+    const int r = row % m.R_cap, vb = row / m.R_cap;
+    const int b = vb % m.batch, v = vb / m.batch;
+    const int Lb = m.last_len[b], W = m.win_len[b];
+    if (r == 0 && v == 0) {
+      int bad = 0;
+      for (int i = threadIdx.x; i < Lb + W; i += blockDim.x) {
+        const int id = i < Lb ? last_ids[b * max_last + i] : win_ids[b * max_window + i - Lb];
+        bad |= (id < 0 || id >= vocab);
+      }
+      bad = __syncthreads_or(bad);
+      if (threadIdx.x == 0) status[b] = bad ? DC_ERR_INDEX : DC_OK;
+    }
+    int tok = mask_id;
+    if (r < Lb) tok = (v == 0) ? last_ids[b * max_last + r] : mask_id;
+    else if (r < Lb + W) tok = win_ids[b * max_window + (r - Lb)];
+    if (tok < 0 || tok >= vocab) tok = mask_id;
+    const T* e = embed + (size_t)tok * d;
+    float* xr = x + (size_t)row * d;
+    // d is a multiple of 4: four elements per thread and step
+#pragma unroll 8
+    for (int i = threadIdx.x * 4; i < d; i += 128 * 4) {
+      float w[4];
+      load4<T>(e + i, w);
+      *reinterpret_cast<float4*>(xr + i) = make_float4(w[0], w[1], w[2], w[3]);
+    }
+    return;
+  }
+  if (row == M)
+    for (int i = threadIdx.x; i < n_words; i += blockDim.x) words[i] = 0u;
+  const int half = hd / 2;
+  const int idx = (row - M) * 128 + threadIdx.x;
+  const int rows = m.batch * m.R_cap;
+  if (idx >= (rows + 1) * half) return;   // one extra row: cos / sin of the per-row angle step
+  const int i = idx % half, br = idx / half;
+  const int r = br % m.R_cap, b = br / m.R_cap;
+  const double inv_freq = pow((double)theta, -2.0 * (double)i / (double)hd);
+  const double ang = (br < rows) ? (double)(m.pos0[b] + r) * inv_freq : inv_freq;
+  double sn, cs;
+  sincos(ang, &sn, &cs);
+  cos_sin[(size_t)br * hd + i] = (float)cs;
+  cos_sin[(size_t)br * hd + half + i] = (float)sn;
 }
 
-// ---- embedding gather: x[row] = E[token of row] -----------------------------------------------
-// Variant 0 (curr): [last block ; window]; variant 1 (prev): the last block's ids replaced by
-// the mask id, everything else fixed, which makes p_prev = p(Z_k | c) (Section 4.4).
 template <typename T>
-__global__ void k_embed(const T* __restrict__ embed, const int32_t* __restrict__ last_ids,
-                        const int32_t* __restrict__ win_ids, int max_last, int max_window,
-                        int mask_id, int vocab, int d, SeqMeta m, float* __restrict__ x,
-                        int32_t* __restrict__ status) {
-  const int row = blockIdx.x;
-  const int r = row % m.R_cap;
-  const int vb = row / m.R_cap;
-  const int b = vb % m.batch, v = vb / m.batch;
-  const int Lb = m.last_len[b], W = m.win_len[b];
-  int tok = mask_id;
-  if (r < Lb) tok = (v == 0) ? last_ids[b * max_last + r] : mask_id;
-  else if (r < Lb + W) tok = win_ids[b * max_window + (r - Lb)];
-  if (tok < 0 || tok >= vocab) {
-    if (threadIdx.x == 0) status[b] = DC_ERR_INDEX;
-    tok = mask_id;
-  }
-  const T* e = embed + (size_t)tok * d;
-  float* xr = x + (size_t)row * d;
-  // d is a multiple of 4: four elements per thread and step
-  for (int i = threadIdx.x * 4; i < d; i += blockDim.x * 4) {
-    float v[4];
-    load4<T>(e + i, v);
-    *reinterpret_cast<float4*>(xr + i) = make_float4(v[0], v[1], v[2], v[3]);
-  }
-}
-
-template <typename T>
-void launch_embed(const T* embed, const int32_t* last_ids, const int32_t* win_ids, int max_last,
-                  int max_window, int mask_id, int vocab, int d, const SeqMeta& m, float* x,
-                  int32_t* status, cudaStream_t s) {
-  const int M = m.nv * m.batch * m.R_cap;
-  k_embed<T><<<M, 128, 0, s>>>(embed, last_ids, win_ids, max_last, max_window, mask_id, vocab, d,
-                               m, x, status);
+void launch_step_begin(const T* embed, const int32_t* last_ids, const int32_t* win_ids, int max_last, int max_window,
+                       int mask_id, int vocab, int d, const SeqMeta& m, float* x, int32_t* status, int head_dim,
+                       float theta, float* cos_sin, unsigned int* words, int n_words, cudaStream_t s) {
+  const int M = m.nv * m.batch * m.R_cap, table = (m.batch * m.R_cap + 1) * (head_dim / 2);
+  k_step_begin<T><<<M + (table + 127) / 128, 128, 0, s>>>(embed, last_ids, win_ids, max_last, max_window, mask_id, vocab,
+                                                          d, m, x, status, head_dim, theta, cos_sin, words, n_words);
 }
 
 // ---- RMSNorm (with the split-K partial sums of the preceding GEMM folded into x) --------------
@@ -241,32 +227,6 @@ void launch_lm_rows(const float* x, const float* part, int nsplit, size_t part_s
 // A tile's 32 columns are either 32 consecutive rows of W, or - for the epilogues that combine two
 // output features - 16 features and their partners: i and i + head_dim / 2 of a head (RoPE), or
 // gate and up of an MLP feature.
-template <typename T> struct GemmIo {
-  static constexpr int kPiece = 16 / (int)sizeof(T);   // elements of a 16-byte copy
-  static constexpr int kPad = kPiece;                  // row padding: no bank conflicts between 8 rows
-};
-__device__ __forceinline__ void cp_async16(void* dst, const void* src, int bytes) {   // the rest of the 16 bytes is zeroed
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;"
-               ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src), "r"(bytes) : "memory");
-}
-typedef unsigned long long f2;
-__device__ __forceinline__ f2 pack2(float lo, float hi) {
-  f2 r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-  return r;
-}
-__device__ __forceinline__ void fma2(f2& d, f2 a, f2 b) {
-  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
-}
-__device__ __forceinline__ float sum2(f2 v) {
-  float lo, hi;
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
-  return lo + hi;
-}
-
-template <typename T>
-__device__ __forceinline__ void simt_store_qkv(const SimtGemm<T>& g, int m, int head, int e, float y1, float y2);
-
 template <typename T, int WM, int WN, int WK, int KC, int STAGES, int EPI>
 __global__ void __launch_bounds__(256) k_gemm_simt(const SimtGemm<T> g) {
   constexpr int BM = 16 * WM, BN = 32 * WN, PITCH = KC + GemmIo<T>::kPad, PIECE = GemmIo<T>::kPiece;
@@ -401,49 +361,6 @@ __global__ void __launch_bounds__(256) k_gemm_simt(const SimtGemm<T> g) {
   }
 }
 
-// One rotated pair (features e and e + head_dim / 2 of a head) of activation row m: bias, rotation,
-// store, and the copy into the context cache when the row belongs to an exported last block.
-template <typename T>
-__device__ __forceinline__ void simt_store_qkv(const SimtGemm<T>& g, int m, int head, int e, float y1, float y2) {
-  const int hd = g.hd, half = hd >> 1;
-  const int rv = g.m.batch * g.m.R_cap, br = m % rv;   // (b, r): the RoPE table is shared by both variants
-  if (g.bq != nullptr) {   // projection bias, before the rotation
-    const T* bb = head < g.nq ? g.bq + head * hd : head < g.nq + g.nkv ? g.bk + (head - g.nq) * hd
-                                                                       : g.bv + (head - g.nq - g.nkv) * hd;
-    y1 += to_f<T>(bb[e]); y2 += to_f<T>(bb[half + e]);
-  }
-  const bool is_v = head >= g.nq + g.nkv;
-  if (!is_v) {
-    const float c = g.cos_sin[(size_t)br * hd + e], sn = g.cos_sin[(size_t)br * hd + half + e];
-    const float t = y1 * c - y2 * sn;
-    y2 = y2 * c + y1 * sn;
-    y1 = t;
-  }
-  const T o1 = from_f<T>(y1), o2 = from_f<T>(y2);
-  if (head < g.nq) {
-    T* dst = g.q + (size_t)m * g.nq * hd + head * hd + e;
-    dst[0] = o1; dst[half] = o2;
-    return;
-  }
-  const int hk = is_v ? head - g.nq - g.nkv : head - g.nq;
-  T* dst = (is_v ? g.v : g.k) + (size_t)m * g.nkv * hd + hk * hd + e;
-  dst[0] = o1; dst[half] = o2;
-  if (g.k_cache != nullptr && m < rv) {
-    const int b = br / g.m.R_cap, r = br - b * g.m.R_cap;
-    if (r < g.m.last_len[b]) {
-      const size_t kv = (size_t)b * g.nkv + hk;
-      const int key = g.m.ctx_len[b] + r;
-      if (is_v) {
-        g.v_cache[(kv * hd + e) * g.max_ctx + key] = o1;
-        g.v_cache[(kv * hd + half + e) * g.max_ctx + key] = o2;
-      } else {
-        g.k_cache[(kv * g.max_ctx + key) * hd + e] = o1;
-        g.k_cache[(kv * g.max_ctx + key) * hd + half + e] = o2;
-      }
-    }
-  }
-}
-
 constexpr long long kSmallTiles = 148 * 8;
 
 template <typename T, int EPI>
@@ -471,38 +388,6 @@ void launch_gemm_simt(const SimtGemm<T>& g, int epi, cudaStream_t s) {
     case EPI_SWIGLU: launch_gemm_epi<T, EPI_SWIGLU>(g, (g.N + 15) / 16, s); break;
     default: launch_gemm_epi<T, EPI_QKV>(g, (g.nq + 2 * g.nkv) * (g.hd / 32), s);
   }
-}
-
-// ---- start of a step: RoPE table, cleared words --------------------------------------------------
-// cos_sin[(b * R_cap + r) * hd + i] = cos(angle), [.. + hd/2 + i] = sin(angle),
-// angle = (pos0[b] + r) * theta^(-2i/hd), evaluated in double precision.  Row batch * R_cap
-// holds cos / sin of theta^(-2i/hd) itself, the angle step between consecutive rows.
-// The first block also clears status[batch] and the synchronisation words of the dense chain.
-__global__ void k_step_begin(const SeqMeta m, int hd, float theta, float* __restrict__ cos_sin,
-                             int32_t* __restrict__ status, unsigned int* __restrict__ words, int n_words) {
-  if (blockIdx.x == 0) {
-    for (int i = threadIdx.x; i < m.batch; i += blockDim.x) status[i] = 0;
-    for (int i = threadIdx.x; i < n_words; i += blockDim.x) words[i] = 0u;
-  }
-  const int half = hd / 2;
-  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  const int rows = m.batch * m.R_cap;
-  const int total = (rows + 1) * half;   // one extra row: cos / sin of the per-row angle step
-  if (idx >= total) return;
-  const int i = idx % half, br = idx / half;
-  const int r = br % m.R_cap, b = br / m.R_cap;
-  const double inv_freq = pow((double)theta, -2.0 * (double)i / (double)hd);
-  const double ang = (br < rows) ? (double)(m.pos0[b] + r) * inv_freq : inv_freq;
-  double sn, cs;
-  sincos(ang, &sn, &cs);
-  cos_sin[(size_t)br * hd + i] = (float)cs;
-  cos_sin[(size_t)br * hd + half + i] = (float)sn;
-}
-
-void launch_step_begin(const SeqMeta& m, int head_dim, float theta, float* cos_sin, int32_t* status,
-                       unsigned int* words, int n_words, cudaStream_t s) {
-  const int total = (m.batch * m.R_cap + 1) * (head_dim / 2);
-  k_step_begin<<<(total + 255) / 256, 256, 0, s>>>(m, head_dim, theta, cos_sin, status, words, n_words);
 }
 
 // head_dim not a multiple of 32: the projections go through `tmp` [M, (nq + 2 nkv) hd] and this
@@ -725,109 +610,15 @@ bool simt_init(bool bf16, int head_dim) {
   return ok && attn_simt_shape(head_dim).smem <= kSimtSmemMax;
 }
 
-// ---- per-position signals from full logits (CUDA-core LM head only) ------------------------------
-// One block per window position.  c = max_v p(v), yhat = argmax (lowest id on ties),
-// H = lse - sum p z, I = sum p [(z - lse) - (z' - lse')] clamped at 0 (Eq. 3).
+// ---- per-position signals from full logits (CUDA-core LM head only): one block per window position --
 constexpr int kSigThreads = 512;
-__global__ void __launch_bounds__(kSigThreads) k_signals(const float* __restrict__ logits, int V,
-                                                 int mask_id, int forbid, SeqMeta m,
-                                                 int32_t* __restrict__ ws_pred,
-                                                 float* __restrict__ ws_conf,
-                                                 float* __restrict__ ws_ent,
-                                                 float* __restrict__ ws_infl,
-                                                 float* __restrict__ ws_lse, SignalOut out,
-                                                 int32_t* __restrict__ status) {
-  __shared__ float red[32];
-  __shared__ float s_m[kSigThreads / 32], s_m2[kSigThreads / 32];
-  __shared__ int s_i[kSigThreads / 32];
-  const int p = blockIdx.x;
-  const int b = p / m.W_cap, k = p % m.W_cap;
-  if (b >= m.batch || k >= m.win_len[b]) return;
-  const bool prev = (m.nv == 2);
-  const float* z = logits + (size_t)lm_row(m, 0, p) * V;
-  const float* z2 = prev ? logits + (size_t)lm_row(m, 1, p) * V : nullptr;
-  const int skip = forbid ? mask_id : -1;
-  float mx = -INFINITY, mx2 = -INFINITY;
-  int am = 0x7fffffff;
-  // four logits at a time where the rows are 16-byte aligned
-  auto each = [&](auto&& f) {
-    if (V % 4 == 0) {
-      for (int v = threadIdx.x * 4; v < V; v += kSigThreads * 4) {
-        const float4 a = *reinterpret_cast<const float4*>(z + v);
-        const float4 p4 = prev ? *reinterpret_cast<const float4*>(z2 + v) : make_float4(0.f, 0.f, 0.f, 0.f);
-        f(v, a.x, p4.x); f(v + 1, a.y, p4.y); f(v + 2, a.z, p4.z); f(v + 3, a.w, p4.w);
-      }
-    } else {
-      for (int v = threadIdx.x; v < V; v += kSigThreads) f(v, z[v], prev ? z2[v] : 0.f);
-    }
-  };
-  each([&](int v, float a, float a2) {
-    if (v == skip) return;
-    if (a > mx) { mx = a; am = v; }  // strided ascending: the first maximum kept per thread
-    if (prev) mx2 = fmaxf(mx2, a2);
-  });
-  // reduce (max, lowest index) across the block
-  for (int o = 16; o > 0; o >>= 1) {
-    const float om = __shfl_xor_sync(0xffffffffu, mx, o);
-    const int oi = __shfl_xor_sync(0xffffffffu, am, o);
-    if (om > mx || (om == mx && oi < am)) { mx = om; am = oi; }
-    mx2 = fmaxf(mx2, __shfl_xor_sync(0xffffffffu, mx2, o));
-  }
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  if (l == 0) { s_m[w] = mx; s_i[w] = am; s_m2[w] = mx2; }
-  __syncthreads();
-  mx = s_m[0]; am = s_i[0]; mx2 = s_m2[0];
-  for (int i = 1; i < kSigThreads / 32; ++i) {
-    if (s_m[i] > mx || (s_m[i] == mx && s_i[i] < am)) { mx = s_m[i]; am = s_i[i]; }
-    mx2 = fmaxf(mx2, s_m2[i]);
-  }
-  float S = 0.f, Az = 0.f, Ad = 0.f, S2 = 0.f;
-  each([&](int v, float a, float a2) {
-    if (v == skip) return;
-    const float e = expf(a - mx);
-    S += e;
-    if (e > 0.f) {
-      Az = fmaf(e, a, Az);
-      if (prev) Ad = fmaf(e, a - a2, Ad);
-    }
-    if (prev) S2 += expf(a2 - mx2);
-  });
-  S = block_sum(S, red);
-  Az = block_sum(Az, red);
-  Ad = block_sum(Ad, red);
-  S2 = block_sum(S2, red);
-  if (threadIdx.x == 0) {
-    const float lse = mx + logf(S);
-    const float conf = 1.f / S;
-    const float ent = lse - Az / S;
-    float infl = 0.f;
-    if (prev && m.have_prev[b]) {
-      const float lse2 = mx2 + logf(S2);
-      infl = fmaxf(Ad / S - lse + lse2, 0.f);
-    }
-    // no finite admissible logit (a NaN / inf hidden row): the argmax sentinel must not reach
-    // the kernels that index the vocabulary matrix with the id
-    if (am < 0 || am >= V || !isfinite(lse)) {
-      am = mask_id;
-      if (status) atomicMax(status + b, (int)DC_ERR_NUMERIC);
-    }
-    const int wi = b * m.W_cap + k;
-    ws_pred[wi] = am; ws_conf[wi] = conf; ws_ent[wi] = ent; ws_infl[wi] = infl; ws_lse[wi] = lse;
-    const int oi = b * out.max_window + k;
-    if (out.pred_id) out.pred_id[oi] = am;
-    if (out.conf) out.conf[oi] = conf;
-    if (out.entropy) out.entropy[oi] = ent;
-    if (out.influence) out.influence[oi] = infl;
-    if (out.lse) out.lse[oi] = lse;
-  }
+__global__ void __launch_bounds__(kSigThreads) k_signals(const SimtSignals sg, const SeqMeta m) {
+  __shared__ SignalsShared<kSigThreads> sh;
+  signals_pos<kSigThreads>(sg, m, blockIdx.x, threadIdx.x, sh, [] { __syncthreads(); });
 }
 
-void launch_signals_from_logits(const float* logits, int V, int mask_id, int forbid,
-                                const SeqMeta& m, int32_t* ws_pred, float* ws_conf,
-                                float* ws_ent, float* ws_infl, float* ws_lse, SignalOut out,
-                                int32_t* status, cudaStream_t s) {
-  k_signals<<<m.batch * m.W_cap, kSigThreads, 0, s>>>(logits, V, mask_id, forbid, m, ws_pred, ws_conf,
-                                              ws_ent, ws_infl, ws_lse, out, status);
+void launch_signals_from_logits(const SimtSignals& sg, const SeqMeta& m, cudaStream_t s) {
+  k_signals<<<m.batch * m.W_cap, kSigThreads, 0, s>>>(sg, m);
 }
 
 // ---- cross log-probabilities: xlogp[b,i,j] = h_i . W_lm[yhat_j] - lse_i  (Eq. 6 halves) ---------
@@ -895,8 +686,9 @@ void launch_xlogp(const T* h, const T* lm_head, const int32_t* ws_pred, const fl
 
 // explicit instantiations
 #define DC_INST(T)                                                                              \
-  template void launch_embed<T>(const T*, const int32_t*, const int32_t*, int, int, int, int,   \
-                                int, const SeqMeta&, float*, int32_t*, cudaStream_t);           \
+  template void launch_step_begin<T>(const T*, const int32_t*, const int32_t*, int, int, int, int, \
+                                     int, const SeqMeta&, float*, int32_t*, int, float, float*,   \
+                                     unsigned int*, int, cudaStream_t);                           \
   template void launch_rmsnorm<T>(float*, const float*, int, size_t, const T*, float, int, int, \
                                   T*, cudaStream_t);                                            \
   template void launch_lm_rows<T>(const float*, const float*, int, size_t, const T*, float, int,  \
