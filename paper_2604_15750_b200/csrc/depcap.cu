@@ -73,6 +73,8 @@ struct dc_ctx {
   int R_cap_max = 0, M_max = 0, Mlm_max = 0;
   // workspace (device)
   std::vector<void*> allocs;
+  char* block = nullptr;     // what is left of the block that small arrays come from
+  size_t block_left = 0;
   float* x = nullptr;        // residual stream [M, d] fp32
   void* a = nullptr;         // normed activations [M, d]
   void* q = nullptr;         // [M, nq*hd] rotated
@@ -118,14 +120,22 @@ inline int round_up(int v, int m) { return (v + m - 1) / m * m; }
 
 template <typename T>
 T* ws_alloc(dc_ctx* c, size_t n, bool* ok) {
+  // small arrays share blocks: a cudaMalloc costs 10..60 us of dc_create, whatever its size
+  const size_t bytes = ((n ? n : 1) * sizeof(T) + 255) / 256 * 256;
+  constexpr size_t kBlock = 2u << 20, kSmall = 512u << 10;
+  if (bytes <= kSmall && bytes <= c->block_left) {
+    char* q = c->block;
+    c->block += bytes; c->block_left -= bytes;
+    return reinterpret_cast<T*>(q);
+  }
   void* p = nullptr;
-  if (n == 0) n = 1;
-  if (cudaMalloc(&p, n * sizeof(T)) != cudaSuccess) {
+  if (cudaMalloc(&p, bytes <= kSmall ? kBlock : bytes) != cudaSuccess) {
     *ok = false;
     cudaGetLastError();
     return nullptr;
   }
   c->allocs.push_back(p);
+  if (bytes <= kSmall) { c->block = static_cast<char*>(p) + bytes; c->block_left = kBlock - bytes; }
   return reinterpret_cast<T*>(p);
 }
 

@@ -123,6 +123,7 @@ __device__ __forceinline__ void simt_store_qkv(const G& g, int m, int head, int 
 // ---- per-position signals from full logits ---------------------------------------------------------
 // c = max_v p(v), yhat = argmax (lowest id on ties), H = lse - sum p z,
 // I = sum p [(z - lse) - (z' - lse')] clamped at 0 (Eq. 3).  NT threads work on one window position.
+// One pass: every thread keeps its own reference points and scales its sums when they move.
 template <int NT> struct SignalsShared { float red[4][NT / 32], m[NT / 32], m2[NT / 32]; int i[NT / 32]; };
 template <int NT, typename Sync>
 __device__ __forceinline__ void signals_pos(const SimtSignals& sg, const SeqMeta& m, int p, int t, SignalsShared<NT>& sh,
@@ -135,24 +136,59 @@ __device__ __forceinline__ void signals_pos(const SimtSignals& sg, const SeqMeta
   const int skip = sg.forbid ? sg.mask_id : -1;
   float mx = -INFINITY, mx2 = -INFINITY;
   int am = 0x7fffffff;
-  // four logits at a time where the rows are 16-byte aligned
-  auto each = [&](auto&& f) {
-    if (V % 4 == 0) {
-      for (int v = t * 4; v < V; v += NT * 4) {
-        const float4 a = __ldcg(reinterpret_cast<const float4*>(z + v));
-        const float4 p4 = prev ? __ldcg(reinterpret_cast<const float4*>(z2 + v)) : make_float4(0.f, 0.f, 0.f, 0.f);
-        f(v, a.x, p4.x); f(v + 1, a.y, p4.y); f(v + 2, a.z, p4.z); f(v + 3, a.w, p4.w);
+  float sum[4] = {0.f, 0.f, 0.f, 0.f};   // S, A, D, S'
+  auto four = [&](int v, const float (&a)[4], const float (&a2)[4], int n) {
+    float top = -INFINITY, top2 = -INFINITY;
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if (i < n && v + i != skip) {
+        if (a[i] > fmaxf(mx, top)) am = v + i;     // ascending ids: the first maximum is kept
+        top = fmaxf(top, a[i]);
+        top2 = fmaxf(top2, a2[i]);
       }
-    } else {
-      for (int v = t; v < V; v += NT) f(v, __ldcg(z + v), prev ? __ldcg(z2 + v) : 0.f);
+    if (top > mx) {
+      const float c = expf(mx - top);
+      sum[0] *= c; sum[1] *= c; sum[2] *= c;
+      mx = top;
     }
+    if (prev && top2 > mx2) { sum[3] *= expf(mx2 - top2); mx2 = top2; }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if (i < n && v + i != skip) {
+        const float e = a[i] == -INFINITY ? 0.f : expf(a[i] - mx);   // (the reference point may still be -inf)
+        sum[0] += e;
+        if (e > 0.f) {
+          sum[1] = fmaf(e, a[i], sum[1]);
+          if (prev) sum[2] = fmaf(e, a[i] - a2[i], sum[2]);
+        }
+        if (prev && a2[i] != -INFINITY) sum[3] += expf(a2[i] - mx2);
+      }
   };
-  each([&](int v, float a, float a2) {
-    if (v == skip) return;
-    if (a > mx) { mx = a; am = v; }  // strided ascending: the first maximum kept per thread
-    if (prev) mx2 = fmaxf(mx2, a2);
-  });
+  // four logits at a time where the rows are 16-byte aligned
+  if (V % 4 == 0) {
+    float4 na = make_float4(0.f, 0.f, 0.f, 0.f), nq = na;
+    auto fetch = [&](int v) {
+      if (v >= V) return;
+      na = __ldcg(reinterpret_cast<const float4*>(z + v));
+      if (prev) nq = __ldcg(reinterpret_cast<const float4*>(z2 + v));
+    };
+    fetch(t * 4);
+#pragma unroll 1
+    for (int v = t * 4; v < V; v += NT * 4) {
+      const float4 a = na, q = nq;
+      fetch(v + NT * 4);
+      const float av[4] = {a.x, a.y, a.z, a.w}, qv[4] = {q.x, q.y, q.z, q.w};
+      four(v, av, qv, 4);
+    }
+  } else {
+    for (int v = t; v < V; v += NT) {
+      const float av[4] = {__ldcg(z + v)}, qv[4] = {prev ? __ldcg(z2 + v) : 0.f};
+      four(v, av, qv, 1);
+    }
+  }
+  const float own = mx, own2 = mx2;
   // reduce (max, lowest index) across the threads
+#pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     const float om = __shfl_xor_sync(0xffffffffu, mx, o);
     const int oi = __shfl_xor_sync(0xffffffffu, am, o);
@@ -167,20 +203,10 @@ __device__ __forceinline__ void signals_pos(const SimtSignals& sg, const SeqMeta
     if (sh.m[i] > mx || (sh.m[i] == mx && sh.i[i] < am)) { mx = sh.m[i]; am = sh.i[i]; }
     mx2 = fmaxf(mx2, sh.m2[i]);
   }
-  float sum[4] = {0.f, 0.f, 0.f, 0.f};   // S, A, D, S'
-  each([&](int v, float a, float a2) {
-    if (v == skip) return;
-    const float e = expf(a - mx);
-    sum[0] += e;
-    if (e > 0.f) {
-      sum[1] = fmaf(e, a, sum[1]);
-      if (prev) sum[2] = fmaf(e, a - a2, sum[2]);
-    }
-    if (prev) sum[3] += expf(a2 - mx2);
-  });
+  const float c = own > -INFINITY ? expf(own - mx) : 0.f, c2 = own2 > -INFINITY ? expf(own2 - mx2) : 0.f;
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
-    sum[i] = warp_sum(sum[i]);
+    sum[i] = warp_sum(sum[i] * (i < 3 ? c : c2));
     if (l == 0) sh.red[i][w] = sum[i];
   }
   sync();

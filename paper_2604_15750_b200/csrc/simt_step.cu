@@ -4,7 +4,9 @@
 // third of that launch, ramp and drain, and the host needs 4 us for every launch.  Here the phases of
 // all layers, the LM head, the signals, the cross log-probs and the boundary rule run in one kernel
 // of one CTA per SM, with a counting grid barrier between phases.  Two-layer fp32 model (d 256, 96 rows,
-// vocab 4096): 22 launches and 157 us per step -> 3 launches and 124 us; a generation step 183 -> 125 us.
+// vocab 4096): 22 launches and 157 us per step -> 3 launches and 108 us; a generation step 183 -> 110 us.
+// What is left: about 1.5 us per barrier (12), and in a phase two L2 latencies (rows, weights) and the
+// issue of some 1000 instructions per warp, four warps to a scheduler.
 //
 //   per layer   norm1 + QKV + rotation + cache append | attention | O projection + residual |
 //               norm2 + gate / up + SwiGLU | down projection + residual
@@ -16,6 +18,8 @@
 // barrier (they depend on nothing).  Data of other CTAs is read past L1 (ld.cg, cp.async.cg).
 #include <cuda_runtime.h>
 
+#include <atomic>
+
 #include "decisions.cuh"
 #include "simt_dev.cuh"
 #include "simt_step.h"
@@ -25,8 +29,7 @@ namespace dc {
 namespace {
 
 constexpr int kGroups = 2, kFuseThreads = 256 * kGroups;
-constexpr int kKC = 128, kStages = 3;          // k-chunk of the GEMM tiles (16 k per warp), ring stages
-constexpr int kCsPitch = 33;
+constexpr int kKC = 256, kStages = 3;          // k-chunk of the GEMM tiles (32 k per warp), ring stages
 constexpr size_t kGroupSmemMax = 112 * 1024;   // shared memory of a group
 constexpr int kMaxNormD = 1024;                // a warp holds a row in registers while it norms it
 
@@ -57,72 +60,80 @@ struct FuseGemm {
   int M, N, K, ldc;
   float* C;
   T* act;
+  int epi, src;
 };
 enum { SRC_GLOBAL = 0, SRC_NORM = 1, SRC_LM = 2 };
 
-// dst_i = T(rmsnorm(row) * gain) by one warp, into up to three places (null: skipped); columns d ..
-// pad_to of s0 are zeroed
+// dst_i = T(rmsnorm(row) * gain) by half a warp (lane l of 16), into up to three places (null: skipped);
+// columns d .. pad_to of s0 are zeroed.  `row` null: nothing but zeros in s0.  (Loops stay rolled all
+// over this file: code that runs once or twice per phase costs its instruction fetches, about 14
+// clocks an instruction; unrolled it took 4500 clocks for 256 columns.)
 template <typename T>
 __device__ __forceinline__ void norm_row(const float* row, const T* gain, float eps, int d, T* s0, int pad_to, T* g0, T* g1,
-                                         int lane) {
-  float4 v[kMaxNormD / 128];
+                                         int l) {
   float ss = 0.f;
-#pragma unroll
-  for (int i = 0; i < kMaxNormD / 128; ++i) {
-    const int e = lane * 4 + 128 * i;
-    if (e < d) {
-      v[i] = __ldcg(reinterpret_cast<const float4*>(row + e));
-      ss += v[i].x * v[i].x + v[i].y * v[i].y + v[i].z * v[i].z + v[i].w * v[i].w;
-    }
-  }
-  ss = warp_sum(ss);
-  const float inv = rsqrtf(ss / (float)d + eps);
-#pragma unroll
-  for (int i = 0; i < kMaxNormD / 128; ++i) {
-    const int e = lane * 4 + 128 * i;
-    float o[4] = {0.f, 0.f, 0.f, 0.f};
-    if (e < d) {
+#pragma unroll 4
+  for (int e = l * 4; e < d; e += 64) {
+    const float4 v = row != nullptr ? __ldcg(reinterpret_cast<const float4*>(row + e)) : make_float4(0.f, 0.f, 0.f, 0.f);
+    ss += v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w;
+    if (sizeof(T) == 4 && s0) {   // the gain now: its latency would follow the row's otherwise
       float gv[4];
       load4<T>(gain + e, gv);
-      o[0] = v[i].x * inv * gv[0]; o[1] = v[i].y * inv * gv[1]; o[2] = v[i].z * inv * gv[2]; o[3] = v[i].w * inv * gv[3];
-      if (g0) store4<T>(g0 + e, o);
-      if (g1) store4<T>(g1 + e, o);
+      *reinterpret_cast<float4*>(s0 + e) = make_float4(v.x * gv[0], v.y * gv[1], v.z * gv[2], v.w * gv[3]);
     }
-    if (s0 && e < pad_to) store4<T>(s0 + e, o);
   }
-}
-template <typename T>
-__device__ __forceinline__ void copy_row(const T* src, int d, T* s0, int pad_to, T* g0, int lane) {   // src null: zeros
-  for (int e = lane * 4; e < pad_to; e += 128) {
-    float o[4] = {0.f, 0.f, 0.f, 0.f};
-    if (src != nullptr && e < d) ldcg4<T>(src + e, o);
-    store4<T>(s0 + e, o);
-    if (g0 && e < d) store4<T>(g0 + e, o);
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+  const float inv = rsqrtf(ss / (float)d + eps);
+#pragma unroll 2
+  for (int e = l * 4; e < d; e += 64) {
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    float gv[4] = {1.f, 1.f, 1.f, 1.f};
+    if (sizeof(T) == 4 && s0) v = *reinterpret_cast<const float4*>(s0 + e);
+    else {
+      if (row != nullptr) v = __ldcg(reinterpret_cast<const float4*>(row + e));
+      load4<T>(gain + e, gv);
+    }
+    const float o[4] = {v.x * inv * gv[0], v.y * inv * gv[1], v.z * inv * gv[2], v.w * inv * gv[3]};
+    if (s0) store4<T>(s0 + e, o);
+    if (g0) store4<T>(g0 + e, o);
+    if (g1) store4<T>(g1 + e, o);
   }
+  const float z[4] = {0.f, 0.f, 0.f, 0.f};
+  if (s0)
+    for (int e = d + l * 4; e < pad_to; e += 64) store4<T>(s0 + e, z);
 }
 
-// LM-head input row lrow (see k_lm_rows) into s0; `own`: also into h (and the curr rows into h_out)
+// LM-head input row lrow (see k_lm_rows), by half a warp.  A copied row goes into s0 here and false is
+// returned; otherwise xr (null: zeros) is the row to norm.  g0, g1: where the normed row goes besides -
+// with `own` h, and h_out for the curr rows.
 template <typename T>
-__device__ __forceinline__ void lm_row_to(const SimtStep<T>& p, int lrow, T* s0, int pad_to, bool own, int lane) {
+__device__ __forceinline__ bool lm_row(const SimtStep<T>& p, int lrow, T* s0, int pad_to, bool own, int l, const float*& xr,
+                                       T*& g0, T*& g1) {
   const SeqMeta& m = p.ml;
   const int grp = lrow / (m.nv * m.G), in = lrow % (m.nv * m.G);
   const int v = in / m.G, pos = grp * m.G + in % m.G;
   const int b = pos / m.W_cap, k = pos % m.W_cap;
-  T* hr = own ? p.h + (size_t)lrow * p.d : nullptr;
-  if (lrow >= m.nv * m.npos_pad || b >= m.batch || k >= m.win_len[b]) {
-    copy_row<T>(nullptr, p.d, s0, pad_to, lrow < m.nv * m.npos_pad ? hr : nullptr, lane);
-    return;
-  }
-  T* ho = (own && v == 0 && p.io.h_out != nullptr) ? p.io.h_out + ((size_t)b * p.max_window + k) * p.d : nullptr;
+  const bool row_ok = lrow < m.nv * m.npos_pad;
+  g0 = own && row_ok ? p.h + (size_t)lrow * p.d : nullptr;
+  if (!row_ok || b >= m.batch || k >= m.win_len[b]) return true;
+  if (own && v == 0 && p.io.h_out != nullptr) g1 = p.io.h_out + ((size_t)b * p.max_window + k) * p.d;
+  xr = p.x + (size_t)act_row(p.m, v < p.m.nv ? v : 0, b, p.m.last_len[b] + k) * p.d;
   const T* src = p.io.h_in != nullptr ? p.io.h_in + (((size_t)b * 2 + v) * p.max_window + k) * p.d
-               : (v >= p.m.nv && k < p.io.prev.n[b]) ? p.io.h_prev_in + ((size_t)b * p.max_window + k) * p.d : nullptr;
-  if (src != nullptr) {
-    copy_row<T>(src, p.d, s0, pad_to, hr, lane);
-    if (ho == nullptr || p.io.h_in == nullptr) return;
-    s0 = nullptr; hr = nullptr;
+                 : (v >= p.m.nv && k < p.io.prev.n[b]) ? p.io.h_prev_in + ((size_t)b * p.max_window + k) * p.d : nullptr;
+  if (src == nullptr) return true;
+#pragma unroll 4
+  for (int e = l * 4; e < p.d; e += 64) {
+    float o[4];
+    ldcg4<T>(src + e, o);
+    store4<T>(s0 + e, o);
+    if (g0) store4<T>(g0 + e, o);
   }
-  norm_row<T>(p.x + (size_t)act_row(p.m, v < p.m.nv ? v : 0, b, p.m.last_len[b] + k) * p.d, p.final_norm, p.eps, p.d, s0,
-              pad_to, hr, ho, lane);
+  const float z[4] = {0.f, 0.f, 0.f, 0.f};
+  for (int e = p.d + l * 4; e < pad_to; e += 64) store4<T>(s0 + e, z);
+  g0 = nullptr;
+  if (p.io.h_in == nullptr) g1 = nullptr;
+  return false;
 }
 
 // what simt_store_qkv needs
@@ -135,166 +146,191 @@ struct QkvView {
   T *q, *k, *v, *k_cache, *v_cache;
 };
 
-// All tiles (16 rows x 32 columns, as in k_gemm_simt) of one GEMM; `wait` is the barrier in front of the
-// phase: every thread of the CTA calls it once.  Returns false if it gave up.
-template <typename T, int EPI, int SRC, typename Wait>
-__device__ bool gemm_phase(const SimtStep<T>& p, const FuseGemm<T>& g, const QkvView<T>* qv, const Group& gr, Wait&& wait) {
-  constexpr int PIECE = GemmIo<T>::kPiece, PITCH = kKC + GemmIo<T>::kPad, PPR = kKC / PIECE;   // pieces per row of a chunk
-  constexpr int WR = 32 * PPR / 256, AR = 16 * PPR / 256;      // rows of W / A that a thread copies a piece of
-  constexpr int RSTEP = 256 / PPR;
-  const int chunks = (g.K + kKC - 1) / kKC, apitch = SRC == SRC_GLOBAL ? PITCH : chunks * kKC + GemmIo<T>::kPad;
-  T* ring_w = reinterpret_cast<T*>(gr.smem);                    // [stages][32][PITCH]
-  T* as = ring_w + kStages * 32 * PITCH;                        // [stages][16][PITCH], or the 16 whole rows
-  float* cs = reinterpret_cast<float*>(as + (SRC == SRC_GLOBAL ? kStages * 16 * PITCH : 16 * apitch));   // [8][16][33]
-  const int units = EPI == EPI_QKV ? (p.nq + 2 * p.nkv) * (p.hd / 32) : EPI == EPI_SWIGLU ? (g.N + 15) / 16 : (g.N + 31) / 32;
-  const int MT = (g.M + 15) / 16, tiles = MT * units;
-  const int r_t = gr.t / PPR, k_t = (gr.t % PPR) * PIECE;
+// All tiles (16 rows x 16 columns; for the epilogues that combine two features 8 and their partners) of
+// one GEMM; `wait` is the barrier in front of the phase: every thread of the CTA calls it once.  Returns
+// false if it gave up.
+//
+// A group keeps one row tile and walks through column units, so its rows are normed once; the k-chunks
+// of all of its units are one stream through the ring, so that a unit's first loads run under the
+// unit before.  Epilogue and source of A are run-time values: one piece of code serves all GEMMs of the
+// step and stays in the instruction cache (five instances of it: 5000 clocks for the first chunk of a
+// phase, 1500 for the fourth).
+template <typename T, typename Wait>
+__device__ __forceinline__ bool gemm_phase(const SimtStep<T>& p, const FuseGemm<T>& g, const QkvView<T>& qv, const Group& gr, Wait&& wait) {
+  constexpr int KC = kKC, ST = kStages, NC = 16;
+  constexpr int PIECE = GemmIo<T>::kPiece, PITCH = KC + GemmIo<T>::kPad, PPR = KC / PIECE;  // pieces per row of a chunk
+  constexpr int NP = NC * PPR / 256, RS = 256 / PPR;            // pieces of W (and of A) that a thread copies, rows apart
+  constexpr int CP = NC + 1;
+  const int chunks = (g.K + KC - 1) / KC, epi = g.epi;
+  const bool stream_a = g.src == SRC_GLOBAL;
+  const int apitch = stream_a ? PITCH : chunks * KC + GemmIo<T>::kPad;
+  T* ring_w = reinterpret_cast<T*>(gr.smem);                    // [ST][16][PITCH]
+  T* as = ring_w + ST * NC * PITCH;                             // [ST][16][PITCH], or the 16 whole rows
+  float* cs = reinterpret_cast<float*>(as + (stream_a ? ST * 16 * PITCH : 16 * apitch));   // [8][16][CP]
+  const int per_head = p.hd >> 4, half = p.hd >> 1;
+  const int units = epi == EPI_QKV ? (p.nq + 2 * p.nkv) * per_head : epi == EPI_SWIGLU ? (g.N + 7) / 8 : (g.N + NC - 1) / NC;
+  const int MT = (g.M + 15) / 16;
+  // a long K and few tiles: the two groups of a CTA take half of the chunks of one tile each
+  const bool split = chunks > 1 && MT * units <= (int)gridDim.x;
+  const int cb = split ? gr.id * (chunks / 2) : 0, ce = split && gr.id == 0 ? chunks / 2 : chunks;
+  const int vid = split ? (int)blockIdx.x : gr.vid, nv = split ? (int)gridDim.x : gr.nv;
+  const int per = MT <= nv ? nv / MT : 1;   // groups (CTAs) on a row tile
+  const int pr = gr.t / PPR, pk = (gr.t % PPR) * PIECE;         // this thread's piece of a chunk: row, column
   const int ty = gr.lane >> 3, tx = gr.lane & 7;
   bool waited = false;
-  for (int tile = gr.vid; tile < tiles || !waited; tile += gr.nv) {
-    const bool has = tile < tiles;
-    const int u = tile / MT, m0 = (tile - u * MT) * 16;
-    const T* wsrc[WR];
-    auto load_w = [&](int c) {
-      T* dst = ring_w + (size_t)(c % kStages) * 32 * PITCH;
-      const int k0 = c * kKC + k_t, bytes = max(0, min(16, (g.K - k0) * (int)sizeof(T)));
-#pragma unroll
-      for (int i = 0; i < WR; ++i)
-        cp_async16(dst + (r_t + i * RSTEP) * PITCH + k_t, wsrc[i] != nullptr && bytes ? wsrc[i] + k0 : g.w0,
-                   wsrc[i] != nullptr ? bytes : 0);
-    };
-    auto load_a = [&](int c) {
-      T* dst = as + (size_t)(c % kStages) * 16 * PITCH;
-      const int k0 = c * kKC + k_t, bytes = max(0, min(16, (g.K - k0) * (int)sizeof(T)));
-#pragma unroll
-      for (int i = 0; i < (AR > 0 ? AR : 1); ++i) {
-        const int r = r_t + i * RSTEP;
-        const bool in = m0 + r < g.M && bytes > 0;
-        cp_async16(dst + r * PITCH + k_t, in ? g.A + (size_t)(m0 + r) * g.K + k0 : g.A, in ? bytes : 0);
-      }
-    };
-    if (has) {
-#pragma unroll
-      for (int i = 0; i < WR; ++i) {
-        const int jj = r_t + i * RSTEP;
-        const T* src = nullptr;
-        if (EPI == EPI_QKV) {
-          const int half = p.hd >> 1, per_head = p.hd >> 5, head = u / per_head;
-          const int e = (u - head * per_head) * 16 + (jj & 15) + (jj >> 4) * half;
-          if (head < p.nq) src = g.w0 + (size_t)(head * p.hd + e) * g.K;
-          else if (head < p.nq + p.nkv) src = g.w1 + (size_t)((head - p.nq) * p.hd + e) * g.K;
-          else src = g.w2 + (size_t)((head - p.nq - p.nkv) * p.hd + e) * g.K;
-        } else if (EPI == EPI_SWIGLU) {
-          const int f = u * 16 + (jj & 15);
-          if (f < g.N) src = (jj < 16 ? g.w0 : g.w1) + (size_t)f * g.K;
-        } else {
-          const int n = u * 32 + jj;
-          if (n < g.N) src = g.w0 + (size_t)n * g.K;
-        }
-        wsrc[i] = src;
-      }
-      for (int c = 0; c < kStages - 1 && c < chunks; ++c) load_w(c);
-    }
-    if (!waited) {
-      if (!wait()) return false;
-      waited = true;
-    }
-    if (!has) break;
-    float old[2];   // residual values that the epilogue adds to
-    if (EPI == EPI_ADD_F32) {
-#pragma unroll
-      for (int i = 0; i < 2; ++i) {
-        const int pos = gr.t + 256 * i, r = pos >> 5, n = u * 32 + (pos & 31);
-        old[i] = (m0 + r < g.M && n < g.N) ? __ldcg(g.C + (size_t)(m0 + r) * g.ldc + n) : 0.f;
-      }
-    }
-    if (SRC == SRC_GLOBAL) {   // group c: W chunk c (all W loads so far with the first) and A chunk c
-      for (int c = 0; c < kStages - 1; ++c) {
-        if (c < chunks) load_a(c);
-        asm volatile("cp.async.commit_group;" ::: "memory");
-      }
-    } else {
-      for (int c = 0; c < kStages - 1; ++c) asm volatile("cp.async.commit_group;" ::: "memory");
 #pragma unroll 1
-      for (int i = 0; i < 2; ++i) {
-        const int r = gr.warp * 2 + i, row = m0 + r;
-        T* dst = as + (size_t)r * apitch;
-        if (SRC == SRC_LM) lm_row_to<T>(p, row, dst, chunks * kKC, u == 0, gr.lane);
-        else if (row < g.M) norm_row<T>(p.x + (size_t)row * p.d, g.gain, p.eps, p.d, dst, chunks * kKC, (T*)nullptr, (T*)nullptr, gr.lane);
-        else copy_row<T>(nullptr, p.d, dst, chunks * kKC, nullptr, gr.lane);
+  for (int mt = MT <= nv ? vid % MT : vid; !waited || mt < MT; mt += (MT <= nv ? MT : nv)) {
+    const int first = MT <= nv ? vid / MT : 0, m0 = mt * 16;
+    const int mine = (mt < MT && first < per && first < units) ? (units - first + per - 1) / per : 0;
+    const int total = mine * (ce - cb);
+    int iu = first, ic = cb, is = 0, issued = 0;   // next step to load: unit, chunk, ring slot
+    auto issue = [&](bool with_w, bool with_a, int u, int c, int s) {
+      const int k0 = c * KC + pk, full = max(0, min(16, (g.K - k0) * (int)sizeof(T)));
+#pragma unroll 1
+      for (int i = 0; i < NP; ++i) {
+        const int r = pr + i * RS;
+        if (with_w) {
+          const T* w = g.w0;
+          int n = u * NC + r, N = g.N;
+          if (epi == EPI_QKV) {
+            const int head = u / per_head, e = (u - head * per_head) * 8 + (r & 7) + (r >> 3) * half;
+            const int hh = head < p.nq ? head : head < p.nq + p.nkv ? head - p.nq : head - p.nq - p.nkv;
+            w = head < p.nq ? g.w0 : head < p.nq + p.nkv ? g.w1 : g.w2;
+            n = hh * p.hd + e; N = n + 1;
+          } else if (epi == EPI_SWIGLU) {
+            n = u * 8 + (r & 7);
+            if (r >= 8) w = g.w1;
+          }
+          const int bytes = n < N ? full : 0;
+          cp_async16(ring_w + ((size_t)s * NC + r) * PITCH + pk, bytes ? w + (size_t)n * g.K + k0 : g.w0, bytes);
+        }
+        if (with_a && stream_a) {
+          const int bytes = m0 + r < g.M ? full : 0;
+          cp_async16(as + ((size_t)s * 16 + r) * PITCH + pk, bytes ? g.A + (size_t)(m0 + r) * g.K + k0 : g.A, bytes);
+        }
+      }
+    };
+    const bool before = !waited;   // the weights of the first steps are on their way while the CTA waits
+    if (!before) gsync(gr);        // the rows of the tile before have been read
+#pragma unroll 1
+    for (int pass = before ? 0 : 1; pass < 2; ++pass) {
+      if (pass == 1 && before) {
+        if (!wait()) return false;
+        waited = true;
+      }
+      iu = first; ic = cb; is = 0; issued = 0;
+#pragma unroll 1
+      for (int s = 0; s < ST - 1; ++s) {
+        if (issued < total) {
+          issue(pass == 0 || !before, pass == 1, iu, ic, is);
+          if (++ic == ce) { ic = cb; iu += per; }
+          ++is; ++issued;
+        }
+        if (pass == 1) asm volatile("cp.async.commit_group;" ::: "memory");
       }
     }
-    f2 acc[4][4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) acc[i][j] = 0ull;
-    for (int c = 0; c < chunks; ++c) {
-      asm volatile("cp.async.wait_group %0;" ::"n"(kStages - 2) : "memory");
-      gsync(gr);               // chunk c has landed for every thread; the stage of chunk c - 1 is free
-      if (c + kStages - 1 < chunks) {
-        load_w(c + kStages - 1);
-        if (SRC == SRC_GLOBAL) load_a(c + kStages - 1);
+    if (total == 0) continue;
+    if (!stream_a) {
+      const int r = gr.warp * 2 + (gr.lane >> 4), row = m0 + r;
+      T* dst = as + (size_t)r * apitch;
+      const float* xr = nullptr;
+      T *g0 = nullptr, *g1 = nullptr;
+      bool norm = true;
+      if (g.src == SRC_LM) norm = lm_row<T>(p, row, dst, chunks * KC, first == 0, gr.lane & 15, xr, g0, g1);
+      else if (row < g.M) xr = p.x + (size_t)row * p.d;
+      if (__any_sync(0xffffffffu, norm || g1 != nullptr))       // both halves of the warp take part
+        norm_row<T>(xr, g.gain, p.eps, p.d, norm ? dst : nullptr, chunks * KC, g0, g1, gr.lane & 15);
+    }
+    f2 acc[4][2];
+    float old = 0.f;             // residual value that the epilogue adds to
+    int u = first, c = cb, slot = 0;
+#pragma unroll 1
+    for (int step = 0; step < total; ++step) {
+      asm volatile("cp.async.wait_group %0;" ::"n"(ST - 2) : "memory");
+      gsync(gr);                 // this step's chunk has landed for every thread; the slot of the last one is free
+      if (issued < total) {
+        issue(true, true, iu, ic, is);
+        if (++ic == ce) { ic = cb; iu += per; }
+        if (++is == ST) is = 0;
+        ++issued;
       }
       asm volatile("cp.async.commit_group;" ::: "memory");
-      const T* wp = ring_w + (size_t)(c % kStages) * 32 * PITCH + tx * PITCH + gr.warp * (kKC / 8);
-      const T* ap = (SRC == SRC_GLOBAL ? as + (size_t)(c % kStages) * 16 * PITCH : as + c * kKC) + ty * 4 * apitch + gr.warp * (kKC / 8);
+      const int er = gr.t >> 4, ec = gr.t & 15;                 // the epilogue's element of this thread
+      if (c == cb) {
 #pragma unroll
-      for (int k = 0; k < kKC / 8; k += 4) {
-        f2 av[4][2], wv[4][2];
+        for (int i = 0; i < 4; ++i) acc[i][0] = acc[i][1] = 0ull;
+        if (epi == EPI_ADD_F32 && m0 + er < g.M && u * NC + ec < g.N) old = __ldcg(g.C + (size_t)(m0 + er) * g.ldc + u * NC + ec);
+      }
+      const T* wp = ring_w + ((size_t)slot * NC + tx) * PITCH + gr.warp * (KC / 8);
+      const T* ap = (stream_a ? as + (size_t)slot * 16 * PITCH : as + c * KC) + ty * 4 * apitch + gr.warp * (KC / 8);
+#pragma unroll 2
+      for (int k = 0; k < KC / 8; k += 4) {
+        f2 av[4][2], wv[2][2];
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
           float v[4];
           load4<T>(ap + i * apitch + k, v);
           av[i][0] = pack2(v[0], v[1]); av[i][1] = pack2(v[2], v[3]);
-          load4<T>(wp + i * 8 * PITCH + k, v);
-          wv[i][0] = pack2(v[0], v[1]); wv[i][1] = pack2(v[2], v[3]);
+        }
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+          float v[4];
+          load4<T>(wp + j * 8 * PITCH + k, v);
+          wv[j][0] = pack2(v[0], v[1]); wv[j][1] = pack2(v[2], v[3]);
         }
 #pragma unroll
         for (int i = 0; i < 4; ++i)
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
+          for (int j = 0; j < 2; ++j) {
             fma2(acc[i][j], av[i][0], wv[j][0]);
             fma2(acc[i][j], av[i][1], wv[j][1]);
           }
       }
-    }
+      if (++slot == ST) slot = 0;
+      if (++c < ce) continue;
+      c = cb;
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+      for (int i = 0; i < 4; ++i)
 #pragma unroll
-      for (int j = 0; j < 4; ++j) cs[(gr.warp * 16 + ty * 4 + i) * kCsPitch + tx + 8 * j] = sum2(acc[i][j]);
-    gsync(gr);                 // the sums are there, and the ring and the rows have been read
-    auto value = [&](int r, int c) {
-      float v = cs[r * kCsPitch + c];
+        for (int j = 0; j < 2; ++j) cs[(gr.warp * 16 + ty * 4 + i) * CP + tx + 8 * j] = sum2(acc[i][j]);
+      float y = 0.f;
+      if (split) {     // (one tile per CTA, so the sums are not overwritten)
+        asm volatile("bar.sync 3, %0;" ::"n"(kFuseThreads) : "memory");
+        if (gr.id != 0) break;
+        const float* ct = cs + p.group_smem / (int)sizeof(float);
 #pragma unroll
-      for (int w = 1; w < 8; ++w) v += cs[(w * 16 + r) * kCsPitch + c];
-      return v;
-    };
-    if (EPI == EPI_STORE_F32 || EPI == EPI_ADD_F32) {
-#pragma unroll
-      for (int i = 0; i < 2; ++i) {
-        const int pos = gr.t + 256 * i, r = pos >> 5, c = pos & 31, n = u * 32 + c;
-        if (m0 + r < g.M && n < g.N) g.C[(size_t)(m0 + r) * g.ldc + n] = EPI == EPI_ADD_F32 ? old[i] + value(r, c) : value(r, c);
+        for (int w = 0; w < 8; ++w) y += ct[(w * 16 + er) * CP + ec];
+      } else {
+        gsync(gr);
       }
-    } else {
-      const int r = gr.t >> 4, i = gr.t & 15, m = m0 + r;
-      if (m < g.M) {
-        const float y1 = value(r, i), y2 = value(r, 16 + i);
-        if (EPI == EPI_SWIGLU) {
-          const int f = u * 16 + i;
-          if (f < g.N) g.act[(size_t)m * g.N + f] = from_f<T>(y1 / (1.f + expf(-y1)) * y2);
-        } else {
-          const int per_head = p.hd >> 5, head = u / per_head;
-          simt_store_qkv<T>(*qv, m, head, (u - head * per_head) * 16 + i, y1, y2);
+#pragma unroll
+      for (int w = 0; w < 8; ++w) y += cs[(w * 16 + er) * CP + ec];
+      const int m = m0 + er;
+      if (epi <= EPI_ADD_F32) {
+        if (m < g.M && u * NC + ec < g.N) g.C[(size_t)m * g.ldc + u * NC + ec] = epi == EPI_ADD_F32 ? old + y : y;
+      } else {
+        const float y2 = __shfl_down_sync(0xffffffffu, y, 8);   // the partner feature's column
+        if (ec < 8 && m < g.M) {
+          if (epi == EPI_SWIGLU) {
+            const int f = u * 8 + ec;
+            if (f < g.N) g.act[(size_t)m * g.N + f] = from_f<T>(y / (1.f + expf(-y)) * y2);
+          } else {
+            const int head = u / per_head;
+            simt_store_qkv<T>(qv, m, head, (u - head * per_head) * 8 + ec, y, y2);
+          }
         }
       }
+      u += per;
     }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
   }
   return true;
 }
 
-// Bidirectional attention: a unit is 8 query rows of one head and variant, a row per warp.  Tiles of
-// p.kt keys arrive in two buffers as they lie in memory (cached V transposed, active V row-major).
+// Bidirectional attention: a unit is 4 query rows of one head and variant, two warps per row with half of
+// the keys of every tile each.  (It is bound by shared-memory reads, every warp reads its keys' K and V:
+// with a row per warp and all keys a tile of 64 keys took 6300 clocks.)  Tiles of p.kt keys arrive in two
+// buffers as they lie in memory (cached V transposed, active V row-major).
 template <typename T, typename Wait>
 __device__ bool attn_phase(const SimtStep<T>& p, int layer, const Group& gr, Wait&& wait) {
   constexpr int PIECE = GemmIo<T>::kPiece;
@@ -303,14 +339,18 @@ __device__ bool attn_phase(const SimtStep<T>& p, int layer, const Group& gr, Wai
   const int vbuf = max(kt * kp, hd * vp);
   T* kb = reinterpret_cast<T*>(gr.smem);             // [2][kt][kp]
   T* vb = kb + 2 * kt * kp;                          // [2][vbuf]
-  float* qs = reinterpret_cast<float*>(vb + 2 * vbuf) + gr.warp * (hd + kt);   // this warp's query row, then its probabilities
+  float* qs = reinterpret_cast<float*>(vb + 2 * vbuf) + gr.warp * (hd + 32);   // this warp's query row, then its probabilities
   float* ps = qs + hd;
-  const int nrt = (m.R_cap + 7) / 8, units = nrt * p.nq * m.nv * m.batch, ld = p.nkv * hd;
+  float* other = reinterpret_cast<float*>(vb + 2 * vbuf) + (gr.warp ^ 1) * (hd + 32);
+  const int kw = kt / 2, kb0 = (gr.warp & 1) * kw;              // this warp's keys of a tile (32 or 16)
+  const int nrt = (m.R_cap + 3) / 4, units = nrt * p.nq * m.nv * m.batch, ld = p.nkv * hd;
+  const int hq = hd / PIECE, kj = gr.t / hq, kq0 = gr.t % hq;   // this thread's first piece of a K tile
   const float scale = rsqrtf((float)hd);
   bool waited = false;
+#pragma unroll 1
   for (int unit = gr.vid; unit < units || !waited; unit += gr.nv) {
     const bool has = unit < units;
-    const int vbi = unit / (nrt * p.nq), rem = unit - vbi * nrt * p.nq, h = rem / nrt, r0 = (rem - h * nrt) * 8;
+    const int vbi = unit / (nrt * p.nq), rem = unit - vbi * nrt * p.nq, h = rem / nrt, r0 = (rem - h * nrt) * 4;
     const int b = has ? vbi % m.batch : 0, vv = vbi / m.batch;
     const int P = m.ctx_len[b], R = m.last_len[b] + m.win_len[b], kvh = h / (p.nq / p.nkv);
     const int row0 = act_row(m, vv, b, 0);
@@ -319,11 +359,13 @@ __device__ bool attn_phase(const SimtStep<T>& p, int layer, const Group& gr, Wai
     auto load = [&](int t) {
       if (t < nt) {
         const bool ctx = t < tc;
-        const int j0 = (ctx ? t : t - tc) * kt, n = min(kt, (ctx ? P : R) - j0), hq = hd / PIECE;
+        const int j0 = (ctx ? t : t - tc) * kt, n = min(kt, (ctx ? P : R) - j0);
         T* kd = kb + (size_t)(t & 1) * kt * kp;
         T* vd = vb + (size_t)(t & 1) * vbuf;
-        for (int i = gr.t; i < kt * hq; i += 256) {
-          const int j = i / hq, e = (i - j * hq) * PIECE;
+#pragma unroll 1
+        for (int j = kj, q = kq0; j < kt; j += 256 / hq, q += 256 % hq) {
+          if (q >= hq) { q -= hq; if (++j >= kt) break; }
+          const int e = q * PIECE;
           const T* src = ctx ? p.k_cache + kv + (size_t)(j0 + j) * hd + e : p.k + (size_t)(row0 + j0 + j) * ld + kvh * hd + e;
           cp_async16(kd + j * kp + e, j < n ? src : p.k, j < n ? 16 : 0);
           if (!ctx) {
@@ -333,8 +375,9 @@ __device__ bool attn_phase(const SimtStep<T>& p, int layer, const Group& gr, Wai
         }
         if (ctx) {   // keys are contiguous; what the cache holds beyond ctx_len is not read
           const int kq = kt / PIECE;
-          for (int i = gr.t; i < hd * kq; i += 256) {
-            const int e = i / kq, j = (i - e * kq) * PIECE, bytes = max(0, min(16, (n - j) * (int)sizeof(T)));
+#pragma unroll 1
+          for (int e = gr.t / kq; e < hd; e += 256 / kq) {   // kq is a power of two
+            const int j = (gr.t % kq) * PIECE, bytes = max(0, min(16, (n - j) * (int)sizeof(T)));
             cp_async16(vd + e * vp + j, bytes ? p.v_cache + kv + (size_t)e * p.max_ctx + j0 + j : p.v, bytes);
           }
         }
@@ -350,7 +393,7 @@ __device__ bool attn_phase(const SimtStep<T>& p, int layer, const Group& gr, Wai
     if (!has) break;
     if (nt == 0) continue;
     if (!early) load(0);
-    const int row = r0 + gr.warp;
+    const int row = r0 + (gr.warp >> 1);
     const bool live = row < R;
     if (live)
       for (int e = gr.lane * 4; e < hd; e += 128) {
@@ -359,6 +402,7 @@ __device__ bool attn_phase(const SimtStep<T>& p, int layer, const Group& gr, Wai
         *reinterpret_cast<float4*>(qs + e) = make_float4(v[0], v[1], v[2], v[3]);
       }
     float mx = -INFINITY, sum = 0.f, o[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 1
     for (int t = 0; t < nt; ++t) {
       load(t + 1);
       asm volatile("cp.async.wait_group 1;" ::: "memory");
@@ -368,75 +412,73 @@ __device__ bool attn_phase(const SimtStep<T>& p, int layer, const Group& gr, Wai
         const int n = min(kt, ctx ? P - t * kt : R - (t - tc) * kt);
         const T* kd = kb + (size_t)(t & 1) * kt * kp;
         const T* vd = vb + (size_t)(t & 1) * vbuf;
-        float tm = -INFINITY;
-        for (int j = gr.lane; j < kt; j += 32) {   // one key per lane and step
-          float s = -INFINITY;
-          if (j < n) {
-            float a0 = 0.f, a1 = 0.f;
-            const T* kr = kd + j * kp;
+        const int key = kb0 + gr.lane;                          // one key per lane
+        const bool mine = gr.lane < kw && key < n;
+        const T* kr = kd + (gr.lane < kw ? key : kb0) * kp;
+        float a0 = 0.f, a1 = 0.f;
 #pragma unroll 4
-            for (int e = 0; e < hd; e += 4) {
-              float x[4];
-              load4<T>(kr + e, x);
-              const float4 qv = *reinterpret_cast<const float4*>(qs + e);
-              a0 = fmaf(qv.x, x[0], a0); a1 = fmaf(qv.y, x[1], a1); a0 = fmaf(qv.z, x[2], a0); a1 = fmaf(qv.w, x[3], a1);
-            }
-            s = (a0 + a1) * scale;
-          }
-          ps[j] = s;
-          tm = fmaxf(tm, s);
+        for (int e = 0; e < hd; e += 4) {
+          float x[4];
+          load4<T>(kr + e, x);
+          const float4 qv = *reinterpret_cast<const float4*>(qs + e);
+          a0 = fmaf(qv.x, x[0], a0); a1 = fmaf(qv.y, x[1], a1); a0 = fmaf(qv.z, x[2], a0); a1 = fmaf(qv.w, x[3], a1);
         }
-        const float nm = fmaxf(mx, warp_max(tm)), corr = expf(mx - nm);   // 0 on the first tile
-        float ts = 0.f;
-        for (int j = gr.lane; j < kt; j += 32) {
-          const float e = expf(ps[j] - nm);
-          ps[j] = e;
-          ts += e;
-        }
-        sum = sum * corr + warp_sum(ts);
+        const float s0 = mine ? (a0 + a1) * scale : -INFINITY;
+        const float nm = fmaxf(mx, warp_max(s0));
+        // (a warp may have no valid key so far: its reference point is still -inf, its sums are 0)
+        const float corr = nm > -INFINITY ? expf(mx - nm) : 1.f, e0 = mine ? expf(s0 - nm) : 0.f;
+        __syncwarp();
+        ps[gr.lane] = e0;
+        sum = sum * corr + warp_sum(e0);
         mx = nm;
         __syncwarp();
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const int e = gr.lane + 32 * i;
-          if (e < hd) {
-            float x0 = 0.f, x1 = 0.f;
-            if (ctx) {
-              const T* vr = vd + e * vp;
-#pragma unroll 4
-              for (int j = 0; j < kt; j += 4) {
-                float w[4];
-                load4<T>(vr + j, w);
-                const float4 pv = *reinterpret_cast<const float4*>(ps + j);
-                x0 = fmaf(pv.x, w[0], x0); x1 = fmaf(pv.y, w[1], x1); x0 = fmaf(pv.z, w[2], x0); x1 = fmaf(pv.w, w[3], x1);
-              }
-            } else {
-#pragma unroll 8
-              for (int j = 0; j < kt; j += 2) {
-                x0 = fmaf(ps[j], to_f<T>(vd[j * kp + e]), x0);
-                x1 = fmaf(ps[j + 1], to_f<T>(vd[(j + 1) * kp + e]), x1);
-              }
+        for (int i = 0; i < 4; ++i) o[i] *= corr;
+        // features lane, lane + 32, ..: cached V has the keys contiguous, active V the features
+        const T* vr = ctx ? vd + gr.lane * vp + kb0 : vd + kb0 * kp + gr.lane;
+#pragma unroll 2
+        for (int j = 0; j < kw; j += 4) {
+          const float4 pv = *reinterpret_cast<const float4*>(ps + j);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            if (32 * i >= hd) break;
+            float w[4];
+            if (ctx) load4<T>(vr + 32 * i * vp + j, w);
+            else {
+#pragma unroll
+              for (int c = 0; c < 4; ++c) w[c] = to_f<T>(vr[(j + c) * kp + 32 * i]);
             }
-            o[i] = o[i] * corr + (x0 + x1);
+            o[i] = fmaf(pv.x, w[0], o[i]); o[i] = fmaf(pv.y, w[1], o[i]); o[i] = fmaf(pv.z, w[2], o[i]); o[i] = fmaf(pv.w, w[3], o[i]);
           }
         }
       }
       gsync(gr);
     }
     asm volatile("cp.async.wait_group 0;" ::: "memory");
-    if (live) {
-      const float inv = 1.f / sum;
+    // the two halves of a row meet: the odd warp leaves its sums where its query row was
+    if (gr.warp & 1) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        if (32 * i < hd) qs[gr.lane + 32 * i] = o[i];
+      if (gr.lane == 0) { ps[0] = mx; ps[1] = sum; }
+    }
+    gsync(gr);
+    if (live && !(gr.warp & 1)) {
+      const float m2 = other[hd], s2 = other[hd + 1], top = fmaxf(mx, m2);
+      const float c1 = expf(mx - top), c2 = m2 > -INFINITY ? expf(m2 - top) : 0.f;   // (this warp has the first key)
+      const float inv = 1.f / (sum * c1 + s2 * c2);
       T* dst = p.o + (size_t)(row0 + row) * p.nq * hd + (size_t)h * hd;
 #pragma unroll
       for (int i = 0; i < 4; ++i)
-        if (gr.lane + 32 * i < hd) dst[gr.lane + 32 * i] = from_f<T>(o[i] * inv);
+        if (32 * i < hd) dst[gr.lane + 32 * i] = from_f<T>((o[i] * c1 + other[gr.lane + 32 * i] * c2) * inv);
     }
+    gsync(gr);
   }
   return true;
 }
 
 // Cross log-probs (Eq. 6 halves): xlogp[b,i,j] = h_i . W_lm[yhat_j] - lse_i.  A unit is a column j and 16
-// rows; every warp keeps its part of W_lm[yhat_j] in registers.
+// rows, two per warp.
 template <typename T>
 __device__ __forceinline__ void xlogp_phase(const SimtStep<T>& p, const Group& gr) {
   const SeqMeta& m = p.ml;
@@ -446,27 +488,27 @@ __device__ __forceinline__ void xlogp_phase(const SimtStep<T>& p, const Group& g
     if (j >= W) continue;
     const int tok = __ldcg(p.sig.ws_pred + b * m.W_cap + j);
     const bool ok = tok >= 0 && tok < p.V;   // never index the vocabulary matrix with an id outside it
-    float w[kMaxNormD / 128][4];
+    const T* wr = p.lm_head + (size_t)(ok ? tok : 0) * p.d;
+    const int i0 = (unit - bj * it) * 16 + gr.warp * 2;
+    if (i0 >= W) continue;
+    const bool two = i0 + 1 < W;
+    const T* h0 = p.h + (size_t)lm_row(m, 0, b * m.W_cap + i0) * p.d;
+    const T* h1 = p.h + (size_t)lm_row(m, 0, b * m.W_cap + i0 + (two ? 1 : 0)) * p.d;
+    float a0 = 0.f, a1 = 0.f;
+#pragma unroll 2
+    for (int e = gr.lane * 4; e < p.d; e += 128) {
+      float w[4], x[4], y[4];
+      load4<T>(wr + e, w);
+      ldcg4<T>(h0 + e, x);
+      ldcg4<T>(h1 + e, y);
 #pragma unroll
-    for (int i = 0; i < kMaxNormD / 128; ++i)
-      if (ok && gr.lane * 4 + 128 * i < p.d) load4<T>(p.lm_head + (size_t)tok * p.d + gr.lane * 4 + 128 * i, w[i]);
-#pragma unroll
-    for (int r = 0; r < 2; ++r) {
-      const int i0 = (unit - bj * it) * 16 + gr.warp * 2 + r;
-      if (i0 >= W) continue;
-      const T* hr = p.h + (size_t)lm_row(m, 0, b * m.W_cap + i0) * p.d;
-      float acc = 0.f;
-#pragma unroll
-      for (int i = 0; i < kMaxNormD / 128; ++i)
-        if (gr.lane * 4 + 128 * i < p.d) {
-          float hv[4];
-          ldcg4<T>(hr + gr.lane * 4 + 128 * i, hv);
-#pragma unroll
-          for (int c = 0; c < 4; ++c) acc = fmaf(hv[c], ok ? w[i][c] : 0.f, acc);
-        }
-      acc = warp_sum(acc);
-      if (gr.lane == 0)
-        p.xlogp[((size_t)b * p.max_window + i0) * p.max_window + j] = ok ? acc - __ldcg(p.sig.ws_lse + b * m.W_cap + i0) : -INFINITY;
+      for (int c = 0; c < 4; ++c) { a0 = fmaf(x[c], w[c], a0); a1 = fmaf(y[c], w[c], a1); }
+    }
+    a0 = warp_sum(a0); a1 = warp_sum(a1);
+    if (gr.lane < (two ? 2 : 1)) {
+      const int i = i0 + gr.lane;
+      p.xlogp[((size_t)b * p.max_window + i) * p.max_window + j] =
+          ok ? (gr.lane ? a1 : a0) - __ldcg(p.sig.ws_lse + b * m.W_cap + i) : -INFINITY;
     }
   }
 }
@@ -518,25 +560,36 @@ __global__ void __launch_bounds__(kFuseThreads, 1) k_simt_step(const __grid_cons
     return go != 0;
   };
 
-  const int M = p.m.nv * p.m.batch * p.m.R_cap;
-  for (int l = 0; l < p.n_layers; ++l) {
-    const SimtLayer<T> L = p.layers[l];
+  const int M = p.m.nv * p.m.batch * p.m.R_cap, n_phases = 5 * p.n_layers;
+#pragma unroll 1
+  for (int ph = 0; ph <= n_phases; ++ph) {
+    const int l = ph / 5, kind = ph == n_phases ? 5 : ph - 5 * l;   // QKV, attention, O, gate / up, down; LM head
+    if (ph > 0) arrive();
+    if (kind == 1) {
+      if (!attn_phase<T>(p, l, gr, wait)) return;
+      continue;
+    }
+    const SimtLayer<T>* L = p.layers + l;
     const size_t cache = (size_t)l * p.cache_layer;
-    const QkvView<T> qv{p.m, p.nq, p.nkv, p.hd, p.max_ctx, p.cos_sin, L.bq, L.bk, L.bv, p.q, p.k, p.v,
-                        p.export_kv ? p.k_cache + cache : nullptr, p.export_kv ? p.v_cache + cache : nullptr};
-    if (!gemm_phase<T, EPI_QKV, SRC_NORM>(p, FuseGemm<T>{nullptr, L.wq, L.wk, L.wv, L.n1, M, 0, p.d, 0, nullptr, nullptr}, &qv, gr, wait)) return;
-    if (p.kv_only && l + 1 == p.n_layers) return;
-    arrive();
-    if (!attn_phase<T>(p, l, gr, wait)) return;
-    arrive();
-    if (!gemm_phase<T, EPI_ADD_F32, SRC_GLOBAL>(p, FuseGemm<T>{p.o, L.wo, nullptr, nullptr, nullptr, M, p.d, p.nq * p.hd, p.d, p.x, nullptr}, nullptr, gr, wait)) return;
-    arrive();
-    if (!gemm_phase<T, EPI_SWIGLU, SRC_NORM>(p, FuseGemm<T>{nullptr, L.wg, L.wu, nullptr, L.n2, M, p.F, p.d, 0, nullptr, p.act}, nullptr, gr, wait)) return;
-    arrive();
-    if (!gemm_phase<T, EPI_ADD_F32, SRC_GLOBAL>(p, FuseGemm<T>{p.act, L.wd, nullptr, nullptr, nullptr, M, p.d, p.F, p.d, p.x, nullptr}, nullptr, gr, wait)) return;
-    arrive();
+    QkvView<T> qv{p.m, p.nq, p.nkv, p.hd, p.max_ctx, p.cos_sin, nullptr, nullptr, nullptr, p.q, p.k, p.v,
+                  p.export_kv ? p.k_cache + cache : nullptr, p.export_kv ? p.v_cache + cache : nullptr};
+    FuseGemm<T> g{nullptr, nullptr, nullptr, nullptr, nullptr, M, p.d, p.d, p.d, p.x, p.act, EPI_ADD_F32, SRC_GLOBAL};
+    if (kind == 0) {
+      g.w0 = L->wq; g.w1 = L->wk; g.w2 = L->wv; g.gain = L->n1; g.epi = EPI_QKV; g.src = SRC_NORM;
+      qv.bq = L->bq; qv.bk = L->bk; qv.bv = L->bv;
+    } else if (kind == 2) {
+      g.A = p.o; g.w0 = L->wo; g.K = p.nq * p.hd;
+    } else if (kind == 3) {
+      g.w0 = L->wg; g.w1 = L->wu; g.gain = L->n2; g.N = p.F; g.epi = EPI_SWIGLU; g.src = SRC_NORM;
+    } else if (kind == 4) {
+      g.A = p.act; g.w0 = L->wd; g.K = p.F;
+    } else {
+      g.w0 = p.lm_head; g.gain = p.final_norm; g.M = p.ml.nv * p.ml.npos_pad; g.N = p.V; g.C = p.logits; g.ldc = p.V;
+      g.epi = EPI_STORE_F32; g.src = SRC_LM;
+    }
+    if (!gemm_phase<T>(p, g, qv, gr, wait)) return;
+    if (p.kv_only && ph == n_phases - 5) return;   // prefill: nothing after the last layer's K / V is used
   }
-  if (!gemm_phase<T, EPI_STORE_F32, SRC_LM>(p, FuseGemm<T>{nullptr, p.lm_head, nullptr, nullptr, p.final_norm, p.ml.nv * p.ml.npos_pad, p.V, p.d, p.V, p.logits, nullptr}, nullptr, gr, wait)) return;
   arrive();
   if (!wait()) return;
   for (int pos = gr.vid; pos < p.ml.batch * p.ml.W_cap; pos += gr.nv) {
@@ -548,17 +601,17 @@ __global__ void __launch_bounds__(kFuseThreads, 1) k_simt_step(const __grid_cons
   if (p.xlogp != nullptr) xlogp_phase<T>(p, gr);
   if (p.bnd.block_len != nullptr && gr.id == 0 && gr.warp == 0)   // the SMs that get the fewest cross log-prob units
     for (int b = gridDim.x - 1 - blockIdx.x; b < p.ml.batch; b += gridDim.x)
-      boundary_seq<DC_MAX_WINDOW / 32>(p.sig.ws_infl, p.sig.ws_ent, b, p.ml, DevLens{}, p.hp, p.bnd, bnd[0], bnd[1]);
+      if (p.max_window <= 64) boundary_seq<2>(p.sig.ws_infl, p.sig.ws_ent, b, p.ml, DevLens{}, p.hp, p.bnd, bnd[0], bnd[1]);
+      else boundary_seq<DC_MAX_WINDOW / 32>(p.sig.ws_infl, p.sig.ws_ent, b, p.ml, DevLens{}, p.hp, p.bnd, bnd[0], bnd[1]);
 }
 
 template <typename T>
 size_t group_smem(int d, int hd, int kt) {
   const size_t pitch = kKC + GemmIo<T>::kPad, rows = (size_t)(d + kKC - 1) / kKC * kKC + GemmIo<T>::kPad;
-  const size_t a = 16 * (kStages * pitch > rows ? kStages * pitch : rows);
-  const size_t gemm = (kStages * 32 * pitch + a) * sizeof(T) + 8 * 16 * kCsPitch * sizeof(float);
+  const size_t gemm = 16 * (kStages * pitch + (kStages * pitch > rows ? kStages * pitch : rows)) * sizeof(T) + 8 * 16 * 17 * sizeof(float);
   const size_t kp = hd + GemmIo<T>::kPiece, vp = kt + GemmIo<T>::kPiece;
   const size_t vb = kt * kp > hd * vp ? kt * kp : hd * vp;
-  const size_t attn = 2 * (kt * kp + vb) * sizeof(T) + 8 * (size_t)(hd + kt) * sizeof(float);
+  const size_t attn = 2 * (kt * kp + vb) * sizeof(T) + 8 * (size_t)(hd + 32) * sizeof(float);
   return ((gemm > attn ? gemm : attn) + 127) / 128 * 128;
 }
 
@@ -577,17 +630,24 @@ bool simt_step_init(SimtFuse* f, int d, int F, int nq, int nkv, int hd, int voca
     f->group_smem = (int)group_smem<T>(d, hd, f->kt);
   }
   if ((size_t)f->group_smem > kGroupSmemMax) return true;
-  int dev = 0, coop = 0, sms = 0, per_sm = 0;
+  // the answer is the device's, not the context's: asked once (a racing context finds the same)
+  static std::atomic<int> sms_of[64];
+  int dev = 0, sms = 0, coop = 0;
   cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (!coop || sms < 1) return true;
-  if (cudaFuncSetAttribute(k_simt_step<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kGroups * kGroupSmemMax)) != cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_simt_step<T>, kFuseThreads, kGroups * f->group_smem) != cudaSuccess) {
-    cudaGetLastError();
-    return false;
+  if (dev < 64) sms = sms_of[dev].load(std::memory_order_acquire);
+  if (sms == 0) {
+    cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    int per_sm = 0;
+    if (cudaFuncSetAttribute(k_simt_step<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kGroups * kGroupSmemMax)) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_simt_step<T>, kFuseThreads, kGroups * kGroupSmemMax) != cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
+    if (!coop || sms < 1 || per_sm < 1) sms = -1;
+    if (dev < 64) sms_of[dev].store(sms, std::memory_order_release);
   }
-  if (per_sm >= 1) f->grid = sms;
+  if (sms > 0) f->grid = sms;
   return true;
 }
 
@@ -597,8 +657,8 @@ bool simt_step_ok(const SimtFuse& f, const SimtStep<T>& p) {
   // GEMMs that take many rounds of small tiles are better off as kernels of their own, with the larger tile
   const long long M = (long long)p.m.nv * p.m.batch * p.m.R_cap, Mlm = (long long)p.ml.nv * p.ml.npos_pad;
   const long long mt = (M + 15) / 16;
-  long long most = mt * ((p.F + 15) / 16);
-  const long long qkv = mt * (p.nq + 2 * p.nkv) * (p.hd / 32), lm = p.kv_only ? 0 : (Mlm + 15) / 16 * ((p.V + 31) / 32);
+  long long most = mt * ((p.F + 7) / 8);
+  const long long qkv = mt * (p.nq + 2 * p.nkv) * (p.hd / 16), lm = p.kv_only ? 0 : (Mlm + 15) / 16 * ((p.V + 15) / 16);
   most = most > qkv ? most : qkv;
   most = most > lm ? most : lm;
   return most <= kFuseMaxTiles;
