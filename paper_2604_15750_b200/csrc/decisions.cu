@@ -9,6 +9,7 @@
 #include <type_traits>
 
 #include "decisions.cuh"
+#include "pdl.cuh"
 
 namespace dc {
 
@@ -19,6 +20,8 @@ __global__ void __launch_bounds__(32 * kSeqWarps) k_boundary(const float* influe
                                                              const __grid_constant__ SeqMeta m, DevLens dl, Hyper hp,
                                                              BoundaryIo io) {
   __shared__ float sI[kSeqWarps][33 * NQ], sH[kSeqWarps][33 * NQ];
+  pdl_trigger();
+  pdl_wait();
   const int w = threadIdx.x >> 5, b = blockIdx.x * (blockDim.x >> 5) + w;
   if (b < batch) boundary_seq<NQ>(influence, entropy, b, m, dl, hp, io, sI[w], sH[w]);
 }
@@ -38,7 +41,7 @@ static void boundary(const float* influence, const float* entropy, int ld, int b
                      int32_t* block_len, cudaStream_t s) {
   const BoundaryIo io = make_boundary_io(influence, entropy, ld, max_window, score, cum_i, cum_s, block_len);
   decide_launch(batch, max_window, [&](auto nq, dim3 grid, int threads) {
-    k_boundary<decltype(nq)::value><<<grid, threads, 0, s>>>(influence, entropy, batch, m, dl, hp, io);
+    launch_chained(k_boundary<decltype(nq)::value>, grid, threads, 0, s, influence, entropy, batch, m, dl, hp, io);
   });
 }
 
@@ -142,6 +145,7 @@ __global__ void __launch_bounds__(32 * kSeqWarps, 5) k_select(
   __shared__ __align__(16) int members[kSeqWarps][32 * NQ + NA];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int b = blockIdx.x * (blockDim.x >> 5) + w;
+  pdl_wait();
   if (b >= batch) return;
   const int W = len_of(dl.win_len, m.win_len, b);
   const int kept = cm.win_ids != nullptr ? cm.keep.n[b] : -1;   // the length of a block that a generation is in the middle of
@@ -228,8 +232,8 @@ static void select(const float* conf, const int32_t* win_ids, const float* xlogp
                    uint8_t* sel_mask, int32_t* sel_idx, int32_t* sel_count, cudaStream_t s,
                    const SelectCommit& cm = SelectCommit{}) {
   decide_launch(batch, max_window, [&](auto nq, dim3 grid, int threads) {
-    k_select<decltype(nq)::value><<<grid, threads, 0, s>>>(conf, win_ids, xlogp, block_len, batch, m, dl, hp, mask_id,
-                                                           max_window, sel_mask, sel_idx, sel_count, cm);
+    launch_chained(k_select<decltype(nq)::value>, grid, threads, 0, s, conf, win_ids, xlogp, block_len, batch, m, dl, hp,
+                   mask_id, max_window, sel_mask, sel_idx, sel_count, cm);
   });
 }
 

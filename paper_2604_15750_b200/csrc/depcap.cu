@@ -279,7 +279,7 @@ int run_step(dc_ctx* c, const dc_step_in* in, const dc_step_out* out, const SeqM
       const bool last = l + 1 == L;
       pf.begin(DC_STAGE_ATTN, 1);
       rc = tc_attention(c->tc, l, m, (const __nv_bfloat16*)in->k_cache,
-                        (const __nv_bfloat16*)in->v_cache, export_kv, kv_only && last);
+                        (const __nv_bfloat16*)in->v_cache, export_kv, kv_only && last, false);
       pf.end();
       if (rc != DC_OK) return fail(c, rc, "attention failed: %s", tc_error(c->tc));
       if (kv_only && last) break;   // prefill: nothing after the last layer's K / V is used
@@ -618,7 +618,7 @@ int dc_create(const dc_config* cfg, const dc_weights* w, void* cuda_stream, dc_c
       if (c->fuse.grid == 0) return true;
       c->simt_bar = ws_alloc<unsigned int>(c, 2, &ok);
       c->simt_layers = ws_alloc<SimtLayer<T>>(c, g.n_layers, &ok);
-      return ok && (g.n_layers == 0 || cudaMemcpy(c->simt_layers, ls.data(), ls.size() * sizeof(ls[0]), cudaMemcpyHostToDevice) == cudaSuccess);
+      return ok && (g.n_layers == 0 || cudaMemcpyAsync(c->simt_layers, ls.data(), ls.size() * sizeof(ls[0]), cudaMemcpyHostToDevice, c->stream) == cudaSuccess);   // (pageable: staged before the call returns)
     };
     if (!(c->bf16 ? init(__nv_bfloat16{}) : init(0.f)) && ok) {
       cudaGetLastError();

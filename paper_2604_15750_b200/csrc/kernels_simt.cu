@@ -7,6 +7,7 @@
 #include <atomic>
 #include <type_traits>
 
+#include "pdl.cuh"
 #include "simt_dev.cuh"
 
 namespace dc {
@@ -41,6 +42,7 @@ __global__ void __launch_bounds__(128) k_step_begin(const T* __restrict__ embed,
                                                     int mask_id, int vocab, int d, const __grid_constant__ SeqMeta m,
                                                     float* __restrict__ x, int32_t* __restrict__ status, int hd, float theta,
                                                     float* __restrict__ cos_sin, unsigned int* __restrict__ words, int n_words) {
+  pdl_trigger();
   const int M = m.nv * m.batch * m.R_cap, row = blockIdx.x;
   if (row < M) {
     const int r = row % m.R_cap, vb = row / m.R_cap;
@@ -131,6 +133,8 @@ __global__ void __launch_bounds__(256) k_rmsnorm(float* __restrict__ x,
                                                  size_t part_stride, const T* __restrict__ g,
                                                  float eps, int d, T* __restrict__ out) {
   __shared__ float red[32];
+  pdl_trigger();
+  pdl_wait();
   const size_t off = (size_t)blockIdx.x * d;
   rmsnorm_row<T>(x + off, part ? part + off : nullptr, nsplit, part_stride, g, eps, d, out + off,
                  red);
@@ -139,7 +143,7 @@ __global__ void __launch_bounds__(256) k_rmsnorm(float* __restrict__ x,
 template <typename T>
 void launch_rmsnorm(float* x, const float* part, int nsplit, size_t part_stride, const T* g,
                     float eps, int M, int d, T* out, cudaStream_t s) {
-  k_rmsnorm<T><<<M, 256, 0, s>>>(x, part, nsplit, part_stride, g, eps, d, out);
+  launch_chained(k_rmsnorm<T>, M, 256, 0, s, x, part, nsplit, part_stride, g, eps, d, out);
 }
 
 // LM-head input rows, one block per row of the LM head's order (groups of G positions: curr rows, then
@@ -154,6 +158,8 @@ __global__ void __launch_bounds__(256) k_lm_rows(const float* __restrict__ x, co
                                                  const SeqMeta m, int nv_x, const LmRowsIo<T> io, T* __restrict__ h) {
   extern __shared__ __align__(16) float lm_row_s[];   // the row with the partial sums folded in
   __shared__ float red[32];
+  pdl_trigger();
+  pdl_wait();
   const int lrow = blockIdx.x;
   const int grp = lrow / (m.nv * m.G), in = lrow % (m.nv * m.G);
   const int v = in / m.G, p = grp * m.G + in % m.G;
@@ -207,7 +213,7 @@ __global__ void __launch_bounds__(256) k_lm_rows(const float* __restrict__ x, co
 template <typename T>
 void launch_lm_rows(const float* x, const float* part, int nsplit, size_t part_stride, const T* g, float eps, int d,
                     const SeqMeta& m, int nv_x, const LmRowsIo<T>& io, T* h, cudaStream_t s) {
-  k_lm_rows<T><<<m.nv * m.npos_pad, 256, d * sizeof(float), s>>>(x, part, nsplit, part_stride, g, eps, d, m, nv_x, io, h);
+  launch_chained(k_lm_rows<T>, m.nv * m.npos_pad, 256, d * sizeof(float), s, x, part, nsplit, part_stride, g, eps, d, m, nv_x, io, h);
 }
 
 // ---- CUDA-core GEMM: acc[m, n] = sum_k A[m, k] W[n, k], fp32 FMAs, with the epilogues of a layer ----
@@ -630,6 +636,8 @@ __global__ void __launch_bounds__(256) k_xlogp(const T* __restrict__ h,
                                                SeqMeta m, int max_window,
                                                float* __restrict__ xlogp) {
   extern __shared__ __align__(16) float wrow[];  // W_lm[yhat_j] as fp32
+  pdl_trigger();
+  pdl_wait();
   const int b = blockIdx.y, j = blockIdx.x;
   const int W = m.win_len[b];
   if (j >= W) return;
@@ -680,8 +688,7 @@ template <typename T>
 void launch_xlogp(const T* h, const T* lm_head, const int32_t* ws_pred, const float* ws_lse, int d,
                   int V, const SeqMeta& m, int max_window, float* xlogp, cudaStream_t s) {
   dim3 grid(m.W_cap, m.batch, (m.W_cap + 7) / 8);
-  k_xlogp<T><<<grid, 256, d * sizeof(float), s>>>(h, lm_head, ws_pred, ws_lse, d, V, m, max_window,
-                                                  xlogp);
+  launch_chained(k_xlogp<T>, grid, 256, d * sizeof(float), s, h, lm_head, ws_pred, ws_lse, d, V, m, max_window, xlogp);
 }
 
 // explicit instantiations

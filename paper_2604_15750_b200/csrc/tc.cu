@@ -325,14 +325,15 @@ static int launch_gemm(TcState* t, const CUtensorMap& w0, const CUtensorMap& w1,
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(2 * workers); cfg.blockDim = dim3(kGemmThreads);
     cfg.dynamicSmemBytes = smem; cfg.stream = t->s;
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeClusterDimension;
-    attr.val.clusterDim.x = 2; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
-    cfg.attrs = &attr; cfg.numAttrs = 1;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr; cfg.numAttrs = 2;
     e = cudaLaunchKernelEx(&cfg, k_gemm_tc<EPI, true>, w0, w1, w2, *ma_half, p, stages);
   } else {
-    k_gemm_tc<EPI, false><<<workers, kGemmThreads, smem, t->s>>>(w0, w1, w2, ma, p, stages);
-    e = cudaGetLastError();
+    e = launch_chained(k_gemm_tc<EPI, false>, workers, kGemmThreads, smem, t->s, w0, w1, w2, ma, p, stages);
   }
   if (e != cudaSuccess) {
     cudaGetLastError();
@@ -374,7 +375,7 @@ static int pick_split_rounds(const TcState* t, int tiles, int M, int BN, int N, 
 }
 
 int tc_attention(TcState* t, int layer, const SeqMeta& m, const __nv_bfloat16* k_cache,
-                 const __nv_bfloat16* v_cache, bool export_kv, bool export_only) {
+                 const __nv_bfloat16* v_cache, bool export_kv, bool export_only, bool chained) {
   const dc_config& g = t->g;
   const int nq = g.n_q_heads, nkv = g.n_kv_heads, hd = g.head_dim;
   bool any_ctx = false;
@@ -407,9 +408,15 @@ int tc_attention(TcState* t, int layer, const SeqMeta& m, const __nv_bfloat16* k
   ap.units = export_only ? 0 : m.nv == 2 ? 2 * nqt : nqt;
   if (ap.units + export_tiles == 0) return DC_OK;
   dim3 grid(ap.units + export_tiles, nq, m.batch);
-  k_attn_tc<<<grid, kAttnThreads, kAttnSmem, t->s>>>(t->map_q, t->map_k, t->map_vt, t->map_kc,
-                                                     t->map_vc, ap);
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e;
+  if (chained) {
+    e = launch_chained(k_attn_tc, grid, kAttnThreads, kAttnSmem, t->s, t->map_q, t->map_k, t->map_vt, t->map_kc, t->map_vc, ap);
+  } else {
+    // between two launches of the dense chain (programmatic launches there cost 1..3% of a step: 4523 ->
+    // 4658 us on one LLaDA-8B sequence)
+    k_attn_tc<<<grid, kAttnThreads, kAttnSmem, t->s>>>(t->map_q, t->map_k, t->map_vt, t->map_kc, t->map_vc, ap);
+    e = cudaGetLastError();
+  }
   if (e != cudaSuccess) return tfail(t, DC_ERR_CUDA, "attention launch failed: %s", cudaGetErrorString(e));
   return DC_OK;
 }
@@ -570,7 +577,7 @@ int tc_layer(TcState* t, int layer, const SeqMeta& m, float* x, const __nv_bfloa
   if (rc != DC_OK) return rc;
 
   hook.begin(DC_STAGE_ATTN, 1);
-  rc = tc_attention(t, layer, m, k_cache, v_cache, export_kv, kv_only);
+  rc = tc_attention(t, layer, m, k_cache, v_cache, export_kv, kv_only, true);
   hook.end();
   if (rc != DC_OK || kv_only) return rc;   // prefill, last layer: only its K / V were wanted
 
@@ -615,12 +622,12 @@ int tc_lmhead(TcState* t, const SeqMeta& m, const __nv_bfloat16* h, int mask_id,
   if (nctas < 1) nctas = 1;
   if (nctas > ntiles) nctas = ntiles;
   p.ngroups = groups;
-  k_lmhead_tc<<<groups * nctas, kLmThreads, t->lm_stages * kLmStageBytes + 1024, t->s>>>(t->map_h, t->map_lm,
-                                                                                      p, t->lm_stages);
+  cudaError_t e = launch_chained(k_lmhead_tc, groups * nctas, kLmThreads, t->lm_stages * kLmStageBytes + 1024, t->s,
+                                 t->map_h, t->map_lm, p, t->lm_stages);
   const int npos = m.batch * m.W_cap;
-  k_lm_combine<<<(npos + 3) / 4, 128, 0, t->s>>>(t->lm_part, nctas, m, g.vocab, mask_id, status, 1, ws_pred,
-                                                 ws_conf, ws_ent, ws_infl, ws_lse, out);
-  cudaError_t e = cudaGetLastError();
+  if (e == cudaSuccess)
+    e = launch_chained(k_lm_combine, (npos + 3) / 4, 128, 0, t->s, t->lm_part, nctas, m, g.vocab, mask_id, status, 1,
+                       ws_pred, ws_conf, ws_ent, ws_infl, ws_lse, out);
   if (e != cudaSuccess) return tfail(t, DC_ERR_CUDA, "LM-head launch failed: %s", cudaGetErrorString(e));
   return DC_OK;
 }
@@ -628,6 +635,8 @@ int tc_lmhead(TcState* t, const SeqMeta& m, const __nv_bfloat16* h, int mask_id,
 bool tc_has_lmhead(const dc_config& g) { return tc_supported(g); }
 
 __global__ void k_flush_status(int32_t* tc_status, int32_t* status, int batch) {
+  pdl_trigger();
+  pdl_wait();
   if (*tc_status != 0) {
     for (int b = threadIdx.x; b < batch; b += blockDim.x) status[b] = *tc_status;
     __syncthreads();
@@ -636,7 +645,7 @@ __global__ void k_flush_status(int32_t* tc_status, int32_t* status, int batch) {
 }
 
 void tc_flush_status(TcState* t, int32_t* status, int batch) {
-  k_flush_status<<<1, 32, 0, t->s>>>(t->status, status, batch);
+  launch_chained(k_flush_status, 1, 32, 0, t->s, t->status, status, batch);
 }
 
 }  // namespace dc

@@ -49,8 +49,9 @@ int tc_layer(TcState* t, int layer, const SeqMeta& m, float* x, const __nv_bfloa
 // Attention of one layer alone (reads the rotated q / k / transposed v the QKV epilogue wrote).
 // export_kv: the same launch also appends the curr variant's K / V of the last-block rows of `layer`
 // to the caches (base pointers of the whole caches, written then); export_only: nothing but that.
+// chained: programmatic launch behind the kernel before it (pdl.cuh).
 int tc_attention(TcState* t, int layer, const SeqMeta& m, const __nv_bfloat16* k_cache,
-                 const __nv_bfloat16* v_cache, bool export_kv, bool export_only);
+                 const __nv_bfloat16* v_cache, bool export_kv, bool export_only, bool chained);
 
 // Launch the dense chain with (default) or without the cooperative attribute; see DC_OPT_COOPERATIVE.
 void tc_set_cooperative(TcState* t, bool on);

@@ -35,6 +35,7 @@
 // about 2270 clocks per tile for MMAs that keep the tensor pipe busy for 1024.
 #pragma once
 #include "kernels.h"
+#include "pdl.cuh"
 #include "tc_ptx.cuh"
 
 namespace dc {
@@ -195,13 +196,15 @@ k_attn_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
   __shared__ float xm[3][128];     // [slot][row]: maximum raw score of the slot's tiles
 
   const int b = blockIdx.z, h = blockIdx.y;
+  pdl_trigger();
   if ((int)blockIdx.x >= p.units) {
+    pdl_wait();
     const int r0 = ((int)blockIdx.x - p.units) * kBK;
     if (h < p.nkv && r0 < p.m.last_len[b]) attn_export_tile(p, b, h, r0);
     return;
   }
   AttnUnit un;
-  if (!attn_unit(p.m, b, blockIdx.x, un)) return;   // nothing of this sequence in this unit (uniform)
+  if (!attn_unit(p.m, b, blockIdx.x, un)) { pdl_wait(); return; }   // nothing of this sequence in this unit (uniform)
 
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~static_cast<uintptr_t>(1023));
@@ -233,6 +236,7 @@ k_attn_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
   __syncthreads();
   ptx::tc_fence_after();
   const uint32_t tmem_base = tmem_base_s;
+  pdl_wait();
   // TMEM columns: S / P of tile J in buffer J % 3 (columns 0..127, 128..255, 256..383), O 384..511
 
   // softmax threads: row, slot and per-pass state (other warps carry the variables along)

@@ -24,6 +24,7 @@
 // starts when the epilogue has drained them.
 #pragma once
 #include "kernels.h"
+#include "pdl.cuh"
 #include "tc_ptx.cuh"
 
 namespace dc {
@@ -87,6 +88,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w0, const __grid_constant__ CU
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~static_cast<uintptr_t>(1023));
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  pdl_trigger();
   // Column blocks of one weight tile sit next to each other in the unit order, so that the
   // CTAs that share a weight tile run together and all but one read it from L2.
   const int n_cblk = (p.M + p.BN - 1) / p.BN;
@@ -147,6 +149,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w0, const __grid_constant__ CU
     ptx::cluster_sync();
   }
 
+  pdl_wait();   // everything below reads or writes what other kernels of the step share
   // One thread issues every TMA load and one every MMA, so their own instruction streams are on
   // the critical path: slot indices, addresses and descriptors advance by additions only.
   if (warp == 0) {

@@ -20,6 +20,7 @@
 // row; k_lm_combine merges the records of all CTAs.
 #pragma once
 #include "kernels.h"
+#include "pdl.cuh"
 #include "tc_ptx.cuh"
 
 namespace dc {
@@ -49,6 +50,7 @@ k_lmhead_tc(const __grid_constant__ CUtensorMap map_h, const __grid_constant__ C
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~static_cast<uintptr_t>(1023));
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  pdl_trigger();
   // CTA -> (group of LM rows, vocabulary slice), groups fastest: the CTAs that stream the same
   // vocabulary tiles for different groups run at the same time, so a tile crosses HBM once and is
   // served to the other groups from L2
@@ -77,6 +79,7 @@ k_lmhead_tc(const __grid_constant__ CUtensorMap map_h, const __grid_constant__ C
   ptx::tc_fence_after();
   const uint32_t tmem_base = tmem_base_s;
 
+  pdl_wait();
   // (lean single-thread loops: addresses and descriptors advance by additions only)
   if (warp == 0) {
     if (lane == 0) {
@@ -240,6 +243,8 @@ __global__ void k_lm_combine(const float* __restrict__ part, int nctas, SeqMeta 
                              int32_t* __restrict__ ws_pred, float* __restrict__ ws_conf,
                              float* __restrict__ ws_ent, float* __restrict__ ws_infl,
                              float* __restrict__ ws_lse, SignalOut out) {
+  pdl_trigger();
+  pdl_wait();
   const int pos = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (pos >= m.batch * m.W_cap) return;
