@@ -513,21 +513,23 @@ __device__ __forceinline__ void chain_gemm(ChainCtx& c, const ChainParams& p, co
 }
 
 // x[row] += sum of the partial sums (in split order); out[row] = bf16(rmsnorm(x[row]) * g).
-// Two rows per CTA at a time: warps 0..3 take one, warps 4..7 the other.  The rows of x and of
-// the partial sums are brought into the (idle) ring by bulk copies, so that a CTA has all of its
-// 160 KB in flight at once instead of a few loads per thread.
+// Two rows per CTA at a time, or one while there are as many CTAs as rows (half the bytes per SM: 80 KB
+// take 1 us): the first half of the threads has one row, the second the other, or all the same.
+// The rows of x and of the partial sums are brought into the (idle) ring by bulk copies, so that a CTA
+// has all of them in flight at once instead of a few loads per thread.
 __device__ __forceinline__ void chain_norm(ChainCtx& c, const ChainParams& p, int nsplit,
                                            const __nv_bfloat16* __restrict__ g, float* red) {
-  constexpr int kGrp = kChainThreads / 2;          // threads per row
+  const int per = p.M <= (int)gridDim.x ? 1 : 2;   // rows at a time
+  const int kGrp = kChainThreads / per;            // threads per row
   const int grp = threadIdx.x / kGrp;              // 0 or 1
   const int t = threadIdx.x - grp * kGrp;          // index inside the group
   const int d = p.d;
   const int narr = 1 + nsplit;
   float* stage = reinterpret_cast<float*>(c.ring);  // [grp][narr][d], then the gain vector
   __nv_bfloat16* sg = reinterpret_cast<__nv_bfloat16*>(stage + (size_t)2 * narr * d);
-  for (int r0 = 2 * blockIdx.x; r0 < p.M; r0 += 2 * gridDim.x) {
+  for (int r0 = per * blockIdx.x; r0 < p.M; r0 += per * gridDim.x) {
     if (threadIdx.x == 0) {
-      const int rows = (r0 + 1 < p.M) ? 2 : 1;
+      const int rows = min(per, p.M - r0);
       ptx::fence_proxy_async_smem();  // earlier generic accesses to the staging space come first
       ptx::mbar_expect_tx(c.norm_bar, (uint32_t)(rows * narr * d * 4 + d * 2));
       ptx::bulk_load(sg, g, d * 2, c.norm_bar);
@@ -564,9 +566,9 @@ __device__ __forceinline__ void chain_norm(ChainCtx& c, const ChainParams& p, in
     for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
     if (c.lane == 0) red[c.warp] = ss;
     // group-wide exchange: named barriers 5 and 6 (1..4 belong to the QKV epilogue)
-    asm volatile("bar.sync %0, %1;" ::"r"(grp + 5), "n"(kGrp) : "memory");
+    asm volatile("bar.sync %0, %1;" ::"r"(grp + 5), "r"(kGrp) : "memory");
     float tot = 0.f;
-#pragma unroll
+#pragma unroll 8
     for (int i = 0; i < kGrp / 32; ++i) tot += red[grp * (kGrp / 32) + i];
     if (live) {
       const float inv = rsqrtf(tot / (float)d + p.eps);
