@@ -72,6 +72,7 @@ constexpr int kStaticOther = 512;
 
 struct LayerMaps {
   CUtensorMap wq, wk, wv, wo, w_gate, w_up, w_down;
+  CUtensorMap w_gate_c, w_up_c;   // gate / up with the dense chain's tile height
 };
 
 struct ActMaps {
@@ -142,6 +143,14 @@ int pick_bn(int M) {
 }
 
 }  // namespace
+
+// Weight rows per gate / up tile of the dense chain: as many tiles as the grid has CTAs, in swizzle atoms of
+// 8 rows.  All SMs then stream weights instead of d_ff / 128 of them (d_ff 12288: 140 tiles of 88 rows
+// instead of 96 of 128; llada carried b1 4306 -> 4263 us, denoise b1 3885 -> 3836, 192 rows the same).
+static int gate_up_rows(const TcState* t) {
+  const int r = ((t->g.d_ff + t->chain_grid - 1) / t->chain_grid + 7) / 8 * 8;
+  return r < 32 ? 32 : r;
+}
 
 bool tc_supported(const dc_config& g) {
   return g.dtype == DC_BF16 && g.head_dim == 128 && g.d_model % 128 == 0 && g.d_ff % 128 == 0 &&
@@ -272,6 +281,12 @@ int tc_create(const dc_config& g, cudaStream_t s, int M_max, int Mlm_max,
       }
     }
     cudaGetLastError();
+    if (t->chain_grid > 0) {
+      const int rows = gate_up_rows(t);
+      for (int l = 0; l < g.n_layers && rows <= kChainTile; ++l)
+        if (!make_map_2d(&t->layers[l].w_gate_c, w_gate[l], F, d, rows) || !make_map_2d(&t->layers[l].w_up_c, w_up[l], F, d, rows))
+          return tfail(t, DC_ERR_CUDA, "tensor map encoding failed for layer %d (gate / up)", l);
+    }
   }
   return DC_OK;
 }
@@ -449,12 +464,12 @@ bool tc_chain_ok(const TcState* t, const SeqMeta& m) {
   // norm phases reuse the TMA ring as
   // staging space, which needs at most one GEMM unit per CTA and phase, and both rows of a norm
   // step (x plus the split-K partial sums) inside the ring.
-  const int units_qkv = g.n_q_heads + 2 * g.n_kv_heads, units_f = g.d_ff / kChainTile;
+  if (t->chain_grid <= 0) return false;
+  const int units_qkv = g.n_q_heads + 2 * g.n_kv_heads;
   const int units_d = (g.d_model / kChainTile) * t->max_split;
   const size_t norm_bytes = (size_t)2 * (1 + t->max_split) * g.d_model * sizeof(float) + g.d_model * 2;
-  const bool even = g.n_q_heads % 2 == 0 && g.n_kv_heads % 2 == 0 && (g.d_model / kChainTile) % 2 == 0 &&
-                    (g.d_ff / kChainTile) % 2 == 0;   // a CTA pair takes two adjacent tiles of one matrix
-  return t->chain_grid > 0 && even && M <= 256 && units_qkv <= t->chain_grid && units_f <= t->chain_grid &&
+  const bool even = g.n_q_heads % 2 == 0 && g.n_kv_heads % 2 == 0 && (g.d_model / kChainTile) % 2 == 0;   // a CTA pair takes two adjacent tiles of one matrix
+  return even && M <= 256 && units_qkv <= t->chain_grid && gate_up_rows(t) <= kChainTile &&
          units_d <= t->chain_grid && norm_bytes <= (size_t)kChainRing;
 }
 
@@ -479,7 +494,7 @@ int tc_chain(TcState* t, int layer, int qkv_layer, int phase_begin, int phase_en
   ChainMaps maps;
   const LayerMaps& L = t->layers[layer];
   const LayerMaps& Lq = t->layers[qkv_layer < g.n_layers ? qkv_layer : layer];
-  maps.wo = L.wo; maps.wg = L.w_gate; maps.wu = L.w_up; maps.wd = L.w_down;
+  maps.wo = L.wo; maps.wg = L.w_gate_c; maps.wu = L.w_up_c; maps.wd = L.w_down;
   maps.wq = Lq.wq; maps.wk = Lq.wk; maps.wv = Lq.wv;
   maps.wo_n = Lq.wo;
   maps.a = am->a; maps.o = am->o; maps.act = am->act;
@@ -488,7 +503,7 @@ int tc_chain(TcState* t, int layer, int qkv_layer, int phase_begin, int phase_en
   p.phase_begin = phase_begin; p.phase_end = phase_end;
   p.split_o = pick_split(d / kChainTile, nq * g.head_dim / kChainTileK, t->max_split);
   p.split_down = pick_split(d / kChainTile, F / kChainTileK, t->max_split);
-  p.fold_norm1 = fold_norm1;
+  p.fold_norm1 = fold_norm1; p.gu_rows = gate_up_rows(t);
   p.x = x; p.a = const_cast<__nv_bfloat16*>(a); p.act = t->act;
   p.part = t->part; p.part_stride = t->part_stride;
   p.g2 = g2; p.g1 = g1; p.eps = g.rms_eps;

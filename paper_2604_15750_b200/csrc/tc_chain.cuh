@@ -59,6 +59,7 @@ struct ChainParams {
   int d, F, nq, nkv;            // model width, MLP width, query / kv heads (head_dim 128)
   int phase_begin, phase_end;
   int split_o, split_down;      // split-K factors of the two projections back to d
+  int gu_rows;                  // weight rows per gate / up tile (a multiple of 8, <= 128)
   int fold_norm1;               // partial sums phase 4 folds (0 when the launch starts there)
   float* x;                     // residual stream [M, d] fp32
   __nv_bfloat16* a;             // normed activations [M, d]
@@ -119,6 +120,7 @@ struct GemmPhase {
   int nsplit;                       // K splits
   int KB;                           // k-blocks of 64
   int N;                            // output features (row pitch of the output)
+  int rows;                         // weight rows per tile that are stored (the MMAs take 128)
   int bal_h;                        // k-blocks of every tile that helper CTA pairs compute (0: none)
   // what the producer prefetches into L2 once its own loads are issued: the first pf_kb
   // k-blocks of its unit in the phase named here (tiles == 0: nothing)
@@ -179,7 +181,7 @@ struct RopeBase { float c, s, cd, sd; };
 
 // Epilogue of 16 accumulator columns (activation rows c0 .. c0+15) of feature f of a tile.
 template <int EPI>
-__device__ __forceinline__ void chain_emit(ChainCtx& c, const ChainParams& p, const int N,
+__device__ __forceinline__ void chain_emit(ChainCtx& c, const ChainParams& p, const int N, const int rows,
                                            const int tile, const int split, const int f,
                                            const int c0, float (&v0)[16], float (&v1)[16],
                                            const RopeBase rb, const int half) {
@@ -189,7 +191,8 @@ __device__ __forceinline__ void chain_emit(ChainCtx& c, const ChainParams& p, co
 #pragma unroll
     for (int j = 0; j < 16; ++j) dst[(size_t)j * N] = v0[j] + v1[j];
   } else if (EPI == CEPI_SWIGLU) {
-    __nv_bfloat16* dst = p.act + (size_t)(tile * kChainTile + f) + (size_t)c0 * N;
+    if (f >= rows || tile * rows + f >= N) return;   // lanes beyond the tile or the matrix
+    __nv_bfloat16* dst = p.act + (size_t)(tile * rows + f) + (size_t)c0 * N;
 #pragma unroll
     for (int j = 0; j < 16; ++j) {
       // silu(g) = g * sigmoid(g) = g * (0.5 + 0.5 * tanh(g / 2)): one special-function
@@ -271,7 +274,10 @@ __device__ __forceinline__ void chain_gemm(ChainCtx& c, const ChainParams& p, co
   const bool has = chain_item(g.tiles, g.nsplit, g.KB, g.bal_h, w);
   // weight tiles per k-block: gate and up, or the two tiles of a helper pair in a balanced QKV
   const int nw = (EPI == CEPI_SWIGLU) ? 2 : (EPI == CEPI_QKV && has && w.tile2 >= 0) ? 2 : 1;
-  const int slot_bytes = nw * kChainTile * kChainTileK * 2 + half_rows * kChainTileK * 2;
+  // a tile of fewer than 128 rows takes that much less of a slot: the MMAs read on into what lies behind
+  // it (inside shared memory: the exchange buffers follow the ring), and nobody reads those lanes
+  const int tile_bytes = (EPI == CEPI_SWIGLU ? g.rows : kChainTile) * kChainTileK * 2;
+  const int slot_bytes = nw * tile_bytes + half_rows * kChainTileK * 2;
   int stages = kChainRing / slot_bytes;
   if (stages > 8) stages = 8;
   // map and first row of a QKV tile (q tiles, then k, then v)
@@ -293,7 +299,7 @@ __device__ __forceinline__ void chain_gemm(ChainCtx& c, const ChainParams& p, co
       const uint64_t pol_w = ptx::l2_policy_evict_first(), pol_a = ptx::l2_policy_evict_last();
       if (has) {
         const CUtensorMap *mw = g.w0, *mw2 = g.w1;
-        int wrow = w.tile * kChainTile, wrow2 = wrow;
+        int wrow = w.tile * (EPI == CEPI_SWIGLU ? g.rows : kChainTile), wrow2 = wrow;
         if (EPI == CEPI_QKV) {
           qkv_src(w.tile, mw, wrow);
           if (nw == 2) qkv_src(w.tile2, mw2, wrow2);
@@ -312,8 +318,8 @@ __device__ __forceinline__ void chain_gemm(ChainCtx& c, const ChainParams& p, co
           // weights pass through L2 once (evict first); the activation tile is re-read by every CTA
           // and the small buffers between phases should stay resident (evict last): -5% step time
           ptx::tma_load_2d_pair_hint(pslot, mw, bar, kc, wrow, pol_w);
-          if (nw == 2) ptx::tma_load_2d_pair_hint(pslot + kChainTile * kChainTileK * 2, mw2, bar, kc, wrow2, pol_w);
-          ptx::tma_load_2d_pair_hint(pslot + nw * kChainTile * kChainTileK * 2, g.amap, bar, kc, arow, pol_a);
+          if (nw == 2) ptx::tma_load_2d_pair_hint(pslot + tile_bytes, mw2, bar, kc, wrow2, pol_w);
+          ptx::tma_load_2d_pair_hint(pslot + nw * tile_bytes, g.amap, bar, kc, arow, pol_a);
           if (++ps == (uint32_t)stages) { ps = 0; pslot = ring0; } else pslot += (uint32_t)slot_bytes;
         }
       }
@@ -328,7 +334,7 @@ __device__ __forceinline__ void chain_gemm(ChainCtx& c, const ChainParams& p, co
         const int kb1 = n.kb1 > n.kb0 + g.pf_kb ? n.kb0 + g.pf_kb : n.kb1;
         const bool both = g.pf_w1 != nullptr && g.pf_t1 == 0;  // gate and up: same rows of two maps
         auto src = [&](int tile, const CUtensorMap*& m, int& row) {
-          m = g.pf_w0; row = tile * kChainTile;
+          m = g.pf_w0; row = tile * (both ? p.gu_rows : kChainTile);
           if (!both && g.pf_w2 != nullptr && tile >= g.pf_t2) { m = g.pf_w2; row = (tile - g.pf_t2) * kChainTile; }
           else if (!both && g.pf_w1 != nullptr && tile >= g.pf_t1) { m = g.pf_w1; row = (tile - g.pf_t1) * kChainTile; }
         };
@@ -366,8 +372,8 @@ __device__ __forceinline__ void chain_gemm(ChainCtx& c, const ChainParams& p, co
         ok = ptx::mbar_wait_a(mfull0 + 8u * ms, par, c.abort_flag);
         if (!ok) break;
         const uint64_t dw0 = desc_hi | (uint64_t)(mslot >> 4);
-        const uint64_t dw1 = dw0 + (kChainTile * kChainTileK * 2 >> 4);
-        const uint64_t da = dw0 + ((uint64_t)nw * (kChainTile * kChainTileK * 2 >> 4));
+        const uint64_t dw1 = dw0 + (uint32_t)(tile_bytes >> 4);
+        const uint64_t da = dw0 + (uint32_t)(nw * tile_bytes >> 4);
         if (nw == 2) {
           ptx::umma_bf16_pair(c.tmem_base, dw0, da, idesc, acc_first);
           ptx::umma_bf16_pair(c.tmem_base + 256, dw1, da, idesc, acc_first);
@@ -477,7 +483,7 @@ __device__ __forceinline__ void chain_gemm(ChainCtx& c, const ChainParams& p, co
             for (int k = 0; k < 4; ++k) {
               a0[4 * k] += ha[k].x; a0[4 * k + 1] += ha[k].y; a0[4 * k + 2] += ha[k].z; a0[4 * k + 3] += ha[k].w;
             }
-            chain_emit<EPI>(c, p, g.N, tile, split, f, c0, a0, a1, rb, half);
+            chain_emit<EPI>(c, p, g.N, g.rows, tile, split, f, c0, a0, a1, rb, half);
 #pragma unroll
             for (int k = 0; k < 4; ++k) ha[k] = hn[k];
             rb.c = rn.c; rb.s = rn.s;
@@ -500,7 +506,7 @@ __device__ __forceinline__ void chain_gemm(ChainCtx& c, const ChainParams& p, co
           ptx::tmem_ld_32x16(t_lane + 256 + c0, a1);
           if (rope && c0 + 16 < col1) rope_base(c0 + 16, rn);   // one chunk ahead
           ptx::tmem_ld_wait();
-          chain_emit<EPI>(c, p, g.N, tile, split, f, c0, a0, a1, rb, half);
+          chain_emit<EPI>(c, p, g.N, g.rows, tile, split, f, c0, a0, a1, rb, half);
           rb.c = rn.c; rb.s = rn.s;
         }
       }
@@ -638,7 +644,7 @@ k_dense_chain(const __grid_constant__ ChainMaps maps, const ChainParams p) {
   ptx::cluster_sync();
 
   const int KBd = p.d / kChainTileK, KBq = p.nq * 128 / kChainTileK, KBf = p.F / kChainTileK;
-  const int tiles_d = p.d / kChainTile, tiles_f = p.F / kChainTile, tiles_qkv = p.nq + 2 * p.nkv;
+  const int tiles_d = p.d / kChainTile, tiles_f = ((p.F + p.gu_rows - 1) / p.gu_rows + 1) & ~1, tiles_qkv = p.nq + 2 * p.nkv;
   const bool has_qkv = p.phase_end > CH_QKV;
 
   unsigned int n_barriers = 0;
@@ -656,7 +662,7 @@ k_dense_chain(const __grid_constant__ ChainMaps maps, const ChainParams p) {
         chain_norm(c, p, p.split_o, p.g2, red);
         break;
       case CH_GATEUP:
-        g.w0 = &maps.wg; g.w1 = &maps.wu; g.amap = &maps.a; g.tiles = tiles_f; g.nsplit = 1; g.KB = KBd; g.N = p.F;
+        g.w0 = &maps.wg; g.w1 = &maps.wu; g.amap = &maps.a; g.tiles = tiles_f; g.nsplit = 1; g.KB = KBd; g.N = p.F; g.rows = p.gu_rows;
         g.pf_w0 = &maps.wd; g.pf_tiles = tiles_d; g.pf_nsplit = p.split_down; g.pf_KB = KBf; g.pf_kb = kPfDown;
         chain_gemm<CEPI_SWIGLU>(c, p, g);
         break;

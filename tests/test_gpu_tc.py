@@ -154,3 +154,23 @@ def test_fused_chain_qkv_helper_layouts(n_q, n_kv):
     _, launches = eng.step_profiled(**di)
     assert launches["dense"] == case.n_layers + 1
     eng.close()
+
+
+@pytest.mark.parametrize("ff,last,win,influence", [(7040, 32, 96, True), (7040, 0, 16, False), (4864, 16, 32, True)])
+def test_fused_chain_gate_up_tile_heights(ff, last, win, influence):
+    """Gate / up tiles of fewer than 128 rows: d_ff 7040 in 147 tiles of 48 (the 148th lies beyond the
+    matrix), 4864 in 122 of 40 with a remainder; 256, 16 and 96 activation rows."""
+    wl = _wl(1, ff=ff, last=max(last, 1), win=win)
+    lengths = dict(ctx_len=[100], last_len=[last], win_len=[win], remain_len=[128])
+    case = Case(wl, lengths=lengths)
+    eng = case.make_engine(max_window=win)
+    di = case.device_inputs(eng)
+    out = eng.step(influence=influence, boundary=True, **di)
+    sel = eng.select(di["win_ids"], di["win_len"])
+    eng.synchronize()
+    gpu = {k_: v_.cpu().numpy() for k_, v_ in out.items()}
+    gpu.update({k_: v_.cpu().numpy() for k_, v_ in sel.items()})
+    compare(case, gpu, case.run_oracle(influence=influence))
+    _, launches = eng.step_profiled(influence=influence, boundary=True, **di)
+    assert launches["dense"] == case.n_layers + 1
+    eng.close()
