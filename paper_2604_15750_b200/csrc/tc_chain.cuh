@@ -350,49 +350,46 @@ __device__ __forceinline__ void chain_gemm(ChainCtx& c, const ChainParams& p, co
       }
     }
   } else if (c.warp == 1) {
-    if (c.lane == 0 && c.rank == 0 && has) {
+    if (c.rank == 0 && has) {
       // ---------------- MMA issuer (even CTA of the pair, for both) ----------------
-      // (A ring unrolled over its slots with split 32-bit descriptors issues an MMA every 97 clk at
-      // N = 192 in isolation, against 140 for this loop, but these GEMMs wait for their data, not
-      // for the issue, and the larger code made the launch 4% slower: measured and taken out.)
+      // The whole warp runs the loop and one elected lane issues: the operands then stay in uniform
+      // registers.  In a branch of a single lane a k-block of four MMAs takes 484 clocks at N = 192 and
+      // 481 at N = 16 (gate / up's eight: 749 and 664), this way 390 and 360 (773 and 388), the first
+      // being the tensor core's own time.
+      const bool el = ptx::elect_one();
       const uint32_t idesc = ptx::idesc_bf16(2 * kChainTile, BN);
       bool ok = true;
-      const uint32_t mring0 = ptx::smem_u32(c.ring);
       const uint32_t mfull0 = ptx::smem_u32(&c.full[0]), mempty0 = ptx::smem_u32(&c.empty[0]);
-      const uint64_t desc_hi = ptx::smem_desc_sw128_hi();
-      uint32_t ms = 0, mslot = mring0;
+      const uint32_t desc_hi = ptx::smem_desc_hi32(), lo0 = ptx::smem_desc_lo(ptx::smem_u32(c.ring));
+      const uint32_t up = (uint32_t)tile_bytes >> 4, act = (uint32_t)(nw * tile_bytes) >> 4, step = (uint32_t)slot_bytes >> 4;
+      uint32_t ms = 0, lo = lo0;
       if (c.mma_units > 0) {  // the epilogue has drained both accumulators of the last unit
         ok = ptx::mbar_wait(c.acc_empty, (c.mma_units - 1) & 1u, c.abort_flag);
       }
       ptx::tc_fence_after();
-      uint32_t acc_first = 0;   // 0 until the first k-block of the unit has been issued
       for (int kb = w.kb0; kb < w.kb1 && ok; ++kb) {
         const uint32_t par = (c.use_bits >> ms) & 1u;
         c.use_bits ^= 1u << ms;
-        ok = ptx::mbar_wait_a(mfull0 + 8u * ms, par, c.abort_flag);
+        ok = __all_sync(0xffffffffu, ptx::mbar_wait_a(mfull0 + 8u * ms, par, c.abort_flag));
         if (!ok) break;
-        const uint64_t dw0 = desc_hi | (uint64_t)(mslot >> 4);
-        const uint64_t dw1 = dw0 + (uint32_t)(tile_bytes >> 4);
-        const uint64_t da = dw0 + (uint32_t)(nw * tile_bytes >> 4);
-        if (nw == 2) {
-          ptx::umma_bf16_pair(c.tmem_base, dw0, da, idesc, acc_first);
-          ptx::umma_bf16_pair(c.tmem_base + 256, dw1, da, idesc, acc_first);
+        const uint32_t more = kb > w.kb0 ? 1u : 0u;   // the first MMA of an accumulator overwrites it
+        if (el) {
+          if (nw == 2) {
 #pragma unroll
-          for (int kk = 1; kk < kChainTileK / 16; ++kk) {
-            ptx::umma_bf16_pair_acc(c.tmem_base, dw0 + 2 * kk, da + 2 * kk, idesc);
-            ptx::umma_bf16_pair_acc(c.tmem_base + 256, dw1 + 2 * kk, da + 2 * kk, idesc);
+            for (int kk = 0; kk < kChainTileK / 16; ++kk) {
+              ptx::umma_bf16_pair_lo(c.tmem_base, lo + 2 * kk, lo + act + 2 * kk, desc_hi, idesc, kk > 0 ? 1u : more);
+              ptx::umma_bf16_pair_lo(c.tmem_base + 256, lo + up + 2 * kk, lo + act + 2 * kk, desc_hi, idesc, kk > 0 ? 1u : more);
+            }
+          } else {
+#pragma unroll
+            for (int kk = 0; kk < kChainTileK / 16; ++kk)
+              ptx::umma_bf16_pair_lo(c.tmem_base + (kk & 1) * 256, lo + 2 * kk, lo + act + 2 * kk, desc_hi, idesc, kk > 1 ? 1u : more);
           }
-        } else {
-          ptx::umma_bf16_pair(c.tmem_base, dw0, da, idesc, acc_first);
-          ptx::umma_bf16_pair(c.tmem_base + 256, dw0 + 2, da + 2, idesc, acc_first);
-          ptx::umma_bf16_pair_acc(c.tmem_base, dw0 + 4, da + 4, idesc);
-          ptx::umma_bf16_pair_acc(c.tmem_base + 256, dw0 + 6, da + 6, idesc);
+          ptx::umma_commit_pair_a(mempty0 + 8u * ms);   // frees the slot in both CTAs
         }
-        acc_first = 1;
-        ptx::umma_commit_pair_a(mempty0 + 8u * ms);   // frees the slot in both CTAs
-        if (++ms == (uint32_t)stages) { ms = 0; mslot = mring0; } else mslot += (uint32_t)slot_bytes;
+        if (++ms == (uint32_t)stages) { ms = 0; lo = lo0; } else lo += step;
       }
-      if (ok) ptx::umma_commit_pair(c.acc_full);  // both epilogues start
+      if (ok && el) ptx::umma_commit_pair(c.acc_full);  // both epilogues start
       ++c.mma_units;
     }
   }
@@ -611,7 +608,8 @@ k_dense_chain(const __grid_constant__ ChainMaps maps, const ChainParams p) {
   c.full = bar_full; c.empty = bar_empty; c.acc_full = &bar_acc_full; c.acc_empty = &bar_acc_empty; c.norm_bar = &bar_norm;
   c.abort_flag = &abort_flag;
   c.fill_bits = 0; c.use_bits = 0; c.units_done = 0; c.mma_units = 0; c.norm_uses = 0;
-  c.warp = threadIdx.x >> 5; c.lane = threadIdx.x & 31;
+  c.warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);   // warp-uniform for the compiler too
+  c.lane = threadIdx.x & 31;
   c.rank = ptx::cluster_ctarank();
 
   if (threadIdx.x == 0) {
