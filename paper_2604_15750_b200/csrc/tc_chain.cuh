@@ -94,9 +94,12 @@ constexpr int kChainXch = kChainParts * 128 * kXchRow * 4;  // RoPE exchange buf
 constexpr int kChainSmem = kChainRing + kChainXch + 1024;
 constexpr int kChainTile = 128;                 // weight rows per unit
 constexpr int kChainTileK = 64;
-// k-blocks of its next unit that a CTA prefetches into L2 when its own loads are issued (measured:
-// 8 / 12 / 24 k-blocks cost +0.03 / +0.04 / +0.25 ms per step against 4)
-constexpr int kPfGateUp = 4, kPfDown = 4, kPfQkv = 4;
+// k-blocks of its next item that a CTA prefetches into L2 at a grid barrier, and of the O projection while
+// attention runs.  Gate / up, down, QKV 4 / 8 / 8 against 4 / 4 / 4 against the same issued before the
+// epilogue: carried b1 (96 rows) 4161 / 4192 / 4252 us, denoise b1 (16 rows) 3710 / 3728 / 3766; boundary b1
+// (192 rows) 4715 / 4660 / 4696; 16 / 12 / 16: +1.5% there.
+constexpr int kPfGateUp = 4, kPfOproj = 64;
+__device__ __forceinline__ int chain_pf_deep(int BN) { return BN <= 128 ? 8 : 4; }   // down, QKV
 
 struct ChainCtx {
   uint8_t* ring;
@@ -122,10 +125,9 @@ struct GemmPhase {
   int N;                            // output features (row pitch of the output)
   int rows;                         // weight rows per tile that are stored (the MMAs take 128)
   int bal_h;                        // k-blocks of every tile that helper CTA pairs compute (0: none)
-  // what the producer prefetches into L2 once its own loads are issued: the first pf_kb
-  // k-blocks of its unit in the phase named here (tiles == 0: nothing)
+  // the phase whose first k-blocks chain_prefetch brings into L2 (tiles == 0: none)
   const CUtensorMap *pf_w0, *pf_w1, *pf_w2;
-  int pf_tiles, pf_nsplit, pf_KB, pf_kb, pf_t1, pf_t2;  // pf_t1 / pf_t2: first tile of w1 / w2
+  int pf_tiles, pf_nsplit, pf_KB, pf_t1, pf_t2;  // pf_t1 / pf_t2: first tile of w1 / w2
   int pf_bal_h;
 };
 
@@ -266,6 +268,29 @@ __device__ __forceinline__ void chain_emit(ChainCtx& c, const ChainParams& p, co
 }
 
 
+// Starts the first pf_kb k-blocks of this CTA's item in the phase that g.pf_* names on their way into L2.
+// Called by one warp, a k-block per lane: a prefetch instruction occupies its thread for a while.
+__device__ __forceinline__ void chain_prefetch(ChainCtx& c, const ChainParams& p, const GemmPhase& g, const int pf_kb) {
+  ChainItem n;
+  if (g.pf_tiles == 0 || !chain_item(g.pf_tiles, g.pf_nsplit, g.pf_KB, g.pf_bal_h, n)) return;
+  const int kb1 = n.kb1 > n.kb0 + pf_kb ? n.kb0 + pf_kb : n.kb1;
+  const bool both = g.pf_w1 != nullptr && g.pf_t1 == 0;  // gate and up: same rows of two maps
+  auto src = [&](int tile, const CUtensorMap*& m, int& row) {
+    m = g.pf_w0; row = tile * (both ? p.gu_rows : kChainTile);
+    if (!both && g.pf_w2 != nullptr && tile >= g.pf_t2) { m = g.pf_w2; row = (tile - g.pf_t2) * kChainTile; }
+    else if (!both && g.pf_w1 != nullptr && tile >= g.pf_t1) { m = g.pf_w1; row = (tile - g.pf_t1) * kChainTile; }
+  };
+  const CUtensorMap *m0, *m1 = nullptr;
+  int r0, r1 = 0;
+  src(n.tile, m0, r0);
+  if (both) { m1 = g.pf_w1; r1 = r0; }
+  else if (n.tile2 >= 0) src(n.tile2, m1, r1);
+  for (int kb = n.kb0 + c.lane; kb < kb1; kb += 32) {
+    ptx::tma_prefetch_l2_2d(m0, kb * kChainTileK, r0);
+    if (m1 != nullptr) ptx::tma_prefetch_l2_2d(m1, kb * kChainTileK, r1);
+  }
+}
+
 template <int EPI>
 __device__ __forceinline__ void chain_gemm(ChainCtx& c, const ChainParams& p, const GemmPhase& g) {
   const int BN = p.BN;
@@ -324,31 +349,9 @@ __device__ __forceinline__ void chain_gemm(ChainCtx& c, const ChainParams& p, co
         }
       }
     }
-    ok = __shfl_sync(0xffffffffu, (int)ok, 0) != 0;
-    {
-      // ---------------- L2 prefetch of this CTA's item in the next GEMM phase ----------------
-      // Issued by all lanes of the warp, a k-block each: a prefetch instruction occupies its thread
-      // for a while, and the producer lane is needed again right after the grid barrier.
-      ChainItem n;
-      if (ok && g.pf_tiles > 0 && chain_item(g.pf_tiles, g.pf_nsplit, g.pf_KB, g.pf_bal_h, n)) {
-        const int kb1 = n.kb1 > n.kb0 + g.pf_kb ? n.kb0 + g.pf_kb : n.kb1;
-        const bool both = g.pf_w1 != nullptr && g.pf_t1 == 0;  // gate and up: same rows of two maps
-        auto src = [&](int tile, const CUtensorMap*& m, int& row) {
-          m = g.pf_w0; row = tile * (both ? p.gu_rows : kChainTile);
-          if (!both && g.pf_w2 != nullptr && tile >= g.pf_t2) { m = g.pf_w2; row = (tile - g.pf_t2) * kChainTile; }
-          else if (!both && g.pf_w1 != nullptr && tile >= g.pf_t1) { m = g.pf_w1; row = (tile - g.pf_t1) * kChainTile; }
-        };
-        const CUtensorMap *m0, *m1 = nullptr;
-        int r0, r1 = 0;
-        src(n.tile, m0, r0);
-        if (both) { m1 = g.pf_w1; r1 = r0; }
-        else if (n.tile2 >= 0) src(n.tile2, m1, r1);
-        for (int kb = n.kb0 + c.lane; kb < kb1; kb += 32) {
-          ptx::tma_prefetch_l2_2d(m0, kb * kChainTileK, r0);
-          if (m1 != nullptr) ptx::tma_prefetch_l2_2d(m1, kb * kChainTileK, r1);
-        }
-      }
-    }
+    // attention runs after QKV; meanwhile the O projection of that layer streams into L2 (gate / up of that
+    // layer on top of it was measured slower: +2..4% per step for 8..32 k-blocks)
+    if (EPI == CEPI_QKV && __shfl_sync(0xffffffffu, (int)ok, 0) != 0) chain_prefetch(c, p, g, kPfOproj);
   } else if (c.warp == 1) {
     if (c.rank == 0 && has) {
       // ---------------- MMA issuer (even CTA of the pair, for both) ----------------
@@ -653,7 +656,7 @@ k_dense_chain(const __grid_constant__ ChainMaps maps, const ChainParams p) {
       case CH_OPROJ:
         g.w0 = &maps.wo; g.amap = &maps.o; g.tiles = tiles_d; g.nsplit = p.split_o; g.KB = KBq; g.N = p.d;
         g.pf_w0 = &maps.wg; g.pf_w1 = &maps.wu; g.pf_t1 = 0; g.pf_tiles = tiles_f; g.pf_nsplit = 1;
-        g.pf_KB = KBd; g.pf_kb = kPfGateUp;
+        g.pf_KB = KBd;
         chain_gemm<CEPI_PARTIAL>(c, p, g);
         break;
       case CH_NORM2:
@@ -661,14 +664,14 @@ k_dense_chain(const __grid_constant__ ChainMaps maps, const ChainParams p) {
         break;
       case CH_GATEUP:
         g.w0 = &maps.wg; g.w1 = &maps.wu; g.amap = &maps.a; g.tiles = tiles_f; g.nsplit = 1; g.KB = KBd; g.N = p.F; g.rows = p.gu_rows;
-        g.pf_w0 = &maps.wd; g.pf_tiles = tiles_d; g.pf_nsplit = p.split_down; g.pf_KB = KBf; g.pf_kb = kPfDown;
+        g.pf_w0 = &maps.wd; g.pf_tiles = tiles_d; g.pf_nsplit = p.split_down; g.pf_KB = KBf;
         chain_gemm<CEPI_SWIGLU>(c, p, g);
         break;
       case CH_DOWN:
         g.w0 = &maps.wd; g.amap = &maps.act; g.tiles = tiles_d; g.nsplit = p.split_down; g.KB = KBf; g.N = p.d;
         if (has_qkv) {
           g.pf_w0 = &maps.wq; g.pf_w1 = &maps.wk; g.pf_w2 = &maps.wv; g.pf_t1 = p.nq; g.pf_t2 = p.nq + p.nkv;
-          g.pf_tiles = tiles_qkv; g.pf_nsplit = 1; g.pf_KB = KBd; g.pf_kb = kPfQkv; g.pf_bal_h = p.bal_h;
+          g.pf_tiles = tiles_qkv; g.pf_nsplit = 1; g.pf_KB = KBd; g.pf_bal_h = p.bal_h;
         }
         chain_gemm<CEPI_PARTIAL>(c, p, g);
         break;
@@ -678,9 +681,7 @@ k_dense_chain(const __grid_constant__ ChainMaps maps, const ChainParams p) {
       default:  // CH_QKV
         g.w0 = &maps.wq; g.w1 = &maps.wk; g.w2 = &maps.wv; g.amap = &maps.a; g.tiles = tiles_qkv;
         g.nsplit = 1; g.KB = KBd; g.N = 0; g.bal_h = p.bal_h;
-        // attention runs next; meanwhile the O projection of that layer streams into L2 (gate / up
-        // of that layer on top of it was measured slower: +2..4% per step for 8..32 k-blocks)
-        g.pf_w0 = &maps.wo_n; g.pf_tiles = tiles_d; g.pf_nsplit = p.split_o; g.pf_KB = KBq; g.pf_kb = 64;
+        g.pf_w0 = &maps.wo_n; g.pf_tiles = tiles_d; g.pf_nsplit = p.split_o; g.pf_KB = KBq;
         chain_gemm<CEPI_QKV>(c, p, g);
         break;
     }
@@ -692,6 +693,10 @@ k_dense_chain(const __grid_constant__ ChainMaps maps, const ChainParams p) {
           abort_flag = 1;
         if (abort_flag) atomicExch(p.status, DC_ERR_TIMEOUT);
         ptx::fence_proxy_async_all();
+      } else if (c.warp == 3) {
+        // While the CTA waits the first weights of its next GEMM start into L2.  In a warp of its own and not
+        // before this point: the release of the arrival waits for what its thread has in flight.
+        chain_prefetch(c, p, g, ph == CH_OPROJ ? kPfGateUp : chain_pf_deep(p.BN));
       }
       __syncthreads();
     }
