@@ -72,7 +72,7 @@ constexpr int kStaticOther = 512;
 
 struct LayerMaps {
   CUtensorMap wq, wk, wv, wo, w_gate, w_up, w_down;
-  CUtensorMap w_gate_c, w_up_c;   // gate / up with the dense chain's tile height
+  CUtensorMap w_gate_c, w_up_c;   // gate / up with the dense chain's lower tiles (gate_up_rows)
 };
 
 struct ActMaps {
@@ -144,11 +144,14 @@ int pick_bn(int M) {
 
 }  // namespace
 
-// Weight rows per gate / up tile of the dense chain: as many tiles as the grid has CTAs, in swizzle atoms of
-// 8 rows.  All SMs then stream weights instead of d_ff / 128 of them (d_ff 12288: 140 tiles of 88 rows
-// instead of 96 of 128; llada carried b1 4306 -> 4263 us, denoise b1 3885 -> 3836, 192 rows the same).
-static int gate_up_rows(const TcState* t) {
-  const int r = ((t->g.d_ff + t->chain_grid - 1) / t->chain_grid + 7) / 8 * 8;
+// Weight rows per gate / up tile of the dense chain.  Up to 128 activation rows as many tiles as the grid has
+// CTAs, in swizzle atoms of 8 rows: all SMs then stream weights instead of d_ff / 128 of them (d_ff 12288:
+// 140 tiles of 88 rows instead of 96 of 128; llada carried b1 4306 -> 4263 us, denoise b1 3885 -> 3836).  With
+// more rows whole tiles where they fit: the MMAs take 128 rows anyway, and the power that the surplus
+// ones cost is what such a step is short of (llada boundary b1, 192 rows: 4736 -> 4685).
+static int gate_up_rows(const TcState* t, int BN) {
+  const int r = ((t->g.d_ff + t->chain_grid - 1) / t->chain_grid + 7) / 8 * 8, tiles = t->g.d_ff / kChainTile;
+  if (BN > 128 && tiles % 2 == 0 && tiles <= t->chain_grid) return kChainTile;
   return r < 32 ? 32 : r;
 }
 
@@ -282,7 +285,7 @@ int tc_create(const dc_config& g, cudaStream_t s, int M_max, int Mlm_max,
     }
     cudaGetLastError();
     if (t->chain_grid > 0) {
-      const int rows = gate_up_rows(t);
+      const int rows = gate_up_rows(t, 0);
       for (int l = 0; l < g.n_layers && rows <= kChainTile; ++l)
         if (!make_map_2d(&t->layers[l].w_gate_c, w_gate[l], F, d, rows) || !make_map_2d(&t->layers[l].w_up_c, w_up[l], F, d, rows))
           return tfail(t, DC_ERR_CUDA, "tensor map encoding failed for layer %d (gate / up)", l);
@@ -469,7 +472,7 @@ bool tc_chain_ok(const TcState* t, const SeqMeta& m) {
   const int units_d = (g.d_model / kChainTile) * t->max_split;
   const size_t norm_bytes = (size_t)2 * (1 + t->max_split) * g.d_model * sizeof(float) + g.d_model * 2;
   const bool even = g.n_q_heads % 2 == 0 && g.n_kv_heads % 2 == 0 && (g.d_model / kChainTile) % 2 == 0;   // a CTA pair takes two adjacent tiles of one matrix
-  return even && M <= 256 && units_qkv <= t->chain_grid && gate_up_rows(t) <= kChainTile &&
+  return even && M <= 256 && units_qkv <= t->chain_grid && gate_up_rows(t, M) <= kChainTile &&
          units_d <= t->chain_grid && norm_bytes <= (size_t)kChainRing;
 }
 
@@ -494,7 +497,7 @@ int tc_chain(TcState* t, int layer, int qkv_layer, int phase_begin, int phase_en
   ChainMaps maps;
   const LayerMaps& L = t->layers[layer];
   const LayerMaps& Lq = t->layers[qkv_layer < g.n_layers ? qkv_layer : layer];
-  maps.wo = L.wo; maps.wg = L.w_gate_c; maps.wu = L.w_up_c; maps.wd = L.w_down;
+  maps.wo = L.wo; maps.wd = L.w_down;
   maps.wq = Lq.wq; maps.wk = Lq.wk; maps.wv = Lq.wv;
   maps.wo_n = Lq.wo;
   maps.a = am->a; maps.o = am->o; maps.act = am->act;
@@ -503,7 +506,7 @@ int tc_chain(TcState* t, int layer, int qkv_layer, int phase_begin, int phase_en
   p.phase_begin = phase_begin; p.phase_end = phase_end;
   p.split_o = pick_split(d / kChainTile, nq * g.head_dim / kChainTileK, t->max_split);
   p.split_down = pick_split(d / kChainTile, F / kChainTileK, t->max_split);
-  p.fold_norm1 = fold_norm1; p.gu_rows = gate_up_rows(t);
+  p.fold_norm1 = fold_norm1; p.gu_rows = gate_up_rows(t, BN);
   p.x = x; p.a = const_cast<__nv_bfloat16*>(a); p.act = t->act;
   p.part = t->part; p.part_stride = t->part_stride;
   p.g2 = g2; p.g1 = g1; p.eps = g.rms_eps;
@@ -514,6 +517,8 @@ int tc_chain(TcState* t, int layer, int qkv_layer, int phase_begin, int phase_en
     p.bq = (const __nv_bfloat16*)t->bq[lq]; p.bk = (const __nv_bfloat16*)t->bk[lq]; p.bv = (const __nv_bfloat16*)t->bv[lq];
   }
   p.bar = t->grid_bar; p.status = t->status;
+  maps.wg = p.gu_rows == kChainTile ? L.w_gate : L.w_gate_c;
+  maps.wu = p.gu_rows == kChainTile ? L.w_up : L.w_up_c;
   // QKV has nq + 2 nkv tiles; when that is fewer than the grid has CTAs, the CTA pairs left over
   // take a share of every tile's k-blocks
   p.bal_h = 0;
