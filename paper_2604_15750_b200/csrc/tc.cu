@@ -11,6 +11,7 @@
 #include <string>
 
 #include "tc_attn.cuh"
+#include "tc_attn_few.cuh"
 #include "tc_chain.cuh"
 #include "tc_gemm.cuh"
 #include "tc_lmhead.cuh"
@@ -96,7 +97,7 @@ struct TcState {
   int max_split = 4;
   int32_t* status = nullptr;
   int ldv = 0;  // row pitch of the transposed active V
-  CUtensorMap map_q, map_k, map_vt, map_kc, map_vc;
+  CUtensorMap map_q, map_q_few, map_k, map_vt, map_kc, map_vc;
   const void *kc_base = nullptr, *vc_base = nullptr;
   CUtensorMap map_h, map_lm;
   float* lm_part = nullptr;
@@ -206,7 +207,7 @@ int tc_create(const dc_config& g, cudaStream_t s, int M_max, int Mlm_max,
   cudaMemsetAsync(t->k, 0, M * hkv * 2, s);
   cudaMemsetAsync(t->v, 0, (size_t)t->ldv * hkv * 2, s);
   cudaMemsetAsync(t->o, 0, M * hq * 2, s);
-  if (!(make_map_2d(&t->map_q, t->q, M, hq, 64) && make_map_2d(&t->map_k, t->k, M, hkv, 128) &&
+  if (!(make_map_2d(&t->map_q, t->q, M, hq, 64) && make_map_2d(&t->map_q_few, t->q, M, hq, kFewRows) && make_map_2d(&t->map_k, t->k, M, hkv, 128) &&
         make_map_2d(&t->map_vt, t->v, hkv, t->ldv, 128)))
     return tfail(t, DC_ERR_CUDA, "attention tensor map encoding failed");
   t->map_kc = t->map_k; t->map_vc = t->map_vt;  // placeholders until a cache is supplied
@@ -230,10 +231,11 @@ int tc_create(const dc_config& g, cudaStream_t s, int M_max, int Mlm_max,
       return tfail(t, DC_ERR_CUDA, "cannot opt in to shared memory for the LM head");
     }
   }
-  if (cudaFuncSetAttribute(k_attn_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, kAttnSmem) !=
-      cudaSuccess) {
+  if (cudaFuncSetAttribute(k_attn_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, kAttnSmem) != cudaSuccess ||
+      cudaFuncSetAttribute(k_attn_few, cudaFuncAttributeMaxDynamicSharedMemorySize, few_smem(kFewSlotsMax)) != cudaSuccess ||
+      cudaFuncSetAttribute(k_attn_few, cudaFuncAttributePreferredSharedMemoryCarveout, 100) != cudaSuccess) {
     cudaGetLastError();
-    return tfail(t, DC_ERR_CUDA, "cannot opt in to %d bytes of shared memory", kAttnSmem);
+    return tfail(t, DC_ERR_CUDA, "cannot opt in to %d bytes of shared memory", few_smem(kFewSlotsMax));
   }
   cudaError_t e1 = cudaFuncSetAttribute(k_gemm_tc<GEMM_EPI_QKV, false>,
                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -420,20 +422,32 @@ int tc_attention(TcState* t, int layer, const SeqMeta& m, const __nv_bfloat16* k
       export_tiles = n > export_tiles ? n : export_tiles;
     }
   }
-  const int nqt = (m.R_cap + 127) / 128;
+  // few rows: keys on the lanes (tc_attn_few.cuh)
+  int few_ctas = 0;
+  for (int b = 0; b < m.batch; ++b) few_ctas += m.nv * nq * ((m.last_len[b] + m.win_len[b] + kFewRows - 1) / kFewRows);
+  const bool few = few_rows_rule(m, few_ctas, t->n_sm);
+  const int nqt = few ? (m.R_cap + kFewRows - 1) / kFewRows : (m.R_cap + 127) / 128;
   // one CTA per query tile: (row tile, variant) with two variants in the pass (a row tile with 64
   // rows or fewer packs both variants into the curr CTA, the prev CTA returns at once)
   ap.units = export_only ? 0 : m.nv == 2 ? 2 * nqt : nqt;
   if (ap.units + export_tiles == 0) return DC_OK;
   dim3 grid(ap.units + export_tiles, nq, m.batch);
+  // programmatic launch not between two launches of the dense chain: there it cost 1..3% of a step (4523 ->
+  // 4658 us on one LLaDA-8B sequence)
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid; cfg.stream = t->s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr; cfg.numAttrs = chained ? 1 : 0;
   cudaError_t e;
-  if (chained) {
-    e = launch_chained(k_attn_tc, grid, kAttnThreads, kAttnSmem, t->s, t->map_q, t->map_k, t->map_vt, t->map_kc, t->map_vc, ap);
+  if (few) {
+    const int slots = few_ctas > t->n_sm ? 3 : kFewSlotsMax;   // two CTAs on an SM, or one with a deeper ring
+    cfg.blockDim = dim3(kFewThreads); cfg.dynamicSmemBytes = few_smem(slots);
+    e = cudaLaunchKernelEx(&cfg, k_attn_few, t->map_q_few, t->map_k, t->map_vt, t->map_kc, t->map_vc, ap, slots);
   } else {
-    // between two launches of the dense chain (programmatic launches there cost 1..3% of a step: 4523 ->
-    // 4658 us on one LLaDA-8B sequence)
-    k_attn_tc<<<grid, kAttnThreads, kAttnSmem, t->s>>>(t->map_q, t->map_k, t->map_vt, t->map_kc, t->map_vc, ap);
-    e = cudaGetLastError();
+    cfg.blockDim = dim3(kAttnThreads); cfg.dynamicSmemBytes = kAttnSmem;
+    e = cudaLaunchKernelEx(&cfg, k_attn_tc, t->map_q, t->map_k, t->map_vt, t->map_kc, t->map_vc, ap);
   }
   if (e != cudaSuccess) return tfail(t, DC_ERR_CUDA, "attention launch failed: %s", cudaGetErrorString(e));
   return DC_OK;

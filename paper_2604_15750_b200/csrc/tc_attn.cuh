@@ -135,6 +135,7 @@ __device__ __forceinline__ AttnTile attn_tile(const AttnUnit& a, int j) {
 // SMs that a small batch leaves idle.  As a kernel of its own, with a row per CTA and element-wise
 // stores of V at a stride of max_ctx, this took 11 us of each layer of a one-sequence step and 59 us
 // of a 1024-token prefill, plus a launch.
+template <int THREADS>
 __device__ __forceinline__ void attn_export_tile(const AttnParams& p, int b, int g, int r0) {
   const int n = min(kBK, p.m.last_len[b] - r0);
   const int row = act_row(p.m, 0, b, r0), key = p.m.ctx_len[b] + r0;
@@ -142,7 +143,7 @@ __device__ __forceinline__ void attn_export_tile(const AttnParams& p, int b, int
   const __nv_bfloat16* ks = p.k + (size_t)row * p.nkv * kHd + g * kHd;
   __nv_bfloat16* kd = p.k_cache + (kv * p.max_ctx + key) * kHd;
 #pragma unroll 4
-  for (int i = threadIdx.x; i < n * (kHd / 8); i += kAttnThreads) {
+  for (int i = threadIdx.x; i < n * (kHd / 8); i += THREADS) {
     const int r = i / (kHd / 8), c = i % (kHd / 8) * 8;
     *reinterpret_cast<uint4*>(kd + (size_t)r * kHd + c) =
         *reinterpret_cast<const uint4*>(ks + (size_t)r * p.nkv * kHd + c);
@@ -153,7 +154,7 @@ __device__ __forceinline__ void attn_export_tile(const AttnParams& p, int b, int
     const __nv_bfloat16* vs = p.v + (size_t)g * kHd * p.ldv + row;
     __nv_bfloat16* vd = p.v_cache + kv * kHd * p.max_ctx + key;
 #pragma unroll 4
-    for (int i = threadIdx.x; i < kHd * (kBK / 8); i += kAttnThreads) {
+    for (int i = threadIdx.x; i < kHd * (kBK / 8); i += THREADS) {
       const int e = i / (kBK / 8), c = i % (kBK / 8) * 8;
       if (c < n)
         *reinterpret_cast<uint4*>(vd + (size_t)e * p.max_ctx + c) = *reinterpret_cast<const uint4*>(vs + (size_t)e * p.ldv + c);
@@ -162,7 +163,7 @@ __device__ __forceinline__ void attn_export_tile(const AttnParams& p, int b, int
   }
   const int odd = key & 1, pairs = (n + odd + 1) >> 1, lane = threadIdx.x & 31;
 #pragma unroll 2
-  for (int e = threadIdx.x >> 5; e < kHd; e += kAttnThreads / 32) {
+  for (int e = threadIdx.x >> 5; e < kHd; e += THREADS / 32) {
     const __nv_bfloat16* vs = p.v + (size_t)(g * kHd + e) * p.ldv + row;
     __nv_bfloat16* vd = p.v_cache + (kv * kHd + e) * p.max_ctx + key;
 #pragma unroll 3
@@ -200,7 +201,7 @@ k_attn_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
   if ((int)blockIdx.x >= p.units) {
     pdl_wait();
     const int r0 = ((int)blockIdx.x - p.units) * kBK;
-    if (h < p.nkv && r0 < p.m.last_len[b]) attn_export_tile(p, b, h, r0);
+    if (h < p.nkv && r0 < p.m.last_len[b]) attn_export_tile<kAttnThreads>(p, b, h, r0);
     return;
   }
   AttnUnit un;

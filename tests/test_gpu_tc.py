@@ -2,7 +2,10 @@
 on sizes that span several weight tiles, k-blocks, column blocks and ragged tails."""
 import numpy as np
 import pytest
+import torch
 
+from oracle import adapters
+from oracle import depcap_oracle as O
 from paper_2604_15750_b200 import inputs
 
 from parity import Case, compare
@@ -174,3 +177,86 @@ def test_fused_chain_gate_up_tile_heights(ff, last, win, influence):
     _, launches = eng.step_profiled(influence=influence, boundary=True, **di)
     assert launches["dense"] == case.n_layers + 1
     eng.close()
+
+
+@pytest.mark.parametrize("n_q,n_kv,ctx,last,win", [
+    (4, 2, [0], [0], [16]),                  # active keys only
+    (4, 2, [1], [1], [1]),                   # one cached key; two rows
+    (4, 2, [128], [0], [7]),                 # whole context tile
+    (4, 4, [129], [5], [27]),                # one key in the second tile, 32 rows, append at an odd position
+    (4, 2, [700], [31], [33]),               # 64 rows: two row tiles; six tiles through the deep ring
+    (40, 20, [513, 40, 300, 250], [16, 5, 0, 9], [32, 17, 9, 24]),   # more CTAs than SMs: two on an SM
+    (32, 32, [1200, 1163, 1126, 1000, 960, 1190, 900, 1024], [0] * 8, [24, 19, 14, 9, 32, 8, 24, 1]),   # as above, caches larger than L2
+])
+def test_tc_attention_few_rows(n_q, n_kv, ctx, last, win):
+    """One variant of few rows: keys on the lanes, 32 rows a CTA.  With the last block
+    appended: its keys and values at the 2e-2 of a bf16 stack, nothing else of the cache written."""
+    B = len(ctx)
+    wl = _wl(B, n_q=n_q, n_kv=n_kv, ctx=(max(max(ctx), 1), max(max(ctx), 1)), last=max(max(last), 1), win=max(win))
+    case = Case(wl, lengths=dict(ctx_len=ctx, last_len=last, win_len=win, remain_len=[64] * B))
+    eng = case.make_engine(max_ctx=1280, max_window=(max(win) + 15) // 16 * 16)
+    di = case.device_inputs(eng, poison=True)
+    k0, v0 = di["k_cache"].clone(), di["v_cache"].clone()
+    out = eng.step(influence=False, boundary=True, export_kv=True, **di)
+    sel = eng.select(di["win_ids"], di["win_len"])
+    eng.synchronize()
+    gpu = {k_: v_.cpu().numpy() for k_, v_ in {**out, **sel}.items()}
+    ora = {b: O.step(case.ocfg, case.ow, adapters.to_np(case.k_log[:, b]), adapters.to_np(case.v_log[:, b]), ctx[b],
+                     case.last_ids[b, :last[b]].numpy(), case.win_ids[b, :win[b]].numpy(), 64, influence=False,
+                     return_kv=True) for b in range(B)}
+    compare(case, gpu, ora)
+    for b in range(B):
+        end = ctx[b] + last[b]
+        for new, old in ((di["k_cache"][:, b], k0[:, b]), (di["v_cache"][:, b].transpose(-1, -2), v0[:, b].transpose(-1, -2))):
+            assert torch.equal(new[:, :, :ctx[b]], old[:, :, :ctx[b]]) and new[:, :, end:].isnan().all()
+            which = 0 if new.data_ptr() == di["k_cache"][:, b].data_ptr() else 1
+            for l in range(case.n_layers if last[b] else 0):
+                ref = ora[b]["kv_last"][l][which]                    # [last, nkv, hd]
+                got = new[l, :, ctx[b]:end].float().permute(1, 0, 2).cpu().numpy()
+                assert np.abs(got - ref).max() / max(np.abs(ref).max(), 1.0) <= 2e-2, (b, l)
+    eng.close()
+
+
+@pytest.mark.parametrize("batch,ctx,last,win", [
+    (2, [300, 300], [32, 32], [128, 128]),                 # two query tiles, the second of both variants
+    (4, [128, 40, 77, 0], [16, 5, 0, 9], [32, 17, 9, 27]), # both variants in one tile, ragged
+    (1, [513], [32], [96]),                                # 128 rows a variant
+])
+def test_tc_attention_many_heads(batch, ctx, last, win):
+    """40 heads: more (row tile, head) units than the few-rows kernel is given, so rows on the lanes.  Poisoned
+    caches, and cached keys (where there are 300) that make the pass run again."""
+    wl = _wl(batch, n_q=40, n_kv=20, ctx=(max(ctx), max(ctx)), last=max(last), win=max(win))
+    case = Case(wl, lengths=dict(ctx_len=ctx, last_len=last, win_len=win, remain_len=[128] * batch))
+    eng = case.make_engine(max_window=(max(win) + 15) // 16 * 16)
+    gpu, ora = case.run_gpu(eng, poison=True), case.run_oracle()
+    compare(case, gpu, ora)
+    if ctx[0] == 300:
+        for pos in (150, 210, 290):
+            case.k_log[:, :, :, pos, :] *= 2000.0
+        gpu, ora = case.run_gpu(eng), case.run_oracle()
+        for b in range(batch):   # (tolerances as in the test above of scores far from the first)
+            W = win[b]
+            for name in ("conf", "entropy", "lse"):
+                ref = ora[b][name]
+                assert (np.abs(gpu[name][b, :W] - ref) / np.maximum(np.abs(ref), 1.0)).max() <= 2e-2, (name, b)
+            assert (gpu["pred_id"][b, :W] == ora[b]["pred"]).mean() >= 0.95
+    eng.close()
+
+
+def test_tc_attention_few_rows_with_scores_far_above_the_first():
+    """Keys behind the first 32 that lie hundreds of log2 units above them: the passes that find the maxima and
+    use them.  Tolerances as in the test of the other kernel above."""
+    wl = _wl(2, ctx=(300, 300), last=1, win=40)
+    case = Case(wl, lengths=dict(ctx_len=[300, 290], last_len=[0, 0], win_len=[40, 33], remain_len=[64, 64]))
+    for pos in (50, 150, 270):
+        case.k_log[:, :, :, pos, :] *= 2000.0
+    eng = case.make_engine()
+    gpu, ora = case.run_gpu(eng, influence=False), case.run_oracle(influence=False)
+    eng.close()
+    for b in range(2):
+        W = case.len["win_len"][b]
+        for name in ("conf", "entropy", "lse"):
+            ref = ora[b][name]
+            err = np.abs(gpu[name][b, :W] - ref) / np.maximum(np.abs(ref), 1.0)
+            assert np.isfinite(gpu[name][b, :W]).all() and err.max() <= 2e-2, (name, b, err.max())
+        assert (gpu["pred_id"][b, :W] == ora[b]["pred"]).mean() >= 0.95
