@@ -260,12 +260,7 @@ k_attn_few(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CU
           const int s = (2 * J + 1) % slots;
           ok = __all_sync(0xffffffffu, ptx::mbar_wait(&c.v_full[J % 3], (uint32_t)(J / 3) & 1u, abort_flag));
           if (!ok) break;
-          uint8_t* base = ring + (size_t)s * kFewSlot + key * 128;
-          for (int cc = nvalid; cc < kBK;) {
-            uint8_t* at = base + (cc >> 6) * kSub + ((((cc & 63) >> 3) ^ (key & 7)) << 4) + (cc & 7) * 2;
-            if ((cc & 7) == 0) { *reinterpret_cast<uint4*>(at) = make_uint4(0, 0, 0, 0); cc += 8; }
-            else { *reinterpret_cast<uint16_t*>(at) = 0; ++cc; }
-          }
+          attn_clear_v(ring + (size_t)s * kFewSlot, key, nvalid);
         }
         ptx::fence_proxy_async_smem();
         __syncwarp();
