@@ -164,6 +164,8 @@ int build_meta(dc_ctx* c, int batch, int flags, const int32_t* ctx_len, const in
     m->remain[b] = remain_len ? remain_len[b] : W;
     m->have_prev[b] = (m->nv == 2 && Lb > 0) ? 1 : 0;
     maxR = maxR > Lb + W ? maxR : Lb + W;
+    m->row0[b] = m->rows;
+    m->rows += round_up(Lb + W, 16);
     maxW = maxW > W ? maxW : W;
   }
   m->R_cap = round_up(maxR, 16);
@@ -204,7 +206,7 @@ int run_step(dc_ctx* c, const dc_step_in* in, const dc_step_out* out, const SeqM
   cudaStream_t s = c->stream;
   Profiler& pf = c->prof;
   const int d = g.d_model, nq = g.n_q_heads, nkv = g.n_kv_heads, hd = g.head_dim, F = g.d_ff;
-  const int M = m.nv * m.batch * m.R_cap;
+  const int M = m.nv * m.rows;
   const bool carried = (in->flags & DC_STEP_CARRIED_PREV) != 0;
   const SeqMeta ml = carried ? carried_meta(m, in->prev_len) : m;   // what the LM-head stage sees
   const int Mlm = ml.nv * ml.npos_pad;

@@ -21,7 +21,13 @@ struct SeqMeta {
   int pos0[DC_MAX_BATCH];   // absolute position of active row 0 (ctx_len unless a prefill says otherwise)
   int batch;     // B
   int nv;        // variants in the pass: 1 (curr) or 2 (curr, prev)
-  int R_cap;     // active rows per (variant, sequence), multiple of 16: [last ; window ; pad]
+  int R_cap;     // the most active rows of a sequence, rounded up to 16
+  // active rows [last ; window ; pad] of a sequence, rounded up to 16 each (the dense chain rotates 16 rows in
+  // a step), lie behind those of the one before: a ragged batch has no rows that only fill it up to its longest
+  // sequence (eight denoising steps of 8..24 rows are 192 rows instead of 256: 5925 -> 5303 us; four prompts
+  // of 450..600 tokens 33.4 -> 29.1 ms).
+  int rows;                     // rows of one variant
+  int row0[DC_MAX_BATCH];       // first row of each sequence in its variant
   int W_cap;     // window rows per sequence, multiple of 16
   int G;         // LM-head group: positions per group (<= 128)
   int npos_pad;  // B * W_cap rounded up to a multiple of G
@@ -29,7 +35,13 @@ struct SeqMeta {
 
 // active row index of (variant v, sequence b, row r)
 __host__ __device__ inline int act_row(const SeqMeta& m, int v, int b, int r) {
-  return (v * m.batch + b) * m.R_cap + r;
+  return v * m.rows + m.row0[b] + r;
+}
+// sequence of row br of a variant
+__host__ __device__ inline int act_seq(const SeqMeta& m, int br) {
+  int b = 0;
+  while (b + 1 < m.batch && br >= m.row0[b + 1]) ++b;
+  return b;
 }
 // LM-head row of (variant v, flattened position p = b * W_cap + k): groups of G positions,
 // inside a group the curr rows come first, then the prev rows.

@@ -31,8 +31,8 @@ __device__ __forceinline__ float block_sum(float v, float* red) {
 // the last block's ids replaced by the mask id, everything else fixed, which makes p_prev =
 // p(Z_k | c) (Section 4.4).  The block of a sequence's first curr row checks all of its ids and writes
 // status[b] (so that nothing has to clear it first).
-// The other blocks: cos_sin[(b * R_cap + r) * hd + i] = cos(angle), [.. + hd/2 + i] = sin(angle), angle =
-// (pos0[b] + r) * theta^(-2i/hd), evaluated in double precision; row batch * R_cap holds cos / sin of
+// The other blocks: cos_sin[(row0[b] + r) * hd + i] = cos(angle), [.. + hd/2 + i] = sin(angle), angle =
+// (pos0[b] + r) * theta^(-2i/hd), evaluated in double precision; row `rows` holds cos / sin of
 // theta^(-2i/hd) itself, the angle step between consecutive rows.  The first of them also clears the
 // grid-barrier words of the kernels that follow.
 // (One launch: as a memset and two kernels the start of a step took 8 us, most of it launch latency.)
@@ -43,10 +43,9 @@ __global__ void __launch_bounds__(128) k_step_begin(const T* __restrict__ embed,
                                                     float* __restrict__ x, int32_t* __restrict__ status, int hd, float theta,
                                                     float* __restrict__ cos_sin, unsigned int* __restrict__ words, int n_words) {
   pdl_trigger();
-  const int M = m.nv * m.batch * m.R_cap, row = blockIdx.x;
+  const int M = m.nv * m.rows, row = blockIdx.x;
   if (row < M) {
-    const int r = row % m.R_cap, vb = row / m.R_cap;
-    const int b = vb % m.batch, v = vb / m.batch;
+    const int v = row / m.rows, br = row - v * m.rows, b = act_seq(m, br), r = br - m.row0[b];
     const int Lb = m.last_len[b], W = m.win_len[b];
     if (r == 0 && v == 0) {
       int bad = 0;
@@ -76,10 +75,10 @@ __global__ void __launch_bounds__(128) k_step_begin(const T* __restrict__ embed,
     for (int i = threadIdx.x; i < n_words; i += blockDim.x) words[i] = 0u;
   const int half = hd / 2;
   const int idx = (row - M) * 128 + threadIdx.x;
-  const int rows = m.batch * m.R_cap;
+  const int rows = m.rows;
   if (idx >= (rows + 1) * half) return;   // one extra row: cos / sin of the per-row angle step
   const int i = idx % half, br = idx / half;
-  const int r = br % m.R_cap, b = br / m.R_cap;
+  const int b = act_seq(m, br), r = br - m.row0[b];
   const double inv_freq = pow((double)theta, -2.0 * (double)i / (double)hd);
   const double ang = (br < rows) ? (double)(m.pos0[b] + r) * inv_freq : inv_freq;
   double sn, cs;
@@ -92,7 +91,7 @@ template <typename T>
 void launch_step_begin(const T* embed, const int32_t* last_ids, const int32_t* win_ids, int max_last, int max_window,
                        int mask_id, int vocab, int d, const SeqMeta& m, float* x, int32_t* status, int head_dim,
                        float theta, float* cos_sin, unsigned int* words, int n_words, cudaStream_t s) {
-  const int M = m.nv * m.batch * m.R_cap, table = (m.batch * m.R_cap + 1) * (head_dim / 2);
+  const int M = m.nv * m.rows, table = (m.rows + 1) * (head_dim / 2);
   k_step_begin<T><<<M + (table + 127) / 128, 128, 0, s>>>(embed, last_ids, win_ids, max_last, max_window, mask_id, vocab,
                                                           d, m, x, status, head_dim, theta, cos_sin, words, n_words);
 }

@@ -81,7 +81,7 @@ __device__ __forceinline__ float sum2(f2 v) {
 template <typename T, typename G>
 __device__ __forceinline__ void simt_store_qkv(const G& g, int m, int head, int e, float y1, float y2) {
   const int hd = g.hd, half = hd >> 1;
-  const int rv = g.m.batch * g.m.R_cap, br = m % rv;   // (b, r): the RoPE table is shared by both variants
+  const int rv = g.m.rows, br = m % rv;   // (b, r): the RoPE table is shared by both variants
   if (g.bq != nullptr) {   // projection bias, before the rotation
     const T* bb = head < g.nq ? g.bq + head * hd : head < g.nq + g.nkv ? g.bk + (head - g.nq) * hd
                                                                        : g.bv + (head - g.nq - g.nkv) * hd;
@@ -104,7 +104,7 @@ __device__ __forceinline__ void simt_store_qkv(const G& g, int m, int head, int 
   T* dst = (is_v ? g.v : g.k) + (size_t)m * g.nkv * hd + hk * hd + e;
   dst[0] = o1; dst[half] = o2;
   if (g.k_cache != nullptr && m < rv) {
-    const int b = br / g.m.R_cap, r = br - b * g.m.R_cap;
+    const int b = act_seq(g.m, br), r = br - g.m.row0[b];
     if (r < g.m.last_len[b]) {
       const size_t kv = (size_t)b * g.nkv + hk;
       const int key = g.m.ctx_len[b] + r;

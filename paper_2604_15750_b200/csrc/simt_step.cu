@@ -560,7 +560,7 @@ __global__ void __launch_bounds__(kFuseThreads, 1) k_simt_step(const __grid_cons
     return go != 0;
   };
 
-  const int M = p.m.nv * p.m.batch * p.m.R_cap, n_phases = 5 * p.n_layers;
+  const int M = p.m.nv * p.m.rows, n_phases = 5 * p.n_layers;
 #pragma unroll 1
   for (int ph = 0; ph <= n_phases; ++ph) {
     const int l = ph / 5, kind = ph == n_phases ? 5 : ph - 5 * l;   // QKV, attention, O, gate / up, down; LM head
@@ -655,7 +655,7 @@ template <typename T>
 bool simt_step_ok(const SimtFuse& f, const SimtStep<T>& p) {
   if (f.grid == 0) return false;
   // GEMMs that take many rounds of small tiles are better off as kernels of their own, with the larger tile
-  const long long M = (long long)p.m.nv * p.m.batch * p.m.R_cap, Mlm = (long long)p.ml.nv * p.ml.npos_pad;
+  const long long M = (long long)p.m.nv * p.m.rows, Mlm = (long long)p.ml.nv * p.ml.npos_pad;
   const long long mt = (M + 15) / 16;
   long long most = mt * ((p.F + 7) / 8);
   const long long qkv = mt * (p.nq + 2 * p.nkv) * (p.hd / 16), lm = p.kv_only ? 0 : (Mlm + 15) / 16 * ((p.V + 15) / 16);

@@ -139,8 +139,8 @@ T* talloc(TcState* t, size_t n, bool* ok) {
 
 int pick_bn(int M) {
   const int nblk = (M + 255) / 256;
-  const int bn = ((M + nblk - 1) / nblk + 15) / 16 * 16;
-  return bn;
+  const int step = nblk > 1 ? 32 : 16;   // several blocks: what the MMAs of CTA pairs take
+  return ((M + nblk - 1) / nblk + step - 1) / step * step;
 }
 
 }  // namespace
@@ -474,7 +474,7 @@ void tc_set_cooperative(TcState* t, bool on) { t->chain_coop = on && t->coop_sup
 
 bool tc_chain_ok(const TcState* t, const SeqMeta& m) {
   const dc_config& g = t->g;
-  const int M = m.nv * m.batch * m.R_cap;
+  const int M = m.nv * m.rows;
   // One column block of 16 to 256 activation rows (N of a pair MMA is any multiple of 16 there).  A
   // LLaDA-8B denoising step over a block of up to 16 positions takes 4640 us on the per-op kernels
   // (7 launches per layer, 2 us of gap each, no weight stream across them) and 4006 us here.  The
@@ -503,7 +503,7 @@ int tc_chain(TcState* t, int layer, int qkv_layer, int phase_begin, int phase_en
              size_t* part_stride) {
   const dc_config& g = t->g;
   const int d = g.d_model, nq = g.n_q_heads, nkv = g.n_kv_heads, F = g.d_ff;
-  const int M = m.nv * m.batch * m.R_cap;
+  const int M = m.nv * m.rows;
   const int BN = (M + 15) / 16 * 16;
   ActMaps* am = nullptr;
   int rc = get_act_maps(t, a, BN / 2, &am);  // every CTA of a pair stages half of the rows
@@ -524,7 +524,7 @@ int tc_chain(TcState* t, int layer, int qkv_layer, int phase_begin, int phase_en
   p.x = x; p.a = const_cast<__nv_bfloat16*>(a); p.act = t->act;
   p.part = t->part; p.part_stride = t->part_stride;
   p.g2 = g2; p.g1 = g1; p.eps = g.rms_eps;
-  p.cos_sin = cos_sin; p.rows_per_variant = m.batch * m.R_cap;
+  p.cos_sin = cos_sin; p.rows_per_variant = m.rows;
   p.q = t->q; p.k = t->k; p.v = t->v; p.ldv = t->ldv;
   if (!t->bq.empty()) {
     const int lq = qkv_layer < g.n_layers ? qkv_layer : layer;
@@ -583,7 +583,7 @@ int tc_layer(TcState* t, int layer, const SeqMeta& m, float* x, const __nv_bfloa
              StageHook& hook, bool export_kv, bool kv_only) {
   const dc_config& g = t->g;
   const int d = g.d_model, nq = g.n_q_heads, nkv = g.n_kv_heads, hd = g.head_dim, F = g.d_ff;
-  const int M = m.nv * m.batch * m.R_cap;
+  const int M = m.nv * m.rows;
   const int BN = pick_bn(M);
   ActMaps *am = nullptr, *amh = nullptr;
   int rc = get_act_maps(t, a, BN, &am);
@@ -597,7 +597,7 @@ int tc_layer(TcState* t, int layer, const SeqMeta& m, float* x, const __nv_bfloa
   const LayerMaps& L = t->layers[layer];
   GemmParams p{};
   p.M = M; p.BN = BN; p.nq = nq; p.nkv = nkv; p.hd = hd;
-  p.cos_sin = cos_sin; p.rows_per_variant = m.batch * m.R_cap;
+  p.cos_sin = cos_sin; p.rows_per_variant = m.rows;
   p.q = t->q; p.k = t->k; p.v = t->v; p.ldv = t->ldv; p.act = t->act;
   if (!t->bq.empty()) {
     p.bq = (const __nv_bfloat16*)t->bq[layer]; p.bk = (const __nv_bfloat16*)t->bk[layer]; p.bv = (const __nv_bfloat16*)t->bv[layer];
@@ -751,7 +751,7 @@ extern "C" int dc_signals_static(const dc_signals_in* in, const dc_signals_out* 
     maxW = maxW > W ? maxW : W;
   }
   m.W_cap = (maxW + 15) / 16 * 16;
-  m.R_cap = m.W_cap;
+  m.R_cap = m.W_cap;   // (no stack: no active rows)
   const int npos = in->batch * m.W_cap;
   if (npos > DC_STATIC_MAX_POS)
     return sfail(DC_ERR_SHAPE, "more than DC_STATIC_MAX_POS window positions: the fixed scratch array cannot hold them");

@@ -46,7 +46,7 @@ struct GemmParams {
   // QKV epilogue
   int nq, nkv, hd;          // tiles [0,nq) are q heads, [nq,nq+nkv) k heads, rest v heads
   const float* cos_sin;     // RoPE table [(b, r)][hd]
-  int rows_per_variant;     // batch * R_cap: the table is shared by the variants
+  int rows_per_variant;     // the table is shared by the variants
   const __nv_bfloat16 *bq, *bk, *bv;  // projection biases [nq*hd], [nkv*hd], [nkv*hd], or null
   __nv_bfloat16 *q, *k, *v; // outputs q [M, nq*hd], k [M, nkv*hd], v TRANSPOSED [nkv*hd, ldv]
   int ldv;                  // row pitch of the transposed v (elements, multiple of 8)

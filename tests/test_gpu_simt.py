@@ -1,6 +1,10 @@
 """CUDA-core kernels at the shapes where their tiles can go wrong, against the oracle."""
+import numpy as np
 import pytest
+import torch
 
+from oracle import adapters
+from oracle import depcap_oracle as O
 from paper_2604_15750_b200 import inputs
 
 from parity import Case, compare
@@ -61,4 +65,35 @@ def test_fused_step_and_separate_launches(wl):
         n = lengths["win_len"][b]
         for k in ("conf", "entropy", "lse"):
             assert abs(gpu[k][b, :n] - one[k][b, :n]).max() <= tol * max(1.0, abs(one[k][b, :n]).max()), (k, b)
+    eng.close()
+
+
+@pytest.mark.parametrize("cooperative", [1, 0])   # the fused step, separate launches
+def test_ragged_rows_lie_behind_one_another(cooperative):
+    """Sequences of 48, 16 and 32 rows (rounded up) in a batch, fp32: signals at 1e-4, the appended keys and values at
+    1e-4, nothing else of the cache written."""
+    ctx, last, win = [40, 64, 7], [16, 0, 5], [32, 3, 12]
+    wl = inputs.Workload("ragged_f32", 2, 64, 4, 2, 16, 128, 300, "f32", 3, 64, 64, 16, 32, 64, 515)
+    case = Case(wl, lengths=dict(ctx_len=ctx, last_len=last, win_len=win, remain_len=[64] * 3))
+    eng = case.make_engine(max_ctx=128)
+    eng.set_option(1, cooperative)             # DC_OPT_COOPERATIVE
+    di = case.device_inputs(eng)
+    k0, v0 = di["k_cache"].clone(), di["v_cache"].clone()
+    out = eng.step(influence=True, boundary=True, export_kv=True, **di)
+    sel = eng.select(di["win_ids"], di["win_len"])
+    eng.synchronize()
+    gpu = {k_: v_.cpu().numpy() for k_, v_ in {**out, **sel}.items()}
+    ora = {b: O.step(case.ocfg, case.ow, adapters.to_np(case.k_log[:, b]), adapters.to_np(case.v_log[:, b]), ctx[b],
+                     case.last_ids[b, :last[b]].numpy(), case.win_ids[b, :win[b]].numpy(), 64, return_kv=True)
+           for b in range(3)}
+    compare(case, gpu, ora)
+    for b in range(3):
+        end = ctx[b] + last[b]
+        for which, (new, old) in enumerate(((di["k_cache"][:, b], k0[:, b]),
+                                            (di["v_cache"][:, b].transpose(-1, -2), v0[:, b].transpose(-1, -2)))):
+            assert torch.equal(new[:, :, :ctx[b]], old[:, :, :ctx[b]]) and torch.equal(new[:, :, end:], old[:, :, end:])
+            for l in range(2 if last[b] else 0):
+                ref = ora[b]["kv_last"][l][which]                    # [last, nkv, hd]
+                got = new[l, :, ctx[b]:end].permute(1, 0, 2).cpu().numpy()
+                assert np.abs(got - ref).max() / max(np.abs(ref).max(), 1.0) <= 1e-4, (b, l)
     eng.close()

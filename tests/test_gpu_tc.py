@@ -185,6 +185,7 @@ def test_fused_chain_gate_up_tile_heights(ff, last, win, influence):
     (4, 2, [128], [0], [7]),                 # whole context tile
     (4, 4, [129], [5], [27]),                # one key in the second tile, 32 rows, append at an odd position
     (4, 2, [700], [31], [33]),               # 64 rows: two row tiles; six tiles through the deep ring
+    (4, 2, [40, 64, 7], [16, 0, 5], [32, 3, 12]),   # 48, 16 and 32 rows, one sequence behind the other
     (40, 20, [513, 40, 300, 250], [16, 5, 0, 9], [32, 17, 9, 24]),   # more CTAs than SMs: two on an SM
     (32, 32, [1200, 1163, 1126, 1000, 960, 1190, 900, 1024], [0] * 8, [24, 19, 14, 9, 32, 8, 24, 1]),   # as above, caches larger than L2
 ])
