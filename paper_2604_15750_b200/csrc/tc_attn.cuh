@@ -129,9 +129,9 @@ __device__ __forceinline__ AttnTile attn_tile(const AttnUnit& a, int j) {
 }
 
 
-// Clears keys valid .. 127 of row rr of a V^T tile, eight at a time.  (One at a time by one warp, the tile with
-// the last cached keys took 8 us longer: two variants behind 513 cached keys
-// 21.4 -> 17.1 us a layer, eight ragged sequences 150.7 -> 140.8.)
+// Clears keys valid .. 127 of row rr of a V^T tile, eight at a time.  (One at a time, by one warp, on the serial
+// chain of the pass: two variants behind 513 cached keys 21.4 us a layer instead of 17.1, eight ragged
+// sequences 150.7 instead of 140.8.)
 __device__ __forceinline__ void attn_clear_v(uint8_t* tile, int rr, int valid) {
   for (int cc = valid; cc < kBK;) {
     uint8_t* at = tile + (cc >> 6) * kSub + rr * 128 + ((((cc & 63) >> 3) ^ (rr & 7)) << 4) + (cc & 7) * 2;
