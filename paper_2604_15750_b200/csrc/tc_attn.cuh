@@ -29,7 +29,7 @@
 //
 // Warp roles (512 threads): warp 0 = TMA producer for Q and K, warp 1 = TMEM owner + issuer of the
 // score MMAs (Q K^T), warp 2 = TMA producer for V^T, warp 3 = issuer of the output MMAs (P V; all
-// its lanes first clear the V^T columns beyond ctx_len in the one tile that has any), warps 4..15 =
+// its lanes first clear the V^T columns beyond the valid keys, attn_clear_v), warps 4..15 =
 // softmax / output (TMEM lane quarter = warp % 4, slot = (warp - 4) / 4).  Two issuing threads
 // because one was the bottleneck: with its four barrier waits and two commits per tile it needed
 // about 2270 clocks per tile for MMAs that keep the tensor pipe busy for 1024.
@@ -129,15 +129,21 @@ __device__ __forceinline__ AttnTile attn_tile(const AttnUnit& a, int j) {
 }
 
 
-// Clears keys valid .. 127 of row rr of a V^T tile, eight at a time.  (One at a time, by one warp, on the serial
-// chain of the pass: two variants behind 513 cached keys 21.4 us a layer instead of 17.1, eight ragged
-// sequences 150.7 instead of 140.8.)
+// Keys of a tile that the P V product takes: its MMAs are 16 keys each, those without a valid key are left out.
+__device__ __forceinline__ int attn_pv_keys(int valid) { return (valid + 15) & ~15; }
+// Clears what the product takes beyond the valid keys (valid % 16 != 0), in row rr of a V^T tile.  Any tile may
+// hold NaN there, a tile of active keys too (the rows of the next sequence, or what an earlier step left), and
+// the product with their probability 0 must be 0.  In whole 16-byte pieces, because this is on the serial chain
+// of the pass: a Dream-7B prefill of 187 tokens, two tiles of active keys, takes 3836 us like this, 3865 with the
+// keys cleared one at a time, and 3823 with active tiles left as they are.
 __device__ __forceinline__ void attn_clear_v(uint8_t* tile, int rr, int valid) {
-  for (int cc = valid; cc < kBK;) {
-    uint8_t* at = tile + (cc >> 6) * kSub + rr * 128 + ((((cc & 63) >> 3) ^ (rr & 7)) << 4) + (cc & 7) * 2;
-    if ((cc & 7) == 0) { *reinterpret_cast<uint4*>(at) = make_uint4(0, 0, 0, 0); cc += 8; }
-    else { *reinterpret_cast<uint16_t*>(at) = 0; ++cc; }
-  }
+  const int c = valid >> 3, k = valid & 7;   // the piece of eight keys that the valid ones end in, and how many of it are
+  auto piece = [&](int i) { return reinterpret_cast<uint4*>(tile + (i >> 3) * kSub + rr * 128 + (((i & 7) ^ (rr & 7)) << 4)); };
+  auto kept = [&](int e) { return k > e + 1 ? 0xffffffffu : k > e ? 0xffffu : 0u; };   // of keys e and e + 1
+  uint4 w = *piece(c);
+  w.x &= kept(0); w.y &= kept(2); w.z &= kept(4); w.w &= kept(6);
+  *piece(c) = w;
+  if ((c & 1) == 0) *piece(c + 1) = make_uint4(0, 0, 0, 0);
 }
 
 // Appends rows r0 .. r0 + 127 of the last decoded block (curr variant) of one sequence and kv head to
@@ -375,11 +381,10 @@ k_attn_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
         const uint32_t s = (uint32_t)(J % kAttnStagesV), ph = ((uint32_t)(J / kAttnStagesV)) & 1u;
         const uint32_t sb = (uint32_t)J % 3u;
         const AttnTile t = attn_tile(un, j);
-        if (t.is_ctx && t.valid < kBK) {
-          // The one context tile with cached keys beyond ctx_len: all lanes zero those V^T columns
-          // (0 * whatever the cache holds there, NaN included, must not reach O).
+        if (t.valid & 15) {
           ok = __all_sync(0xffffffffu, ptx::mbar_wait_a(b_v_loc + 8u * s, ph, &abort_flag));
           if (!ok) break;
+#pragma unroll
           for (int rr = lane; rr < 128; rr += 32) attn_clear_v(Vs + (size_t)s * 2 * kSub, rr, t.valid);
           ptx::fence_proxy_async_smem();
           __syncwarp();
@@ -390,11 +395,17 @@ k_attn_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
           if (ok) {
             ptx::tc_fence_after();
             const uint32_t d = tmem_base + 384u, a = tmem_base + sb * 128u, bv = v_lo + s * (2 * kSub16);
-#pragma unroll
-            for (int kk = 0; kk < 8; ++kk) {
+            auto mma = [&](int kk) {
               const uint32_t off = (uint32_t)(kk >> 2) * kSub16 + (uint32_t)(kk & 3) * 2u;
               ptx::umma_bf16_ts_lo(d, a + (uint32_t)(kk >> 1) * 32u + (uint32_t)(kk & 1) * 8u, bv + off, hi32, idesc,
                                    (kk > 0 || j > 0) ? 1u : 0u);
+            };
+            if (t.valid == kBK) {   // (the lean path: constants only)
+#pragma unroll
+              for (int kk = 0; kk < 8; ++kk) mma(kk);
+            } else {
+#pragma unroll 1
+              for (int kk = 0; kk < attn_pv_keys(t.valid) >> 4; ++kk) mma(kk);
             }
             // also tells the V^T producer that the slot is free and the score issuer that the
             // buffer is
@@ -502,7 +513,7 @@ k_attn_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
       if (pass == 0 && slot == 0) {
         const float top = fmaxf(fmaxf(xm[0][r], xm[1][r]), xm[2][r]) * scale;
         // (with one tile only the other slots never read m_row: this warp has m0 in any case)
-        const bool far = sm_ok && (top - m0 > kAttnRange);
+        const bool far = sm_ok && (r & 63) < un.n[r >> 6] && top - m0 > kAttnRange;   // (the other rows are not this sequence's)
         m_row[r] = top;          // the reference points of a second pass
         if (__any_sync(0xffffffffu, far) && lane == 0) again_flag = 1;
       }

@@ -180,8 +180,10 @@ k_attn_few(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CU
         if (ptx::elect_one()) {
           const uint32_t d = tmem_base + (pv ? 64u : (uint32_t)(J & 1) * 32u);
           const uint32_t a = ring_lo + (uint32_t)s * (kFewSlot >> 4);
+          const int nk = pv ? attn_pv_keys(min(kBK, j < Tc ? P - j * kBK : R - (j - Tc) * kBK)) >> 4 : 8;
 #pragma unroll
           for (int kk = 0; kk < 8; ++kk) {
+            if (kk >= nk) break;
             const uint32_t k4 = (uint32_t)(kk & 3) * 2u, half = (uint32_t)(kk >> 2);
             ptx::umma_bf16_lo(d, a + half * (kSub >> 4) + k4, b_lo + half * (kFewQ / 2 >> 4) + k4, hi32, idesc,
                               (kk > 0 || (pv && j > 0)) ? 1u : 0u);
@@ -254,9 +256,7 @@ k_attn_few(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CU
         for (int i = 0; i < 32; ++i)
           asm volatile("st.shared.b16 [%0], %1;" ::"r"(p_addr[i & 7] + (uint32_t)(i >> 3) * 1024u),
                        "h"(__bfloat16_as_ushort(__float2bfloat16_rn(v[i]))) : "memory");
-        if (j < Tc && nvalid < kBK) {
-          // the one context tile with cached keys beyond ctx_len: their V^T columns are cleared (0 * NaN), a
-          // row of the tile per thread
+        if (nvalid & 15) {   // V^T columns beyond the valid keys are cleared, a row of the tile per thread
           const int s = (2 * J + 1) % slots;
           ok = __all_sync(0xffffffffu, ptx::mbar_wait(&c.v_full[J % 3], (uint32_t)(J / 3) & 1u, abort_flag));
           if (!ok) break;

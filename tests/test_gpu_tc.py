@@ -7,6 +7,7 @@ import torch
 from oracle import adapters
 from oracle import depcap_oracle as O
 from paper_2604_15750_b200 import inputs
+from paper_2604_15750_b200.binding import DC_ERR_NUMERIC
 
 from parity import Case, compare
 
@@ -261,3 +262,40 @@ def test_tc_attention_few_rows_with_scores_far_above_the_first():
             err = np.abs(gpu[name][b, :W] - ref) / np.maximum(np.abs(ref), 1.0)
             assert np.isfinite(gpu[name][b, :W]).all() and err.max() <= 2e-2, (name, b, err.max())
         assert (gpu["pred_id"][b, :W] == ora[b]["pred"]).mean() >= 0.95
+
+
+@pytest.mark.parametrize("n_q,n_kv,influence", [
+    (4, 2, False), (4, 2, True),     # keys on the lanes, one variant and two
+    (40, 20, True),                  # rows on the lanes, both variants in one tile
+])
+def test_tc_non_finite_keys_of_one_sequence_stay_there(n_q, n_kv, influence):
+    """A sequence whose cached keys and values hold NaN inside ctx_len (and whose own rows become NaN with
+    them): the sequences before and behind it in the batch give the bits of a clean run, and so does a smaller
+    step afterwards, whose last key tile ends in (57 rows, padded to 64) and reads on into rows that the NaN step
+    left in the workspace."""
+    wl = _wl(3, n_q=n_q, n_kv=n_kv)
+    case = Case(wl, lengths=dict(ctx_len=[40, 77, 128], last_len=[16, 16, 3], win_len=[21, 30, 17], remain_len=[64] * 3))
+    eng, ref = case.make_engine(max_window=48), case.make_engine(max_window=48)
+
+    def step(e, di, seqs, **other):
+        args = {k_: v_[:seqs] if isinstance(v_, list) else v_ for k_, v_ in di.items()}
+        out = e.step(influence=influence, boundary=True, **{**args, **other})
+        e.synchronize()
+        return {k_: v_.cpu().numpy() for k_, v_ in out.items()}
+
+    di = case.device_inputs(eng)
+    clean = step(ref, di, 3)
+    bad = dict(di, k_cache=di["k_cache"].clone(), v_cache=di["v_cache"].clone())
+    bad["k_cache"][:, 1, :, 5] = float("nan")
+    bad["v_cache"][:, 1, :, :, 9] = float("nan")
+    got = step(eng, bad, 3)
+    assert got["status"][[0, 2]].tolist() == [0, 0] and got["status"][1] == DC_ERR_NUMERIC
+    for b in (0, 2):
+        W = case.len["win_len"][b]
+        for k_ in ("pred_id", "conf", "entropy", "lse", "influence"):
+            assert np.array_equal(got[k_][b, :W], clean[k_][b, :W]), (k_, b)
+    small, again = (step(e, di, 1, win_len=[41]) for e in (ref, eng))
+    for k_ in ("pred_id", "conf", "entropy", "lse", "influence"):
+        assert np.array_equal(small[k_][0, :41], again[k_][0, :41]), k_
+    assert again["status"][0] == 0
+    eng.close(); ref.close()
