@@ -412,6 +412,7 @@ int tc_attention(TcState* t, int layer, const SeqMeta& m, const __nv_bfloat16* k
   ap.scale_log2 = 1.4426950408889634f / sqrtf((float)hd);
   ap.o = t->o; ap.status = t->status;
   ap.k = t->k; ap.v = t->v; ap.ldv = t->ldv; ap.k_cache = ap.v_cache = nullptr;
+  ap.cache_vec = ((reinterpret_cast<uintptr_t>(k_cache) | reinterpret_cast<uintptr_t>(v_cache)) & 15) == 0;
   int export_tiles = 0;   // tiles of 128 last-block rows to append to the caches
   if (export_kv) {
     const size_t per_layer = (size_t)g.max_batch * nkv * g.max_ctx * hd;

@@ -53,6 +53,7 @@ struct AttnParams {
   const __nv_bfloat16 *k, *v;        // active K [M, nkv * 128], V transposed [nkv * 128, ldv]
   int ldv;
   __nv_bfloat16 *k_cache, *v_cache;  // this layer's caches
+  int cache_vec;                     // they start on 16-byte boundaries
 };
 
 constexpr int kAttnThreads = 512;
@@ -159,6 +160,17 @@ __device__ __forceinline__ void attn_export_tile(const AttnParams& p, int b, int
   const size_t kv = (size_t)b * p.nkv + g;
   const __nv_bfloat16* ks = p.k + (size_t)row * p.nkv * kHd + g * kHd;
   __nv_bfloat16* kd = p.k_cache + (kv * p.max_ctx + key) * kHd;
+  if (!p.cache_vec) {   // no wider accesses (without cached keys to load by TMA a cache may start anywhere)
+    for (int i = threadIdx.x; i < n * kHd; i += THREADS) {
+      const int r = i / kHd, e = i % kHd;
+      kd[i] = ks[(size_t)r * p.nkv * kHd + e];
+    }
+    for (int i = threadIdx.x; i < n * kHd; i += THREADS) {
+      const int e = i / n, j = i % n;
+      p.v_cache[(kv * kHd + e) * p.max_ctx + key + j] = p.v[(size_t)(g * kHd + e) * p.ldv + row + j];
+    }
+    return;
+  }
 #pragma unroll 4
   for (int i = threadIdx.x; i < n * (kHd / 8); i += THREADS) {
     const int r = i / (kHd / 8), c = i % (kHd / 8) * 8;

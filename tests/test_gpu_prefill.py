@@ -153,3 +153,32 @@ def test_dual_cache_suffix_rows_prefilled_at_their_own_positions(tc):
     off = case.run_oracle(influence=False)
     assert np.abs(off[0]["lse"] - ora[0]["lse"]).max() > 1e-4
     eng.close()
+
+
+@pytest.mark.parametrize("shift", [1, 2, 4])
+@pytest.mark.parametrize("n_ids", [[137, 40], [24, 9]])
+def test_prefill_into_caches_that_start_anywhere(n_ids, shift):
+    """Without cached keys nothing loads from the caches by TMA, and they may start at any element: 2, 4 and 8
+    bytes past a 16-byte boundary the bits are those of aligned caches.  With cached keys such caches are refused."""
+    wl = inputs.Workload("prefill_shift", 2, 256, 4, 2, 128, 512, 2048, "bf16", 2, 0, 0, max(n_ids), 16, 64, 5151)
+    case = Case(wl)
+    eng = case.make_engine(max_ctx=192, max_last=max(n_ids))
+    dev, shape = eng.device, (2, 2, 2, 192, 128)
+    size = int(np.prod(shape))
+    ids = torch.randint(0, wl.vocab - 1, (2, eng.max_last), dtype=torch.int32, generator=torch.Generator().manual_seed(7)).to(dev)
+
+    def filled(off):
+        k, v = (torch.full((size + 8,), -7.0, dtype=torch.bfloat16, device=dev) for _ in range(2))
+        kc, vc = k[off:off + size].view(shape), v[off:off + size].view(2, 2, 2, 128, 192)
+        st = eng.prefill(kc, vc, ids, n_ids)
+        eng.synchronize()
+        assert st.cpu().tolist() == [0, 0]
+        return kc, vc
+
+    (k0, v0), (k1, v1) = filled(0), filled(shift)
+    assert torch.equal(k0, k1) and torch.equal(v0, v1)
+    assert (k1[:, 0, :, n_ids[0]:] == -7).all() and (v1[:, 1, :, :, n_ids[1]:] == -7).all()
+    with pytest.raises(DepCapError) as e:
+        eng.prefill(k1, v1, ids, [8, 8], ctx_len=[5, 5])
+    assert "aligned" in str(e.value)
+    eng.close()
