@@ -66,6 +66,7 @@ struct dc_ctx {
   bool bf16 = false;
   bool use_tc = false;  // tensor-core kernels for the transformer layers
   bool tc_lm = false;   // tensor-core LM head fused with the streaming softmax statistics
+  bool gains_vec = true;   // every layer's norm gains start on 16-byte boundaries (the dense chain's bulk copies)
   const void *embed = nullptr, *final_norm = nullptr, *lm_head = nullptr;
   std::vector<const void*> wq, wk, wv, wo, w_gate, w_up, w_down, norm1, norm2;
   std::vector<const void*> bq, bk, bv;   // q / k / v projection biases (cfg.qkv_bias), else empty
@@ -267,7 +268,7 @@ int run_step(dc_ctx* c, const dc_step_in* in, const dc_step_out* out, const SeqM
   size_t part_stride = 0;
 
   const bool export_kv = (in->flags & DC_STEP_EXPORT_KV) != 0;
-  const bool chain = c->use_tc && tc_chain_ok(c->tc, m);
+  const bool chain = c->use_tc && c->gains_vec && tc_chain_ok(c->tc, m);
   if (chain) {
     // persistent dense chain: norm1 + QKV of layer 0, then per layer attention and one launch
     // that runs O projection .. QKV of the next layer
@@ -546,6 +547,8 @@ int dc_create(const dc_config* cfg, const dc_weights* w, void* cuda_stream, dc_c
     cp(c->norm1, w->norm1); cp(c->norm2, w->norm2);
     if (g.qkv_bias) { cp(c->bq, w->bq); cp(c->bk, w->bk); cp(c->bv, w->bv); }
   }
+  for (int l = 0; l < g.n_layers; ++l)
+    if ((reinterpret_cast<uintptr_t>(w->norm1[l]) | reinterpret_cast<uintptr_t>(w->norm2[l])) & 15) c->gains_vec = false;
   c->use_tc = g.impl == DC_IMPL_AUTO && tc_supported(g);
   c->tc_lm = c->use_tc && tc_has_lmhead(g);
   const size_t es = c->bf16 ? 2 : 4;

@@ -299,3 +299,26 @@ def test_tc_non_finite_keys_of_one_sequence_stay_there(n_q, n_kv, influence):
         assert np.array_equal(small[k_][0, :41], again[k_][0, :41]), k_
     assert again["status"][0] == 0
     eng.close(); ref.close()
+
+
+@pytest.mark.parametrize("ff,win,influence", [(512, 16, False), (640, 32, True)])
+def test_norm_gains_on_8_byte_boundaries(ff, win, influence):
+    """The fused chain brings the gains in by bulk copies, which start on 16-byte boundaries; gains on 8-byte
+    boundaries keep the launch per operation (16 rows; 64 rows with an odd number of gate / up tiles)."""
+    wl = _wl(1, ff=ff, last=1, win=win)
+    case = Case(wl, lengths=dict(ctx_len=[100], last_len=[0], win_len=[win], remain_len=[128]))
+    for lw in case.weights["layers"]:
+        for k_ in ("norm1", "norm2"):
+            at = torch.zeros(wl.d_model + 4, dtype=torch.bfloat16, device="cuda:0")[4:]
+            lw[k_] = at.copy_(lw[k_])
+    eng = case.make_engine(max_window=win)
+    assert eng._weights["layers"][0]["norm1"].data_ptr() % 16 == 8
+    di = case.device_inputs(eng)
+    out = eng.step(influence=influence, boundary=True, **di)
+    sel = eng.select(di["win_ids"], di["win_len"])
+    eng.synchronize()
+    gpu = {k_: v_.cpu().numpy() for k_, v_ in {**out, **sel}.items()}
+    compare(case, gpu, case.run_oracle(influence=influence))
+    _, launches = eng.step_profiled(influence=influence, boundary=True, **di)
+    assert launches["dense"] == 0 and launches["qkv"] == case.n_layers
+    eng.close()
