@@ -236,7 +236,8 @@ int run_step(dc_ctx* c, const dc_step_in* in, const dc_step_out* out, const SeqM
   const SimtSignals sg{c->logits, g.vocab, g.mask_id, g.forbid_mask_pred, c->ws_pred, c->ws_conf, c->ws_ent,
                        c->ws_infl, c->ws_lse, so, out->status};
 
-  if (!c->use_tc && c->fuse.grid > 0 && c->coop && !pf.on) {   // (profiling wants the stages apart)
+  // (profiling wants the stages apart; a prefill without layers has no work, and no rows at the LM head either)
+  if (!c->use_tc && c->fuse.grid > 0 && c->coop && !pf.on && !(kv_only && g.n_layers == 0)) {
     SimtStep<T> st{};
     st.layers = (const SimtLayer<T>*)c->simt_layers; st.n_layers = g.n_layers; st.kv_only = kv_only;
     st.export_kv = (in->flags & DC_STEP_EXPORT_KV) != 0;

@@ -8,7 +8,7 @@ import torch
 from oracle import adapters
 from oracle import depcap_oracle as O
 from paper_2604_15750_b200 import DepCapError, inputs
-from paper_2604_15750_b200.binding import DC_IMPL_SIMT
+from paper_2604_15750_b200.binding import DC_ERR_INDEX, DC_IMPL_SIMT
 
 from parity import Case, compare
 
@@ -181,4 +181,20 @@ def test_prefill_into_caches_that_start_anywhere(n_ids, shift):
     with pytest.raises(DepCapError) as e:
         eng.prefill(k1, v1, ids, [8, 8], ctx_len=[5, 5])
     assert "aligned" in str(e.value)
+    eng.close()
+
+
+def test_prefill_of_a_model_without_layers():
+    """A context made for the decision calls alone: a prefill checks the ids, writes the status and nothing else."""
+    case = Case(inputs.scaled(TINY, ctx_min=0, ctx_max=0), n_layers=0)
+    eng = case.make_engine(max_last=16, max_ctx=64)
+    dev = eng.device
+    cache = torch.full((64,), -7.0, device=dev)
+    ids = torch.zeros((1, 16), dtype=torch.int32, device=dev)
+    for first, status in ((3, 0), (TINY.vocab, DC_ERR_INDEX)):
+        ids[0, 0] = first
+        eng.prefill(cache, cache, ids, [16])
+        eng.synchronize()
+        assert int(eng.out["status"][0]) == status
+    assert (cache == -7.0).all()
     eng.close()
