@@ -2,9 +2,12 @@
 // start while the one before it in the stream still runs: its blocks take the SMs that become free, set
 // up barriers, TMEM and tensor maps, and wait in pdl_wait() until everything before has completed and is
 // visible.  Every kernel launched this way calls pdl_wait() in all of its blocks before it touches global
-// memory (so that completion is transitive), and every kernel calls pdl_trigger() first of all, which only
-// allows the next kernel's blocks to be scheduled.  Two kernels of a layer were 2.1 us apart; the 224
-// launches of a 1024-token LLaDA-8B prefill took 15.37 ms and take 14.84 ms.
+// memory (so that completion is transitive).  pdl_trigger() only allows the next kernel's blocks to be scheduled,
+// once every block has called it or ended; a kernel without it counts as triggered when it ends.  A kernel that
+// allocates TMEM triggers behind the allocation: a block of the next kernel that fitted beside one of these
+// would take the columns first and hold them in pdl_wait(), whose end is behind the allocation that waits for
+// them.  Two kernels of a layer were 2.1 us apart; the 224 launches of a 1024-token LLaDA-8B prefill took 15.37 ms
+// and take 14.84 ms.
 #pragma once
 #include <cuda_runtime.h>
 

@@ -222,8 +222,8 @@ k_attn_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
   __shared__ float xm[3][128];     // [slot][row]: maximum raw score of the slot's tiles
 
   const int b = blockIdx.z, h = blockIdx.y;
-  pdl_trigger();
   if ((int)blockIdx.x >= p.units) {
+    pdl_trigger();
     pdl_wait();
     const int r0 = ((int)blockIdx.x - p.units) * kBK;
     if (h < p.nkv && r0 < p.m.last_len[b]) attn_export_tile<kAttnThreads>(p, b, h, r0);
@@ -262,6 +262,7 @@ k_attn_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
   __syncthreads();
   ptx::tc_fence_after();
   const uint32_t tmem_base = tmem_base_s;
+  pdl_trigger();   // (not before the allocation: pdl.cuh)
   pdl_wait();
   // TMEM columns: S / P of tile J in buffer J % 3 (columns 0..127, 128..255, 256..383), O 384..511
 

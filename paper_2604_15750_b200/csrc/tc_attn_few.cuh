@@ -78,8 +78,8 @@ k_attn_few(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CU
            const __grid_constant__ CUtensorMap map_vc, const AttnParams p, const int slots) {
   extern __shared__ uint8_t smem_few[];
   const int b = blockIdx.z, h = blockIdx.y;
-  pdl_trigger();
   if ((int)blockIdx.x >= p.units) {
+    pdl_trigger();
     pdl_wait();
     const int r0 = ((int)blockIdx.x - p.units) * kBK;
     if (h < p.nkv && r0 < p.m.last_len[b]) attn_export_tile<kFewThreads>(p, b, h, r0);
@@ -118,6 +118,7 @@ k_attn_few(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CU
   __syncthreads();
   ptx::tc_fence_after();
   const uint32_t tmem_base = c.tmem_base;   // columns: S^T of tile J in buffer J % 2 (0..31, 32..63), O^T 64..95
+  pdl_trigger();   // (not before the allocation: pdl.cuh)
   pdl_wait();
 
   int* abort_flag = &c.abort_flag;

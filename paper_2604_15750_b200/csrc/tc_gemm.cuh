@@ -88,7 +88,6 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w0, const __grid_constant__ CU
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~static_cast<uintptr_t>(1023));
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  pdl_trigger();
   // Column blocks of one weight tile sit next to each other in the unit order, so that the
   // CTAs that share a weight tile run together and all but one read it from L2.
   const int n_cblk = (p.M + p.BN - 1) / p.BN;
@@ -142,6 +141,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w0, const __grid_constant__ CU
   __syncthreads();
   ptx::tc_fence_after();
   const uint32_t tmem_base = tmem_base_s;
+  pdl_trigger();   // (not before the allocation: pdl.cuh)
   if (PAIR) {
     // both CTAs hold all 512 columns, so the pair MMA's accumulator address names the same columns
     // in both; the partner's barriers are initialised before any load can report to them

@@ -50,7 +50,6 @@ k_lmhead_tc(const __grid_constant__ CUtensorMap map_h, const __grid_constant__ C
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~static_cast<uintptr_t>(1023));
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  pdl_trigger();
   // CTA -> (group of LM rows, vocabulary slice), groups fastest: the CTAs that stream the same
   // vocabulary tiles for different groups run at the same time, so a tile crosses HBM once and is
   // served to the other groups from L2
@@ -79,6 +78,7 @@ k_lmhead_tc(const __grid_constant__ CUtensorMap map_h, const __grid_constant__ C
   ptx::tc_fence_after();
   const uint32_t tmem_base = tmem_base_s;
 
+  pdl_trigger();   // (not before the allocation: pdl.cuh)
   pdl_wait();
   // (lean single-thread loops: addresses and descriptors advance by additions only)
   if (warp == 0) {

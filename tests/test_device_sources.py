@@ -1,0 +1,42 @@
+"""Rules of the device code that a run on a GPU does not show, checked on the sources: breaking one is a hang that
+takes a rare order of events."""
+import os
+import re
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2604_15750_b200", "csrc")
+
+
+def _closing(src, at, pair):
+    """index of the bracket that closes the one at `at`"""
+    depth = 0
+    for i in range(at, len(src)):
+        depth += (src[i] == pair[0]) - (src[i] == pair[1])
+        if depth == 0:
+            return i
+
+
+def _kernel(name, kernel):
+    """the body of a __global__ function, without comments"""
+    src = re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, name)).read())
+    at = re.search(r"__global__[^;{]*?\b" + kernel + r"\(", src).end() - 1
+    head = src.index("{", _closing(src, at, "()"))
+    return src[head:_closing(src, head, "{}") + 1]
+
+
+@pytest.mark.parametrize("name,kernel", [("tc_gemm.cuh", "k_gemm_tc"), ("tc_lmhead.cuh", "k_lmhead_tc"),
+                                         ("tc_attn.cuh", "k_attn_tc"), ("tc_attn_few.cuh", "k_attn_few")])
+def test_the_next_kernel_is_let_in_behind_the_tmem_allocation(name, kernel):
+    """A block of the next kernel that gets an SM before the one it waits for has its TMEM columns could take them
+    and hold them while it waits.  Only blocks that leave without an allocation may trigger before it."""
+    body = _kernel(name, kernel)
+    alloc = body.index("tmem_alloc(")
+    triggers = [m.start() for m in re.finditer(r"pdl_trigger\(\)", body)]
+    assert any(t > alloc for t in triggers)
+    for t in triggers:
+        if t < alloc:
+            end = body.index("return;", t)
+            assert end < alloc and body[t:end].count("{") <= body[t:end].count("}") + 1
+        else:
+            assert "__syncthreads()" in body[alloc:t]
