@@ -367,7 +367,7 @@ __device__ __forceinline__ void chain_gemm(ChainCtx& c, const ChainParams& p, co
       const uint32_t up = (uint32_t)tile_bytes >> 4, act = (uint32_t)(nw * tile_bytes) >> 4, step = (uint32_t)slot_bytes >> 4;
       uint32_t ms = 0, lo = lo0;
       if (c.mma_units > 0) {  // the epilogue has drained both accumulators of the last unit
-        ok = ptx::mbar_wait(c.acc_empty, (c.mma_units - 1) & 1u, c.abort_flag);
+        ok = __all_sync(0xffffffffu, ptx::mbar_wait(c.acc_empty, (c.mma_units - 1) & 1u, c.abort_flag));   // (the lanes go on together)
       }
       ptx::tc_fence_after();
       for (int kb = w.kb0; kb < w.kb1 && ok; ++kb) {

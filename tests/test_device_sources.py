@@ -40,3 +40,20 @@ def test_the_next_kernel_is_let_in_behind_the_tmem_allocation(name, kernel):
             assert end < alloc and body[t:end].count("{") <= body[t:end].count("}") + 1
         else:
             assert "__syncthreads()" in body[alloc:t]
+
+
+@pytest.mark.parametrize("name,first,last", [
+    ("tc_chain.cuh", "const bool el = ptx::elect_one();", "umma_commit_pair(c.acc_full)"),
+    ("tc_attn_few.cuh", "const bool pv = warp == 2;", "umma_commit(pv ? &c.p_empty"),
+])
+def test_a_warp_that_issues_together_gives_up_together(name, first, last):
+    """A bounded wait is decided lane by lane.  Where the whole warp runs the issuing loop, whose votes take all
+    lanes, every wait is voted on: lanes that gave up alone would leave the others in the next vote for good."""
+    src = open(os.path.join(CSRC, name)).read()
+    part = src[src.index(first):src.index(last)]
+    waits = list(re.finditer(r"ptx::mbar_wait", part))
+    assert waits
+    for m in waits:
+        statement = part[max(part.rfind(c, 0, m.start()) for c in ";{}"):part.index(";", m.start())]
+        later = part[m.start():]
+        assert "__all_sync(" in statement or re.search(r"ok = __all_sync\(0xffffffffu, ok\);\s*if \(!ok\) break;", later)
