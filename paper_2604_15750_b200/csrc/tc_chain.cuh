@@ -418,7 +418,7 @@ __device__ __forceinline__ void chain_gemm(ChainCtx& c, const ChainParams& p, co
       const float* dl = p.cos_sin + (size_t)p.rows_per_variant * 128 + (f & 63);  // step row
       rb.cd = __ldg(dl); rb.sd = __ldg(dl + 64);
     }
-    bool ok = ptx::mbar_wait(c.acc_full, c.units_done & 1u, c.abort_flag);
+    bool ok = __all_sync(0xffffffffu, ptx::mbar_wait(c.acc_full, c.units_done & 1u, c.abort_flag));
     ++c.units_done;
     if (ok && EPI == CEPI_QKV && kind == ITEM_MAIN) {
       // the helper pair's part of this tile has been written (its warps have counted up)
@@ -426,6 +426,7 @@ __device__ __forceinline__ void chain_gemm(ChainCtx& c, const ChainParams& p, co
       if (c.lane == 0) got = ptx::flag_wait(p.tile_flags + tile, p.flag_target, c.abort_flag);
       ok = __shfl_sync(0xffffffffu, (int)got, 0) != 0;   // also orders the lanes' loads behind the acquire
     }
+    if (EPI == CEPI_QKV) ok = ptx::all_agree(half + 1, 128, ok);   // the warps of a column part meet in this epilogue
     if (ok) {
       ptx::tc_fence_after();
       // 16 columns (activation rows) per step in a rolled loop (the code runs once per unit, so

@@ -273,7 +273,8 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w0, const __grid_constant__ CU
       const int tile = w.tile, split = w.split;
       const uint32_t set = pp ? (uint32_t)(j & 1) : 0u;
       const uint32_t uses = pp ? (uint32_t)(j >> 1) : (uint32_t)j;
-      ok = ptx::mbar_wait(&acc_full[set], uses & 1u, &abort_flag);
+      ok = __all_sync(0xffffffffu, ptx::mbar_wait(&acc_full[set], uses & 1u, &abort_flag));
+      if (EPI == GEMM_EPI_QKV) ok = ptx::all_agree(1, 128, ok);   // (they meet in this epilogue)
       ptx::tc_fence_after();
       if (!ok) break;
       if (w.nkb > 0) {

@@ -92,6 +92,21 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity,
   return true;
 }
 
+// True for all `threads` threads that meet on named barrier `id` if it holds for every one of them.  Waits are decided
+// thread by thread: threads that go on to a barrier or a warp-wide TMEM access together have to agree first.
+__device__ __forceinline__ bool all_agree(int id, int threads, bool ok) {
+  uint32_t all;
+  asm volatile(
+      "{\n\t.reg .pred P, Q;\n\t"
+      "setp.ne.u32 P, %3, 0;\n\t"
+      "barrier.cta.red.and.pred Q, %1, %2, P;\n\t"
+      "selp.u32 %0, 1, 0, Q;\n\t}"
+      : "=r"(all)
+      : "r"(id), "r"(threads), "r"((uint32_t)ok)
+      : "memory");
+  return all != 0;
+}
+
 // ---- grid-wide barrier for persistent kernels whose CTAs are all resident (cooperative launch) --
 // One arrival counter that only counts up: a CTA adds one (fire-and-forget, release) and polls
 // until the counter reaches `target` (acquire).  The host zeroes the word at the start of a step

@@ -57,3 +57,17 @@ def test_a_warp_that_issues_together_gives_up_together(name, first, last):
         statement = part[max(part.rfind(c, 0, m.start()) for c in ";{}"):part.index(";", m.start())]
         later = part[m.start():]
         assert "__all_sync(" in statement or re.search(r"ok = __all_sync\(0xffffffffu, ok\);\s*if \(!ok\) break;", later)
+
+
+@pytest.mark.parametrize("name,first,last", [
+    ("tc_chain.cuh", "epilogue: all warps", "tc_fence_after"), ("tc_gemm.cuh", "epilogue: warps 2..5", "tc_fence_after"),
+])
+def test_warps_that_meet_in_an_epilogue_give_up_together(name, first, last):
+    """The epilogues read TMEM warp-wide, and the rotation meets on named barriers of four warps: the wait in front of
+    them is voted on in the warp and agreed on among the four."""
+    src = open(os.path.join(CSRC, name)).read()
+    part = src[src.index(first):]
+    part = part[:part.index(last)]
+    waits = re.findall(r"[^;]*ptx::mbar_wait\([^;]*;", part)
+    assert waits and all("__all_sync(" in w for w in waits)
+    assert re.search(r"EPI_QKV\) ok = ptx::all_agree\([^;]*, 128, ok\);", part)
