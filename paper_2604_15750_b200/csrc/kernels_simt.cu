@@ -154,8 +154,9 @@ void launch_rmsnorm(float* x, const float* part, int nsplit, size_t part_stride,
 template <typename T>
 __global__ void __launch_bounds__(256) k_lm_rows(const float* __restrict__ x, const float* __restrict__ part, int nsplit,
                                                  size_t part_stride, const T* __restrict__ g, float eps, int d,
-                                                 const SeqMeta m, int nv_x, const LmRowsIo<T> io, T* __restrict__ h) {
-  extern __shared__ __align__(16) float lm_row_s[];   // the row with the partial sums folded in
+                                                 const SeqMeta m, int nv_x, const LmRowsIo<T> io, T* __restrict__ h,
+                                                 int staged) {
+  extern __shared__ __align__(16) float lm_row_s[];   // staged: the row with the partial sums folded in
   __shared__ float red[32];
   pdl_trigger();
   pdl_wait();
@@ -186,21 +187,25 @@ __global__ void __launch_bounds__(256) k_lm_rows(const float* __restrict__ x, co
   const size_t off = (size_t)act_row(m, v < nv_x ? v : 0, b, m.last_len[b] + k) * d;
   T* dst0 = src == nullptr ? hr : nullptr;
   T* dst1 = (v == 0 && io.h_out != nullptr) ? io.h_out + ((size_t)b * io.max_window + k) * d : nullptr;
-  float ss = 0.f;
-  for (int i = threadIdx.x * 4; i < d; i += blockDim.x * 4) {
+  auto folded = [&](int i) {
     float4 w = *reinterpret_cast<const float4*>(x + off + i);
     if (part)
       for (int sidx = 0; sidx < nsplit; ++sidx) {
         const float4 pv = *reinterpret_cast<const float4*>(part + sidx * part_stride + off + i);
         w.x += pv.x; w.y += pv.y; w.z += pv.z; w.w += pv.w;
       }
-    *reinterpret_cast<float4*>(lm_row_s + i) = w;
+    return w;
+  };
+  float ss = 0.f;
+  for (int i = threadIdx.x * 4; i < d; i += blockDim.x * 4) {
+    const float4 w = folded(i);
+    if (staged) *reinterpret_cast<float4*>(lm_row_s + i) = w;
     ss += w.x * w.x + w.y * w.y + w.z * w.z + w.w * w.w;
   }
   ss = block_sum(ss, red);
   const float inv = rsqrtf(ss / (float)d + eps);
   for (int i = threadIdx.x * 4; i < d; i += blockDim.x * 4) {
-    const float4 w = *reinterpret_cast<const float4*>(lm_row_s + i);
+    const float4 w = staged ? *reinterpret_cast<const float4*>(lm_row_s + i) : folded(i);
     float gv[4];
     load4<T>(g + i, gv);
     const float o[4] = {w.x * inv * gv[0], w.y * inv * gv[1], w.z * inv * gv[2], w.w * inv * gv[3]};
@@ -212,7 +217,12 @@ __global__ void __launch_bounds__(256) k_lm_rows(const float* __restrict__ x, co
 template <typename T>
 void launch_lm_rows(const float* x, const float* part, int nsplit, size_t part_stride, const T* g, float eps, int d,
                     const SeqMeta& m, int nv_x, const LmRowsIo<T>& io, T* h, cudaStream_t s) {
-  launch_chained(k_lm_rows<T>, m.nv * m.npos_pad, 256, d * sizeof(float), s, x, part, nsplit, part_stride, g, eps, d, m, nv_x, io, h);
+  // rows of more than 12256 elements are folded twice instead of staged: they have no room in the 48 KB that a
+  // kernel may use without an opt-in (and 128 bytes are the sums')
+  const size_t row = d * sizeof(float);
+  const int staged = row + 128 <= 48 * 1024;
+  launch_chained(k_lm_rows<T>, m.nv * m.npos_pad, 256, staged ? row : 0, s, x, part, nsplit, part_stride, g, eps, d, m, nv_x, io, h,
+                 staged);
 }
 
 // ---- CUDA-core GEMM: acc[m, n] = sum_k A[m, k] W[n, k], fp32 FMAs, with the epilogues of a layer ----
@@ -595,7 +605,7 @@ static bool simt_init_t() {
     constexpr int E = decltype(epi)::value;
     return opt(k_gemm_simt<T, 1, 1, 8, 128, 3, E>) && opt(k_gemm_simt<T, 4, 2, 1, 32, 3, E>);
   };
-  return opt(k_attn_simt<T>) && opt(k_lm_rows<T>) && gemm(std::integral_constant<int, EPI_STORE_F32>{}) &&
+  return opt(k_attn_simt<T>) && gemm(std::integral_constant<int, EPI_STORE_F32>{}) &&
          gemm(std::integral_constant<int, EPI_ADD_F32>{}) && gemm(std::integral_constant<int, EPI_SWIGLU>{}) &&
          gemm(std::integral_constant<int, EPI_QKV>{});
 }

@@ -322,3 +322,29 @@ def test_norm_gains_on_8_byte_boundaries(ff, win, influence):
     _, launches = eng.step_profiled(influence=influence, boundary=True, **di)
     assert launches["dense"] == 0 and launches["qkv"] == case.n_layers
     eng.close()
+
+
+@pytest.mark.parametrize("d,xlogp", [(12288, True), (12416, False)])
+def test_rows_that_do_not_fit_without_a_shared_memory_opt_in(d, xlogp):
+    """Models wider than 48 KB of fp32 a row: the rows of the LM head, with and without the cross log-probs (which
+    stage a row of 48 KB at most), and the rows that a later step carries."""
+    wl = inputs.Workload("tc_wide", 1, d, 2, 2, 128, 256, 512, "bf16", 1, 40, 40, 3, 16, 32, 77)
+    case = Case(wl)
+    eng = case.make_engine()
+    di = case.device_inputs(eng)
+    h = torch.zeros((1, eng.max_window, d), dtype=torch.bfloat16, device=eng.device)
+    out = eng.step(influence=True, boundary=True, want_xlogp=xlogp, h_out=h, **di)
+    eng.synchronize()
+    assert int(out["status"][0]) == 0
+    ora = case.run_oracle()[0]
+    for name in ("conf", "entropy", "lse"):
+        got = out[name][0, :16].cpu().numpy()
+        assert (np.abs(got - ora[name]) / np.maximum(np.abs(ora[name]), 1.0)).max() <= 2e-2, name
+    if xlogp:
+        got = out["xlogp"][0, :16, :16].cpu().numpy()
+        same = out["pred_id"][0, :16].cpu().numpy() == ora["pred"]
+        assert same.mean() >= 0.9
+        err = np.abs(got - ora["xlogp"]) / np.maximum(np.abs(ora["xlogp"]), 1.0)
+        assert err[:, same].max() <= 2e-2
+    assert np.abs(h[0, :16].float().cpu().numpy()).max() > 0 and torch.isfinite(h).all()
+    eng.close()
