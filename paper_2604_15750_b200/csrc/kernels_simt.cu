@@ -585,11 +585,71 @@ static AttnSimtShape attn_simt_shape(int hd) {
   }
 }
 
+// A head_dim whose tiles do not fit in shared memory (above some 3500): a CTA takes one query row of one head and
+// keeps it and its output there; K and V are read where they lie, 256 keys at a time.
+template <typename T>
+__global__ void __launch_bounds__(256) k_attn_simt_wide(
+    const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ v,
+    const T* __restrict__ k_cache, const T* __restrict__ v_cache, int max_ctx, const SeqMeta m, int nq,
+    int nkv, int hd, T* __restrict__ o) {
+  extern __shared__ __align__(16) float attn_smem[];
+  __shared__ float red[32];
+  const int h = blockIdx.y, b = blockIdx.z % m.batch, vv = blockIdx.z / m.batch, g = h / (nq / nkv), r = blockIdx.x;
+  const int P = m.ctx_len[b], R = m.last_len[b] + m.win_len[b];
+  if (r >= R) return;
+  float *qs = attn_smem, *os = qs + hd, *ps = os + hd;   // [hd], [hd], [256]
+  const int row0 = act_row(m, vv, b, 0), ld = nkv * hd, tid = threadIdx.x, w = tid >> 5, l = tid & 31;
+  const size_t off = (size_t)(row0 + r) * nq * hd + (size_t)h * hd, kvh = (size_t)b * nkv + g;
+  for (int e = tid; e < hd; e += 256) { qs[e] = to_f<T>(q[off + e]); os[e] = 0.f; }
+  const float scale = rsqrtf((float)hd);
+  float mx = -INFINITY, sum = 0.f;
+  const int tc = (P + 255) / 256, tiles = tc + (R + 255) / 256;
+  for (int t = 0; t < tiles; ++t) {
+    const bool ctx = t < tc;
+    const int j0 = (ctx ? t : t - tc) * 256, n = min(256, (ctx ? P : R) - j0);
+    __syncthreads();                            // the tile before has been read
+    float s = -INFINITY;
+    if (tid < n) {
+      const T* kr = ctx ? k_cache + (kvh * max_ctx + j0 + tid) * hd : k + (size_t)(row0 + j0 + tid) * ld + (size_t)g * hd;
+      s = 0.f;
+      for (int e = 0; e < hd; ++e) s = fmaf(qs[e], to_f<T>(kr[e]), s);
+      s *= scale;
+    }
+    float top = warp_max(s);
+    if (l == 0) red[w] = top;
+    __syncthreads();
+    for (int i = 0; i < 8; ++i) top = fmaxf(top, red[i]);
+    top = fmaxf(top, mx);
+    const float corr = expf(mx - top), p = tid < n ? expf(s - top) : 0.f;
+    ps[tid] = p;
+    sum = sum * corr + block_sum(p, red);       // (its barriers also publish ps)
+    mx = top;
+    for (int e = tid; e < hd; e += 256) {
+      float acc = os[e] * corr;
+      if (ctx) {
+        const T* vr = v_cache + (kvh * hd + e) * max_ctx + j0;
+        for (int j = 0; j < n; ++j) acc = fmaf(ps[j], to_f<T>(vr[j]), acc);
+      } else {
+        const T* vr = v + (size_t)(row0 + j0) * ld + (size_t)g * hd + e;
+        for (int j = 0; j < n; ++j) acc = fmaf(ps[j], to_f<T>(vr[(size_t)j * ld]), acc);
+      }
+      os[e] = acc;
+    }
+  }
+  const float inv = 1.f / sum;
+  for (int e = tid; e < hd; e += 256) o[off + e] = from_f<T>(os[e] * inv);
+}
+static size_t attn_wide_smem(int hd) { return sizeof(float) * (2 * (size_t)hd + 256); }
+
 template <typename T>
 void launch_attn_simt(const T* q, const T* k, const T* v, const T* k_cache, const T* v_cache,
                       int max_ctx, const SeqMeta& m, int nq, int nkv, int hd, T* o,
                       cudaStream_t s) {
   const AttnSimtShape a = attn_simt_shape(hd);
+  if (a.smem > kSimtSmemMax) {
+    k_attn_simt_wide<T><<<dim3(m.R_cap, nq, m.nv * m.batch), 256, attn_wide_smem(hd), s>>>(q, k, v, k_cache, v_cache, max_ctx, m, nq, nkv, hd, o);
+    return;
+  }
   auto aligned = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
   const int vec = hd % 4 == 0 && aligned(k_cache) && aligned(v_cache);
   dim3 grid((m.R_cap + a.rows - 1) / a.rows, nq, m.nv * m.batch);
@@ -605,7 +665,7 @@ static bool simt_init_t() {
     constexpr int E = decltype(epi)::value;
     return opt(k_gemm_simt<T, 1, 1, 8, 128, 3, E>) && opt(k_gemm_simt<T, 4, 2, 1, 32, 3, E>);
   };
-  return opt(k_attn_simt<T>) && gemm(std::integral_constant<int, EPI_STORE_F32>{}) &&
+  return opt(k_attn_simt<T>) && opt(k_attn_simt_wide<T>) && gemm(std::integral_constant<int, EPI_STORE_F32>{}) &&
          gemm(std::integral_constant<int, EPI_ADD_F32>{}) && gemm(std::integral_constant<int, EPI_SWIGLU>{}) &&
          gemm(std::integral_constant<int, EPI_QKV>{});
 }
@@ -622,7 +682,7 @@ bool simt_init(bool bf16, int head_dim) {
     if (ok) done[bf16].fetch_or(bit, std::memory_order_release);
     cudaGetLastError();
   }
-  return ok && attn_simt_shape(head_dim).smem <= kSimtSmemMax;
+  return ok && (attn_simt_shape(head_dim).smem <= kSimtSmemMax || attn_wide_smem(head_dim) <= kSimtSmemMax);
 }
 
 // ---- per-position signals from full logits (CUDA-core LM head only): one block per window position --

@@ -27,6 +27,9 @@ def _wl(name, dtype, n_q, n_kv, hd, d, ff, vocab, batch, ctx, last, win):
     _wl("simt_hd6", "f32", 2, 2, 6, 64, 72, 509, 2, (65, 129), 33, 40),
     # bf16 with tiles of both kinds and long contexts
     _wl("simt_bf16", "bf16", 4, 4, 32, 256, 520, 4100, 2, (200, 331), 16, 48),
+    # heads whose tiles do not fit in shared memory: more than one tile of cached keys, and of active ones
+    _wl("simt_hd4096", "f32", 2, 1, 4096, 64, 72, 130, 2, (5, 300), 40, 240),
+    _wl("simt_hd6000", "bf16", 1, 1, 6000, 64, 72, 130, 1, (30, 30), 3, 17),
 ], ids=lambda w: w.name)
 def test_cuda_core_shapes(wl):
     case = Case(wl, ctx_from_oracle=wl.dtype == "f32" and wl.ctx_max > 0, steer="decay")
