@@ -216,7 +216,8 @@ __device__ __forceinline__ void signals_pos(const SimtSignals& sg, const SeqMeta
       sum[i] = 0.f;
       for (int j = 0; j < NT / 32; ++j) sum[i] += sh.red[i][j];
     }
-    const float S = sum[0];
+    // (no logit above -inf: not a sum of 0, whose 1 / S would be the highest confidence of all)
+    const float S = mx > -INFINITY ? sum[0] : __int_as_float(0x7fffffff);
     const float lse = mx + logf(S);
     const float conf = 1.f / S;
     const float ent = lse - sum[1] / S;

@@ -6,6 +6,7 @@ import torch
 from oracle import adapters
 from oracle import depcap_oracle as O
 from paper_2604_15750_b200 import inputs
+from paper_2604_15750_b200.binding import DC_ERR_NUMERIC
 
 from parity import Case, compare
 
@@ -99,4 +100,35 @@ def test_ragged_rows_lie_behind_one_another(cooperative):
                 ref = ora[b]["kv_last"][l][which]                    # [last, nkv, hd]
                 got = new[l, :, ctx[b]:end].permute(1, 0, 2).cpu().numpy()
                 assert np.abs(got - ref).max() / max(np.abs(ref).max(), 1.0) <= 1e-4, (b, l)
+    eng.close()
+
+
+@pytest.mark.parametrize("cooperative", [1, 0])   # the fused step, separate launches
+def test_position_whose_logits_are_all_minus_infinity(cooperative):
+    """Not a confident position: confidence, entropy and log-sum-exp are NaN, so that no threshold is met, and the
+    status says so; the other positions have the bits of a run without it."""
+    wl = _wl("simt_minf", "f32", 4, 4, 32, 128, 256, 515, 1, (40, 40), 5, 16)
+    case = Case(wl, steer="decay")
+    case.weights["lm_head"][:, 0] = -1.0
+    eng = case.make_engine()
+    eng.set_option(1, cooperative)             # DC_OPT_COOPERATIVE
+    di = case.device_inputs(eng)
+    di["h_final"][..., 0] = 0.0
+
+    def run():
+        out = eng.step(influence=True, boundary=True, **di)
+        sel = eng.select(di["win_ids"], [16], block_len=torch.full((1,), 16, dtype=torch.int32, device=eng.device))
+        eng.synchronize()
+        return {k_: v_.cpu().numpy()[0] for k_, v_ in {**out, **sel}.items()}
+
+    clean = run()
+    di["h_final"][0, :, 3] = 0.0
+    di["h_final"][0, :, 3, 0] = float("inf")
+    got = run()
+    assert clean["status"] == 0 and got["status"] == DC_ERR_NUMERIC
+    assert np.isnan([got[k_][3] for k_ in ("conf", "entropy", "lse")]).all()
+    assert got["pred_id"][3] == wl.mask_id and got["influence"][3] == 0 and got["sel_mask"][3] == 0
+    rest = np.arange(16) != 3
+    for k_ in ("pred_id", "conf", "entropy", "lse", "influence"):
+        assert np.array_equal(got[k_][rest], clean[k_][rest]), k_
     eng.close()
