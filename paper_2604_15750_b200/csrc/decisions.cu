@@ -163,7 +163,8 @@ __global__ void __launch_bounds__(32 * kSeqWarps, 5) k_select(
       if (win_ids[o + k] == mask_id) key[q] = c == c ? order_key(c) : 1u;   // NaN: below every threshold
     }
   }
-  const unsigned k_low = order_key(hp.tau_low), k_high = order_key(fmaxf(hp.tau_low, hp.tau_high));
+  auto bar = [](float tau) { return tau == tau ? order_key(tau) : kAll; };   // (nothing reaches a NaN)
+  const unsigned k_low = bar(hp.tau_low), k_high = max(k_low, bar(hp.tau_high));
   unsigned cand[NQ];
   unsigned sel = 0u;
   if (hp.cap_mode == DC_CAP_STRICT) {         // phase 1, greedily with conflict checks

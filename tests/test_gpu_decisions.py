@@ -206,3 +206,25 @@ def test_decisions_one_warp_per_sequence_bit_exact(W, B, cap_mode):
         assert list(g["sel_idx"][b, :int(g["sel_count"][b])]) == want, b
         assert [i for i in range(w) if g["sel_mask"][b, i]] == want, b
     eng.close()
+
+
+@pytest.mark.parametrize("cap_mode", [0, 1])
+def test_select_with_nan_thresholds_as_the_comparisons_have_it(cap_mode):
+    """No confidence is at or above a NaN, of either sign: no pool without tau_low (one token, the most confident),
+    no first phase without tau_high."""
+    eng = _engine(Hyper(cap_mode=cap_mode))
+    r = np.random.default_rng(12)
+    W, B = 100, 4
+    conf = r.random((B, 128)).astype(np.float32)
+    x = (r.standard_normal((B, 128, 128)) * 6 - 9).astype(np.float32)
+    ids = np.full((B, 128), WL.mask_id, dtype=np.int32)
+    nan = float("nan")
+    for tl, th in ((nan, 0.95), (-nan, 0.95), (0.3, nan), (0.3, -nan), (nan, -nan)):
+        g = eng.select(torch.from_numpy(ids).cuda(), [W] * B, conf=torch.from_numpy(conf).cuda(),
+                       xlogp=torch.from_numpy(x).cuda(), block_len=torch.full((B,), W, dtype=torch.int32).cuda(),
+                       thresholds=(tl, th, -8.0))
+        eng.synchronize()
+        for b in range(B):
+            want = O.cap_select(conf[b, :W], ids[b, :W] == WL.mask_id, x[b, :W, :W], W, tl, th, -8.0, cap_mode)
+            assert g["sel_idx"][b, :int(g["sel_count"][b])].tolist() == want, (tl, th, b)
+    eng.close()
