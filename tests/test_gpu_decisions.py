@@ -228,3 +228,36 @@ def test_select_with_nan_thresholds_as_the_comparisons_have_it(cap_mode):
             want = O.cap_select(conf[b, :W], ids[b, :W] == WL.mask_id, x[b, :W, :W], W, tl, th, -8.0, cap_mode)
             assert g["sel_idx"][b, :int(g["sel_count"][b])].tolist() == want, (tl, th, b)
     eng.close()
+
+
+@pytest.mark.parametrize("cap_mode", [0, 1])
+@pytest.mark.parametrize("W", [80, 128, 144, 256])
+@pytest.mark.parametrize("conflicts", [0.0, 0.004, 0.05])
+def test_select_long_greedy_passes_bit_exact(W, cap_mode, conflicts):
+    """Pools of a hundred and more positions of which few or none conflict, ties among the confidences and decoded
+    positions between them; every fourth sequence has a pool of just under or over what goes on in rank order."""
+    hp = Hyper(tau_low=0.5, tau_high=0.9, cap_mode=cap_mode)
+    eng = _engine(hp, max_batch=1, max_window=W)
+    r = np.random.default_rng(W + cap_mode)
+    B, mask_id = 12, WL.mask_id
+    conf = (0.5 + 0.5 * r.random((B, W))).astype(np.float32)
+    conf[:, ::5] = np.float32(0.75)                                            # ties
+    conf[1] = np.float32(0.6)
+    conf[2::4, 30:] = np.float32(0.1)                                          # pools of some 27
+    x = np.where(r.random((B, W, W)) < conflicts, 0.0, -30.0 - 4 * r.random((B, W, W))).astype(np.float32)
+    ids = np.where(r.random((B, W)) < 0.9, mask_id, 5).astype(np.int32)
+    ids[0] = mask_id
+    win = np.where(np.arange(B) % 3 == 2, W - 7, W).astype(np.int32)
+    dev = eng.device
+    t = lambda a: torch.from_numpy(a).to(dev)
+    so = dict(sel_mask=torch.zeros((B, W), dtype=torch.uint8, device=dev),
+              sel_idx=torch.zeros((B, W), dtype=torch.int32, device=dev),
+              sel_count=torch.zeros((B,), dtype=torch.int32, device=dev))
+    eng.select_batched(t(conf), t(ids), t(x), t(win), t(win), so)
+    eng.synchronize()
+    for b in range(B):
+        w = int(win[b])
+        want = O.cap_select(conf[b, :w], ids[b, :w] == mask_id, x[b, :w, :w], w, hp.tau_low, hp.tau_high, hp.gamma, cap_mode)
+        assert so["sel_idx"][b, :int(so["sel_count"][b])].tolist() == want, b
+        assert so["sel_mask"][b, :w].nonzero().flatten().tolist() == want, b
+    eng.close()
