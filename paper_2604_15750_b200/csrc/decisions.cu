@@ -13,6 +13,7 @@
 
 namespace dc {
 
+constexpr int kWideBoundary = 4096;   // sequences that k_boundary_wide takes
 constexpr int kThreads = 256;         // one thread per window position (k_commit)
 
 template <int NQ>
@@ -24,6 +25,18 @@ __global__ void __launch_bounds__(32 * kSeqWarps) k_boundary(const float* influe
   pdl_wait();
   const int w = threadIdx.x >> 5, b = blockIdx.x * (blockDim.x >> 5) + w;
   if (b < batch) boundary_seq<NQ>(influence, entropy, b, m, dl, hp, io, sI[w], sH[w]);
+}
+
+// Windows above 128 on four warps a sequence: eight positions a lane are a chain of their own, and the general
+// smoothing more so (radius 1 / 3, W 256, us a call: 1 sequence 13.7 / 15.6 on one warp, 11.8 / 11.7 here; 4096 sequences
+// 21.8 / 27.5 and 21.1 / 21.8)
+__global__ void __launch_bounds__(128) k_boundary_wide(const float* influence, const float* entropy, const __grid_constant__ SeqMeta m,
+                                                       DevLens dl, Hyper hp, BoundaryIo io) {
+  __shared__ float sI[33 * (kMaxW / 32)], sH[33 * (kMaxW / 32)];
+  __shared__ BoundaryTeam<4> team;
+  pdl_trigger();
+  pdl_wait();
+  boundary_seq<kMaxW / 128, 4>(influence, entropy, blockIdx.x, m, dl, hp, io, sI, sH, &team);
 }
 
 // f(NQ as a constant): positions per lane for a window of max_window, warps per CTA for a batch
@@ -40,6 +53,10 @@ static void boundary(const float* influence, const float* entropy, int ld, int b
                      const DevLens& dl, const Hyper& hp, int max_window, float* score, float* cum_i, float* cum_s,
                      int32_t* block_len, cudaStream_t s) {
   const BoundaryIo io = make_boundary_io(influence, entropy, ld, max_window, score, cum_i, cum_s, block_len);
+  if (max_window > 128 && batch <= kWideBoundary) {
+    launch_chained(k_boundary_wide, batch, 128, 0, s, influence, entropy, m, dl, hp, io);
+    return;
+  }
   decide_launch(batch, max_window, [&](auto nq, dim3 grid, int threads) {
     launch_chained(k_boundary<decltype(nq)::value>, grid, threads, 0, s, influence, entropy, batch, m, dl, hp, io);
   });

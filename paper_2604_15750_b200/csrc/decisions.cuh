@@ -92,17 +92,25 @@ __device__ __forceinline__ int len_of(const int32_t* dev, const int* by_value, i
   return dev != nullptr ? dev[b] : by_value[b];
 }
 
-// The boundary rule for sequence b, by one warp; sI, sH: 33 * NQ floats of shared memory each.
-template <int NQ>
+// What the warps of a sequence tell one another (TW of them).
+template <int TW>
+struct BoundaryTeam { float top[4][TW]; long long sum[2][TW]; int first[TW]; };
+
+// The boundary rule for sequence b, by TW warps that are a CTA of their own, or one warp; sI, sH: 33 * NQ * TW floats of
+// shared memory each.
+template <int NQ, int TW = 1>
 __device__ __forceinline__ void boundary_seq(const float* influence, const float* entropy, int b, const SeqMeta& m,
-                                             const DevLens& dl, const Hyper& hp, const BoundaryIo& io, float* sI, float* sH) {
-  const int lane = threadIdx.x & 31, ld = io.ld, max_window = io.max_window, vec = io.vec;
+                                             const DevLens& dl, const Hyper& hp, const BoundaryIo& io, float* sI, float* sH,
+                                             BoundaryTeam<TW>* team = nullptr) {
+  const int lane = threadIdx.x & (32 * TW - 1), ld = io.ld, max_window = io.max_window, vec = io.vec;
+  const int warp = TW > 1 ? lane >> 5 : 0;
+  auto sync = [] { if (TW > 1) __syncthreads(); else __syncwarp(); };
   float *score = io.score, *cum_i = io.cum_i, *cum_s = io.cum_s;
   int32_t* block_len = io.block_len;
   const int Lw = max(0, min(min(hp.L_max, len_of(dl.remain, m.remain, b)), len_of(dl.win_len, m.win_len, b)));
   const size_t o = (size_t)b * max_window;
   if (!len_of(dl.have_prev, m.have_prev, b)) {  // cold start: the first block uses L_min
-    for (int k = lane; k < Lw; k += 32) {
+    for (int k = lane; k < Lw; k += 32 * TW) {
       if (score) score[o + k] = 0.f;
       if (cum_i) cum_i[o + k] = 0.f;
       if (cum_s) cum_s[o + k] = 0.f;
@@ -117,7 +125,7 @@ __device__ __forceinline__ void boundary_seq(const float* influence, const float
   load_run<NQ>(influence + (size_t)b * ld, k0, Lw, vec, rawI);
   load_run<NQ>(entropy + (size_t)b * ld, k0, Lw, vec, Hs);
   // centred moving average over the in-range taps, added left to right
-  if (hp.smooth_radius == 1) {   // the default: the neighbours are in this lane or the next ones
+  if (TW == 1 && hp.smooth_radius == 1) {   // the default: the neighbours are in this lane or the next ones
     const float lI = __shfl_up_sync(kAll, rawI[NQ - 1], 1), rI = __shfl_down_sync(kAll, rawI[0], 1);
     const float lH = __shfl_up_sync(kAll, Hs[NQ - 1], 1), rH = __shfl_down_sync(kAll, Hs[0], 1);
     float hPrev = lH;
@@ -139,7 +147,7 @@ __device__ __forceinline__ void boundary_seq(const float* influence, const float
     auto at = [](int k) { return k + (k >> 5); };
 #pragma unroll
     for (int q = 0; q < NQ; ++q) { sI[at(k0 + q)] = rawI[q]; sH[at(k0 + q)] = Hs[q]; }
-    __syncwarp();
+    sync();
 #pragma unroll
     for (int q = 0; q < NQ; ++q) {
       const int k = k0 + q;
@@ -162,7 +170,17 @@ __device__ __forceinline__ void boundary_seq(const float* influence, const float
     }
   if (hp.norm_mode != DC_NORM_NONE) {
     hiI = lanes_max(hiI); hiH = lanes_max(hiH);
-    if (hp.norm_mode == DC_NORM_MINMAX) { nlI = -lanes_max(nlI); nlH = -lanes_max(nlH); }
+    if (hp.norm_mode == DC_NORM_MINMAX) { nlI = lanes_max(nlI); nlH = lanes_max(nlH); }
+    if (TW > 1) {
+      if ((lane & 31) == 0) { team->top[0][warp] = hiI; team->top[1][warp] = hiH; team->top[2][warp] = nlI; team->top[3][warp] = nlH; }
+      sync();
+#pragma unroll
+      for (int i = 0; i < TW; ++i) {
+        hiI = fmaxf(hiI, team->top[0][i]); hiH = fmaxf(hiH, team->top[1][i]);
+        nlI = fmaxf(nlI, team->top[2][i]); nlH = fmaxf(nlH, team->top[3][i]);
+      }
+    }
+    nlI = -nlI; nlH = -nlH;
 #pragma unroll
     for (int q = 0; q < NQ; ++q) {
       Is[q] = normalise(Is[q], hiI, nlI, hp.norm_mode);
@@ -179,7 +197,15 @@ __device__ __forceinline__ void boundary_seq(const float* influence, const float
     accS[q] = (q ? accS[q ? q - 1 : 0] : 0) + fS;
     accI[q] = (q ? accI[q ? q - 1 : 0] : 0) + fI;
   }
-  const long long baseS = lanes_scan(accS[NQ - 1]) - accS[NQ - 1], baseI = lanes_scan(accI[NQ - 1]) - accI[NQ - 1];
+  long long baseS = lanes_scan(accS[NQ - 1]), baseI = lanes_scan(accI[NQ - 1]);
+  if (TW > 1) {
+    if ((lane & 31) == 31) { team->sum[0][warp] = baseS; team->sum[1][warp] = baseI; }
+    sync();
+#pragma unroll
+    for (int i = 0; i + 1 < TW; ++i)
+      if (i < warp) { baseS += team->sum[0][i]; baseI += team->sum[1][i]; }
+  }
+  baseS -= accS[NQ - 1]; baseI -= accI[NQ - 1];
   int first = Lw;
   float ci[NQ], cs[NQ];
 #pragma unroll
@@ -189,7 +215,13 @@ __device__ __forceinline__ void boundary_seq(const float* influence, const float
     ci[q] = from_fixed(tI);
     cs[q] = from_fixed(tS);
   }
-  const int kstar = __reduce_min_sync(kAll, first);
+  int kstar = __reduce_min_sync(kAll, first);
+  if (TW > 1) {
+    if ((lane & 31) == 0) team->first[warp] = kstar;
+    sync();
+#pragma unroll
+    for (int i = 0; i < TW; ++i) kstar = min(kstar, team->first[i]);
+  }
   if (score) store_run<NQ>(score + o, k0, Lw, vec, S);
   if (cum_i) store_run<NQ>(cum_i + o, k0, Lw, vec, ci);
   if (cum_s) store_run<NQ>(cum_s + o, k0, Lw, vec, cs);

@@ -245,19 +245,52 @@ def test_select_long_greedy_passes_bit_exact(W, cap_mode, conflicts):
     conf[1] = np.float32(0.6)
     conf[2::4, 30:] = np.float32(0.1)                                          # pools of some 27
     x = np.where(r.random((B, W, W)) < conflicts, 0.0, -30.0 - 4 * r.random((B, W, W))).astype(np.float32)
+    shift = 1 if conflicts == 0.004 else 0      # (also from a buffer that does not start on a 16-byte boundary)
     ids = np.where(r.random((B, W)) < 0.9, mask_id, 5).astype(np.int32)
     ids[0] = mask_id
     win = np.where(np.arange(B) % 3 == 2, W - 7, W).astype(np.int32)
     dev = eng.device
     t = lambda a: torch.from_numpy(a).to(dev)
+    xd = torch.empty(x.size + 4, device=dev)[shift:shift + x.size].view(x.shape).copy_(t(x))
     so = dict(sel_mask=torch.zeros((B, W), dtype=torch.uint8, device=dev),
               sel_idx=torch.zeros((B, W), dtype=torch.int32, device=dev),
               sel_count=torch.zeros((B,), dtype=torch.int32, device=dev))
-    eng.select_batched(t(conf), t(ids), t(x), t(win), t(win), so)
+    eng.select_batched(t(conf), t(ids), xd, t(win), t(win), so)
     eng.synchronize()
     for b in range(B):
         w = int(win[b])
         want = O.cap_select(conf[b, :w], ids[b, :w] == mask_id, x[b, :w, :w], w, hp.tau_low, hp.tau_high, hp.gamma, cap_mode)
         assert so["sel_idx"][b, :int(so["sel_count"][b])].tolist() == want, b
         assert so["sel_mask"][b, :w].nonzero().flatten().tolist() == want, b
+    eng.close()
+
+
+@pytest.mark.parametrize("mode,norm", [(0, 0), (0, 1), (1, 2), (1, 1)])
+@pytest.mark.parametrize("radius", [0, 1, 3, 8])
+@pytest.mark.parametrize("W,B", [(144, 24), (256, 24), (256, 4097)])
+def test_boundary_of_wide_windows_bit_exact(W, B, mode, norm, radius):
+    """Windows above 128: four warps a sequence up to 4096 sequences, one beyond; lengths that end in any warp."""
+    hp = Hyper(boundary_mode=mode, norm_mode=norm, smooth_radius=radius, L_max=256)
+    eng = _engine(hp, max_batch=1, max_window=W)
+    r = np.random.default_rng(W + B + 7 * radius + norm)
+    win = r.integers(1, W + 1, B).astype(np.int32)
+    win[:8] = [1, 2, 63, 64, 65, 128, 129, W]
+    remain = r.integers(200, 300, B).astype(np.int32)
+    have = (r.random(B) < 0.9).astype(np.int32)
+    I = (np.abs(r.standard_normal((B, W))) * np.exp(-np.arange(W) / 60.0)).astype(np.float32)
+    H = (r.random((B, W)) * r.uniform(0.01, 1.0, (B, 1))).astype(np.float32)   # boundaries far out, too
+    dev = eng.device
+    t = lambda a: torch.from_numpy(a).to(dev)
+    f = lambda: torch.zeros((B, W), device=dev)
+    bo = dict(score=f(), cum_influence=f(), cum_score=f(), block_len=torch.zeros((B,), dtype=torch.int32, device=dev))
+    eng.boundary_batched(t(I), t(H), t(win), t(remain), bo, have_prev=t(have))
+    eng.synchronize()
+    g = {k: v.cpu().numpy() for k, v in bo.items()}
+    for b in list(range(24)) + [B - 1]:
+        L, score, ci, cs = O.boundary(I[b], H[b], int(win[b]), int(remain[b]), bool(have[b]), _ocfg(hp))
+        n = len(score)
+        assert int(g["block_len"][b]) == L, b
+        for name, want in (("score", score), ("cum_influence", ci), ("cum_score", cs)):
+            assert np.array_equal(g[name][b, :n].view(np.uint32), want.view(np.uint32)), (b, name)
+        assert not g["score"][b, n:].any()
     eng.close()
