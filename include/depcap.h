@@ -352,11 +352,13 @@ DC_API int dc_generate(dc_ctx* ctx, const dc_generate_in* in, const dc_generate_
  *     barrier, the grid barrier, a hand-over flag) polls before the kernel gives up, frees what it
  *     holds, returns and reports DC_ERR_TIMEOUT in status[b]; 1000 .. 60 000 000.  The value is
  *     kept on the device and is shared by every context of the process on that device.
- *   DC_OPT_TEST_STALL_LMHEAD (default 0): test hook for the path above.  1 makes the LM-head
+ *   DC_OPT_TEST_STALL_LMHEAD (default 0): test hook for the path above.  1 makes the tensor-core LM-head
  *     kernel skip all of its loads, so that nothing is in flight and every one of its waits runs
  *     out: the step then ends with DC_ERR_TIMEOUT in every status[b] and the context stays usable.
+ *   DC_OPT_TEST_STALL_STEP (default 0): the same for the fused CUDA-core step.  1 makes one of its CTAs leave
+ *     at once, so that the grid barrier of the others runs out.
  * Returns DC_ERR_INVALID_ARG for an unknown option or a value out of range. */
-enum { DC_OPT_COOPERATIVE = 1, DC_OPT_WAIT_LIMIT_US = 2, DC_OPT_TEST_STALL_LMHEAD = 3 };
+enum { DC_OPT_COOPERATIVE = 1, DC_OPT_WAIT_LIMIT_US = 2, DC_OPT_TEST_STALL_LMHEAD = 3, DC_OPT_TEST_STALL_STEP = 4 };
 DC_API int dc_set_option(dc_ctx* ctx, int32_t option, int32_t value);
 
 /* Frees the workspace.  The caller must have synchronised the stream.  Null is a no-op. */

@@ -22,7 +22,7 @@ STAGE_NAMES = ["embed", "norm", "qkv", "attn", "oproj", "gateup", "down", "lmhea
 EXPORTS = ["dc_create", "dc_step", "dc_boundary", "dc_select", "dc_destroy", "dc_last_error",
            "dc_debug_logits", "dc_step_profiled", "dc_signals_static", "dc_commit", "dc_generate", "dc_prefill",
            "dc_set_option", "dc_boundary_batched", "dc_select_batched"]
-DC_OPT_COOPERATIVE, DC_OPT_WAIT_LIMIT_US, DC_OPT_TEST_STALL_LMHEAD = 1, 2, 3
+DC_OPT_COOPERATIVE, DC_OPT_WAIT_LIMIT_US, DC_OPT_TEST_STALL_LMHEAD, DC_OPT_TEST_STALL_STEP = 1, 2, 3, 4
 
 
 class DepCapError(RuntimeError):

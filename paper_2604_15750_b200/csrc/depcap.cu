@@ -94,6 +94,7 @@ struct dc_ctx {
   void* simt_layers = nullptr;      // device [n_layers] SimtLayer
   unsigned int* simt_bar = nullptr; // its grid-barrier words
   bool coop = true;                 // DC_OPT_COOPERATIVE
+  bool stall_step = false;          // DC_OPT_TEST_STALL_STEP
   // workspace of dc_generate: window / last-block ids, step and selection outputs, counters
   int32_t *g_win = nullptr, *g_last = nullptr, *g_pred = nullptr, *g_blk = nullptr, *g_status = nullptr;
   float *g_conf = nullptr, *g_xlogp = nullptr;
@@ -246,7 +247,7 @@ int run_step(dc_ctx* c, const dc_step_in* in, const dc_step_out* out, const SeqM
     st.x = c->x; st.q = q; st.k = k; st.v = v; st.o = o; st.act = act; st.h = h; st.cos_sin = c->cos_sin;
     st.k_cache = (T*)in->k_cache; st.v_cache = (T*)in->v_cache;
     st.final_norm = (const T*)c->final_norm; st.lm_head = (const T*)c->lm_head; st.io = io; st.logits = c->logits;
-    st.sig = sg; st.xlogp = out->xlogp; st.hp = c->hp; st.bar = c->simt_bar;
+    st.sig = sg; st.xlogp = out->xlogp; st.hp = c->hp; st.bar = c->simt_bar; st.stall = c->stall_step;
     if ((in->flags & DC_STEP_BOUNDARY) && out->block_len)
       st.bnd = make_boundary_io(c->ws_infl, c->ws_ent, ml.W_cap, g.max_window, out->score, out->cum_influence,
                                 out->cum_score, out->block_len);
@@ -922,13 +923,19 @@ int dc_set_option(dc_ctx* c, int32_t option, int32_t value) {
   }
   if (option == DC_OPT_WAIT_LIMIT_US) {
     if (value < 1000 || value > 60000000) return fail(c, DC_ERR_INVALID_ARG, "wait limit outside [1000, 60000000] us");
-    if (!c->tc)
-      return simt_set_wait_limit_us(value, c->stream) == 0 ? DC_OK : fail(c, DC_ERR_CUDA, "setting the wait limit failed");
-    const int rc = tc_set_wait_limit_us(c->tc, value);
-    return rc == DC_OK ? DC_OK : fail(c, rc, "%s", tc_error(c->tc));
+    // (the tensor-core kernels and the fused CUDA-core step have a word each on the device)
+    if (simt_set_wait_limit_us(value, c->stream) != 0 || tc_set_wait_limit_us(value, c->stream) != 0) {
+      cudaGetLastError();
+      return fail(c, DC_ERR_CUDA, "setting the wait limit failed");
+    }
+    return DC_OK;
   }
   if (option == DC_OPT_TEST_STALL_LMHEAD) {
     if (c->tc) tc_set_stall_lmhead(c->tc, value != 0);
+    return DC_OK;
+  }
+  if (option == DC_OPT_TEST_STALL_STEP) {
+    c->stall_step = value != 0;
     return DC_OK;
   }
   return fail(c, DC_ERR_INVALID_ARG, "unknown option %d", option);

@@ -557,8 +557,10 @@ __global__ void __launch_bounds__(kFuseThreads, 1) k_simt_step(const __grid_cons
       go = ok;
     }
     __syncthreads();
+    if (go == 0) asm volatile("cp.async.wait_all;" ::: "memory");   // the copies that the next phase had under way
     return go != 0;
   };
+  if (p.stall && blockIdx.x == 0) return;
 
   const int M = p.m.nv * p.m.rows, n_phases = 5 * p.n_layers;
 #pragma unroll 1

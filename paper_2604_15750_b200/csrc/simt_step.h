@@ -30,6 +30,7 @@ struct SimtStep {
   Hyper hp;
   unsigned int* bar;            // arrivals, and a word that a CTA which gave up sets; zero at the start
   int kt, group_smem;           // set by the launcher
+  int stall;                    // test hook: one CTA leaves at once, so that the others wait for it in vain
 };
 
 // What the fused step needs to know about a context; grid == 0: the shape or the device does not take it

@@ -461,14 +461,11 @@ void tc_set_qkv_bias(TcState* t, const std::vector<const void*>& bq, const std::
 
 void tc_set_stall_lmhead(TcState* t, bool on) { t->stall_lmhead = on; }
 
-int tc_set_wait_limit_us(TcState* t, long long us) {
+int tc_set_wait_limit_us(long long us, cudaStream_t s) {
   const unsigned long long ns = (unsigned long long)us * 1000ull;
-  if (cudaMemcpyToSymbolAsync(ptx::g_wait_limit_ns, &ns, sizeof(ns), 0, cudaMemcpyHostToDevice, t->s) != cudaSuccess ||
-      cudaStreamSynchronize(t->s) != cudaSuccess) {
-    cudaGetLastError();
-    return tfail(t, DC_ERR_CUDA, "setting the wait limit failed");
-  }
-  return DC_OK;
+  cudaError_t e = cudaMemcpyToSymbolAsync(ptx::g_wait_limit_ns, &ns, sizeof(ns), 0, cudaMemcpyHostToDevice, s);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  return (int)e;
 }
 
 void tc_set_cooperative(TcState* t, bool on) { t->chain_coop = on && t->coop_supported; }

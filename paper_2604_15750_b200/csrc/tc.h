@@ -56,7 +56,7 @@ int tc_attention(TcState* t, int layer, const SeqMeta& m, const __nv_bfloat16* k
 // Launch the dense chain with (default) or without the cooperative attribute; see DC_OPT_COOPERATIVE.
 void tc_set_cooperative(TcState* t, bool on);
 // Bound of every device-side wait of the tensor-core kernels, microseconds (device-wide).
-int tc_set_wait_limit_us(TcState* t, long long us);
+int tc_set_wait_limit_us(long long us, cudaStream_t s);   // cudaError_t
 // Test hook: the LM-head kernel issues no loads, so that its bounded waits run out.
 void tc_set_stall_lmhead(TcState* t, bool on);
 // true if the persistent dense chain takes this step (all activation rows in one column block)
