@@ -28,23 +28,25 @@ __device__ __forceinline__ float from_fixed(long long v) {
 constexpr int kSeqWarps = 8;          // sequences per CTA of a call with more sequences than kSpread
 constexpr int kSpread = 4 * 148;
 
-// NQ consecutive values of a row from position k0 on; positions >= n are 0 / not written
-template <int NQ>
-__device__ __forceinline__ void load_run(const float* __restrict__ row, int k0, int n, int vec, float (&v)[NQ]) {
+// NQ consecutive values of a row from position k0 on; positions >= n are 0 / not written.  SAME: the row may have been
+// written earlier in this launch, by another CTA: it is read past L1, and never as constant data
+template <int NQ, bool SAME>
+__device__ __forceinline__ void load_run(const float* row, int k0, int n, int vec, float (&v)[NQ]) {
   constexpr int V = NQ >= 4 ? 4 : 2;
+  auto get = [](const auto* p) { return SAME ? __ldcg(p) : *p; };
 #pragma unroll
   for (int q = 0; q < NQ; q += V) {
     if (vec && k0 + q + V <= n) {
       if (V == 4) {
-        const float4 t = *reinterpret_cast<const float4*>(row + k0 + q);
+        const float4 t = get(reinterpret_cast<const float4*>(row + k0 + q));
         v[q] = t.x; v[q + 1] = t.y; v[q + V / 2] = t.z; v[q + V - 1] = t.w;
       } else {
-        const float2 t = *reinterpret_cast<const float2*>(row + k0 + q);
+        const float2 t = get(reinterpret_cast<const float2*>(row + k0 + q));
         v[q] = t.x; v[q + 1] = t.y;
       }
     } else {
 #pragma unroll
-      for (int u = 0; u < V; ++u) v[q + u] = k0 + q + u < n ? row[k0 + q + u] : 0.f;
+      for (int u = 0; u < V; ++u) v[q + u] = k0 + q + u < n ? get(row + k0 + q + u) : 0.f;
     }
   }
 }
@@ -97,8 +99,8 @@ template <int TW>
 struct BoundaryTeam { float top[4][TW]; long long sum[2][TW]; int first[TW]; };
 
 // The boundary rule for sequence b, by TW warps that are a CTA of their own, or one warp; sI, sH: 33 * NQ * TW floats of
-// shared memory each.
-template <int NQ, int TW = 1>
+// shared memory each.  SAME: see load_run.
+template <int NQ, int TW = 1, bool SAME = false>
 __device__ __forceinline__ void boundary_seq(const float* influence, const float* entropy, int b, const SeqMeta& m,
                                              const DevLens& dl, const Hyper& hp, const BoundaryIo& io, float* sI, float* sH,
                                              BoundaryTeam<TW>* team = nullptr) {
@@ -122,8 +124,8 @@ __device__ __forceinline__ void boundary_seq(const float* influence, const float
   // one scan over the lanes' totals instead of NQ scans (the kernel is bound by instruction issue)
   const int k0 = NQ * lane;
   float rawI[NQ], Is[NQ], Hs[NQ];
-  load_run<NQ>(influence + (size_t)b * ld, k0, Lw, vec, rawI);
-  load_run<NQ>(entropy + (size_t)b * ld, k0, Lw, vec, Hs);
+  load_run<NQ, SAME>(influence + (size_t)b * ld, k0, Lw, vec, rawI);
+  load_run<NQ, SAME>(entropy + (size_t)b * ld, k0, Lw, vec, Hs);
   // centred moving average over the in-range taps, added left to right
   if (TW == 1 && hp.smooth_radius == 1) {   // the default: the neighbours are in this lane or the next ones
     const float lI = __shfl_up_sync(kAll, rawI[NQ - 1], 1), rI = __shfl_down_sync(kAll, rawI[0], 1);

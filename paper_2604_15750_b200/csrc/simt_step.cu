@@ -603,8 +603,8 @@ __global__ void __launch_bounds__(kFuseThreads, 1) k_simt_step(const __grid_cons
   if (p.xlogp != nullptr) xlogp_phase<T>(p, gr);
   if (p.bnd.block_len != nullptr && gr.id == 0 && gr.warp == 0)   // the SMs that get the fewest cross log-prob units
     for (int b = gridDim.x - 1 - blockIdx.x; b < p.ml.batch; b += gridDim.x)
-      if (p.max_window <= 64) boundary_seq<2>(p.sig.ws_infl, p.sig.ws_ent, b, p.ml, DevLens{}, p.hp, p.bnd, bnd[0], bnd[1]);
-      else boundary_seq<DC_MAX_WINDOW / 32>(p.sig.ws_infl, p.sig.ws_ent, b, p.ml, DevLens{}, p.hp, p.bnd, bnd[0], bnd[1]);
+      if (p.max_window <= 64) boundary_seq<2, 1, true>(p.sig.ws_infl, p.sig.ws_ent, b, p.ml, DevLens{}, p.hp, p.bnd, bnd[0], bnd[1]);
+      else boundary_seq<DC_MAX_WINDOW / 32, 1, true>(p.sig.ws_infl, p.sig.ws_ent, b, p.ml, DevLens{}, p.hp, p.bnd, bnd[0], bnd[1]);
 }
 
 template <typename T>
