@@ -578,7 +578,8 @@ def main():
     # dense layers: every weight byte once per step; 2 flops per parameter and activation row
     gemm_ms = sum(stage_ms[n] for n in ("qkv", "oproj", "gateup", "down", "dense"))
     w_bytes = 2.0 * _layer_param_count(wl) * n_layers
-    dense_name = ("k_dense_chain: O projection, norms, gate/up + SwiGLU, down projection, QKV + RoPE of the "
+    dense_name = ("k_simt_step: the whole CUDA-core step behind the embedding in one launch" if fused and wl.dtype == "f32" else
+                  "k_dense_chain: O projection, norms, gate/up + SwiGLU, down projection, QKV + RoPE of the "
                   "next layer in one persistent launch per layer" if fused else
                   "k_gemm_tc: per-op QKV + RoPE, O projection, gate/up + SwiGLU, down projection")
     roof = roof_entry(dense_name, gemm_ms, w_bytes, w_bytes * M,

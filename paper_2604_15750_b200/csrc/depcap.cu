@@ -237,8 +237,8 @@ int run_step(dc_ctx* c, const dc_step_in* in, const dc_step_out* out, const SeqM
   const SimtSignals sg{c->logits, g.vocab, g.mask_id, g.forbid_mask_pred, c->ws_pred, c->ws_conf, c->ws_ent,
                        c->ws_infl, c->ws_lse, so, out->status};
 
-  // (profiling wants the stages apart; a prefill without layers has no work, and no rows at the LM head either)
-  if (!c->use_tc && c->fuse.grid > 0 && c->coop && !pf.on && !(kv_only && g.n_layers == 0)) {
+  // (a prefill without layers has no work, and no rows at the LM head either)
+  if (!c->use_tc && c->fuse.grid > 0 && c->coop && !(kv_only && g.n_layers == 0)) {
     SimtStep<T> st{};
     st.layers = (const SimtLayer<T>*)c->simt_layers; st.n_layers = g.n_layers; st.kv_only = kv_only;
     st.export_kv = (in->flags & DC_STEP_EXPORT_KV) != 0;
@@ -254,7 +254,9 @@ int run_step(dc_ctx* c, const dc_step_in* in, const dc_step_out* out, const SeqM
     auto aligned = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
     if (simt_step_ok<T>(c->fuse, st) && aligned(in->k_cache) && aligned(in->v_cache) && aligned(io.h_in) &&
         aligned(io.h_prev_in) && aligned(io.h_out)) {
+      pf.begin(DC_STAGE_DENSE, 1);
       const cudaError_t e = (cudaError_t)launch_simt_step<T>(c->fuse, st, s);
+      pf.end();
       if (e != cudaSuccess) {
         cudaGetLastError();
         return fail(c, DC_ERR_CUDA, "fused step launch failed: %s", cudaGetErrorString(e));

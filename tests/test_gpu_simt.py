@@ -13,6 +13,13 @@ from parity import Case, compare
 pytestmark = pytest.mark.gpu
 
 
+def _fused(eng, case):
+    """whether a step of the case runs as one launch"""
+    _, launches = eng.step_profiled(**case.device_inputs(eng, poison=case.wl.ctx_max > 0))
+    assert (launches["dense"] == 1) == (launches["qkv"] == 0) and launches["dense"] <= 1
+    return launches["dense"] == 1
+
+
 def _wl(name, dtype, n_q, n_kv, hd, d, ff, vocab, batch, ctx, last, win):
     return inputs.Workload(name, 2, d, n_q, n_kv, hd, ff, vocab, dtype, batch, ctx[0], ctx[1], last, win, 64, 31337)
 
@@ -60,9 +67,14 @@ def test_fused_step_and_separate_launches(wl):
                    win_len=[wl.win_len, 1, 17][:wl.batch], remain_len=[64, 8, 30][:wl.batch])
     case = Case(wl, lengths=lengths, n_decoded=0)
     eng = case.make_engine()
+    assert _fused(eng, case)
     gpu, ora = case.run_gpu(eng, poison=True), case.run_oracle()
     compare(case, gpu, ora)
+    eng.step_profiled(**case.device_inputs(eng, poison=True))   # (the call that is profiled is the same one)
+    for k in ("conf", "entropy", "lse", "influence", "block_len"):
+        assert np.array_equal(eng.out[k].cpu().numpy(), gpu[k]), k
     eng.set_option(1, 0)                       # DC_OPT_COOPERATIVE off: one launch per operation
+    assert not _fused(eng, case)
     one = case.run_gpu(eng, poison=True)
     tol = 1e-5 if wl.dtype == "f32" else 2e-2
     for b in range(wl.batch):
