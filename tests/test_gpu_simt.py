@@ -84,15 +84,17 @@ def test_fused_step_and_separate_launches(wl):
     eng.close()
 
 
-@pytest.mark.parametrize("cooperative", [1, 0])   # the fused step, separate launches
-def test_ragged_rows_lie_behind_one_another(cooperative):
+@pytest.mark.parametrize("hd,cooperative,fused", [(32, 1, True), (32, 0, False), (16, 1, False)])
+def test_ragged_rows_lie_behind_one_another(hd, cooperative, fused):
     """Sequences of 48, 16 and 32 rows (rounded up) in a batch, fp32: signals at 1e-4, the appended keys and values at
-    1e-4, nothing else of the cache written."""
+    1e-4, nothing else of the cache written.  The fused step, separate launches, and separate launches with the
+    rotation outside the GEMM."""
     ctx, last, win = [40, 64, 7], [16, 0, 5], [32, 3, 12]
-    wl = inputs.Workload("ragged_f32", 2, 64, 4, 2, 16, 128, 300, "f32", 3, 64, 64, 16, 32, 64, 515)
+    wl = inputs.Workload("ragged_f32", 2, 64, 4, 2, hd, 128, 300, "f32", 3, 64, 64, 16, 32, 64, 515)
     case = Case(wl, lengths=dict(ctx_len=ctx, last_len=last, win_len=win, remain_len=[64] * 3))
     eng = case.make_engine(max_ctx=128)
     eng.set_option(1, cooperative)             # DC_OPT_COOPERATIVE
+    assert _fused(eng, case) == fused
     di = case.device_inputs(eng)
     k0, v0 = di["k_cache"].clone(), di["v_cache"].clone()
     out = eng.step(influence=True, boundary=True, export_kv=True, **di)
