@@ -257,12 +257,15 @@ int run_step(dc_ctx* c, const dc_step_in* in, const dc_step_out* out, const SeqM
       pf.begin(DC_STAGE_DENSE, 1);
       const cudaError_t e = (cudaError_t)launch_simt_step<T>(c->fuse, st, s);
       pf.end();
-      if (e != cudaSuccess) {
-        cudaGetLastError();
-        return fail(c, DC_ERR_CUDA, "fused step launch failed: %s", cudaGetErrorString(e));
+      if (e != cudaSuccess) cudaGetLastError();
+      if (e == cudaSuccess) {
+        if (!kv_only) { c->have_logits = true; c->last_meta = ml; }
+        return DC_OK;
       }
-      if (!kv_only) { c->have_logits = true; c->last_meta = ml; }
-      return DC_OK;
+      if (e != cudaErrorCooperativeLaunchTooLarge)
+        return fail(c, DC_ERR_CUDA, "fused step launch failed: %s", cudaGetErrorString(e));
+      c->fuse.grid = 0;   // the stream has fewer SMs than the device: separate launches from now on
+      pf.launches[DC_STAGE_DENSE] = 0;
     }
   }
 
@@ -272,16 +275,24 @@ int run_step(dc_ctx* c, const dc_step_in* in, const dc_step_out* out, const SeqM
   size_t part_stride = 0;
 
   const bool export_kv = (in->flags & DC_STEP_EXPORT_KV) != 0;
-  const bool chain = c->use_tc && c->gains_vec && tc_chain_ok(c->tc, m);
+  bool chain = c->use_tc && c->gains_vec && tc_chain_ok(c->tc, m);
   if (chain) {
     // persistent dense chain: norm1 + QKV of layer 0, then per layer attention and one launch
     // that runs O projection .. QKV of the next layer
-    const int L = g.n_layers;
     pf.begin(DC_STAGE_DENSE, 1);
-    int rc = tc_chain(c->tc, 0, 0, CH_NORM1, CH_END, m, c->x, (const __nv_bfloat16*)a, c->cos_sin,
-                      nullptr, (const __nv_bfloat16*)c->norm1[0], 0, &part, &nsplit, &part_stride);
+    const int rc = tc_chain(c->tc, 0, 0, CH_NORM1, CH_END, m, c->x, (const __nv_bfloat16*)a, c->cos_sin,
+                            nullptr, (const __nv_bfloat16*)c->norm1[0], 0, &part, &nsplit, &part_stride);
     pf.end();
-    if (rc != DC_OK) return fail(c, rc, "dense chain failed: %s", tc_error(c->tc));
+    if (rc == kTooFewSms) {
+      chain = false; part = nullptr; nsplit = 0;
+      pf.launches[DC_STAGE_DENSE] = 0;
+    } else if (rc != DC_OK) {
+      return fail(c, rc, "dense chain failed: %s", tc_error(c->tc));
+    }
+  }
+  if (chain) {
+    const int L = g.n_layers;
+    int rc = DC_OK;
     for (int l = 0; l < L; ++l) {
       const bool last = l + 1 == L;
       pf.begin(DC_STAGE_ATTN, 1);

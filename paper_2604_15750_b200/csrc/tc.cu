@@ -569,6 +569,10 @@ int tc_chain(TcState* t, int layer, int qkv_layer, int phase_begin, int phase_en
   cudaError_t e = cudaLaunchKernelEx(&cfg, k_dense_chain, maps, p);
   if (e != cudaSuccess) {
     cudaGetLastError();
+    if (e == cudaErrorCooperativeLaunchTooLarge) {   // the stream has fewer SMs than the device
+      t->chain_grid = 0;
+      return kTooFewSms;
+    }
     return tfail(t, DC_ERR_CUDA, "dense chain launch failed: %s", cudaGetErrorString(e));
   }
   *part = t->part; *nsplit = p.split_down; *part_stride = t->part_stride;

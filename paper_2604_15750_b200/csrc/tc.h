@@ -63,6 +63,9 @@ void tc_set_stall_lmhead(TcState* t, bool on);
 bool tc_chain_ok(const TcState* t, const SeqMeta& m);
 // once at the start of a step: the words of the chain's grid barrier that must be cleared before it
 void tc_step_begin(TcState* t, unsigned int** words, int* n_words);
+// what tc_chain returns, before it has launched anything, when the stream does not have the SMs for it; tc_chain_ok is
+// false then
+constexpr int kTooFewSms = -1;
 // Phases [phase_begin, phase_end) of the dense chain (CH_* in tc_chain.cuh): O projection,
 // residual + norm2 (gain g2), gate/up, down projection of `layer`; residual + norm1 (gain g1,
 // folding fold_norm1 partial sums) and the rotated QKV of `qkv_layer`.  The partial sums of the

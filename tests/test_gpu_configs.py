@@ -14,6 +14,7 @@ GPU stack produced.
 """
 import numpy as np
 import pytest
+import torch
 
 from paper_2604_15750_b200 import inputs
 
@@ -66,3 +67,26 @@ def test_llada8b_long_context_batch16_bimodal():
     """B = 16, 4096 cached keys per sequence (32 context tiles), M = 5120 rows, 4096 LM-head rows,
     max-probability bimodal (half the positions peaked above 0.9, half flat)."""
     near, worst, near_r, worst_r, strict = _run("llada8b_long", "bimodal", "per-op", 32)
+
+
+@pytest.mark.parametrize("dtype,hd,win", [("f32", 32, 32), ("bf16", 128, 16), ("bf16", 128, 32)])
+def test_a_stream_with_fewer_sms_than_the_device(dtype, hd, win):
+    """The fused CUDA-core step and the dense chain need a CTA on every SM at once.  On a stream of 16 SMs their
+    launches are refused, and the steps run as separate launches."""
+    gc = pytest.importorskip("torch.cuda.green_contexts")
+    if not gc.SUPPORTED:
+        pytest.skip("no green contexts")
+    wl = inputs.Workload("few_sms", 2, 256, 4, 2, hd, 512, 2048, dtype, 1, 100, 100, 16, win, 64, 31337)
+    case = Case(wl)
+    green = gc.GreenContext.create(16, 0)
+    green.set_context()
+    try:
+        with torch.cuda.stream(green.Stream()):
+            eng = case.make_engine()
+            gpu = case.run_gpu(eng)
+            _, launches = eng.step_profiled(**case.device_inputs(eng))
+            eng.close()
+    finally:
+        green.pop_context()
+    assert launches["dense"] == 0 and launches["qkv"] == case.n_layers
+    compare(case, gpu, case.run_oracle())
