@@ -125,6 +125,12 @@ int tfail(TcState* t, int code, const char* fmt, ...) {
   return code;
 }
 
+// a launch that failed: reported here, so that the error is not found again behind the next launch
+int launch_fail(TcState* t, const char* what, cudaError_t e) {
+  cudaGetLastError();
+  return tfail(t, DC_ERR_CUDA, "%s launch failed: %s", what, cudaGetErrorString(e));
+}
+
 template <typename T>
 T* talloc(TcState* t, size_t n, bool* ok) {
   void* p = nullptr;
@@ -355,10 +361,7 @@ static int launch_gemm(TcState* t, const CUtensorMap& w0, const CUtensorMap& w1,
   } else {
     e = launch_chained(k_gemm_tc<EPI, false>, workers, kGemmThreads, smem, t->s, w0, w1, w2, ma, p, stages);
   }
-  if (e != cudaSuccess) {
-    cudaGetLastError();
-    return tfail(t, DC_ERR_CUDA, "GEMM launch failed: %s", cudaGetErrorString(e));
-  }
+  if (e != cudaSuccess) return launch_fail(t, "GEMM", e);
   return DC_OK;
 }
 
@@ -450,7 +453,7 @@ int tc_attention(TcState* t, int layer, const SeqMeta& m, const __nv_bfloat16* k
     cfg.blockDim = dim3(kAttnThreads); cfg.dynamicSmemBytes = kAttnSmem;
     e = cudaLaunchKernelEx(&cfg, k_attn_tc, t->map_q, t->map_k, t->map_vt, t->map_kc, t->map_vc, ap);
   }
-  if (e != cudaSuccess) return tfail(t, DC_ERR_CUDA, "attention launch failed: %s", cudaGetErrorString(e));
+  if (e != cudaSuccess) return launch_fail(t, "attention", e);
   return DC_OK;
 }
 
@@ -568,12 +571,10 @@ int tc_chain(TcState* t, int layer, int qkv_layer, int phase_begin, int phase_en
   cfg.attrs = attrs; cfg.numAttrs = t->chain_coop ? 2 : 1;
   cudaError_t e = cudaLaunchKernelEx(&cfg, k_dense_chain, maps, p);
   if (e != cudaSuccess) {
-    cudaGetLastError();
-    if (e == cudaErrorCooperativeLaunchTooLarge) {   // the stream has fewer SMs than the device
-      t->chain_grid = 0;
-      return kTooFewSms;
-    }
-    return tfail(t, DC_ERR_CUDA, "dense chain launch failed: %s", cudaGetErrorString(e));
+    const int rc = launch_fail(t, "dense chain", e);
+    if (e != cudaErrorCooperativeLaunchTooLarge) return rc;
+    t->chain_grid = 0;   // the stream has fewer SMs than the device
+    return kTooFewSms;
   }
   *part = t->part; *nsplit = p.split_down; *part_stride = t->part_stride;
   return DC_OK;
@@ -664,7 +665,7 @@ int tc_lmhead(TcState* t, const SeqMeta& m, const __nv_bfloat16* h, int mask_id,
   if (e == cudaSuccess)
     e = launch_chained(k_lm_combine, (npos + 3) / 4, 128, 0, t->s, t->lm_part, nctas, m, g.vocab, mask_id, status, 1,
                        ws_pred, ws_conf, ws_ent, ws_infl, ws_lse, out);
-  if (e != cudaSuccess) return tfail(t, DC_ERR_CUDA, "LM-head launch failed: %s", cudaGetErrorString(e));
+  if (e != cudaSuccess) return launch_fail(t, "LM-head", e);
   return DC_OK;
 }
 
