@@ -49,7 +49,7 @@ struct FewCtl {
   // let the parity of a K tile's phase be taken for that of the phase before the V^T tile in between.
   uint64_t q_full, k_full[3], v_full[3], empty[kFewSlotsMax], s_full[2], s_empty[2], p_full, p_empty;
   uint32_t tmem_base;
-  int abort_flag, again_flag;
+  int abort_flag, again_flag, late_flag;
   alignas(16) float m0[kFewRows];      // the rows' reference points (log2 units)
   float part[4][kFewRows];             // per softmax warp: the rows' sums (or maxima) over its keys
   alignas(16) float inv[kFewRows];
@@ -101,7 +101,7 @@ k_attn_few(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CU
   const int Tc = (P + kBK - 1) / kBK, T = Tc + (R + kBK - 1) / kBK;   // context tiles, then tiles of active keys
 
   if (threadIdx.x == 0) {
-    c.abort_flag = 0; c.again_flag = 0;
+    c.abort_flag = 0; c.again_flag = 0; c.late_flag = 0;
     ptx::mbar_init(&c.q_full, 1);
     for (int i = 0; i < slots; ++i) ptx::mbar_init(&c.empty[i], 1);
     for (int i = 0; i < 3; ++i) { ptx::mbar_init(&c.k_full[i], 1); ptx::mbar_init(&c.v_full[i], 1); }
@@ -122,6 +122,7 @@ k_attn_few(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CU
   pdl_wait();
 
   int* abort_flag = &c.abort_flag;
+  int loads = 0;   // of the producer thread: Q, then K and V^T tiles
   // Tiles are counted through all passes (J = pass * T + j); the ring holds items 2 J (K) and 2 J + 1 (V^T).
   for (int pass = 0; pass < 3; ++pass) {
     const int J0 = pass * T;
@@ -133,6 +134,7 @@ k_attn_few(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CU
           ptx::mbar_expect_tx(&c.q_full, kFewQ);
           ptx::tma_load_2d(Qs, &map_q, &c.q_full, h * kHd, row);
           ptx::tma_load_2d(Qs + kFewQ / 2, &map_q, &c.q_full, h * kHd + 64, row);
+          loads = 1;
         }
         int s = (2 * J0) % slots;
         uint32_t ph = (uint32_t)((2 * J0) / slots) & 1u;
@@ -161,6 +163,7 @@ k_attn_few(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CU
             ptx::tma_load_2d(dst, &map_vt, bar, col, g * kHd);
             ptx::tma_load_2d(dst + kSub, &map_vt, bar, col + 64, g * kHd);
           }
+          ++loads;
           if (++s == slots) { s = 0; ph ^= 1u; }
         }
       }
@@ -298,6 +301,14 @@ k_attn_few(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CU
         if (i < n) dst[(size_t)i * p.nq * kHd] = __float2bfloat16_rn(o[i] * c.inv[i]);
     }
     break;
+  }
+  if (loads > 0 && c.abort_flag != 0) {
+    // given up: what is still on its way lands before another CTA gets this shared memory (with a limit of its own)
+    ptx::mbar_wait(&c.q_full, 0, &c.late_flag);
+    for (int it = max(0, loads - 7); it < loads - 1; ++it) {   // the last three tiles of each kind
+      const int J = it >> 1;
+      ptx::mbar_wait((it & 1) == 0 ? &c.k_full[J % 3] : &c.v_full[J % 3], (uint32_t)(J / 3) & 1u, &c.late_flag);
+    }
   }
   ptx::tc_fence_before();
   __syncthreads();
