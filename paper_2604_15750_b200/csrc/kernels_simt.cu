@@ -133,7 +133,7 @@ __global__ void __launch_bounds__(256) k_rmsnorm(float* __restrict__ x,
                                                  float eps, int d, T* __restrict__ out) {
   __shared__ float red[32];
   pdl_trigger();
-  pdl_wait();
+  pdl_wait(x, part);
   const size_t off = (size_t)blockIdx.x * d;
   rmsnorm_row<T>(x + off, part ? part + off : nullptr, nsplit, part_stride, g, eps, d, out + off,
                  red);
@@ -159,7 +159,7 @@ __global__ void __launch_bounds__(256) k_lm_rows(const float* __restrict__ x, co
   extern __shared__ __align__(16) float lm_row_s[];   // staged: the row with the partial sums folded in
   __shared__ float red[32];
   pdl_trigger();
-  pdl_wait();
+  pdl_wait(x, part);
   const int lrow = blockIdx.x;
   const int grp = lrow / (m.nv * m.G), in = lrow % (m.nv * m.G);
   const int v = in / m.G, p = grp * m.G + in % m.G;
@@ -706,7 +706,7 @@ __global__ void __launch_bounds__(256) k_xlogp(const T* __restrict__ h,
                                                float* __restrict__ xlogp) {
   extern __shared__ __align__(16) float wrow[];  // W_lm[yhat_j] as fp32
   pdl_trigger();
-  pdl_wait();
+  pdl_wait(h, ws_pred, ws_lse);
   const int b = blockIdx.y, j = blockIdx.x;
   const int W = m.win_len[b];
   if (j >= W) return;

@@ -14,6 +14,15 @@
 namespace dc {
 
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// The same for a kernel that reads what earlier kernels wrote through __restrict__ pointers, which it passes here: the
+// compiler may move a load through such a pointer in front of a statement that cannot change what it points to.
+template <typename P0, typename... P>
+__device__ __forceinline__ void pdl_wait(P0& p0, P&... p) {
+  pdl_wait();
+  auto behind = [](auto& q) { asm volatile("" : "+l"(q) : : "memory"); };
+  behind(p0);
+  (behind(p), ...);
+}
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 template <typename... P, typename... A>

@@ -244,7 +244,7 @@ __global__ void k_lm_combine(const float* __restrict__ part, int nctas, SeqMeta 
                              float* __restrict__ ws_ent, float* __restrict__ ws_infl,
                              float* __restrict__ ws_lse, SignalOut out) {
   pdl_trigger();
-  pdl_wait();
+  pdl_wait(part);
   const int pos = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (pos >= m.batch * m.W_cap) return;
