@@ -228,6 +228,8 @@ typedef struct dc_ctx dc_ctx; /* opaque */
  * cuda_stream: a cudaStream_t (null = the legacy default stream); all work is ordered on it.
  * Tensor-core kernels need dtype bf16, head_dim 128, d_model and d_ff multiples of 128; any
  * other shape runs on the CUDA-core kernels.  Errors: INVALID_ARG, UNSUPPORTED, NOMEM, CUDA.
+ * The first context of a process on a device also loads and sets up its kernels, which takes some
+ * milliseconds (7 .. 16 for a small CUDA-core model, whose later contexts take 1).
  * The backbone is the pre-norm transformer the paper's backbones share (Section 5.1). */
 DC_API int dc_create(const dc_config* cfg, const dc_weights* w, void* cuda_stream, dc_ctx** out);
 
@@ -342,12 +344,14 @@ typedef struct dc_generate_out {
 DC_API int dc_generate(dc_ctx* ctx, const dc_generate_in* in, const dc_generate_out* out);
 
 /* Options of a context.  No paper counterpart.
- *   DC_OPT_COOPERATIVE (default 1): the fused dense-layer kernel synchronises its CTAs through a
- *     counter in global memory, which needs all of them resident at once; a cooperative launch
- *     guarantees that (or fails).  0 launches the same grid without the attribute - for profilers
- *     that cannot replay cooperative cluster launches.  All CTAs are still resident when the GPU
- *     runs nothing else, and every wait in the kernel is bounded (DC_ERR_TIMEOUT in status[b]
- *     otherwise), but the guarantee is gone: not for production use.
+ *   DC_OPT_COOPERATIVE (default 1): the fused kernels synchronise their CTAs through a counter in
+ *     global memory, which needs all of them resident at once; a cooperative launch guarantees
+ *     that.  A stream without the SMs for it (a green context's) gets a launch per operation instead.
+ *     0 is for profilers that cannot replay cooperative launches.  The fused dense-layer
+ *     kernel of the tensor-core path is then launched on the same grid without the attribute: all
+ *     CTAs are still resident when the GPU runs nothing else, and every wait in the kernel is bounded
+ *     (DC_ERR_TIMEOUT in status[b] otherwise), but the guarantee is gone: not for production use.
+ *     The CUDA-core step runs as a launch per operation, with fp32 sums in another order.
  *   DC_OPT_WAIT_LIMIT_US (default 2 000 000): how long a device-side wait (on a TMA / MMA
  *     barrier, the grid barrier, a hand-over flag) polls before the kernel gives up, frees what it
  *     holds, returns and reports DC_ERR_TIMEOUT in status[b]; 1000 .. 60 000 000.  The value is

@@ -1,5 +1,6 @@
 // Decision kernels: the DepGA-Block boundary scan (Section 4.2, cumulative form Section 4.4)
-// and CAP-Decoding (Section 4.3, Algorithm 1).  One warp per sequence.
+// and CAP-Decoding (Section 4.3, Algorithm 1).  One warp per sequence, more where that is too long a chain
+// (k_boundary_wide, select_long).
 //
 // Every floating-point step that decides an integer is written with explicit round-to-nearest
 // intrinsics (no contraction into FMA) and a fixed operation order, so the decisions are a
@@ -80,7 +81,7 @@ void launch_boundary_dev(const float* influence, const float* entropy, int ld, i
 // position, never the matrix of the whole pool (Eq. 6: conflict iff xlogp[i,j] + xlogp[j,i] > gamma).
 // Position 32 q + lane belongs to the lane; a set of candidates is the array of their sort keys, 0 where
 // a position is not in it.  The kernel is bound by instruction issue and by the latency of those
-// rows and columns, so the code is kept to few instructions and five CTAs of eight warps per SM.
+// rows and columns, so the code is kept to few instructions and to the registers of 40 warps per SM.
 // (Loading the conflicts of the last 16 candidates at once instead of a round per selected position
 // was slower: 63 against 40 us, most of its loads were for pairs that never meet; prefetching the
 // pool's rows into L2 changed nothing at 8192 x 128 and cost 8 us at 1000 x 256.)

@@ -20,11 +20,11 @@ __device__ __forceinline__ float from_fixed(long long v) {
 
 // Both decisions are a few hundred dependent operations per sequence, so a sequence is one warp with
 // NQ positions per lane, every reduction and scan is a shuffle, and nothing waits on a block-wide
-// barrier.  A call over many sequences is
-// then bound by its memory traffic: all 8192 sequences of a large call are resident at once and
-// their load latencies overlap (8192 x 128: k_boundary 26 -> 13 us, k_select 222 -> 39 us against
-// one block with a thread per position).  With few sequences - a step - every warp is a CTA of its
-// own, so that they spread over the SMs.
+// barrier (8192 x 128: k_boundary 26 -> 13 us, k_select 222 -> 37 us against one block with a thread per
+// position).  What bounds a call over many sequences is instruction issue and latency: 63 registers a
+// thread let 32 warps of k_boundary on an SM, 48 let 40 of k_select, so 8192 sequences are 1.7 and 1.4 rounds; 63% and
+// 52% of the issue slots are used, 6% and 24% of the DRAM throughput.  With few sequences - a step - every warp is a
+// CTA of its own, so that they spread over the SMs.
 constexpr int kSeqWarps = 8;          // sequences per CTA of a call with more sequences than kSpread
 constexpr int kSpread = 4 * 148;
 

@@ -4,9 +4,10 @@
 // third of that launch, ramp and drain, and the host needs 4 us for every launch.  Here the phases of
 // all layers, the LM head, the signals, the cross log-probs and the boundary rule run in one kernel
 // of one CTA per SM, with a counting grid barrier between phases.  Two-layer fp32 model (d 256, 96 rows,
-// vocab 4096): 22 launches and 157 us per step -> 3 launches and 108 us; a generation step 183 -> 110 us.
+// vocab 4096): 22 launches and 157 us per step -> 3 launches and 106 us; a generation step 183 -> 107 us.
 // What is left: about 1.5 us per barrier (12), and in a phase two L2 latencies (rows, weights) and the
-// issue of some 1000 instructions per warp, four warps to a scheduler.
+// issue of some 1000 instructions per warp, four warps to a scheduler.  The first context of a process on a
+// device loads the kernel when it is made (dc_create 7..16 ms instead of 0.9).
 //
 //   per layer   norm1 + QKV + rotation + cache append | attention | O projection + residual |
 //               norm2 + gate / up + SwiGLU | down projection + residual
@@ -31,7 +32,7 @@ namespace {
 constexpr int kGroups = 2, kFuseThreads = 256 * kGroups;
 constexpr int kKC = 256, kStages = 3;          // k-chunk of the GEMM tiles (32 k per warp), ring stages
 constexpr size_t kGroupSmemMax = 112 * 1024;   // shared memory of a group
-constexpr int kMaxNormD = 1024;                // a warp holds a row in registers while it norms it
+constexpr int kMaxNormD = 1024;                // half a warp norms a row (norm_row), 64 elements of it at this width
 
 // How long a thread waits at the grid barrier before it gives up (as in the tensor-core kernels).
 __device__ unsigned long long g_simt_wait_ns = 2000000000ull;

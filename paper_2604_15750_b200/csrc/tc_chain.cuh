@@ -14,9 +14,9 @@
 //
 // Why one kernel: at 192 activation rows a layer is 436 MB of weights (67 us of HBM time) cut
 // into four GEMMs of 5..30 us each; as separate launches every one of them pays its own launch,
-// pipeline ramp, and an epilogue that nothing overlaps.  Here the weight stream of the next phase
-// is already on its way into L2 (cp.async.bulk.prefetch) while the current phase drains, and the
-// only cost between phases is the barrier.
+// pipeline ramp, and an epilogue that nothing overlaps.  Here phases are a barrier apart, and while a
+// CTA waits at it the first weights of its next phase are on their way into L2
+// (cp.async.bulk.prefetch, from the arrival on).
 //
 // GEMM orientation (as in tc_gemm.cuh): a CTA owns 128 weight rows (MMA M, one TMEM lane per
 // output feature) and all activation rows (MMA N <= 256, one TMEM column per row).  Every unit
@@ -34,8 +34,9 @@
 // CTA of a pair issues the MMAs; TMA loads of both CTAs report to the even CTA's full barrier,
 // tcgen05.commit releases the ring slot in both CTAs.  No load is multicast.
 //
-// Warp roles (512 threads): warp 0 lane 0 = TMA producer, warp 1 lane 0 = MMA issuer (warp 1
-// owns the TMEM allocation).  All sixteen warps run the epilogue: warp w reads the TMEM lanes
+// Warp roles (512 threads): warp 0 lane 0 = TMA producer, warp 1 = MMA issuer (the whole warp runs the
+// loop, one elected lane issues; it also owns the TMEM allocation), warp 3 = L2 prefetch at the
+// barriers.  All sixteen warps run the epilogue: warp w reads the TMEM lanes
 // 32 * (w % 4) .. +31 (the only ones it can reach) and the column part w / 4, so four warps share
 // every lane quarter.  The RoPE epilogue is a chain of dependent shared-memory exchanges and
 // barriers: with four warps per scheduler instead of two it takes 7.2 k instead of 12.2 k clocks.
