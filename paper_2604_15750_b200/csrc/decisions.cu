@@ -6,6 +6,7 @@
 // intrinsics (no contraction into FMA) and a fixed operation order, so the decisions are a
 // function of the input bits alone; running sums use 2^40 fixed point, which is order-free.
 #include <math.h>
+#include <string.h>
 
 #include <type_traits>
 
@@ -14,6 +15,7 @@
 
 namespace dc {
 
+const SeqMeta kNoLengths{};            // (the lengths are in device memory)
 constexpr int kWideBoundary = 4096;   // sequences that k_boundary_wide takes
 constexpr int kThreads = 256;         // one thread per window position (k_commit)
 
@@ -72,7 +74,7 @@ void launch_boundary(const float* influence, const float* entropy, int ld, const
 void launch_boundary_dev(const float* influence, const float* entropy, int ld, int batch, const DevLens& dl,
                          const Hyper& hp, int max_window, float* score, float* cum_i, float* cum_s,
                          int32_t* block_len, cudaStream_t s) {
-  boundary(influence, entropy, ld, batch, SeqMeta{}, dl, hp, max_window, score, cum_i, cum_s, block_len, s);
+  boundary(influence, entropy, ld, batch, kNoLengths, dl, hp, max_window, score, cum_i, cum_s, block_len, s);
 }
 
 // ---- CAP-Decoding ------------------------------------------------------------------------------
@@ -185,8 +187,8 @@ struct SelectArgs {
 };
 
 // lengths of sequence b: window, block
-__device__ __forceinline__ void select_lengths(const SelectArgs& p, const SeqMeta& m, const SelectCommit& cm, int b, int& W, int& blk) {
-  W = len_of(p.dl.win_len, m.win_len, b);
+__device__ __forceinline__ void select_lengths(const SelectArgs& p, const PrevLen& win, const SelectCommit& cm, int b, int& W, int& blk) {
+  W = len_of(p.dl.win_len, win.n, b);
   const int kept = cm.win_ids != nullptr ? cm.keep.n[b] : -1;   // the length of a block that a generation is in the middle of
   blk = kept >= 0 ? kept : p.block_len[b];
 }
@@ -294,7 +296,7 @@ __device__ __forceinline__ void long_matrix(const float* __restrict__ xb, unsign
 // one while the others make that of the next.  It starts from the inputs again: nothing of the sequences that end
 // without it has to be kept for it.
 template <int NQ>
-__device__ __forceinline__ void select_long(const SelectArgs& p, const SeqMeta& m, const SelectCommit& cm, int first, unsigned todo,
+__device__ __forceinline__ void select_long(const SelectArgs& p, const PrevLen& win, const SelectCommit& cm, int first, unsigned todo,
                                             unsigned team, LongPass<NQ> (&sm)[2], int& next) {
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int me = __popc(team & ((1u << w) - 1u)), n_team = __popc(team);
@@ -309,7 +311,7 @@ __device__ __forceinline__ void select_long(const SelectArgs& p, const SeqMeta& 
     todo &= todo - 1u;
     if (cur >= 0) {
       int W, blk;
-      select_lengths(p, m, cm, cur, W, blk);
+      select_lengths(p, win, cm, cur, W, blk);
       const int L = min(max(blk, 0), W);
 #pragma unroll 1
       for (int q = me; q < NQ; q += n_team) {
@@ -358,7 +360,7 @@ __device__ __forceinline__ void select_long(const SelectArgs& p, const SeqMeta& 
         masked |= (lw.key[32 * q + lane] != 0u ? 1u : 0u) << q;
       }
       int W, blk;
-      select_lengths(p, m, cm, before, W, blk);
+      select_lengths(p, win, cm, before, W, blk);
       select_store<NQ>(p, cm, before, W, blk, sel, masked);
     }
     if (cur < 0) return;
@@ -369,7 +371,7 @@ __device__ __forceinline__ void select_long(const SelectArgs& p, const SeqMeta& 
 }
 
 template <int NQ>
-__global__ void __launch_bounds__(32 * kSeqWarps, 5) k_select(const __grid_constant__ SelectArgs p, const __grid_constant__ SeqMeta m,
+__global__ void __launch_bounds__(32 * kSeqWarps, 5) k_select(const __grid_constant__ SelectArgs p, const __grid_constant__ PrevLen win,
                                                               const __grid_constant__ SelectCommit cm) {
   constexpr int NA = 4;
   constexpr bool kCoop = NQ >= 4;             // (shorter windows have no long passes)
@@ -382,7 +384,7 @@ __global__ void __launch_bounds__(32 * kSeqWarps, 5) k_select(const __grid_const
   pdl_wait();
   if (w < p.seqs && b < p.batch) {
     int W, blk;
-    select_lengths(p, m, cm, b, W, blk);
+    select_lengths(p, win, cm, b, W, blk);
     const int L = min(max(blk, 0), W);
     const size_t o = (size_t)b * p.max_window;
     const float* xb = p.xlogp + o * p.max_window;
@@ -454,7 +456,7 @@ __global__ void __launch_bounds__(32 * kSeqWarps, 5) k_select(const __grid_const
     asm volatile("barrier.cta.sync 1, %0;" ::"r"(blockDim.x) : "memory");
     const unsigned todo = __ballot_sync(kAll, lane < p.seqs && lp_pending[lane & (kSeqWarps - 1)] != 0);
     const unsigned idle = (1u << (blockDim.x >> 5)) - (1u << p.seqs);
-    if (todo != 0u) select_long<NQ>(p, m, cm, blockIdx.x * p.seqs, todo, todo | idle, lp, lp_next);
+    if (todo != 0u) select_long<NQ>(p, win, cm, blockIdx.x * p.seqs, todo, todo | idle, lp, lp_next);
   }
 }
 
@@ -462,19 +464,25 @@ static void select(const float* conf, const int32_t* win_ids, const float* xlogp
                    const SeqMeta& m, const DevLens& dl, const Hyper& hp, int mask_id, int max_window,
                    uint8_t* sel_mask, int32_t* sel_idx, int32_t* sel_count, cudaStream_t s,
                    const SelectCommit& cm = SelectCommit{}) {
+  PrevLen win;
+  memcpy(win.n, m.win_len, sizeof(win.n));
   SelectArgs p{conf, win_ids, xlogp, block_len, batch, mask_id, max_window, sel_mask, sel_idx, sel_count, 0,
                (reinterpret_cast<uintptr_t>(xlogp) & 15) == 0 ? 1 : 0, dl, hp};
   decide_launch(batch, max_window, [&](auto nq, dim3 grid, int threads) {
     constexpr int NQ = decltype(nq)::value;
     p.seqs = threads / 32;
-    if (NQ >= 4) {   // whole CTAs, which end long passes together: the machine is filled before a CTA gets a second sequence
-      const int warps = NQ == 4 && batch > kSelectCtas ? kSeqWarps / 2 : kSeqWarps, ctas = kSelectCtas * kSeqWarps / warps;
+    if (NQ >= 4) {
+      // Whole CTAs, which end long passes together: the machine is filled before a CTA gets a second sequence.  Calls that
+      // would put more than six into one have CTAs of four warps, whose slots are free sooner (boundary and
+      // selection of 6000 x 128: 35.9 us against 38.4; below, the larger CTAs are the better spread: 1500 x 128 16.3
+      // against 18.0, 4000 x 128 27.8 and 27.8).
+      const int warps = NQ == 4 && batch > 6 * kSelectCtas ? kSeqWarps / 2 : kSeqWarps, ctas = kSelectCtas * kSeqWarps / warps;
       p.seqs = (batch + ctas - 1) / ctas;
       if (p.seqs > warps) p.seqs = warps;
       threads = 32 * warps;
       grid = dim3((batch + p.seqs - 1) / p.seqs);
     }
-    launch_chained(k_select<NQ>, grid, threads, 0, s, p, m, cm);
+    launch_chained(k_select<NQ>, grid, threads, 0, s, p, win, cm);
   });
 }
 
@@ -489,7 +497,7 @@ void launch_select_dev(const float* conf, const int32_t* win_ids, const float* x
                        const int32_t* block_len, int batch, const DevLens& dl, const Hyper& hp, int mask_id,
                        int max_window, uint8_t* sel_mask, int32_t* sel_idx, int32_t* sel_count,
                        cudaStream_t s) {
-  select(conf, win_ids, xlogp, block_len, batch, SeqMeta{}, dl, hp, mask_id, max_window, sel_mask, sel_idx, sel_count, s);
+  select(conf, win_ids, xlogp, block_len, batch, kNoLengths, dl, hp, mask_id, max_window, sel_mask, sel_idx, sel_count, s);
 }
 
 // ---- commit (Eq. 2): y_i <- yhat_i for the selected positions; masked positions left in the block --
