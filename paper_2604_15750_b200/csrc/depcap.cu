@@ -614,7 +614,7 @@ int dc_create(const dc_config* cfg, const dc_weights* w, void* cuda_stream, dc_c
     c->act = ws_alloc<char>(c, M * g.d_ff * es, &ok);
     if (hd % 32) c->tmp = ws_alloc<float>(c, M * (nq + 2 * nkv) * hd, &ok);
   }
-  if ((!c->use_tc || !c->tc_lm) && !simt_init(c->bf16, hd)) {
+  if ((!c->use_tc || !c->tc_lm) && !simt_init(c->bf16, g.n_layers > 0 ? hd : 0)) {
     dc_destroy(c);
     return fail(nullptr, DC_ERR_UNSUPPORTED, "head_dim %d needs more shared memory than the CUDA-core kernels have", hd);
   }

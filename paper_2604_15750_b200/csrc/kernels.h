@@ -118,7 +118,8 @@ void launch_attn_simt(const T* q, const T* k, const T* v, const T* k_cache, cons
                       int max_ctx, const SeqMeta& m, int nq, int nkv, int hd, T* o,
                       cudaStream_t s);
 
-// once per context: shared-memory opt-in of the CUDA-core kernels on the current device
+// once per context: shared-memory opt-in of the CUDA-core kernels on the current device; false when the attention of
+// this head_dim (0: none) does not fit
 bool simt_init(bool bf16, int head_dim);
 
 struct SignalOut {

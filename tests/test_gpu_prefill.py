@@ -184,9 +184,11 @@ def test_prefill_into_caches_that_start_anywhere(n_ids, shift):
     eng.close()
 
 
-def test_prefill_of_a_model_without_layers():
-    """A context made for the decision calls alone: a prefill checks the ids, writes the status and nothing else."""
-    case = Case(inputs.scaled(TINY, ctx_min=0, ctx_max=0), n_layers=0)
+@pytest.mark.parametrize("head_dim", [TINY.head_dim, 40000])
+def test_prefill_of_a_model_without_layers(head_dim):
+    """A context made for the decision calls alone: a prefill checks the ids, writes the status and nothing else.  No
+    attention will run, so its heads may be of any size."""
+    case = Case(inputs.scaled(TINY, ctx_min=0, ctx_max=0, head_dim=head_dim), n_layers=0)
     eng = case.make_engine(max_last=16, max_ctx=64)
     dev = eng.device
     cache = torch.full((64,), -7.0, device=dev)
