@@ -18,7 +18,8 @@
 // lies too far above m0: then one more pass finds the rows' maxima and a third uses them.
 //
 // Warp roles (256 threads): warp 0 = TMA producer (Q, then K and V^T tiles in turn through one ring), warp
-// 1 = TMEM owner + issuer of S^T, warp 2 = issuer of O^T, warps 4..7 = softmax and output.
+// 1 = TMEM owner + issuer of S^T, warp 2 = issuer of O^T, warp 3 = clears V^T beyond the valid keys, warps 4..7 =
+// softmax and output.
 #pragma once
 #include "tc_attn.cuh"
 
@@ -106,7 +107,7 @@ k_attn_few(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CU
     for (int i = 0; i < slots; ++i) ptx::mbar_init(&c.empty[i], 1);
     for (int i = 0; i < 3; ++i) { ptx::mbar_init(&c.k_full[i], 1); ptx::mbar_init(&c.v_full[i], 1); }
     for (int i = 0; i < 2; ++i) { ptx::mbar_init(&c.s_full[i], 1); ptx::mbar_init(&c.s_empty[i], 4); }
-    ptx::mbar_init(&c.p_full, 4);
+    ptx::mbar_init(&c.p_full, 5);   // the softmax warps, and warp 3
     ptx::mbar_init(&c.p_empty, 1);
     ptx::fence_barrier_init();
   }
@@ -197,6 +198,21 @@ k_attn_few(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CU
         }
         __syncwarp();
       }
+    } else if (warp == 3) {
+      // ---------------- V^T columns beyond the valid keys: cleared while the softmax warps make P ----------------
+      for (int j = 0; j < T; ++j) {
+        const int J = J0 + j, nvalid = min(kBK, j < Tc ? P - j * kBK : R - (j - Tc) * kBK);
+        if (nvalid & 15) {
+          if (!__all_sync(0xffffffffu, ptx::mbar_wait(&c.v_full[J % 3], (uint32_t)(J / 3) & 1u, abort_flag))) break;
+#pragma unroll
+          for (int rr = lane; rr < 128; rr += 32) attn_clear_v(ring + (size_t)((2 * J + 1) % slots) * kFewSlot, rr, nvalid);
+          ptx::fence_proxy_async_smem();
+          __syncwarp();
+        }
+        if (lane == 0) ptx::mbar_arrive(&c.p_full);
+        // (not ahead of the tile: its next arrival belongs to the next phase)
+        if (!__all_sync(0xffffffffu, ptx::mbar_wait(&c.p_full, (uint32_t)J & 1u, abort_flag))) break;
+      }
     } else if (warp >= 4) {
       // ---------------- softmax: one thread per key of the tile ----------------
       const int quarter = warp & 3, key = quarter * 32 + lane;
@@ -260,12 +276,6 @@ k_attn_few(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CU
         for (int i = 0; i < 32; ++i)
           asm volatile("st.shared.b16 [%0], %1;" ::"r"(p_addr[i & 7] + (uint32_t)(i >> 3) * 1024u),
                        "h"(__bfloat16_as_ushort(__float2bfloat16_rn(v[i]))) : "memory");
-        if (nvalid & 15) {   // V^T columns beyond the valid keys are cleared, a row of the tile per thread
-          const int s = (2 * J + 1) % slots;
-          ok = __all_sync(0xffffffffu, ptx::mbar_wait(&c.v_full[J % 3], (uint32_t)(J / 3) & 1u, abort_flag));
-          if (!ok) break;
-          attn_clear_v(ring + (size_t)s * kFewSlot, key, nvalid);
-        }
         ptx::fence_proxy_async_smem();
         __syncwarp();
         if (lane == 0) ptx::mbar_arrive(&c.p_full);
