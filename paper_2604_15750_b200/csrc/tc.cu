@@ -65,15 +65,29 @@ bool make_map_3d(CUtensorMap* m, const void* base, uint64_t n0, uint64_t n1, uin
              CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// The q / k / v weight rows [heads * 128, K] as {K, 16 rows, 4 groups, 2 halves of every head}: a box brings rows
+// 16 q .. + 15 of both halves of a head, one TMEM lane quarter of a tile (head_feature)
+bool make_map_heads(CUtensorMap* m, const void* base, uint64_t heads, uint64_t K) {
+  EncodeTiledFn enc = get_encode();
+  if (!enc) return false;
+  cuuint64_t dims[4] = {K, 16, 4, 2 * heads};
+  cuuint64_t strides[3] = {K * 2, 16 * K * 2, 64 * K * 2};
+  cuuint32_t box[4] = {64, 16, 1, 2};
+  cuuint32_t estr[4] = {1, 1, 1, 1};
+  return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, box,
+             estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 constexpr int kSmemBudget = 232448 - 1024;  // opt-in shared memory per CTA, minus alignment slack
-constexpr int kStaticQkv = 128 * 33 * 4 + 512;  // static shared memory of the kernels (upper bounds)
-constexpr int kStaticOther = 512;
+constexpr int kGemmStatic = 512;            // static shared memory of k_gemm_tc (upper bound)
 
 }  // namespace
 
 struct LayerMaps {
   CUtensorMap wq, wk, wv, wo, w_gate, w_up, w_down;
   CUtensorMap w_gate_c, w_up_c;   // gate / up with the dense chain's lower tiles (gate_up_rows)
+  CUtensorMap wq_h, wk_h, wv_h;   // q / k / v in the row order of make_map_heads
 };
 
 struct ActMaps {
@@ -143,12 +157,6 @@ T* talloc(TcState* t, size_t n, bool* ok) {
   return reinterpret_cast<T*>(p);
 }
 
-int pick_bn(int M) {
-  const int nblk = (M + 255) / 256;
-  const int step = nblk > 1 ? 32 : 16;   // several blocks: what the MMAs of CTA pairs take
-  return ((M + nblk - 1) / nblk + step - 1) / step * step;
-}
-
 }  // namespace
 
 // Weight rows per gate / up tile of the dense chain.  Up to 128 activation rows as many tiles as the grid has
@@ -192,7 +200,9 @@ int tc_create(const dc_config& g, cudaStream_t s, int M_max, int Mlm_max,
     bool ok = make_map_2d(&L.wq, wq[l], hq, d, 128) && make_map_2d(&L.wk, wk[l], hkv, d, 128) &&
               make_map_2d(&L.wv, wv[l], hkv, d, 128) && make_map_2d(&L.wo, wo[l], d, hq, 128) &&
               make_map_2d(&L.w_gate, w_gate[l], F, d, 128) &&
-              make_map_2d(&L.w_up, w_up[l], F, d, 128) && make_map_2d(&L.w_down, w_down[l], d, F, 128);
+              make_map_2d(&L.w_up, w_up[l], F, d, 128) && make_map_2d(&L.w_down, w_down[l], d, F, 128) &&
+              make_map_heads(&L.wq_h, wq[l], g.n_q_heads, d) && make_map_heads(&L.wk_h, wk[l], g.n_kv_heads, d) &&
+              make_map_heads(&L.wv_h, wv[l], g.n_kv_heads, d);
     if (!ok) return tfail(t, DC_ERR_CUDA, "tensor map encoding failed for layer %d (weights must be 16-byte aligned)", l);
   }
   bool ok = true;
@@ -243,28 +253,14 @@ int tc_create(const dc_config& g, cudaStream_t s, int M_max, int Mlm_max,
     cudaGetLastError();
     return tfail(t, DC_ERR_CUDA, "cannot opt in to %d bytes of shared memory", few_smem(kFewSlotsMax));
   }
-  cudaError_t e1 = cudaFuncSetAttribute(k_gemm_tc<GEMM_EPI_QKV, false>,
-                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        kSmemBudget + 1024 - kStaticQkv);
-  cudaError_t e2 = cudaFuncSetAttribute(k_gemm_tc<GEMM_EPI_PARTIAL, false>,
-                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        kSmemBudget + 1024 - kStaticOther);
-  cudaError_t e3 = cudaFuncSetAttribute(k_gemm_tc<GEMM_EPI_SWIGLU, false>,
-                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        kSmemBudget + 1024 - kStaticOther);
-  if (e1 == cudaSuccess) e1 = cudaFuncSetAttribute(k_gemm_tc<GEMM_EPI_QKV, true>,
-                                                   cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   kSmemBudget + 1024 - kStaticQkv);
-  if (e2 == cudaSuccess) e2 = cudaFuncSetAttribute(k_gemm_tc<GEMM_EPI_PARTIAL, true>,
-                                                   cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   kSmemBudget + 1024 - kStaticOther);
-  if (e3 == cudaSuccess) e3 = cudaFuncSetAttribute(k_gemm_tc<GEMM_EPI_SWIGLU, true>,
-                                                   cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   kSmemBudget + 1024 - kStaticOther);
-  if (e1 != cudaSuccess || e2 != cudaSuccess || e3 != cudaSuccess) {
-    cudaGetLastError();
-    return tfail(t, DC_ERR_CUDA, "cannot opt in to %d bytes of shared memory", kSmemBudget);
-  }
+  const void* gemms[6] = {(const void*)k_gemm_tc<GEMM_EPI_QKV, false>,     (const void*)k_gemm_tc<GEMM_EPI_QKV, true>,
+                          (const void*)k_gemm_tc<GEMM_EPI_PARTIAL, false>, (const void*)k_gemm_tc<GEMM_EPI_PARTIAL, true>,
+                          (const void*)k_gemm_tc<GEMM_EPI_SWIGLU, false>,  (const void*)k_gemm_tc<GEMM_EPI_SWIGLU, true>};
+  for (const void* fn : gemms)
+    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget + 1024 - kGemmStatic) != cudaSuccess) {
+      cudaGetLastError();
+      return tfail(t, DC_ERR_CUDA, "cannot opt in to %d bytes of shared memory", kSmemBudget);
+    }
   // the persistent dense chain needs every CTA resident at once (cooperative launch)
   {
     t->grid_bar = talloc<unsigned int>(t, 2 + kFlagWords, &ok);
@@ -320,32 +316,35 @@ static int get_act_maps(TcState* t, const __nv_bfloat16* a, int BN, ActMaps** ou
   return DC_OK;
 }
 
-// ma: activation map with a box of BN rows; ma_half: with BN / 2 rows (CTA pairs), or null
+// CTA pairs (each CTA stages half of the activation block): two adjacent weight tiles of the call
+static bool gemm_pair(const TcState* t, int tiles) { return tiles % 2 == 0 && t->n_sm >= 2; }
+
+// How a GEMM of the per-op path is cut: activation rows per column block, K splits.
+struct GemmCut { int BN, nsplit; };
+
+enum { ACT_A = 0, ACT_O = 1, ACT_MLP = 2 };
+
 template <int EPI>
-static int launch_gemm(TcState* t, const CUtensorMap& w0, const CUtensorMap& w1,
-                       const CUtensorMap& w2, const CUtensorMap& ma, const CUtensorMap* ma_half,
-                       GemmParams p, int tiles, int static_smem) {
+static int launch_gemm(TcState* t, const CUtensorMap& w0, const CUtensorMap& w1, const CUtensorMap& w2,
+                       const __nv_bfloat16* a, int operand, GemmParams p, int tiles, GemmCut cut) {
   const int nw = (EPI == GEMM_EPI_SWIGLU) ? 2 : 1;
+  const bool pair = gemm_pair(t, tiles);
+  p.BN = cut.BN; p.nsplit = cut.nsplit; p.tiles = tiles; p.status = t->status;
+  const int a_rows = pair ? p.BN / 2 : p.BN;
+  ActMaps* am = nullptr;
+  const int rc = get_act_maps(t, a, a_rows, &am);
+  if (rc != DC_OK) return rc;
+  const CUtensorMap& ma = operand == ACT_A ? am->a : operand == ACT_O ? am->o : am->act;
   const int n_cblk = (p.M + p.BN - 1) / p.BN;
-  // CTA pairs (each CTA stages half of the activation block) when the shapes allow it and there
-  // is more than one column block: below that the fused chain is the path that matters
-  const bool pair = ma_half != nullptr && tiles % 2 == 0 && p.BN % 32 == 0 &&
-                    p.BN >= 64 && n_cblk > 1 && t->n_sm >= 2;
-  const int sb = gemm_stage_bytes(nw, pair ? p.BN / 2 : p.BN);
-  int stages = (kSmemBudget - static_smem) / sb;
+  const int sb = gemm_stage_bytes(nw, a_rows);
+  int stages = (kSmemBudget - kGemmStatic) / sb;
   if (stages > 8) stages = 8;
   if (stages < 2) return tfail(t, DC_ERR_UNSUPPORTED, "activation block too large for the smem ring");
   const size_t smem = (size_t)stages * sb + 1024;
-  // persistent: one CTA (pair) per SM (pair) works through the units; with more units than
-  // workers the accumulators of consecutive units alternate between two TMEM sets
+  // persistent: one CTA (pair) per SM (pair) works through the units
   const int n_units = (pair ? tiles / 2 : tiles) * n_cblk * p.nsplit;
   const int workers_max = pair ? t->n_sm / 2 : t->n_sm;
   const int workers = n_units < workers_max ? n_units : workers_max;
-  p.tiles = tiles;
-  // gate / up keep both TMEM sets for one unit (column blocks of 256 rows: with 128-row blocks
-  // every weight tile is pulled from L2 twice as often, which cost more than the overlap gained)
-  p.pingpong = (n_units > workers && nw == 1) ? 1 : 0;
-  p.status = t->status;
   cudaError_t e;
   if (pair) {
     cudaLaunchConfig_t cfg{};
@@ -357,7 +356,7 @@ static int launch_gemm(TcState* t, const CUtensorMap& w0, const CUtensorMap& w1,
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr; cfg.numAttrs = 2;
-    e = cudaLaunchKernelEx(&cfg, k_gemm_tc<EPI, true>, w0, w1, w2, *ma_half, p, stages);
+    e = cudaLaunchKernelEx(&cfg, k_gemm_tc<EPI, true>, w0, w1, w2, ma, p, stages);
   } else {
     e = launch_chained(k_gemm_tc<EPI, false>, workers, kGemmThreads, smem, t->s, w0, w1, w2, ma, p, stages);
   }
@@ -375,24 +374,28 @@ static int pick_split(int tiles, int KB, int max_split) {
   return s;
 }
 
-// K splits of a split-K projection on the per-op path.  With few units (one column block) the
-// splits fill the SMs (pick_split).  With many, units come in rounds over the workers (SMs, or SM
-// pairs) and the last round is partly empty - 160 pair-units on 74 pairs are 3 rounds for 2.16
-// rounds of work; splitting K makes the rounds finer at the price of one more fp32 partial array
-// written and read back per split.  Rough model: GEMM at 1 PFLOP/s, partials at 5 TB/s.
-static int pick_split_rounds(const TcState* t, int tiles, int M, int BN, int N, int K, int max_split) {
-  const int n_cblk = (M + BN - 1) / BN;
-  if (n_cblk <= 1) return pick_split(tiles * n_cblk, K / kTileK, max_split);
-  const bool pair = tiles % 2 == 0 && BN % 32 == 0 && BN >= 64 && t->n_sm >= 2;
-  const int units = (pair ? tiles / 2 : tiles) * n_cblk, workers = pair ? t->n_sm / 2 : t->n_sm;
-  const double t1 = 2.0 * M * N * K / 1e15, work_rounds = (double)units / workers;
-  const double per_split = 2.0 * M * N * 4.0 / 5e12;
-  int best = 1;
+// Units (weight tile, column block, K split) come in rounds over the workers (SMs, or SM pairs), and the last round
+// is partly empty: 96 pair-units on 74 pairs are 2 rounds for 1.3 rounds of work.  Narrower column blocks and K splits
+// make the units finer, at the price of activation traffic and of one more fp32 partial array per split.  The
+// model: a k-block takes what its MMAs do (2 BN clocks a weight tile at 1.9 GHz), what an SM takes in from L2 (108 GB/s)
+// or the issue and ring latencies (200 ns), whichever is longest; gate / up pay for draining their accumulators.
+static GemmCut cut_gemm(const TcState* t, int tiles, int nw, int M, int K, int N, int max_split) {
+  const bool pair = gemm_pair(t, tiles);
+  const int workers = pair ? t->n_sm / 2 : t->n_sm, tp = pair ? tiles / 2 : tiles, KB = K / kTileK;
+  const int blk0 = (M + 255) / 256;
+  GemmCut best{256, 1};
   double best_t = 1e30;
-  for (int s = 1; s <= max_split && (K / kTileK) / s >= 8; ++s) {
-    const double rounds = (double)((units * s + workers - 1) / workers) / s;
-    const double est = t1 * rounds / work_rounds + (s - 1) * per_split;
-    if (est < best_t - 1e-9) { best_t = est; best = s; }
+  for (int nb = blk0; nb <= blk0 + 3; ++nb) {
+    const int BN = ((M + nb - 1) / nb + 15) / 16 * 16, n_cblk = (M + BN - 1) / BN;
+    const double mma = nw * 2.0 * BN / 1.9, in = (nw * 16384.0 + (pair ? BN / 2 : BN) * 128.0) / 108.0;
+    const double t_kb = mma > in ? (mma > 200.0 ? mma : 200.0) : (in > 200.0 ? in : 200.0);
+    for (int s = 1; s <= max_split && (s == 1 || KB / s >= 8); ++s) {
+      const int units = tp * n_cblk * s;
+      const double rounds = (units + workers - 1) / workers;
+      const double est = rounds * ((KB + s - 1) / s * t_kb + (nw == 2 ? 1000.0 + 10.0 * BN : 300.0)) +
+                         (max_split > 1 ? (s - 1) * 2.0 * M * N * 4.0 / 5e3 : 0.0);
+      if (est < best_t * 0.995) { best_t = est; best = GemmCut{BN, s}; }
+    }
   }
   return best;
 }
@@ -587,19 +590,9 @@ int tc_layer(TcState* t, int layer, const SeqMeta& m, float* x, const __nv_bfloa
   const dc_config& g = t->g;
   const int d = g.d_model, nq = g.n_q_heads, nkv = g.n_kv_heads, hd = g.head_dim, F = g.d_ff;
   const int M = m.nv * m.rows;
-  const int BN = pick_bn(M);
-  ActMaps *am = nullptr, *amh = nullptr;
-  int rc = get_act_maps(t, a, BN, &am);
-  if (rc != DC_OK) return rc;
-  if (BN % 32 == 0 && BN >= 64 && M > BN) {
-    rc = get_act_maps(t, a, BN / 2, &amh);
-    if (rc != DC_OK) return rc;
-    rc = get_act_maps(t, a, BN, &am);   // (the cache may have been rebuilt)
-    if (rc != DC_OK) return rc;
-  }
   const LayerMaps& L = t->layers[layer];
   GemmParams p{};
-  p.M = M; p.BN = BN; p.nq = nq; p.nkv = nkv; p.hd = hd;
+  p.M = M; p.nq = nq; p.nkv = nkv;
   p.cos_sin = cos_sin; p.rows_per_variant = m.rows;
   p.q = t->q; p.k = t->k; p.v = t->v; p.ldv = t->ldv; p.act = t->act;
   if (!t->bq.empty()) {
@@ -608,8 +601,9 @@ int tc_layer(TcState* t, int layer, const SeqMeta& m, float* x, const __nv_bfloa
   p.part = t->part; p.part_stride = t->part_stride;
 
   hook.begin(DC_STAGE_QKV, 1);
-  p.N = (nq + 2 * nkv) * hd; p.K = d; p.nsplit = 1;
-  rc = launch_gemm<GEMM_EPI_QKV>(t, L.wq, L.wk, L.wv, am->a, amh ? &amh->a : nullptr, p, nq + 2 * nkv, kStaticQkv);
+  p.N = (nq + 2 * nkv) * hd; p.K = d;
+  int rc = launch_gemm<GEMM_EPI_QKV>(t, L.wq_h, L.wk_h, L.wv_h, a, ACT_A, p, nq + 2 * nkv,
+                                     cut_gemm(t, nq + 2 * nkv, 1, M, p.K, p.N, 1));
   hook.end();
   if (rc != DC_OK) return rc;
 
@@ -619,29 +613,32 @@ int tc_layer(TcState* t, int layer, const SeqMeta& m, float* x, const __nv_bfloa
   if (rc != DC_OK || kv_only) return rc;   // prefill, last layer: only its K / V were wanted
 
   hook.begin(DC_STAGE_OPROJ, 1);
-  p.N = d; p.K = nq * hd; p.nsplit = pick_split_rounds(t, d / kTileN, M, BN, p.N, p.K, t->max_split);
-  rc = launch_gemm<GEMM_EPI_PARTIAL>(t, L.wo, L.wo, L.wo, am->o, amh ? &amh->o : nullptr, p, d / kTileN, kStaticOther);
+  p.N = d; p.K = nq * hd;
+  const GemmCut cut_o = cut_gemm(t, d / kTileN, 1, M, p.K, p.N, t->max_split);
+  rc = launch_gemm<GEMM_EPI_PARTIAL>(t, L.wo, L.wo, L.wo, a, ACT_O, p, d / kTileN, cut_o);
   hook.end();
   if (rc != DC_OK) return rc;
 
   hook.begin(DC_STAGE_NORM, 1);
-  launch_rmsnorm<__nv_bfloat16>(x, t->part, p.nsplit, t->part_stride, norm2, g.rms_eps, M, d,
+  launch_rmsnorm<__nv_bfloat16>(x, t->part, cut_o.nsplit, t->part_stride, norm2, g.rms_eps, M, d,
                                 const_cast<__nv_bfloat16*>(a), t->s);
   hook.end();
 
   hook.begin(DC_STAGE_GATEUP, 1);
-  p.N = F; p.K = d; p.nsplit = 1;
-  rc = launch_gemm<GEMM_EPI_SWIGLU>(t, L.w_gate, L.w_up, L.w_up, am->a, amh ? &amh->a : nullptr, p, F / kTileN, kStaticOther);
+  p.N = F; p.K = d;
+  rc = launch_gemm<GEMM_EPI_SWIGLU>(t, L.w_gate, L.w_up, L.w_up, a, ACT_A, p, F / kTileN,
+                                    cut_gemm(t, F / kTileN, 2, M, p.K, p.N, 1));
   hook.end();
   if (rc != DC_OK) return rc;
 
   hook.begin(DC_STAGE_DOWN, 1);
-  p.N = d; p.K = F; p.nsplit = pick_split_rounds(t, d / kTileN, M, BN, p.N, p.K, t->max_split);
-  rc = launch_gemm<GEMM_EPI_PARTIAL>(t, L.w_down, L.w_down, L.w_down, am->act, amh ? &amh->act : nullptr, p, d / kTileN, kStaticOther);
+  p.N = d; p.K = F;
+  const GemmCut cut_down = cut_gemm(t, d / kTileN, 1, M, p.K, p.N, t->max_split);
+  rc = launch_gemm<GEMM_EPI_PARTIAL>(t, L.w_down, L.w_down, L.w_down, a, ACT_MLP, p, d / kTileN, cut_down);
   hook.end();
   if (rc != DC_OK) return rc;
 
-  *part = t->part; *nsplit = p.nsplit; *part_stride = t->part_stride;
+  *part = t->part; *nsplit = cut_down.nsplit; *part_stride = t->part_stride;
   return DC_OK;
 }
 

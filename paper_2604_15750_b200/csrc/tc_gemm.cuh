@@ -2,26 +2,30 @@
 //
 // out[m, n] = sum_k A[m, k] * W[n, k]        A: activations [M, K], W: weights [N, K]
 //
-// The step has few activation rows (M = 2 * batch * rows, 192 for one sequence) and very many
-// weight rows, so the roles of the MMA operands are swapped: a CTA owns 128 weight rows (the MMA
-// "M" side, one TMEM lane per output feature) and a block of up to 256 activation rows (the MMA
-// "N" side, one TMEM column per row).  Every weight byte is read from HBM exactly once per
-// column block; the activation tile is re-read from L2.
+// The step has few activation rows and very many weight rows, so the roles of the MMA operands are
+// swapped: a CTA owns 128 weight rows (the MMA "M" side, one TMEM lane per output feature) and a block
+// of up to 256 activation rows (the MMA "N" side, one TMEM column per row).  Every weight byte is read
+// from HBM exactly once per column block; the activation tile is re-read from L2.
 //
-// Warp roles (192 threads): warp 0 = TMA producer, warp 1 = TMEM owner + MMA issuer,
-// warps 2..5 = epilogue (TMEM -> registers -> global).  Shared memory is a ring of kStages
-// slots, each {NW weight tiles 128 x 64, one activation tile BN x 64}, all in the 128-byte
-// swizzled K-major layout that both TMA and tcgen05.mma understand.
+// Warp roles (576 threads): warp 0 = TMA producer, warp 1 = TMEM owner + MMA issuer, warps 2..17 =
+// epilogue (TMEM -> registers -> global).  Shared memory is a ring of slots, each {NW weight tiles
+// 128 x 64, one activation tile BN x 64}, all in the 128-byte swizzled K-major layout that both TMA and
+// tcgen05.mma understand.
 //
 // A CTA works through the units (weight tile, column block, K split) blockIdx.x, + gridDim.x, ...
-// With more units than CTAs (`pingpong`) the accumulators of consecutive units alternate
-// between two TMEM sets, the producer and the MMA issuer run on into the next unit, and the
-// epilogue of a unit - which took 25..60% of a unit's time when every unit was a CTA of its own -
-// runs under the MMAs of the next.  A set is one accumulator of up to 256 columns (at N = 256 a
-// single chain of MMAs already runs at the tensor core's rate).  Without `pingpong` (one unit per
-// CTA, or gate / up, which need both sets for one unit) both sets serve a unit - even / odd
-// k-steps, because small N needs two independent chains, or gate / up - and a CTA's next unit
-// starts when the epilogue has drained them.
+// The single-matrix GEMMs keep one accumulator of up to 256 columns per unit and alternate between two
+// TMEM sets: the producer and the MMA issuer run on into the next unit and the epilogue of a unit runs
+// under its MMAs.  Gate / up need both sets for one unit; there a CTA's next unit starts when the
+// epilogue has drained them.
+//
+// What bounds it: an SM takes in 64 bytes a clock from L2, and a k-block of 256 columns needs 32 KB for 512 clocks
+// of MMAs, so the main loops run at 300..320 ns a k-block (108 GB/s an SM) where the MMAs alone would take 270; batches
+// of 2000 rows and more reach the power cap.  Device timestamps with 1024 rows of LLaDA-8B showed three other
+// things before: a lane in a branch of its own issued a k-block in 390 ns (the issuing warps now run their loops
+// together and elect a lane); the rotation through shared memory by four warps took 27 us a unit against 25 of
+// MMAs (shuffles take 3.5: the weight rows arrive in an order that puts the two features of a pair into one warp); gate /
+// up stood still for 11 us of every 51 while four warps drained the accumulators (sixteen take 3).  QKV 83 -> 71
+// us, gate / up 153 -> 133; the whole prefill 15.13 -> 14.01 ms, eight boundary steps 37.4 -> 34.2, 2 x 160 rows 22% less.
 #pragma once
 #include "kernels.h"
 #include "pdl.cuh"
@@ -42,10 +46,9 @@ struct GemmParams {
   int BN;         // activation rows per column block (multiple of 16, <= 256)
   int nsplit;     // split-K factor
   int tiles;      // weight tiles (over all matrices of the call)
-  int pingpong;   // more units than CTAs: one accumulator set per unit, sets alternate
   // QKV epilogue
-  int nq, nkv, hd;          // tiles [0,nq) are q heads, [nq,nq+nkv) k heads, rest v heads
-  const float* cos_sin;     // RoPE table [(b, r)][hd]
+  int nq, nkv;              // tiles [0,nq) are q heads, [nq,nq+nkv) k heads, rest v heads (head_dim 128)
+  const float* cos_sin;     // RoPE table [(b, r)][128]; row rows_per_variant: the angle step between rows
   int rows_per_variant;     // the table is shared by the variants
   const __nv_bfloat16 *bq, *bk, *bv;  // projection biases [nq*hd], [nkv*hd], [nkv*hd], or null
   __nv_bfloat16 *q, *k, *v; // outputs q [M, nq*hd], k [M, nkv*hd], v TRANSPOSED [nkv*hd, ldv]
@@ -58,18 +61,34 @@ struct GemmParams {
   int32_t* status;          // device status word(s); DC_ERR_TIMEOUT on an expired wait
 };
 
-constexpr int kGemmThreads = 192;
+constexpr int kGemmEpiWarps = 16;
+constexpr int kGemmParts = kGemmEpiWarps / 4;           // warps per TMEM lane quarter: they share its columns
+constexpr int kGemmThreads = 64 + 32 * kGemmEpiWarps;
 constexpr int kTileN = 128;  // weight rows per CTA tile
 constexpr int kTileK = 64;   // bf16 elements per k-block (one 128-byte swizzle row)
 
-__host__ __device__ inline int gemm_stage_bytes(int nw, int BN) {
-  return nw * kTileN * kTileK * 2 + BN * kTileK * 2;
+__host__ __device__ inline int gemm_stage_bytes(int nw, int a_rows) {
+  return nw * kTileN * kTileK * 2 + a_rows * kTileK * 2;
+}
+
+// Feature of a head (128 wide) in TMEM lane `lane` of quarter q: the weight rows of a q / k / v tile arrive as
+// {16 q .. + 15, 64 + 16 q .. + 15} per quarter, so that rotate-half's pair (i, i + 64) lies 16 lanes apart.
+__device__ __forceinline__ int head_feature(int quarter, int lane) { return ((lane >> 4) << 6) + 16 * quarter + (lane & 15); }
+
+// The 128 weight rows of head `head` in that order: four boxes of 2 x 16 rows.
+template <bool PAIR>
+__device__ __forceinline__ void load_head_tile(uint32_t slot, const CUtensorMap* map, uint32_t bar, int kc, int head) {
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    if (PAIR) ptx::tma_load_4d_pair_a(slot + q * (32 * kTileK * 2), map, bar, kc, 0, q, 2 * head);
+    else ptx::tma_load_4d_a(slot + q * (32 * kTileK * 2), map, bar, kc, 0, q, 2 * head);
+  }
 }
 
 // PAIR: the launch uses clusters of two CTAs and every MMA is a pair MMA (cta_group::2, M = 256):
 // the two CTAs own adjacent weight tiles and each stages only half of the activation block, so a
 // k-block is 16 KB of weights plus 16 KB of activations per CTA instead of 16 + 32 - the main
-// loops of these GEMMs are bound by what an SM takes in from L2.  The even CTA issues the MMAs;
+// loops of these GEMMs are close to what an SM takes in from L2.  The even CTA issues the MMAs;
 // TMA loads of both CTAs report to its full barrier, tcgen05.commit releases ring slots and
 // signals the accumulators in both; the odd CTA's epilogue warps report the drained accumulators
 // to the even CTA's barrier.  No load is multicast.
@@ -79,15 +98,16 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w0, const __grid_constant__ CU
           const __grid_constant__ CUtensorMap map_w2, const __grid_constant__ CUtensorMap map_a,
           const GemmParams p, const int stages) {
   constexpr int NW = (EPI == GEMM_EPI_SWIGLU) ? 2 : 1;
+  constexpr int NSETS = 2 / NW;          // accumulator sets that units alternate between
+  constexpr int W_BYTES = kTileN * kTileK * 2;
   extern __shared__ uint8_t smem_raw[];
   __shared__ uint64_t bar_full[8], bar_empty[8], acc_full[2], acc_empty[2];
   __shared__ uint32_t tmem_base_s;
-  __shared__ int abort_flag;
-  __shared__ float xch[(EPI == GEMM_EPI_QKV) ? 128 * 33 : 1];
+  __shared__ int abort_flag, late_flag;
 
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~static_cast<uintptr_t>(1023));
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
   // Column blocks of one weight tile sit next to each other in the unit order, so that the
   // CTAs that share a weight tile run together and all but one read it from L2.
   const int n_cblk = (p.M + p.BN - 1) / p.BN;
@@ -99,11 +119,9 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w0, const __grid_constant__ CU
   const int n_units = per_split * p.nsplit;
   const int stage_bytes = gemm_stage_bytes(NW, a_rows);
   const int KB = p.K / kTileK;
-  const bool pp = p.pingpong != 0;
-  const uint32_t up_off = pp ? 128u : 256u;   // second accumulator of a set (gate / up), or the odd k-steps' one
-  const uint32_t tmem_cols = 512u;
+  constexpr uint32_t tmem_cols = 512u;
 
-  struct Unit { int tile, cblk, split, kb0, nkb, wrow; const CUtensorMap* map_w; };
+  struct Unit { int tile, cblk, split, kb0, nkb; };
   auto unit_of = [&](int u) {
     Unit w;
     w.split = u / per_split;
@@ -113,20 +131,13 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w0, const __grid_constant__ CU
     if (PAIR) w.tile = 2 * w.tile + (int)rank;
     w.kb0 = (int)(((long long)w.split * KB) / p.nsplit);
     w.nkb = (int)(((long long)(w.split + 1) * KB) / p.nsplit) - w.kb0;
-    // which weight matrix and which row of it this tile starts at
-    w.map_w = &map_w0;
-    w.wrow = w.tile * kTileN;
-    if (EPI == GEMM_EPI_QKV) {
-      if (w.tile >= p.nq + p.nkv) { w.map_w = &map_w2; w.wrow = (w.tile - p.nq - p.nkv) * kTileN; }
-      else if (w.tile >= p.nq) { w.map_w = &map_w1; w.wrow = (w.tile - p.nq) * kTileN; }
-    }
     return w;
   };
 
   if (threadIdx.x == 0) {
-    abort_flag = 0;
+    abort_flag = 0; late_flag = 0;
     for (int i = 0; i < stages; ++i) { ptx::mbar_init(&bar_full[i], 1); ptx::mbar_init(&bar_empty[i], 1); }
-    for (int i = 0; i < 2; ++i) { ptx::mbar_init(&acc_full[i], 1); ptx::mbar_init(&acc_empty[i], PAIR ? 256 : 128); }
+    for (int i = 0; i < 2; ++i) { ptx::mbar_init(&acc_full[i], 1); ptx::mbar_init(&acc_empty[i], (PAIR ? 2 : 1) * kGemmEpiWarps); }
     ptx::fence_barrier_init();
     ptx::prefetch_tmap(&map_w0);
     ptx::prefetch_tmap(&map_a);
@@ -149,263 +160,222 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w0, const __grid_constant__ CU
     ptx::cluster_sync();
   }
 
-  pdl_wait();   // everything below reads or writes what other kernels of the step share
-  // One thread issues every TMA load and one every MMA, so their own instruction streams are on
-  // the critical path: slot indices, addresses and descriptors advance by additions only.
+  const uint32_t full0 = ptx::smem_u32(&bar_full[0]), empty0 = ptx::smem_u32(&bar_empty[0]);
+  uint32_t fills = 0;   // of the producer: ring slots filled so far
   if (warp == 0) {
     // ---------------- TMA producer ----------------
-    if (lane == 0) {
-      const uint32_t ring0 = ptx::smem_u32(smem);
-      const uint32_t full0 = ptx::smem_u32(&bar_full[0]), empty0 = ptx::smem_u32(&bar_empty[0]);
-      uint32_t s = 0, ph = 0, slot = ring0;
-      bool ok = true;
-      const uint32_t full_r0 = (PAIR && rank != 0) ? ptx::mapa_shared(full0, 0) : full0;   // the even CTA's
-      for (int u = cta; u < n_units && ok; u += n_cta) {
-        const Unit w = unit_of(u);
-        const int arow = w.cblk * p.BN + (int)rank * a_rows;
-        for (int i = 0; i < w.nkb; ++i) {
-          if (!ptx::mbar_wait_a(empty0 + 8u * s, ph ^ 1u, &abort_flag)) { ok = false; break; }
+    // (the whole warp runs the loop and one elected lane issues, as in the MMA issuer)
+    const bool el = ptx::elect_one();
+    const uint32_t ring0 = ptx::smem_u32(smem);
+    const uint32_t full_r0 = (PAIR && rank != 0) ? ptx::mapa_shared(full0, 0) : full0;   // the even CTA's
+    // the weight tile(s) of one k-block, and the bytes that the slot's barrier waits for
+    auto load_w = [&](const Unit& w, int i, uint32_t s, uint32_t slot) {
+      const int kc = (w.kb0 + i) * kTileK;
+      if (rank == 0) ptx::mbar_expect_tx_a(full0 + 8u * s, (PAIR ? 2u : 1u) * (uint32_t)stage_bytes);
+      const uint32_t bar = full_r0 + 8u * s;
+      if (EPI == GEMM_EPI_QKV) {
+        const bool is_v = w.tile >= p.nq + p.nkv, is_q = w.tile < p.nq;
+        load_head_tile<PAIR>(slot, is_q ? &map_w0 : is_v ? &map_w2 : &map_w1, bar, kc,
+                             w.tile - (is_q ? 0 : is_v ? p.nq + p.nkv : p.nq));
+      } else if (PAIR) {
+        ptx::tma_load_2d_pair_a(slot, &map_w0, bar, kc, w.tile * kTileN);
+        if (NW == 2) ptx::tma_load_2d_pair_a(slot + W_BYTES, &map_w1, bar, kc, w.tile * kTileN);
+      } else {
+        ptx::tma_load_2d_a(slot, &map_w0, bar, kc, w.tile * kTileN);
+        if (NW == 2) ptx::tma_load_2d_a(slot + W_BYTES, &map_w1, bar, kc, w.tile * kTileN);
+      }
+    };
+    // The weights of the first slots do not wait for the kernel before this one (nothing in a step writes
+    // them, and the step's first launch has waited for all that was in the stream).
+    int early = 0;
+    if (cta < n_units) {
+      const Unit w = unit_of(cta);
+      early = w.nkb < stages ? w.nkb : stages;
+      for (int i = 0; i < early; ++i)
+        if (el) load_w(w, i, (uint32_t)i, ring0 + (uint32_t)(i * stage_bytes));
+    }
+    pdl_wait();
+    uint32_t s = 0, ph = 0, slot = ring0;
+    bool ok = true;
+    for (int u = cta; u < n_units && ok; u += n_cta) {
+      const Unit w = unit_of(u);
+      const int arow = w.cblk * p.BN + (int)rank * a_rows;
+      for (int i = 0; i < w.nkb; ++i) {
+        const bool have_w = early > 0;
+        if (have_w) --early;
+        else ok = __all_sync(0xffffffffu, ptx::mbar_wait_a(empty0 + 8u * s, ph ^ 1u, &abort_flag));
+        if (!ok) break;
+        if (el) {
+          if (!have_w) load_w(w, i, s, slot);
+          const uint32_t bar = full_r0 + 8u * s;
           const int kc = (w.kb0 + i) * kTileK;
-          if (PAIR) {
-            if (rank == 0) ptx::mbar_expect_tx_a(full0 + 8u * s, 2u * (uint32_t)stage_bytes);
-            const uint32_t bar = full_r0 + 8u * s;
-            ptx::tma_load_2d_pair_a(slot, w.map_w, bar, kc, w.wrow);
-            if (NW == 2) ptx::tma_load_2d_pair_a(slot + kTileN * kTileK * 2, &map_w1, bar, kc, w.wrow);
-            ptx::tma_load_2d_pair_a(slot + NW * kTileN * kTileK * 2, &map_a, bar, kc, arow);
-          } else {
-            ptx::mbar_expect_tx_a(full0 + 8u * s, (uint32_t)stage_bytes);
-            ptx::tma_load_2d_a(slot, w.map_w, full0 + 8u * s, kc, w.wrow);
-            if (NW == 2) ptx::tma_load_2d_a(slot + kTileN * kTileK * 2, &map_w1, full0 + 8u * s, kc, w.wrow);
-            ptx::tma_load_2d_a(slot + NW * kTileN * kTileK * 2, &map_a, full0 + 8u * s, kc, arow);
-          }
-          if (++s == (uint32_t)stages) { s = 0; ph ^= 1u; slot = ring0; } else slot += (uint32_t)stage_bytes;
+          if (PAIR) ptx::tma_load_2d_pair_a(slot + NW * W_BYTES, &map_a, bar, kc, arow);
+          else ptx::tma_load_2d_a(slot + NW * W_BYTES, &map_a, bar, kc, arow);
         }
+        ++fills;
+        if (++s == (uint32_t)stages) { s = 0; ph ^= 1u; slot = ring0; } else slot += (uint32_t)stage_bytes;
       }
     }
   } else if (warp == 1) {
     // ---------------- MMA issuer ----------------
-    if (lane == 0 && rank == 0) {
+    // The whole warp runs the loop and one elected lane issues: the operands then stay in uniform registers (a
+    // k-block of 4 MMAs of 256 columns: 740 clocks in a branch of a single lane, 512 are the tensor core's own).
+    if (rank == 0) {
+      const bool el = ptx::elect_one();
       const uint32_t idesc = ptx::idesc_bf16(PAIR ? 2 * kTileN : kTileN, p.BN);
-      const uint32_t ring0 = ptx::smem_u32(smem);
-      const uint32_t full0 = ptx::smem_u32(&bar_full[0]), empty0 = ptx::smem_u32(&bar_empty[0]);
-      const uint64_t hi = ptx::smem_desc_sw128_hi();
-      uint32_t s = 0, ph = 0, slot = ring0;
+      const uint32_t hi = ptx::smem_desc_hi32(), lo0 = ptx::smem_desc_lo(ptx::smem_u32(smem)), step = (uint32_t)stage_bytes >> 4;
+      uint32_t s = 0, ph = 0, lo = lo0;
       bool ok = true;
       int j = 0;   // units of this CTA so far
       for (int u = cta; u < n_units && ok; u += n_cta, ++j) {
         const Unit w = unit_of(u);
-        const uint32_t set = pp ? (uint32_t)(j & 1) : 0u;
+        const uint32_t set = (uint32_t)(j % NSETS);
         // the epilogue has drained this set (its use before the last one)
-        if (j >= (pp ? 2 : 1)) {
-          const uint32_t uses = pp ? (uint32_t)(j >> 1) : (uint32_t)j;   // completed uses of the set
-          if (!ptx::mbar_wait(&acc_empty[set], (uses - 1) & 1u, &abort_flag)) { ok = false; break; }
-        }
+        if (j >= NSETS) ok = __all_sync(0xffffffffu, ptx::mbar_wait(&acc_empty[set], (uint32_t)(j / NSETS - 1) & 1u, &abort_flag));
+        if (!ok) break;
         ptx::tc_fence_after();
-        const uint32_t acc0 = tmem_base + set * 256u, acc1 = acc0 + up_off;
-        uint32_t acc_first = 0;
+        const uint32_t acc = tmem_base + set * 256u;
         for (int i = 0; i < w.nkb; ++i) {
-          if (!ptx::mbar_wait_a(full0 + 8u * s, ph, &abort_flag)) { ok = false; break; }
-          const uint64_t dw0 = hi | (uint64_t)(slot >> 4);
-          const uint64_t dw1 = dw0 + (kTileN * kTileK * 2 >> 4);
-          const uint64_t da = dw0 + (NW * kTileN * kTileK * 2 >> 4);
-          if (PAIR) {
-            if (NW == 2) {
-              ptx::umma_bf16_pair(acc0, dw0, da, idesc, acc_first);
-              ptx::umma_bf16_pair(acc1, dw1, da, idesc, acc_first);
+          ok = __all_sync(0xffffffffu, ptx::mbar_wait_a(full0 + 8u * s, ph, &abort_flag));
+          if (!ok) break;
+          const uint32_t more = i > 0 ? 1u : 0u;   // the first MMA of an accumulator overwrites it
+          if (el) {
+            const uint32_t da = lo + (NW * W_BYTES >> 4);
 #pragma unroll
-              for (int kk = 1; kk < kTileK / 16; ++kk) {
-                ptx::umma_bf16_pair_acc(acc0, dw0 + 2 * kk, da + 2 * kk, idesc);
-                ptx::umma_bf16_pair_acc(acc1, dw1 + 2 * kk, da + 2 * kk, idesc);
+            for (int kk = 0; kk < kTileK / 16; ++kk) {
+              const uint32_t on = kk > 0 ? 1u : more;
+              if (PAIR) {
+                ptx::umma_bf16_pair_lo(acc, lo + 2 * kk, da + 2 * kk, hi, idesc, on);
+                if (NW == 2) ptx::umma_bf16_pair_lo(acc + 256u, lo + (W_BYTES >> 4) + 2 * kk, da + 2 * kk, hi, idesc, on);
+              } else {
+                ptx::umma_bf16_lo(acc, lo + 2 * kk, da + 2 * kk, hi, idesc, on);
+                if (NW == 2) ptx::umma_bf16_lo(acc + 256u, lo + (W_BYTES >> 4) + 2 * kk, da + 2 * kk, hi, idesc, on);
               }
-            } else if (pp) {
-              ptx::umma_bf16_pair(acc0, dw0, da, idesc, acc_first);
-              ptx::umma_bf16_pair_acc(acc0, dw0 + 2, da + 2, idesc);
-              ptx::umma_bf16_pair_acc(acc0, dw0 + 4, da + 4, idesc);
-              ptx::umma_bf16_pair_acc(acc0, dw0 + 6, da + 6, idesc);
-            } else {
-              ptx::umma_bf16_pair(acc0, dw0, da, idesc, acc_first);
-              ptx::umma_bf16_pair(acc1, dw0 + 2, da + 2, idesc, acc_first);
-              ptx::umma_bf16_pair_acc(acc0, dw0 + 4, da + 4, idesc);
-              ptx::umma_bf16_pair_acc(acc1, dw0 + 6, da + 6, idesc);
             }
-            acc_first = 1;
-            ptx::umma_commit_pair_a(empty0 + 8u * s);   // frees the slot in both CTAs
-          } else {
-          if (NW == 2) {
-            ptx::umma_bf16(acc0, dw0, da, idesc, acc_first);
-            ptx::umma_bf16(acc1, dw1, da, idesc, acc_first);
-#pragma unroll
-            for (int kk = 1; kk < kTileK / 16; ++kk) {
-              ptx::umma_bf16_acc(acc0, dw0 + 2 * kk, da + 2 * kk, idesc);
-              ptx::umma_bf16_acc(acc1, dw1 + 2 * kk, da + 2 * kk, idesc);
-            }
-          } else if (pp) {
-            ptx::umma_bf16(acc0, dw0, da, idesc, acc_first);
-            ptx::umma_bf16_acc(acc0, dw0 + 2, da + 2, idesc);
-            ptx::umma_bf16_acc(acc0, dw0 + 4, da + 4, idesc);
-            ptx::umma_bf16_acc(acc0, dw0 + 6, da + 6, idesc);
-          } else {
-            ptx::umma_bf16(acc0, dw0, da, idesc, acc_first);
-            ptx::umma_bf16(acc1, dw0 + 2, da + 2, idesc, acc_first);
-            ptx::umma_bf16_acc(acc0, dw0 + 4, da + 4, idesc);
-            ptx::umma_bf16_acc(acc1, dw0 + 6, da + 6, idesc);
+            if (PAIR) ptx::umma_commit_pair_a(empty0 + 8u * s);   // frees the slot in both CTAs
+            else ptx::umma_commit_a(empty0 + 8u * s);
           }
-          acc_first = 1;
-          ptx::umma_commit_a(empty0 + 8u * s);  // slot free once these MMAs have read it
-          }
-          if (++s == (uint32_t)stages) { s = 0; ph ^= 1u; slot = ring0; } else slot += (uint32_t)stage_bytes;
+          if (++s == (uint32_t)stages) { s = 0; ph ^= 1u; lo = lo0; } else lo += step;
         }
-        if (ok) {   // this unit's accumulators are complete (in both CTAs of a pair)
+        if (ok && el) {   // this unit's accumulators are complete (in both CTAs of a pair)
           if (PAIR) ptx::umma_commit_pair(&acc_full[set]);
           else ptx::umma_commit(&acc_full[set]);
         }
       }
     }
   } else {
-    // ---------------- epilogue: warps 2..5, TMEM lane quarter = warp % 4 ----------------
-    const int quarter = warp & 3;
-    const int f = quarter * 32 + lane;  // feature (weight row) inside the tile = TMEM lane
+    // ---------------- epilogue: warps 2..5 and the twelve behind them, TMEM lane quarter = warp % 4 ----------------
+    // The four warps of a quarter take chunks of 16 columns (activation rows) in turn.  M is a multiple of 16 (the
+    // rows of a sequence are rounded up to that), so a chunk is valid as a whole, and a chunk's rows are consecutive
+    // positions of one sequence.
+    const int quarter = warp & 3, part = (warp - 2) >> 2;
+    const int f = EPI == GEMM_EPI_QKV ? head_feature(quarter, lane) : quarter * 32 + lane;   // feature of the tile in this lane
+    const uint32_t acc_empty_r0 = (PAIR && rank != 0) ? ptx::mapa_shared(ptx::smem_u32(&acc_empty[0]), 0) : 0u;
+    pdl_wait();
     bool ok = true;
     int j = 0;
-    const uint32_t acc_empty_r0 = (PAIR && rank != 0) ? ptx::mapa_shared(ptx::smem_u32(&acc_empty[0]), 0) : 0u;
     for (int u = cta; u < n_units && ok; u += n_cta, ++j) {
       const Unit w = unit_of(u);
-      const int tile = w.tile, split = w.split;
-      const uint32_t set = pp ? (uint32_t)(j & 1) : 0u;
-      const uint32_t uses = pp ? (uint32_t)(j >> 1) : (uint32_t)j;
-      ok = __all_sync(0xffffffffu, ptx::mbar_wait(&acc_full[set], uses & 1u, &abort_flag));
-      if (EPI == GEMM_EPI_QKV) ok = ptx::all_agree(1, 128, ok);   // (they meet in this epilogue)
+      const uint32_t set = (uint32_t)(j % NSETS);
+      const int m_base = w.cblk * p.BN, cols = min(p.BN, p.M - m_base);
+      const uint32_t t_lane = tmem_base + set * 256u + ((uint32_t)(quarter * 32) << 16);
+      // the rotation of a chunk: (cos, sin) of its first row and of the angle step between rows
+      const bool is_q = w.tile < p.nq, rope = EPI == GEMM_EPI_QKV && w.tile < p.nq + p.nkv;
+      float rc = 1.f, rs = 0.f, dc_ = 1.f, ds = 0.f, bias_f = 0.f;
+      auto rope_row = [&](int c0, float& c, float& s) {
+        int m = m_base + c0;
+        if (m >= p.rows_per_variant) m -= p.rows_per_variant;   // prev variant: same table
+        const float* cs = p.cos_sin + (size_t)m * 128 + (f & 63);
+        c = __ldg(cs); s = __ldg(cs + 64);
+      };
+      if (EPI == GEMM_EPI_QKV) {
+        if (rope) {
+          const float* st = p.cos_sin + (size_t)p.rows_per_variant * 128 + (f & 63);
+          dc_ = __ldg(st); ds = __ldg(st + 64);
+          if (16 * part < cols) rope_row(16 * part, rc, rs);
+        }
+        if (p.bq != nullptr)
+          bias_f = __bfloat162float(is_q ? p.bq[w.tile * 128 + f] : rope ? p.bk[(w.tile - p.nq) * 128 + f]
+                                                                         : p.bv[(w.tile - p.nq - p.nkv) * 128 + f]);
+      }
+      ok = __all_sync(0xffffffffu, ptx::mbar_wait(&acc_full[set], (uint32_t)(j / NSETS) & 1u, &abort_flag));
+      if (EPI == GEMM_EPI_QKV) ok = ptx::all_agree(1 + part, 128, ok);   // (the warps of a column part go on or give up together)
       ptx::tc_fence_after();
       if (!ok) break;
-      if (w.nkb > 0) {
-      const uint32_t t_lane = tmem_base + set * 256u + ((uint32_t)(quarter * 32) << 16);
-      const int m_base = w.cblk * p.BN;
-      float bias_f = 0.f;   // bias of this thread's output feature (q / k / v projections)
-      if (EPI == GEMM_EPI_QKV && p.bq != nullptr) {
-        const __nv_bfloat16* bb = tile >= p.nq + p.nkv ? p.bv + (tile - p.nq - p.nkv) * p.hd
-                                  : tile >= p.nq ? p.bk + (tile - p.nq) * p.hd : p.bq + tile * p.hd;
-        bias_f = __bfloat162float(bb[f]);
-      }
-      for (int c0 = 0; c0 < p.BN; c0 += 32) {
-        float acc[32];
-        // BN is a multiple of 16: the last chunk may be 16 wide
-        const int width = (p.BN - c0 >= 32) ? 32 : 16;
-        if (width == 32) ptx::tmem_ld_32x32(t_lane + c0, acc);
-        else {
-          float a16[16];
-          ptx::tmem_ld_32x16(t_lane + c0, a16);
-#pragma unroll
-          for (int j2 = 0; j2 < 16; ++j2) { acc[j2] = a16[j2]; acc[16 + j2] = 0.f; }
-        }
-        ptx::tmem_ld_wait();
-        if (EPI != GEMM_EPI_SWIGLU && !pp) {
-          // odd k-steps went to the second accumulator
-          float odd[32];
-          if (width == 32) ptx::tmem_ld_32x32(t_lane + up_off + c0, odd);
-          else {
-            float a16[16];
-            ptx::tmem_ld_32x16(t_lane + up_off + c0, a16);
-#pragma unroll
-            for (int j2 = 0; j2 < 16; ++j2) { odd[j2] = a16[j2]; odd[16 + j2] = 0.f; }
-          }
-          ptx::tmem_ld_wait();
-#pragma unroll
-          for (int j2 = 0; j2 < 32; ++j2) acc[j2] += odd[j2];
-        }
+#pragma unroll 1
+      for (int c0 = 16 * part; c0 < cols; c0 += 16 * kGemmParts) {
+        const int m0 = m_base + c0;
+        float v[16];
+        ptx::tmem_ld_32x16(t_lane + c0, v);
         if (EPI == GEMM_EPI_PARTIAL) {
-          float* dst = p.part + (size_t)split * p.part_stride + (size_t)(tile * kTileN + f);
-#pragma unroll
-          for (int j = 0; j < 32; ++j) {
-            const int m = m_base + c0 + j;
-            if (j < width && m < p.M) dst[(size_t)m * p.N] = acc[j];
-          }
-        } else if (EPI == GEMM_EPI_SWIGLU) {
-          float up[32];
-          if (width == 32) ptx::tmem_ld_32x32(t_lane + up_off + c0, up);
-          else {
-            float a16[16];
-            ptx::tmem_ld_32x16(t_lane + up_off + c0, a16);
-#pragma unroll
-            for (int j = 0; j < 16; ++j) { up[j] = a16[j]; up[16 + j] = 0.f; }
-          }
+          float* dst = p.part + (size_t)w.split * p.part_stride + (size_t)m0 * p.N + (size_t)(w.tile * kTileN + f);
           ptx::tmem_ld_wait();
-          __nv_bfloat16* dst = p.act + (size_t)(tile * kTileN + f);
 #pragma unroll
-          for (int j = 0; j < 32; ++j) {
-            const int m = m_base + c0 + j;
-            if (j < width && m < p.M) {
-              // silu(g) = g * (0.5 + 0.5 * tanh(g / 2)): one special-function instruction (as in
-              // the fused chain's epilogue; tanh.approx is good to 2^-11, the result goes to bf16)
-              const float g = acc[j];
-              float th;
-              asm("tanh.approx.f32 %0, %1;" : "=f"(th) : "f"(0.5f * g));
-              dst[(size_t)m * p.N] = __float2bfloat16_rn(g * fmaf(0.5f, th, 0.5f) * up[j]);
-            }
+          for (int i = 0; i < 16; ++i) dst[(size_t)i * p.N] = v[i];
+        } else if (EPI == GEMM_EPI_SWIGLU) {
+          float up[16];
+          ptx::tmem_ld_32x16(t_lane + 256u + c0, up);
+          __nv_bfloat16* dst = p.act + (size_t)m0 * p.N + (size_t)(w.tile * kTileN + f);
+          ptx::tmem_ld_wait();
+#pragma unroll
+          for (int i = 0; i < 16; ++i) {
+            // silu(g) = g * (0.5 + 0.5 * tanh(g / 2)): one special-function instruction (as in
+            // the fused chain's epilogue; tanh.approx is good to 2^-11, the result goes to bf16)
+            float th;
+            asm("tanh.approx.f32 %0, %1;" : "=f"(th) : "f"(0.5f * v[i]));
+            v[i] = v[i] * fmaf(0.5f, th, 0.5f) * up[i];
           }
-        } else {  // GEMM_EPI_QKV
 #pragma unroll
-          for (int j = 0; j < 32; ++j) acc[j] += bias_f;
-          const bool is_v = tile >= p.nq + p.nkv;
-          if (is_v) {
-            // V is stored transposed (keys contiguous): this thread's 32 columns are 32
-            // consecutive keys of feature row f
-            __nv_bfloat16* dst = p.v + (size_t)((tile - p.nq - p.nkv) * p.hd + f) * p.ldv + m_base + c0;
+          for (int i = 0; i < 16; ++i) dst[(size_t)i * p.N] = __float2bfloat16_rn(v[i]);
+        } else if (!rope) {
+          // V is stored transposed (keys contiguous): 16 consecutive keys of feature row f
+          __nv_bfloat16* dst = p.v + (size_t)((w.tile - p.nq - p.nkv) * 128 + f) * p.ldv + m0;
+          ptx::tmem_ld_wait();
 #pragma unroll
-            for (int j = 0; j < 32; j += 8) {
-              if (j < width && m_base + c0 + j < p.M) {
-                uint32_t w[4];
+          for (int h = 0; h < 2; ++h) {
+            uint32_t o[4];
 #pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                  __nv_bfloat162 pr = __floats2bfloat162_rn(acc[j + 2 * e], acc[j + 2 * e + 1]);
-                  w[e] = *reinterpret_cast<uint32_t*>(&pr);
-                }
-                *reinterpret_cast<uint4*>(dst + j) = make_uint4(w[0], w[1], w[2], w[3]);
-              }
+            for (int e = 0; e < 4; ++e) {
+              __nv_bfloat162 pr = __floats2bfloat162_rn(v[8 * h + 2 * e] + bias_f, v[8 * h + 2 * e + 1] + bias_f);
+              o[e] = *reinterpret_cast<uint32_t*>(&pr);
             }
-          } else {
-            // rotate-half RoPE: feature i < hd/2 pairs with i + hd/2, held by the warp two
-            // quarters away; exchange the chunk through shared memory
-#pragma unroll
-            for (int j = 0; j < 32; ++j) xch[f * 33 + j] = acc[j];
-            asm volatile("bar.sync 1, 128;" ::: "memory");
-            const int half = p.hd / 2;
-            const int i = f % half;
-            const bool lo = f < half;
-            const bool is_k = tile >= p.nq;
-            __nv_bfloat16* dst = is_k ? p.k + (size_t)((tile - p.nq) * p.hd + f)
-                                      : p.q + (size_t)(tile * p.hd + f);
-            const int ld = is_k ? p.nkv * p.hd : p.nq * p.hd;
-            // all table reads of the chunk first (independent loads), then the rotation
-            float cv[32], sv[32];
-#pragma unroll
-            for (int j = 0; j < 32; ++j) {
-              int m = m_base + c0 + j;
-              if (m >= p.rows_per_variant) m -= p.rows_per_variant;  // prev variant: same table
-              const bool in = j < width && m_base + c0 + j < p.M;
-              const float* cs = p.cos_sin + (size_t)(in ? m : 0) * p.hd;
-              cv[j] = __ldg(cs + i);
-              sv[j] = __ldg(cs + half + i);
-            }
-#pragma unroll
-            for (int j = 0; j < 32; ++j) {
-              const int m = m_base + c0 + j;
-              if (j < width && m < p.M) {
-                const float other = xch[(f ^ half) * 33 + j];
-                const float y = lo ? (acc[j] * cv[j] - other * sv[j]) : (acc[j] * cv[j] + other * sv[j]);
-                dst[(size_t)m * ld] = __float2bfloat16_rn(y);
-              }
-            }
-            asm volatile("bar.sync 1, 128;" ::: "memory");
+            *reinterpret_cast<uint4*>(dst + 8 * h) = make_uint4(o[0], o[1], o[2], o[3]);
           }
+        } else {
+          // rotate-half: the lane 16 on has the other feature of the pair.  The angle advances by one step a row
+          // (16 rotations in fp32: far below a bf16 ulp).
+          float nc = 1.f, ns = 0.f;
+          if (c0 + 16 * kGemmParts < cols) rope_row(c0 + 16 * kGemmParts, nc, ns);   // one chunk ahead
+          const float sg = lane < 16 ? -1.f : 1.f;
+          const int ld = (is_q ? p.nq : p.nkv) * 128;
+          __nv_bfloat16* dst = (is_q ? p.q + w.tile * 128 : p.k + (w.tile - p.nq) * 128) + (size_t)m0 * ld + f;
+          ptx::tmem_ld_wait();
+#pragma unroll
+          for (int i = 0; i < 16; ++i) {
+            const float y = v[i] + bias_f, other = __shfl_xor_sync(0xffffffffu, y, 16);
+            dst[(size_t)i * ld] = __float2bfloat16_rn(fmaf(y, rc, sg * other * rs));
+            const float cn = rc * dc_ - rs * ds;
+            rs = rs * dc_ + rc * ds;
+            rc = cn;
+          }
+          rc = nc; rs = ns;
         }
-      }
       }
       // the set may be overwritten by the unit after the next; the even CTA's MMA issuer waits
       // for the epilogue warps of both CTAs
       ptx::tc_fence_before();
-      if (PAIR && rank != 0) ptx::mbar_arrive_remote(acc_empty_r0 + 8u * set);
-      else ptx::mbar_arrive(&acc_empty[set]);
+      __syncwarp();
+      if (lane == 0) {
+        if (PAIR && rank != 0) ptx::mbar_arrive_remote(acc_empty_r0 + 8u * set);
+        else ptx::mbar_arrive(&acc_empty[set]);
+      }
     }
+  }
+  if (warp == 0 && lane == 0 && rank == 0 && abort_flag != 0) {
+    // given up: what is still on its way (for the even CTA's barriers, the odd one's loads too) lands before this
+    // shared memory goes to another CTA, with a limit of its own
+    for (uint32_t n = fills > (uint32_t)stages ? fills - stages : 0; n < fills; ++n)
+      ptx::mbar_wait_a(full0 + 8u * (n % stages), (n / stages) & 1u, &late_flag);
   }
   ptx::tc_fence_before();
   __syncthreads();

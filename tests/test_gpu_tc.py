@@ -125,6 +125,25 @@ def test_fused_dense_chain_is_the_path_taken_when_the_rows_fit_one_block():
         eng.close()
 
 
+@pytest.mark.parametrize("n_q,n_kv,d,ff,last,win,influence", [
+    (3, 1, 384, 640, [16] * 3, [32] * 3, True),                          # odd tile counts: no CTA pairs; 288 rows
+    (40, 20, 512, 1024, [16] * 5 + [5], [32, 30, 20, 18, 27, 27], False),  # 272 rows: a last column block with fewer
+    (40, 20, 512, 7680, [16] * 3, [128, 100, 47], True),                 # 672 rows, more units than CTA pairs
+])
+def test_tc_gemms_one_launch_each(n_q, n_kv, d, ff, last, win, influence):
+    """Above 256 rows every GEMM is a launch of its own: column blocks of other widths, single CTAs and pairs,
+    and units that take an accumulator after another one, at the tolerances of the other paths."""
+    B = len(last)
+    wl = _wl(B, n_q=n_q, n_kv=n_kv, d=d, ff=ff, last=max(last), win=max(win))
+    case = Case(wl, lengths=dict(ctx_len=[40] * B, last_len=last, win_len=win, remain_len=[128] * B))
+    eng = case.make_engine(max_window=(max(win) + 15) // 16 * 16)
+    gpu, ora = case.run_gpu(eng, influence=influence), case.run_oracle(influence=influence)
+    compare(case, gpu, ora)
+    _, launches = eng.step_profiled(influence=influence, **case.device_inputs(eng))
+    assert launches["dense"] == 0 and launches["qkv"] == case.n_layers
+    eng.close()
+
+
 @pytest.mark.parametrize("last,win,influence,rows", [(32, 96, True, 256), (0, 16, True, 32), (0, 32, False, 32),
                                                      (0, 7, False, 16), (0, 16, False, 16), (0, 40, False, 48)])
 def test_fused_chain_at_its_row_limits(last, win, influence, rows):
