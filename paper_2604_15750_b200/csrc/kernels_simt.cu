@@ -128,7 +128,50 @@ __device__ __forceinline__ void rmsnorm_row(float* __restrict__ xr, const float*
   }
 }
 
-template <typename T>
+// The same with the row in registers, NI pieces of four a thread: all loads of x and of the partial sums are under way at
+// once, where a piece after the other is a chain of 2 NI memory latencies (the loads of x may not pass its stores).
+template <typename T, int NI>
+__device__ __forceinline__ void rmsnorm_row_regs(float* __restrict__ xr, const float* __restrict__ part,
+                                                 int nsplit, size_t part_stride, const T* __restrict__ g,
+                                                 float eps, int d, T* __restrict__ outr, float* red) {
+  float4 v[NI];
+  const int t4 = threadIdx.x * 4;
+#pragma unroll
+  for (int k = 0; k < NI; ++k)
+    v[k] = t4 + k * 1024 < d ? *reinterpret_cast<const float4*>(xr + t4 + k * 1024) : make_float4(0.f, 0.f, 0.f, 0.f);
+  if (part) {
+#pragma unroll 2
+    for (int sidx = 0; sidx < nsplit; ++sidx) {
+      const float* ps = part + sidx * part_stride;
+      float4 w[NI];
+#pragma unroll
+      for (int k = 0; k < NI; ++k)
+        w[k] = t4 + k * 1024 < d ? __ldg(reinterpret_cast<const float4*>(ps + t4 + k * 1024)) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int k = 0; k < NI; ++k) { v[k].x += w[k].x; v[k].y += w[k].y; v[k].z += w[k].z; v[k].w += w[k].w; }
+    }
+  }
+  float gv[NI][4];
+#pragma unroll
+  for (int k = 0; k < NI; ++k)
+    if (t4 + k * 1024 < d) load4<T>(g + t4 + k * 1024, gv[k]);
+  float ss = 0.f;
+#pragma unroll
+  for (int k = 0; k < NI; ++k) {
+    if (part && t4 + k * 1024 < d) *reinterpret_cast<float4*>(xr + t4 + k * 1024) = v[k];
+    ss += v[k].x * v[k].x + v[k].y * v[k].y + v[k].z * v[k].z + v[k].w * v[k].w;
+  }
+  ss = block_sum(ss, red);
+  const float inv = rsqrtf(ss / (float)d + eps);
+#pragma unroll
+  for (int k = 0; k < NI; ++k)
+    if (t4 + k * 1024 < d) {
+      const float o[4] = {v[k].x * inv * gv[k][0], v[k].y * inv * gv[k][1], v[k].z * inv * gv[k][2], v[k].w * inv * gv[k][3]};
+      store4<T>(outr + t4 + k * 1024, o);
+    }
+}
+
+template <typename T, int NI>   // NI: pieces of 1024 elements of a row, 0: any width
 __global__ void __launch_bounds__(256) k_rmsnorm(float* __restrict__ x,
                                                  const float* __restrict__ part, int nsplit,
                                                  size_t part_stride, const T* __restrict__ g,
@@ -137,14 +180,17 @@ __global__ void __launch_bounds__(256) k_rmsnorm(float* __restrict__ x,
   pdl_trigger();
   pdl_wait(x, part);
   const size_t off = (size_t)blockIdx.x * d;
-  rmsnorm_row<T>(x + off, part ? part + off : nullptr, nsplit, part_stride, g, eps, d, out + off,
-                 red);
+  if constexpr (NI > 0)
+    rmsnorm_row_regs<T, NI>(x + off, part ? part + off : nullptr, nsplit, part_stride, g, eps, d, out + off, red);
+  else
+    rmsnorm_row<T>(x + off, part ? part + off : nullptr, nsplit, part_stride, g, eps, d, out + off, red);
 }
 
 template <typename T>
 void launch_rmsnorm(float* x, const float* part, int nsplit, size_t part_stride, const T* g,
                     float eps, int M, int d, T* out, cudaStream_t s) {
-  launch_chained(k_rmsnorm<T>, M, 256, 0, s, x, part, nsplit, part_stride, g, eps, d, out);
+  auto* k = d <= 1024 ? k_rmsnorm<T, 1> : d <= 2048 ? k_rmsnorm<T, 2> : d <= 4096 ? k_rmsnorm<T, 4> : d <= 8192 ? k_rmsnorm<T, 8> : k_rmsnorm<T, 0>;
+  launch_chained(k, M, 256, 0, s, x, part, nsplit, part_stride, g, eps, d, out);
 }
 
 // LM-head input rows, one block per row of the LM head's order (groups of G positions: curr rows, then

@@ -146,3 +146,15 @@ def test_position_whose_logits_are_all_minus_infinity(cooperative):
     for k_ in ("pred_id", "conf", "entropy", "lse", "influence"):
         assert np.array_equal(got[k_][rest], clean[k_][rest]), k_
     eng.close()
+
+
+@pytest.mark.parametrize("d", [1028, 2052, 4100, 8196])
+def test_norm_of_wide_rows(d):
+    """RMSNorm as a launch of its own: a row in 2, 4 or 8 pieces of registers, with a remainder in the last, and
+    wider ones."""
+    wl = inputs.Workload(f"norm{d}", 1, d, 2, 2, 32, 64, 512, "f32", 1, 16, 16, 4, 16, 32, 900 + d % 7)
+    case = Case(wl, steer=None)
+    eng = case.make_engine()
+    gpu, ora = case.run_gpu(eng), case.run_oracle()
+    compare(case, gpu, ora)
+    eng.close()

@@ -129,6 +129,8 @@ def test_fused_dense_chain_is_the_path_taken_when_the_rows_fit_one_block():
     (3, 1, 384, 640, [16] * 3, [32] * 3, True),                          # odd tile counts: no CTA pairs; 288 rows
     (40, 20, 512, 1024, [16] * 5 + [5], [32, 30, 20, 18, 27, 27], False),  # 272 rows: a last column block with fewer
     (40, 20, 512, 7680, [16] * 3, [128, 100, 47], True),                 # 672 rows, more units than CTA pairs
+    (2, 2, 2176, 256, [16] * 3, [32] * 3, True),                         # norms of wide rows, with K splits folded in
+    (2, 2, 4224, 256, [16] * 3, [32] * 3, True),
 ])
 def test_tc_gemms_one_launch_each(n_q, n_kv, d, ff, last, win, influence):
     """Above 256 rows every GEMM is a launch of its own: column blocks of other widths, single CTAs and pairs,
