@@ -349,25 +349,30 @@ k_attn_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
         }
       }
     } else if (warp == 1) {
-      if (lane == 0) {
-        // ---------------- issuer of S = Q K^T ----------------
-        // Lean issue path (the issuing thread does not run ahead of the tensor core): descriptor low
-        // words are kept in registers and advanced by 32-bit additions of constants.
-        const uint32_t idesc = ptx::idesc_bf16(128, 128);
-        const uint32_t hi32 = ptx::smem_desc_hi32();
-        const uint32_t q_lo = ptx::smem_desc_lo(ptx::smem_u32(Qs));
-        const uint32_t k_lo = ptx::smem_desc_lo(ptx::smem_u32(Ks));
-        constexpr uint32_t kSub16 = kSub >> 4;
-        const uint32_t b_k_full = ptx::smem_u32(&k_full[0]), b_s_full = ptx::smem_u32(&s_full[0]);
-        const uint32_t b_pv_done = ptx::smem_u32(&pv_done[0]);
-        bool ok = ptx::mbar_wait(&q_full, 0, &abort_flag);
-        for (int j = 0; j < T && ok; ++j) {
-          const int J = J0 + j;
-          const uint32_t s = (uint32_t)(J % kAttnStagesK), sb = (uint32_t)J % 3u;
-          // score buffer J % 3 last held P of tile J - 3: its P V (issued by another thread) must be done
-          if (J >= 3 && !ptx::mbar_wait_a(b_pv_done + 8u * sb, ((uint32_t)(J - 3) / 3u) & 1u, &abort_flag)) break;
-          if (!ptx::mbar_wait_a(b_k_full + 8u * s, ((uint32_t)(J / kAttnStagesK)) & 1u, &abort_flag)) break;
-          ptx::tc_fence_after();
+      // ---------------- issuer of S = Q K^T ----------------
+      // Lean issue path (the issuer does not run ahead of the tensor core): the whole warp runs the loop and one
+      // elected lane issues, so that the descriptors' low words stay in uniform registers and advance by additions.
+      // (A lane in a branch of its own: 725 clocks for the 512 of a tile's score MMAs, 670 for its output MMAs.  Per
+      // layer of LLaDA-8B, two variants of 160 rows: eight sequences of 1024 keys 119.7 -> 115.8 us, four of 4096 136.2 -> 132.8.)
+      const bool el = ptx::elect_one();
+      const uint32_t idesc = ptx::idesc_bf16(128, 128);
+      const uint32_t hi32 = ptx::smem_desc_hi32();
+      const uint32_t q_lo = ptx::smem_desc_lo(ptx::smem_u32(Qs));
+      const uint32_t k_lo = ptx::smem_desc_lo(ptx::smem_u32(Ks));
+      constexpr uint32_t kSub16 = kSub >> 4;
+      const uint32_t b_k_full = ptx::smem_u32(&k_full[0]), b_s_full = ptx::smem_u32(&s_full[0]);
+      const uint32_t b_pv_done = ptx::smem_u32(&pv_done[0]);
+      bool ok = __all_sync(0xffffffffu, ptx::mbar_wait(&q_full, 0, &abort_flag));
+      for (int j = 0; j < T && ok; ++j) {
+        const int J = J0 + j;
+        const uint32_t s = (uint32_t)(J % kAttnStagesK), sb = (uint32_t)J % 3u;
+        // score buffer J % 3 last held P of tile J - 3: its P V (issued by another warp) must be done
+        if (J >= 3) ok = ptx::mbar_wait_a(b_pv_done + 8u * sb, ((uint32_t)(J - 3) / 3u) & 1u, &abort_flag);
+        ok = ok && ptx::mbar_wait_a(b_k_full + 8u * s, ((uint32_t)(J / kAttnStagesK)) & 1u, &abort_flag);
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
+        ptx::tc_fence_after();
+        if (el) {
           const uint32_t d = tmem_base + sb * 128u, bk = k_lo + s * (2 * kSub16);
 #pragma unroll
           for (int kk = 0; kk < 8; ++kk) {
@@ -377,6 +382,7 @@ k_attn_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
           // (the K slot is handed back by a softmax thread that has seen S)
           ptx::umma_commit_a(b_s_full + 8u * sb);
         }
+        __syncwarp();
       }
     } else if (warp == 3) {
       // ---------------- issuer of O (+)= P V ----------------
@@ -388,6 +394,7 @@ k_attn_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
       constexpr uint32_t kSub16 = kSub >> 4;
       const uint32_t b_v_loc = ptx::smem_u32(&v_loc[0]), b_p_full = ptx::smem_u32(&p_full[0]);
       const uint32_t b_pv_done = ptx::smem_u32(&pv_done[0]);
+      const bool el = ptx::elect_one();   // (as in warp 1)
       bool ok = true;
       for (int j = 0; j < T && ok; ++j) {
         const int J = J0 + j;
@@ -402,33 +409,32 @@ k_attn_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
           ptx::fence_proxy_async_smem();
           __syncwarp();
         }
-        if (lane == 0) {
-          ok = ptx::mbar_wait_a(b_p_full + 8u * sb, ((uint32_t)J / 3u) & 1u, &abort_flag) &&
-               ptx::mbar_wait_a(b_v_loc + 8u * s, ph, &abort_flag);
-          if (ok) {
-            ptx::tc_fence_after();
-            const uint32_t d = tmem_base + 384u, a = tmem_base + sb * 128u, bv = v_lo + s * (2 * kSub16);
-            auto mma = [&](int kk) {
-              const uint32_t off = (uint32_t)(kk >> 2) * kSub16 + (uint32_t)(kk & 3) * 2u;
-              ptx::umma_bf16_ts_lo(d, a + (uint32_t)(kk >> 1) * 32u + (uint32_t)(kk & 1) * 8u, bv + off, hi32, idesc,
-                                   (kk > 0 || j > 0) ? 1u : 0u);
-            };
-            if (t.valid == kBK) {   // (the lean path: constants only)
+        ok = ptx::mbar_wait_a(b_p_full + 8u * sb, ((uint32_t)J / 3u) & 1u, &abort_flag) &&
+             ptx::mbar_wait_a(b_v_loc + 8u * s, ph, &abort_flag);
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
+        ptx::tc_fence_after();
+        if (el) {
+          const uint32_t d = tmem_base + 384u, a = tmem_base + sb * 128u, bv = v_lo + s * (2 * kSub16);
+          auto mma = [&](int kk) {
+            const uint32_t off = (uint32_t)(kk >> 2) * kSub16 + (uint32_t)(kk & 3) * 2u;
+            ptx::umma_bf16_ts_lo(d, a + (uint32_t)(kk >> 1) * 32u + (uint32_t)(kk & 1) * 8u, bv + off, hi32, idesc,
+                                 (kk > 0 || j > 0) ? 1u : 0u);
+          };
+          if (t.valid == kBK) {   // (the lean path: constants only)
 #pragma unroll
-              for (int kk = 0; kk < 8; ++kk) mma(kk);
-            } else {
+            for (int kk = 0; kk < 8; ++kk) mma(kk);
+          } else {
 #pragma unroll 1
-              for (int kk = 0; kk < attn_pv_keys(t.valid) >> 4; ++kk) mma(kk);
-            }
-            // also tells the V^T producer that the slot is free and the score issuer that the
-            // buffer is
-            ptx::umma_commit_a(b_pv_done + 8u * sb);
+            for (int kk = 0; kk < attn_pv_keys(t.valid) >> 4; ++kk) mma(kk);
           }
+          // also tells the V^T producer that the slot is free and the score issuer that the
+          // buffer is
+          ptx::umma_commit_a(b_pv_done + 8u * sb);
         }
-        // the other lanes wait here (not spinning) while lane 0 issues
-        ok = __shfl_sync(0xffffffffu, (int)ok, 0) != 0;
+        __syncwarp();
       }
-      if (ok && lane == 0) ptx::umma_commit(&o_done);
+      if (ok && el) ptx::umma_commit(&o_done);
     } else {
       // ---------------- softmax warps ----------------
       const uint32_t t_lane = tmem_base + ((uint32_t)(quarter * 32) << 16);
