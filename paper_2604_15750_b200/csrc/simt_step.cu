@@ -177,7 +177,10 @@ __device__ __forceinline__ bool gemm_phase(const SimtStep<T>& p, const FuseGemm<
   const int vid = split ? (int)blockIdx.x : gr.vid, nv = split ? (int)gridDim.x : gr.nv;
   const int per = MT <= nv ? nv / MT : 1;   // groups (CTAs) on a row tile
   const int pr = gr.t / PPR, pk = (gr.t % PPR) * PIECE;         // this thread's piece of a chunk: row, column
-  const int ty = gr.lane >> 3, tx = gr.lane & 7;
+  // A warp has 32 k of a chunk, half of it 16 of them, a lane 4 x 4 outputs: rows ty + 4 i, columns tx + 4 j.  (What a
+  // tile costs is the return path of its shared-memory loads, 4 clocks each: 32 a lane, and 48 with all 32 k in one
+  // lane and 4 x 2 outputs.)
+  const int ty = (gr.lane >> 2) & 3, tx = gr.lane & 3, ko = gr.warp * (KC / 8) + (gr.lane >> 4) * (KC / 16);
   bool waited = false;
 #pragma unroll 1
   for (int mt = MT <= nv ? vid % MT : vid; !waited || mt < MT; mt += (MT <= nv ? MT : nv)) {
@@ -185,29 +188,41 @@ __device__ __forceinline__ bool gemm_phase(const SimtStep<T>& p, const FuseGemm<
     const int mine = (mt < MT && first < per && first < units) ? (units - first + per - 1) / per : 0;
     const int total = mine * (ce - cb);
     int iu = first, ic = cb, is = 0, issued = 0;   // next step to load: unit, chunk, ring slot
+    // A thread copies one column piece of rows pr, pr + RS, .. of a chunk: of W the first eight rows and the other
+    // eight are runs of their own (their partner features, or the same rows of the other matrix).
     auto issue = [&](bool with_w, bool with_a, int u, int c, int s) {
       const int k0 = c * KC + pk, full = max(0, min(16, (g.K - k0) * (int)sizeof(T)));
-#pragma unroll 1
-      for (int i = 0; i < NP; ++i) {
-        const int r = pr + i * RS;
-        if (with_w) {
-          const T* w = g.w0;
-          int n = u * NC + r, N = g.N;
-          if (epi == EPI_QKV) {
-            const int head = u / per_head, e = (u - head * per_head) * 8 + (r & 7) + (r >> 3) * half;
-            const int hh = head < p.nq ? head : head < p.nq + p.nkv ? head - p.nq : head - p.nq - p.nkv;
-            w = head < p.nq ? g.w0 : head < p.nq + p.nkv ? g.w1 : g.w2;
-            n = hh * p.hd + e; N = n + 1;
-          } else if (epi == EPI_SWIGLU) {
-            n = u * 8 + (r & 7);
-            if (r >= 8) w = g.w1;
-          }
-          const int bytes = n < N ? full : 0;
-          cp_async16(ring_w + ((size_t)s * NC + r) * PITCH + pk, bytes ? w + (size_t)n * g.K + k0 : g.w0, bytes);
+      if (with_w) {
+        const T *wa = g.w0, *wb = g.w0;
+        int n = u * NC, run = 8, left = g.N - n;      // first row, the second run's distance, rows of the matrix from n on
+        if (epi == EPI_QKV) {
+          const int head = u / per_head;
+          wa = head < p.nq ? g.w0 : head < p.nq + p.nkv ? g.w1 : g.w2;
+          wb = wa;
+          n = (head < p.nq ? head : head < p.nq + p.nkv ? head - p.nq : head - p.nq - p.nkv) * p.hd + (u - head * per_head) * 8;
+          run = half; left = 8;
+        } else if (epi == EPI_SWIGLU) {
+          wb = g.w1; n = u * 8; run = 0; left = g.N - n;
         }
-        if (with_a && stream_a) {
-          const int bytes = m0 + r < g.M ? full : 0;
-          cp_async16(as + ((size_t)s * 16 + r) * PITCH + pk, bytes ? g.A + (size_t)(m0 + r) * g.K + k0 : g.A, bytes);
+        const int left_b = epi == EPI_STORE_F32 || epi == EPI_ADD_F32 ? left - 8 : left;
+        wa += (size_t)(n + pr) * g.K + k0;
+        wb += (size_t)(n + run + pr) * g.K + k0;
+        T* dst = ring_w + ((size_t)s * NC + pr) * PITCH + pk;
+#pragma unroll
+        for (int i = 0; i < NP / 2; ++i) {
+          const int r = i * RS;                       // row inside the run, from pr on
+          const int ba = pr + r < left ? full : 0, bb = pr + r < left_b ? full : 0;
+          cp_async16(dst + (size_t)r * PITCH, ba ? wa + (size_t)r * g.K : g.w0, ba);
+          cp_async16(dst + (size_t)(r + 8) * PITCH, bb ? wb + (size_t)r * g.K : g.w0, bb);
+        }
+      }
+      if (with_a && stream_a) {
+        const T* src = g.A + (size_t)(m0 + pr) * g.K + k0;
+        T* dst = as + ((size_t)s * 16 + pr) * PITCH + pk;
+#pragma unroll
+        for (int i = 0; i < NP; ++i) {
+          const int bytes = m0 + pr + i * RS < g.M ? full : 0;
+          cp_async16(dst + (size_t)i * RS * PITCH, bytes ? src + (size_t)i * RS * g.K : g.A, bytes);
         }
       }
     };
@@ -242,7 +257,7 @@ __device__ __forceinline__ bool gemm_phase(const SimtStep<T>& p, const FuseGemm<
       if (__any_sync(0xffffffffu, norm || g1 != nullptr))       // both halves of the warp take part
         norm_row<T>(xr, g.gain, p.eps, p.d, norm ? dst : nullptr, chunks * KC, g0, g1, gr.lane & 15);
     }
-    f2 acc[4][2];
+    f2 acc[4][4];
     float old = 0.f;             // residual value that the epilogue adds to
     int u = first, c = cb, slot = 0;
 #pragma unroll 1
@@ -259,41 +274,45 @@ __device__ __forceinline__ bool gemm_phase(const SimtStep<T>& p, const FuseGemm<
       const int er = gr.t >> 4, ec = gr.t & 15;                 // the epilogue's element of this thread
       if (c == cb) {
 #pragma unroll
-        for (int i = 0; i < 4; ++i) acc[i][0] = acc[i][1] = 0ull;
+        for (int i = 0; i < 4; ++i) acc[i][0] = acc[i][1] = acc[i][2] = acc[i][3] = 0ull;
         if (epi == EPI_ADD_F32 && m0 + er < g.M && u * NC + ec < g.N) old = __ldcg(g.C + (size_t)(m0 + er) * g.ldc + u * NC + ec);
       }
-      const T* wp = ring_w + ((size_t)slot * NC + tx) * PITCH + gr.warp * (KC / 8);
-      const T* ap = (stream_a ? as + (size_t)slot * 16 * PITCH : as + c * KC) + ty * 4 * apitch + gr.warp * (KC / 8);
-#pragma unroll 2
-      for (int k = 0; k < KC / 8; k += 4) {
-        f2 av[4][2], wv[2][2];
+      const T* wp = ring_w + ((size_t)slot * NC + tx) * PITCH + ko;
+      const T* ap = (stream_a ? as + (size_t)slot * 16 * PITCH : as + c * KC) + ty * apitch + ko;
+#pragma unroll 1
+      for (int k = 0; k < KC / 16; k += 4) {
+        f2 wv[4][2];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
+        for (int j = 0; j < 4; ++j) {
           float v[4];
-          load4<T>(ap + i * apitch + k, v);
-          av[i][0] = pack2(v[0], v[1]); av[i][1] = pack2(v[2], v[3]);
-        }
-#pragma unroll
-        for (int j = 0; j < 2; ++j) {
-          float v[4];
-          load4<T>(wp + j * 8 * PITCH + k, v);
+          load4<T>(wp + j * 4 * PITCH + k, v);
           wv[j][0] = pack2(v[0], v[1]); wv[j][1] = pack2(v[2], v[3]);
         }
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
+        for (int i = 0; i < 4; ++i) {
+          float v[4];
+          load4<T>(ap + i * 4 * apitch + k, v);
+          const f2 a0 = pack2(v[0], v[1]), a1 = pack2(v[2], v[3]);
 #pragma unroll
-          for (int j = 0; j < 2; ++j) {
-            fma2(acc[i][j], av[i][0], wv[j][0]);
-            fma2(acc[i][j], av[i][1], wv[j][1]);
+          for (int j = 0; j < 4; ++j) {
+            fma2(acc[i][j], a0, wv[j][0]);
+            fma2(acc[i][j], a1, wv[j][1]);
           }
+        }
       }
       if (++slot == ST) slot = 0;
       if (++c < ce) continue;
       c = cb;
+      // the two halves of the warp meet, each keeps two of the four rows
+      const bool hi = gr.lane >= 16;
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+      for (int i = 0; i < 2; ++i)
 #pragma unroll
-        for (int j = 0; j < 2; ++j) cs[(gr.warp * 16 + ty * 4 + i) * CP + tx + 8 * j] = sum2(acc[i][j]);
+        for (int j = 0; j < 4; ++j) {
+          const float lo_v = sum2(acc[i][j]), hi_v = sum2(acc[i + 2][j]);
+          const float got = __shfl_xor_sync(0xffffffffu, hi ? lo_v : hi_v, 16);
+          cs[(gr.warp * 16 + ty + 4 * (i + (hi ? 2 : 0))) * CP + tx + 4 * j] = (hi ? hi_v : lo_v) + got;
+        }
       float y = 0.f;
       if (split) {     // (one tile per CTA, so the sums are not overwritten)
         asm volatile("bar.sync 3, %0;" ::"n"(kFuseThreads) : "memory");
