@@ -48,7 +48,7 @@ struct GemmParams {
   int tiles;      // weight tiles (over all matrices of the call)
   // QKV epilogue
   int nq, nkv;              // tiles [0,nq) are q heads, [nq,nq+nkv) k heads, rest v heads (head_dim 128)
-  const float* cos_sin;     // RoPE table [(b, r)][128]; row rows_per_variant: the angle step between rows
+  const float* cos_sin;     // RoPE table [(b, r)][128]
   int rows_per_variant;     // the table is shared by the variants
   const __nv_bfloat16 *bq, *bk, *bv;  // projection biases [nq*hd], [nkv*hd], [nkv*hd], or null
   __nv_bfloat16 *q, *k, *v; // outputs q [M, nq*hd], k [M, nkv*hd], v TRANSPOSED [nkv*hd, ldv]
@@ -271,7 +271,8 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w0, const __grid_constant__ CU
     const int quarter = warp & 3, part = (warp - 2) >> 2;
     const int f = EPI == GEMM_EPI_QKV ? head_feature(quarter, lane) : quarter * 32 + lane;   // feature of the tile in this lane
     const uint32_t acc_empty_r0 = (PAIR && rank != 0) ? ptx::mapa_shared(ptx::smem_u32(&acc_empty[0]), 0) : 0u;
-    pdl_wait();
+    const float* cos_sin = p.cos_sin;
+    pdl_wait(cos_sin);
     bool ok = true;
     int j = 0;
     for (int u = cta; u < n_units && ok; u += n_cta, ++j) {
@@ -279,25 +280,11 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w0, const __grid_constant__ CU
       const uint32_t set = (uint32_t)(j % NSETS);
       const int m_base = w.cblk * p.BN, cols = min(p.BN, p.M - m_base);
       const uint32_t t_lane = tmem_base + set * 256u + ((uint32_t)(quarter * 32) << 16);
-      // the rotation of a chunk: (cos, sin) of its first row and of the angle step between rows
       const bool is_q = w.tile < p.nq, rope = EPI == GEMM_EPI_QKV && w.tile < p.nq + p.nkv;
-      float rc = 1.f, rs = 0.f, dc_ = 1.f, ds = 0.f, bias_f = 0.f;
-      auto rope_row = [&](int c0, float& c, float& s) {
-        int m = m_base + c0;
-        if (m >= p.rows_per_variant) m -= p.rows_per_variant;   // prev variant: same table
-        const float* cs = p.cos_sin + (size_t)m * 128 + (f & 63);
-        c = __ldg(cs); s = __ldg(cs + 64);
-      };
-      if (EPI == GEMM_EPI_QKV) {
-        if (rope) {
-          const float* st = p.cos_sin + (size_t)p.rows_per_variant * 128 + (f & 63);
-          dc_ = __ldg(st); ds = __ldg(st + 64);
-          if (16 * part < cols) rope_row(16 * part, rc, rs);
-        }
-        if (p.bq != nullptr)
-          bias_f = __bfloat162float(is_q ? p.bq[w.tile * 128 + f] : rope ? p.bk[(w.tile - p.nq) * 128 + f]
-                                                                         : p.bv[(w.tile - p.nq - p.nkv) * 128 + f]);
-      }
+      float bias_f = 0.f;
+      if (EPI == GEMM_EPI_QKV && p.bq != nullptr)
+        bias_f = __bfloat162float(is_q ? p.bq[w.tile * 128 + f] : rope ? p.bk[(w.tile - p.nq) * 128 + f]
+                                                                       : p.bv[(w.tile - p.nq - p.nkv) * 128 + f]);
       ok = __all_sync(0xffffffffu, ptx::mbar_wait(&acc_full[set], (uint32_t)(j / NSETS) & 1u, &abort_flag));
       if (EPI == GEMM_EPI_QKV) ok = ptx::all_agree(1 + part, 128, ok);   // (the warps of a column part go on or give up together)
       ptx::tc_fence_after();
@@ -342,10 +329,14 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w0, const __grid_constant__ CU
             *reinterpret_cast<uint4*>(dst + 8 * h) = make_uint4(o[0], o[1], o[2], o[3]);
           }
         } else {
-          // rotate-half: the lane 16 on has the other feature of the pair.  The angle advances by one step a row
-          // (16 rotations in fp32: far below a bf16 ulp).
-          float nc = 1.f, ns = 0.f;
-          if (c0 + 16 * kGemmParts < cols) rope_row(c0 + 16 * kGemmParts, nc, ns);   // one chunk ahead
+          // rotate-half: the lane 16 on has the other feature of the pair.  Every row has its own factors from the
+          // table, rounded once from fp64: advanced by an angle step from the chunk's first row they were up to 7.7e-7
+          // off instead of 3e-8.
+          const int mt = m0 >= p.rows_per_variant ? m0 - p.rows_per_variant : m0;   // (prev variant: same table)
+          const float* cs = cos_sin + (size_t)mt * 128 + (f & 63);
+          float cv[16], sv[16];
+#pragma unroll
+          for (int i = 0; i < 16; ++i) { cv[i] = __ldg(cs + i * 128); sv[i] = __ldg(cs + i * 128 + 64); }
           const float sg = lane < 16 ? -1.f : 1.f;
           const int ld = (is_q ? p.nq : p.nkv) * 128;
           __nv_bfloat16* dst = (is_q ? p.q + w.tile * 128 : p.k + (w.tile - p.nq) * 128) + (size_t)m0 * ld + f;
@@ -353,12 +344,8 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w0, const __grid_constant__ CU
 #pragma unroll
           for (int i = 0; i < 16; ++i) {
             const float y = v[i] + bias_f, other = __shfl_xor_sync(0xffffffffu, y, 16);
-            dst[(size_t)i * ld] = __float2bfloat16_rn(fmaf(y, rc, sg * other * rs));
-            const float cn = rc * dc_ - rs * ds;
-            rs = rs * dc_ + rc * ds;
-            rc = cn;
+            dst[(size_t)i * ld] = __float2bfloat16_rn(fmaf(y, cv[i], sg * other * sv[i]));
           }
-          rc = nc; rs = ns;
         }
       }
       // the set may be overwritten by the unit after the next; the even CTA's MMA issuer waits
