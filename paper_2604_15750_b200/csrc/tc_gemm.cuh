@@ -286,7 +286,6 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w0, const __grid_constant__ CU
         bias_f = __bfloat162float(is_q ? p.bq[w.tile * 128 + f] : rope ? p.bk[(w.tile - p.nq) * 128 + f]
                                                                        : p.bv[(w.tile - p.nq - p.nkv) * 128 + f]);
       ok = __all_sync(0xffffffffu, ptx::mbar_wait(&acc_full[set], (uint32_t)(j / NSETS) & 1u, &abort_flag));
-      if (EPI == GEMM_EPI_QKV) ok = ptx::all_agree(1 + part, 128, ok);   // (the warps of a column part go on or give up together)
       ptx::tc_fence_after();
       if (!ok) break;
 #pragma unroll 1

@@ -45,6 +45,10 @@ def test_the_next_kernel_is_let_in_behind_the_tmem_allocation(name, kernel):
 @pytest.mark.parametrize("name,first,last", [
     ("tc_chain.cuh", "const bool el = ptx::elect_one();", "umma_commit_pair(c.acc_full)"),
     ("tc_attn_few.cuh", "const bool pv = warp == 2;", "umma_commit(pv ? &c.p_empty"),
+    ("tc_gemm.cuh", "// ---------------- TMA producer", "// ---------------- MMA issuer"),
+    ("tc_gemm.cuh", "// ---------------- MMA issuer", "// ---------------- epilogue"),
+    ("tc_attn.cuh", "// ---------------- issuer of S = Q K^T", "// ---------------- issuer of O (+)= P V"),
+    ("tc_attn.cuh", "// ---------------- issuer of O (+)= P V", "// ---------------- softmax warps"),
 ])
 def test_a_warp_that_issues_together_gives_up_together(name, first, last):
     """A bounded wait is decided lane by lane.  Where the whole warp runs the issuing loop, whose votes take all
@@ -59,15 +63,16 @@ def test_a_warp_that_issues_together_gives_up_together(name, first, last):
         assert "__all_sync(" in statement or re.search(r"ok = __all_sync\(0xffffffffu, ok\);\s*if \(!ok\) break;", later)
 
 
-@pytest.mark.parametrize("name,first,last", [
-    ("tc_chain.cuh", "epilogue: all warps", "tc_fence_after"), ("tc_gemm.cuh", "epilogue: warps 2..5", "tc_fence_after"),
+@pytest.mark.parametrize("name,first,last,meet", [
+    ("tc_chain.cuh", "epilogue: all warps", "tc_fence_after", True), ("tc_gemm.cuh", "epilogue: warps 2..5", "tc_fence_after", False),
 ])
-def test_warps_that_meet_in_an_epilogue_give_up_together(name, first, last):
-    """The epilogues read TMEM warp-wide, and the rotation meets on named barriers of four warps: the wait in front of
-    them is voted on in the warp and agreed on among the four."""
+def test_warps_that_meet_in_an_epilogue_give_up_together(name, first, last, meet):
+    """The epilogues read TMEM warp-wide: the wait in front of them is voted on in the warp.  Where the rotation meets on
+    named barriers of four warps (the chain's; the other one's is an exchange inside a warp) these four agree too."""
     src = open(os.path.join(CSRC, name)).read()
     part = src[src.index(first):]
     part = part[:part.index(last)]
     waits = re.findall(r"[^;]*ptx::mbar_wait\([^;]*;", part)
     assert waits and all("__all_sync(" in w for w in waits)
-    assert re.search(r"EPI_QKV\) ok = ptx::all_agree\([^;]*, 128, ok\);", part)
+    assert bool(re.search(r"EPI_QKV\) ok = ptx::all_agree\([^;]*, 128, ok\);", part)) == meet
+    assert ("bar.sync" in src or "all_agree" in src) == meet
