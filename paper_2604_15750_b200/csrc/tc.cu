@@ -345,6 +345,7 @@ static int launch_gemm(TcState* t, const CUtensorMap& w0, const CUtensorMap& w1,
   const int n_units = (pair ? tiles / 2 : tiles) * n_cblk * p.nsplit;
   const int workers_max = pair ? t->n_sm / 2 : t->n_sm;
   const int workers = n_units < workers_max ? n_units : workers_max;
+  p.dual = EPI == GEMM_EPI_QKV && n_units <= workers;
   cudaError_t e;
   if (pair) {
     cudaLaunchConfig_t cfg{};

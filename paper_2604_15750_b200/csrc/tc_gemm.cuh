@@ -13,10 +13,15 @@
 // tcgen05.mma understand.
 //
 // A CTA works through the units (weight tile, column block, K split) blockIdx.x, + gridDim.x, ...
-// The single-matrix GEMMs keep one accumulator of up to 256 columns per unit and alternate between two
-// TMEM sets: the producer and the MMA issuer run on into the next unit and the epilogue of a unit runs
-// under its MMAs.  Gate / up need both sets for one unit; there a CTA's next unit starts when the
-// epilogue has drained them.
+// The single-matrix GEMMs use one accumulator of up to 256 columns at a time and alternate between two TMEM
+// sets: the producer and the MMA issuer run on into the next accumulator and the epilogue of one runs under its
+// MMAs.  Gate / up need both sets for one unit; there a CTA's next unit starts when the epilogue has drained them.
+//
+// The tensor core truncates the running sum at every MMA, so that the error grows with the MMAs of a chain: sums over K =
+// 4096 of normal numbers are 4.4e-6 off (relative) in one chain, 2.1e-6 in two, 1.0e-6 in four (of positive ones 1.4e-5,
+// 5.3e-6, 2.1e-6); over K = 12288 1.4e-5, 6.7e-6, 3.2e-6.  So the projections back to d go through four accumulators a
+// unit, which the epilogue warps add up in registers (0.3 .. 1 us a GEMM against one), and QKV sends even k-steps to the
+// one set and odd ones to the other where a CTA has no second unit.
 //
 // What bounds it: an SM takes in 64 bytes a clock from L2, and a k-block of 256 columns needs 32 KB for 512 clocks
 // of MMAs, so the main loops run at 300..320 ns a k-block (108 GB/s an SM) where the MMAs alone would take 270; batches
@@ -46,6 +51,7 @@ struct GemmParams {
   int BN;         // activation rows per column block (multiple of 16, <= 256)
   int nsplit;     // split-K factor
   int tiles;      // weight tiles (over all matrices of the call)
+  int dual;       // QKV with a unit a worker: two accumulators, even and odd k-steps
   // QKV epilogue
   int nq, nkv;              // tiles [0,nq) are q heads, [nq,nq+nkv) k heads, rest v heads (head_dim 128)
   const float* cos_sin;     // RoPE table [(b, r)][128]
@@ -66,6 +72,8 @@ constexpr int kGemmParts = kGemmEpiWarps / 4;           // warps per TMEM lane q
 constexpr int kGemmThreads = 64 + 32 * kGemmEpiWarps;
 constexpr int kTileN = 128;  // weight rows per CTA tile
 constexpr int kTileK = 64;   // bf16 elements per k-block (one 128-byte swizzle row)
+constexpr int kGemmChunks = 256 / (16 * kGemmParts);    // chunks of 16 columns that a warp holds
+constexpr int kGemmChains = 4;   // accumulators that a unit of a projection back to d goes through
 
 __host__ __device__ inline int gemm_stage_bytes(int nw, int a_rows) {
   return nw * kTileN * kTileK * 2 + a_rows * kTileK * 2;
@@ -98,7 +106,8 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w0, const __grid_constant__ CU
           const __grid_constant__ CUtensorMap map_w2, const __grid_constant__ CUtensorMap map_a,
           const GemmParams p, const int stages) {
   constexpr int NW = (EPI == GEMM_EPI_SWIGLU) ? 2 : 1;
-  constexpr int NSETS = 2 / NW;          // accumulator sets that units alternate between
+  constexpr int NSETS = 2 / NW;          // accumulator sets that a CTA alternates between
+  constexpr int NCH = EPI == GEMM_EPI_PARTIAL ? kGemmChains : 1;
   constexpr int W_BYTES = kTileN * kTileK * 2;
   extern __shared__ uint8_t smem_raw[];
   __shared__ uint64_t bar_full[8], bar_empty[8], acc_full[2], acc_empty[2];
@@ -226,40 +235,47 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w0, const __grid_constant__ CU
       const uint32_t hi = ptx::smem_desc_hi32(), lo0 = ptx::smem_desc_lo(ptx::smem_u32(smem)), step = (uint32_t)stage_bytes >> 4;
       uint32_t s = 0, ph = 0, lo = lo0;
       bool ok = true;
-      int j = 0;   // units of this CTA so far
-      for (int u = cta; u < n_units && ok; u += n_cta, ++j) {
+      const uint32_t odd = EPI == GEMM_EPI_QKV && p.dual ? 256u : 0u;   // the odd k-steps' accumulator
+      int j = 0;   // accumulators of this CTA so far
+      for (int u = cta; u < n_units && ok; u += n_cta) {
         const Unit w = unit_of(u);
-        const uint32_t set = (uint32_t)(j % NSETS);
-        // the epilogue has drained this set (its use before the last one)
-        if (j >= NSETS) ok = __all_sync(0xffffffffu, ptx::mbar_wait(&acc_empty[set], (uint32_t)(j / NSETS - 1) & 1u, &abort_flag));
-        if (!ok) break;
-        ptx::tc_fence_after();
-        const uint32_t acc = tmem_base + set * 256u;
-        for (int i = 0; i < w.nkb; ++i) {
-          ok = __all_sync(0xffffffffu, ptx::mbar_wait_a(full0 + 8u * s, ph, &abort_flag));
+        const int nch = min(NCH, w.nkb);
+#pragma unroll 1
+        for (int ch = 0; ch < nch; ++ch, ++j) {
+          const uint32_t set = (uint32_t)(j % NSETS);
+          // the epilogue has drained this set (its use before the last one)
+          if (j >= NSETS) ok = __all_sync(0xffffffffu, ptx::mbar_wait(&acc_empty[set], (uint32_t)(j / NSETS - 1) & 1u, &abort_flag));
           if (!ok) break;
-          const uint32_t more = i > 0 ? 1u : 0u;   // the first MMA of an accumulator overwrites it
-          if (el) {
-            const uint32_t da = lo + (NW * W_BYTES >> 4);
+          ptx::tc_fence_after();
+          const uint32_t acc = tmem_base + set * 256u;
+          const int i0 = ch * w.nkb / nch, i1 = (ch + 1) * w.nkb / nch;   // its k-blocks
+          for (int i = i0; i < i1; ++i) {
+            ok = __all_sync(0xffffffffu, ptx::mbar_wait_a(full0 + 8u * s, ph, &abort_flag));
+            if (!ok) break;
+            const uint32_t more = i > i0 ? 1u : 0u;   // the first MMA of an accumulator overwrites it
+            if (el) {
+              const uint32_t da = lo + (NW * W_BYTES >> 4);
 #pragma unroll
-            for (int kk = 0; kk < kTileK / 16; ++kk) {
-              const uint32_t on = kk > 0 ? 1u : more;
-              if (PAIR) {
-                ptx::umma_bf16_pair_lo(acc, lo + 2 * kk, da + 2 * kk, hi, idesc, on);
-                if (NW == 2) ptx::umma_bf16_pair_lo(acc + 256u, lo + (W_BYTES >> 4) + 2 * kk, da + 2 * kk, hi, idesc, on);
-              } else {
-                ptx::umma_bf16_lo(acc, lo + 2 * kk, da + 2 * kk, hi, idesc, on);
-                if (NW == 2) ptx::umma_bf16_lo(acc + 256u, lo + (W_BYTES >> 4) + 2 * kk, da + 2 * kk, hi, idesc, on);
+              for (int kk = 0; kk < kTileK / 16; ++kk) {
+                const uint32_t on = kk > 1 || (kk == 1 && odd == 0) ? 1u : more, to = acc + (kk & 1 ? odd : 0u);
+                if (PAIR) {
+                  ptx::umma_bf16_pair_lo(to, lo + 2 * kk, da + 2 * kk, hi, idesc, on);
+                  if (NW == 2) ptx::umma_bf16_pair_lo(acc + 256u, lo + (W_BYTES >> 4) + 2 * kk, da + 2 * kk, hi, idesc, on);
+                } else {
+                  ptx::umma_bf16_lo(to, lo + 2 * kk, da + 2 * kk, hi, idesc, on);
+                  if (NW == 2) ptx::umma_bf16_lo(acc + 256u, lo + (W_BYTES >> 4) + 2 * kk, da + 2 * kk, hi, idesc, on);
+                }
               }
+              if (PAIR) ptx::umma_commit_pair_a(empty0 + 8u * s);   // frees the slot in both CTAs
+              else ptx::umma_commit_a(empty0 + 8u * s);
             }
-            if (PAIR) ptx::umma_commit_pair_a(empty0 + 8u * s);   // frees the slot in both CTAs
-            else ptx::umma_commit_a(empty0 + 8u * s);
+            if (++s == (uint32_t)stages) { s = 0; ph ^= 1u; lo = lo0; } else lo += step;
           }
-          if (++s == (uint32_t)stages) { s = 0; ph ^= 1u; lo = lo0; } else lo += step;
-        }
-        if (ok && el) {   // this unit's accumulators are complete (in both CTAs of a pair)
-          if (PAIR) ptx::umma_commit_pair(&acc_full[set]);
-          else ptx::umma_commit(&acc_full[set]);
+          if (!ok) break;
+          if (el) {   // this accumulator is complete (in both CTAs of a pair)
+            if (PAIR) ptx::umma_commit_pair(&acc_full[set]);
+            else ptx::umma_commit(&acc_full[set]);
+          }
         }
       }
     }
@@ -270,37 +286,80 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w0, const __grid_constant__ CU
     // positions of one sequence.
     const int quarter = warp & 3, part = (warp - 2) >> 2;
     const int f = EPI == GEMM_EPI_QKV ? head_feature(quarter, lane) : quarter * 32 + lane;   // feature of the tile in this lane
-    const uint32_t acc_empty_r0 = (PAIR && rank != 0) ? ptx::mapa_shared(ptx::smem_u32(&acc_empty[0]), 0) : 0u;
     const float* cos_sin = p.cos_sin;
     pdl_wait(cos_sin);
     bool ok = true;
-    int j = 0;
-    for (int u = cta; u < n_units && ok; u += n_cta, ++j) {
+    int j = 0;   // accumulators so far
+    for (int u = cta; u < n_units && ok; u += n_cta) {
       const Unit w = unit_of(u);
-      const uint32_t set = (uint32_t)(j % NSETS);
       const int m_base = w.cblk * p.BN, cols = min(p.BN, p.M - m_base);
-      const uint32_t t_lane = tmem_base + set * 256u + ((uint32_t)(quarter * 32) << 16);
+      auto wait_full = [&]() -> uint32_t {   // this warp's lanes of the next accumulator
+        const uint32_t set = (uint32_t)(j % NSETS);
+        ok = __all_sync(0xffffffffu, ptx::mbar_wait(&acc_full[set], (uint32_t)(j / NSETS) & 1u, &abort_flag));
+        ptx::tc_fence_after();
+        return tmem_base + set * 256u + ((uint32_t)(quarter * 32) << 16);
+      };
+      auto drained = [&]() {
+        // the set may be overwritten by the next accumulator but one; the even CTA's MMA issuer waits
+        // for the epilogue warps of both CTAs
+        ptx::tc_fence_before();
+        __syncwarp();
+        if (lane == 0) {
+          const uint32_t set = (uint32_t)(j % NSETS);
+          if (PAIR && rank != 0) ptx::mbar_arrive_remote(ptx::mapa_shared(ptx::smem_u32(&acc_empty[set]), 0));
+          else ptx::mbar_arrive(&acc_empty[set]);
+        }
+        ++j;
+      };
+      if constexpr (EPI == GEMM_EPI_PARTIAL) {
+        float sum[kGemmChunks][16];
+#pragma unroll
+        for (int k = 0; k < kGemmChunks; ++k)
+#pragma unroll
+          for (int i = 0; i < 16; ++i) sum[k][i] = 0.f;
+#pragma unroll 1
+        for (int ch = min(NCH, w.nkb); ch > 0; --ch) {
+          const uint32_t t_lane = wait_full();
+          if (!ok) break;
+#pragma unroll
+          for (int k = 0; k < kGemmChunks; ++k)
+            if (16 * part + 16 * k * kGemmParts < cols) {
+#pragma unroll
+              for (int h = 0; h < 16; h += 8) {   // (eight at a time: sixteen more registers are not there)
+                float v[8];
+                ptx::tmem_ld_32x8(t_lane + 16 * part + 16 * k * kGemmParts + h, v);
+                ptx::tmem_ld_wait();
+#pragma unroll
+                for (int i = 0; i < 8; ++i) sum[k][h + i] += v[i];
+              }
+            }
+          drained();
+        }
+        if (!ok) break;
+#pragma unroll
+        for (int k = 0; k < kGemmChunks; ++k) {
+          const int c0 = 16 * part + 16 * k * kGemmParts;
+          if (c0 >= cols) break;
+          float* dst = p.part + (size_t)w.split * p.part_stride + (size_t)(m_base + c0) * p.N + (size_t)(w.tile * kTileN + f);
+#pragma unroll
+          for (int i = 0; i < 16; ++i, dst += p.N) *dst = sum[k][i];
+        }
+        continue;
+      }
       const bool is_q = w.tile < p.nq, rope = EPI == GEMM_EPI_QKV && w.tile < p.nq + p.nkv;
       float bias_f = 0.f;
       if (EPI == GEMM_EPI_QKV && p.bq != nullptr)
         bias_f = __bfloat162float(is_q ? p.bq[w.tile * 128 + f] : rope ? p.bk[(w.tile - p.nq) * 128 + f]
                                                                        : p.bv[(w.tile - p.nq - p.nkv) * 128 + f]);
-      ok = __all_sync(0xffffffffu, ptx::mbar_wait(&acc_full[set], (uint32_t)(j / NSETS) & 1u, &abort_flag));
-      ptx::tc_fence_after();
+      const uint32_t t_lane = wait_full();
       if (!ok) break;
 #pragma unroll 1
       for (int c0 = 16 * part; c0 < cols; c0 += 16 * kGemmParts) {
         const int m0 = m_base + c0;
-        float v[16];
+        float v[16], v2[16];   // v2: up, or the odd k-steps' sums
         ptx::tmem_ld_32x16(t_lane + c0, v);
-        if (EPI == GEMM_EPI_PARTIAL) {
-          float* dst = p.part + (size_t)w.split * p.part_stride + (size_t)m0 * p.N + (size_t)(w.tile * kTileN + f);
-          ptx::tmem_ld_wait();
-#pragma unroll
-          for (int i = 0; i < 16; ++i) dst[(size_t)i * p.N] = v[i];
-        } else if (EPI == GEMM_EPI_SWIGLU) {
-          float up[16];
-          ptx::tmem_ld_32x16(t_lane + 256u + c0, up);
+        if (EPI == GEMM_EPI_SWIGLU || p.dual) ptx::tmem_ld_32x16(t_lane + 256u + c0, v2);
+        if (EPI == GEMM_EPI_SWIGLU) {
           __nv_bfloat16* dst = p.act + (size_t)m0 * p.N + (size_t)(w.tile * kTileN + f);
           ptx::tmem_ld_wait();
 #pragma unroll
@@ -309,14 +368,29 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w0, const __grid_constant__ CU
             // the fused chain's epilogue; tanh.approx is good to 2^-11, the result goes to bf16)
             float th;
             asm("tanh.approx.f32 %0, %1;" : "=f"(th) : "f"(0.5f * v[i]));
-            v[i] = v[i] * fmaf(0.5f, th, 0.5f) * up[i];
+            v[i] = v[i] * fmaf(0.5f, th, 0.5f) * v2[i];
           }
 #pragma unroll
           for (int i = 0; i < 16; ++i) dst[(size_t)i * p.N] = __float2bfloat16_rn(v[i]);
-        } else if (!rope) {
+          continue;
+        }
+        // rotate-half: the lane 16 on has the other feature of the pair.  Every row has its own factors from the
+        // table, rounded once from fp64: advanced by an angle step from the chunk's first row they were up to 7.7e-7
+        // off instead of 3e-8.
+        float cv[16], sv[16];
+        if (rope) {
+          const int mt = m0 >= p.rows_per_variant ? m0 - p.rows_per_variant : m0;   // (prev variant: same table)
+          const float* cs = cos_sin + (size_t)mt * 128 + (f & 63);
+#pragma unroll
+          for (int i = 0; i < 16; ++i) { cv[i] = __ldg(cs + i * 128); sv[i] = __ldg(cs + i * 128 + 64); }
+        }
+        ptx::tmem_ld_wait();
+        if (p.dual)
+#pragma unroll
+          for (int i = 0; i < 16; ++i) v[i] += v2[i];
+        if (!rope) {
           // V is stored transposed (keys contiguous): 16 consecutive keys of feature row f
           __nv_bfloat16* dst = p.v + (size_t)((w.tile - p.nq - p.nkv) * 128 + f) * p.ldv + m0;
-          ptx::tmem_ld_wait();
 #pragma unroll
           for (int h = 0; h < 2; ++h) {
             uint32_t o[4];
@@ -328,18 +402,9 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w0, const __grid_constant__ CU
             *reinterpret_cast<uint4*>(dst + 8 * h) = make_uint4(o[0], o[1], o[2], o[3]);
           }
         } else {
-          // rotate-half: the lane 16 on has the other feature of the pair.  Every row has its own factors from the
-          // table, rounded once from fp64: advanced by an angle step from the chunk's first row they were up to 7.7e-7
-          // off instead of 3e-8.
-          const int mt = m0 >= p.rows_per_variant ? m0 - p.rows_per_variant : m0;   // (prev variant: same table)
-          const float* cs = cos_sin + (size_t)mt * 128 + (f & 63);
-          float cv[16], sv[16];
-#pragma unroll
-          for (int i = 0; i < 16; ++i) { cv[i] = __ldg(cs + i * 128); sv[i] = __ldg(cs + i * 128 + 64); }
           const float sg = lane < 16 ? -1.f : 1.f;
           const int ld = (is_q ? p.nq : p.nkv) * 128;
           __nv_bfloat16* dst = (is_q ? p.q + w.tile * 128 : p.k + (w.tile - p.nq) * 128) + (size_t)m0 * ld + f;
-          ptx::tmem_ld_wait();
 #pragma unroll
           for (int i = 0; i < 16; ++i) {
             const float y = v[i] + bias_f, other = __shfl_xor_sync(0xffffffffu, y, 16);
@@ -347,14 +412,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w0, const __grid_constant__ CU
           }
         }
       }
-      // the set may be overwritten by the unit after the next; the even CTA's MMA issuer waits
-      // for the epilogue warps of both CTAs
-      ptx::tc_fence_before();
-      __syncwarp();
-      if (lane == 0) {
-        if (PAIR && rank != 0) ptx::mbar_arrive_remote(acc_empty_r0 + 8u * set);
-        else ptx::mbar_arrive(&acc_empty[set]);
-      }
+      drained();
     }
   }
   if (warp == 0 && lane == 0 && rank == 0 && abort_flag != 0) {

@@ -1,5 +1,7 @@
 """What the launch-per-GEMM path (more than 256 activation rows) holds and sums in 32 bits, seen through bf16 outputs:
 results that cancel show an error of 1e-6 of their terms, which the rounding of a full-size result hides."""
+import math
+
 import numpy as np
 import pytest
 import torch
@@ -50,3 +52,51 @@ def test_rotated_keys_have_the_tables_precision():
     over = ((np.abs(got[0] - ref) - half_ulp) / terms).max()
     print("largest error past the rounding to bf16, of the terms:", over)
     assert over <= 2.0 ** -23
+
+
+def _cancelling(rows, K, g):
+    """[rows, K] bf16 numbers: random positive ones whose sum the last 64 take back, exactly."""
+    w = (0.5 + torch.rand(rows, K, generator=g)).to(BF16).double()
+    left = w[:, :K - 64].sum(1)
+    for k in range(K - 64, K):
+        take = left / max(K - 8 - k, 1)
+        w[:, k] = (-take).to(BF16).double()
+        left = left + w[:, k]
+    return w
+
+
+@pytest.mark.parametrize("where", ["qkv", "down"])
+def test_sums_are_taken_in_chains_as_short_as_the_fused_chains(where):
+    """The tensor cores truncate a running fp32 sum at every MMA, so its error grows with the MMAs of one
+    accumulator.  The same sums on both paths, 256 rows (two accumulators a GEMM, and K splits) and 1024 rows: the error
+    of the second may not be larger (a factor 1.25 for other orders; one accumulator over all k shows 4)."""
+    err = {}
+    for tokens in (256, 1024):
+        g = torch.Generator().manual_seed(7)
+        if where == "qkv":
+            # a gain of 171 / 128: the products have 16 bits, their sums more than 24; 128 tiles of 128 features for the
+            # fused chain, too many for it to hand a part of k to other CTAs, 36 for the other path, a unit a worker
+            d, nq, nkv = (4096, 64, 32) if tokens == 256 else (4096, 28, 4)
+            w = _cancelling(256, d, g)
+            wv = torch.zeros(nkv * 128, d)
+            wv[:256] = w.float()
+            _, v = _prefill([dict(wv=wv, norm1=torch.full((d,), 171 / 128))], torch.ones(d), nq, nkv, d, 256, tokens)
+            out, ref = v[0][:2].reshape(256, tokens)[:, 0], w.sum(1).numpy()
+        else:
+            # x = (1, 0, ..): the norm gives 32 in feature 0, gate and up make the activations equal; the down projection
+            # of layer 0 adds cancelling sums to x, whose norm (32 of them) layer 1 hands on as its values
+            d, ff = 1024, 8192
+            gate, up, pick = torch.zeros(ff, d), torch.zeros(ff, d), torch.zeros(256, d)
+            gate[:, 0] = 4.0 / 32
+            up[:, 0] = 0.25451 / 32          # 1 / silu(4)
+            pick[torch.arange(256), torch.arange(256) + 1] = 1.0
+            w = _cancelling(d, ff, g)
+            w[0] = 0
+            emb = torch.zeros(d)
+            emb[0] = 1.0
+            _, v = _prefill([dict(w_gate=gate, w_up=up, w_down=w.float()), dict(wv=pick)], emb, 2, 2, d, ff, tokens)
+            out, ref = v[1].reshape(256, tokens)[:, 0] / 32, w[1:257].sum(1).numpy()
+        err[tokens] = math.sqrt(((out - ref) ** 2).mean()) / w[:257].abs().sum(1).max().item()
+    print(where, err)
+    assert 0 < err[256] < 1e-4
+    assert err[1024] <= 1.25 * err[256]
