@@ -113,6 +113,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w0, const __grid_constant__ CU
   __shared__ uint64_t bar_full[8], bar_empty[8], acc_full[2], acc_empty[2];
   __shared__ uint32_t tmem_base_s;
   __shared__ int abort_flag, late_flag;
+  __shared__ uint32_t fills;             // ring slots that the producer has filled
 
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~static_cast<uintptr_t>(1023));
@@ -170,7 +171,6 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w0, const __grid_constant__ CU
   }
 
   const uint32_t full0 = ptx::smem_u32(&bar_full[0]), empty0 = ptx::smem_u32(&bar_empty[0]);
-  uint32_t fills = 0;   // of the producer: ring slots filled so far
   if (warp == 0) {
     // ---------------- TMA producer ----------------
     // (the whole warp runs the loop and one elected lane issues, as in the MMA issuer)
@@ -204,7 +204,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w0, const __grid_constant__ CU
         if (el) load_w(w, i, (uint32_t)i, ring0 + (uint32_t)(i * stage_bytes));
     }
     pdl_wait();
-    uint32_t s = 0, ph = 0, slot = ring0;
+    uint32_t s = 0, ph = 0, slot = ring0, filled = 0;
     bool ok = true;
     for (int u = cta; u < n_units && ok; u += n_cta) {
       const Unit w = unit_of(u);
@@ -221,10 +221,11 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w0, const __grid_constant__ CU
           if (PAIR) ptx::tma_load_2d_pair_a(slot + NW * W_BYTES, &map_a, bar, kc, arow);
           else ptx::tma_load_2d_a(slot + NW * W_BYTES, &map_a, bar, kc, arow);
         }
-        ++fills;
+        ++filled;
         if (++s == (uint32_t)stages) { s = 0; ph ^= 1u; slot = ring0; } else slot += (uint32_t)stage_bytes;
       }
     }
+    if (el) fills = filled;
   } else if (warp == 1) {
     // ---------------- MMA issuer ----------------
     // The whole warp runs the loop and one elected lane issues: the operands then stay in uniform registers (a
@@ -415,14 +416,14 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w0, const __grid_constant__ CU
       drained();
     }
   }
-  if (warp == 0 && lane == 0 && rank == 0 && abort_flag != 0) {
-    // given up: what is still on its way (for the even CTA's barriers, the odd one's loads too) lands before this
-    // shared memory goes to another CTA, with a limit of its own
+  ptx::tc_fence_before();
+  __syncthreads();
+  if (threadIdx.x == 0 && rank == 0 && abort_flag != 0) {
+    // given up, whichever role it was (all of them have decided by now): what is still on its way (for the even CTA's
+    // barriers, the odd one's loads too) lands before this shared memory goes to another CTA, with a limit of its own
     for (uint32_t n = fills > (uint32_t)stages ? fills - stages : 0; n < fills; ++n)
       ptx::mbar_wait_a(full0 + 8u * (n % stages), (n / stages) & 1u, &late_flag);
   }
-  ptx::tc_fence_before();
-  __syncthreads();
   // neither CTA of a pair leaves while the other may still read its shared memory or signal its
   // barriers
   if (PAIR) ptx::cluster_sync();

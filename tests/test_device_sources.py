@@ -76,3 +76,17 @@ def test_warps_that_meet_in_an_epilogue_give_up_together(name, first, last, meet
     assert waits and all("__all_sync(" in w for w in waits)
     assert bool(re.search(r"EPI_QKV\) ok = ptx::all_agree\([^;]*, 128, ok\);", part)) == meet
     assert ("bar.sync" in src or "all_agree" in src) == meet
+
+
+@pytest.mark.parametrize("name,kernel", [("tc_gemm.cuh", "k_gemm_tc"), ("tc_attn_few.cuh", "k_attn_few")])
+def test_what_is_on_its_way_is_waited_for_when_every_role_has_decided(name, kernel):
+    """A CTA that has given up waits for its TMA writes before it leaves, with a limit of its own.  A producer may be
+    through with its loop when another role gives up: the flag is looked at behind a barrier that all roles come to after
+    their last wait, and before the CTA (or its partner) may leave."""
+    body = _kernel(name, kernel)
+    drain = body.index("late_flag)")
+    flag = body.rindex("abort_flag != 0)", 0, drain)
+    role_waits = body.rindex("abort_flag)", 0, flag)
+    assert "__syncthreads();" in body[role_waits:flag]
+    leave = body.find("cluster_sync()", drain)
+    assert leave == -1 or "__syncthreads();" not in body[drain:leave]
