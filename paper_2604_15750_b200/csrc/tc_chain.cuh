@@ -335,7 +335,7 @@ __device__ __forceinline__ void chain_gemm(ChainCtx& c, const ChainParams& p, co
           const uint32_t par = (c.fill_bits >> ps) & 1u;
           c.fill_bits ^= 1u << ps;
           ok = ptx::mbar_wait_a(empty0 + 8u * ps, par ^ 1u, c.abort_flag);
-          if (!ok) break;
+          if (!ok) { c.fill_bits ^= 1u << ps; break; }   // (not filled)
           // the bytes of both CTAs are credited to the even CTA's barrier, which its MMA issuer
           // waits on
           if (c.rank == 0) ptx::mbar_expect_tx_a(full0 + 8u * ps, 2u * (uint32_t)slot_bytes);
@@ -603,7 +603,7 @@ k_dense_chain(const __grid_constant__ ChainMaps maps, const ChainParams p) {
   extern __shared__ uint8_t smem_raw[];
   __shared__ uint64_t bar_full[8], bar_empty[8], bar_acc_full, bar_acc_empty, bar_norm;
   __shared__ uint32_t tmem_base_s;
-  __shared__ int abort_flag;
+  __shared__ int abort_flag, late_flag;
   __shared__ float red[kChainThreads / 32];
 
   ChainCtx c;
@@ -621,6 +621,7 @@ k_dense_chain(const __grid_constant__ ChainMaps maps, const ChainParams p) {
     // an earlier kernel of this step gave up: run through without touching anything (every CTA
     // still reaches the cluster barriers below)
     abort_flag = (*reinterpret_cast<volatile int32_t*>(p.status) != 0) ? 1 : 0;
+    late_flag = 0;
     for (int i = 0; i < 8; ++i) { ptx::mbar_init(&bar_full[i], 1); ptx::mbar_init(&bar_empty[i], 1); }
     ptx::mbar_init(&bar_acc_full, 1);
     ptx::mbar_init(&bar_acc_empty, kChainThreads);
@@ -706,6 +707,13 @@ k_dense_chain(const __grid_constant__ ChainMaps maps, const ChainParams p) {
 
   ptx::tc_fence_before();
   __syncthreads();
+  if (threadIdx.x == 0 && abort_flag != 0) {
+    // given up, whichever role it was: the copies still on their way land before this shared memory goes to another
+    // CTA, with a limit of its own.  The last fill of every ring slot (for the even CTA's barriers, the odd one's loads
+    // too; a slot never filled is no wait), the last rows of a norm.
+    for (int i = 0; i < 8 && c.rank == 0; ++i) ptx::mbar_wait(&bar_full[i], ((c.fill_bits >> i) & 1u) ^ 1u, &late_flag);
+    if (c.norm_uses > 0) ptx::mbar_wait(&bar_norm, (c.norm_uses - 1) & 1u, &late_flag);
+  }
   // neither CTA of a pair leaves while the other may still read its shared memory or signal its
   // barriers
   ptx::cluster_sync();
