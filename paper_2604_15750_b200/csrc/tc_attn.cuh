@@ -216,7 +216,8 @@ k_attn_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
   __shared__ uint64_t q_full, k_full[kAttnStagesK], k_empty[kAttnStagesK], v_loc[kAttnStagesV],
       s_full[3], p_full[3], pv_done[3], o_done, m_ready;
   __shared__ uint32_t tmem_base_s;
-  __shared__ int abort_flag, again_flag;
+  __shared__ int abort_flag, again_flag, late_flag;
+  __shared__ int k_loads, v_loads;  // tiles that the two producers have asked for, over both passes
   __shared__ float m_row[128];     // the rows' reference points of the first pass
   __shared__ float xl[3][128];     // [slot][row]: sum of the probabilities of the slot's tiles
   __shared__ float xm[3][128];     // [slot][row]: maximum raw score of the slot's tiles
@@ -243,7 +244,7 @@ k_attn_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
   const int T = un.T;
 
   if (threadIdx.x == 0) {
-    abort_flag = 0; again_flag = 0;
+    abort_flag = 0; again_flag = 0; late_flag = 0; k_loads = 0; v_loads = 0;
     ptx::mbar_init(&q_full, 1);
     for (int i = 0; i < kAttnStagesK; ++i) { ptx::mbar_init(&k_full[i], 1); ptx::mbar_init(&k_empty[i], 1); }
     for (int i = 0; i < kAttnStagesV; ++i) ptx::mbar_init(&v_loc[i], 1);
@@ -304,6 +305,7 @@ k_attn_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
           const AttnTile t = attn_tile(un, j);
           prefetch_k(j + kAttnStagesK + kAttnPrefetch);
           if (!ptx::mbar_wait(&k_empty[s], (((uint32_t)(J / kAttnStagesK)) & 1u) ^ 1u, &abort_flag)) break;
+          k_loads = J + 1;
           uint8_t* dst = Ks + (size_t)s * 2 * kSub;
           ptx::mbar_expect_tx(&k_full[s], 2 * kSub);
           if (t.is_ctx) {
@@ -335,6 +337,7 @@ k_attn_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
           // the slot held tile J - 2: free once its P V has completed
           if (J >= kAttnStagesV &&
               !ptx::mbar_wait(&pv_done[(J - 2) % 3], ((uint32_t)(J - 2) / 3u) & 1u, &abort_flag)) break;
+          v_loads = J + 1;
           uint8_t* dst = Vs + (size_t)s * 2 * kSub;
           ptx::mbar_expect_tx(&v_loc[s], 2 * kSub);
           if (t.is_ctx) {
@@ -571,6 +574,14 @@ k_attn_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
       }
     }
     break;
+  }
+  if (threadIdx.x == 0 && abort_flag != 0) {
+    // given up: what is still on its way lands before another CTA gets this shared memory (with a limit of its own)
+    ptx::mbar_wait(&q_full, 0, &late_flag);
+    for (int J = max(0, k_loads - kAttnStagesK); J < k_loads; ++J)
+      ptx::mbar_wait(&k_full[J % kAttnStagesK], (uint32_t)(J / kAttnStagesK) & 1u, &late_flag);
+    for (int J = max(0, v_loads - kAttnStagesV); J < v_loads; ++J)
+      ptx::mbar_wait(&v_loc[J % kAttnStagesV], (uint32_t)(J / kAttnStagesV) & 1u, &late_flag);
   }
   ptx::tc_fence_before();
   __syncthreads();
