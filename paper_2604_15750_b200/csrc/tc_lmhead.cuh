@@ -45,7 +45,8 @@ k_lmhead_tc(const __grid_constant__ CUtensorMap map_h, const __grid_constant__ C
   extern __shared__ uint8_t smem_raw[];
   __shared__ uint64_t bar_full[8], bar_empty[8], acc_full[2], acc_empty[2];
   __shared__ uint32_t tmem_base_s;
-  __shared__ int abort_flag;
+  __shared__ int abort_flag, late_flag;
+  __shared__ uint32_t fills;   // ring slots that the producer has filled
   __shared__ float xch[2][64 * 33];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~static_cast<uintptr_t>(1023));
@@ -62,7 +63,7 @@ k_lmhead_tc(const __grid_constant__ CUtensorMap map_h, const __grid_constant__ C
   const int G = p.m.G, nv = p.m.nv;
 
   if (threadIdx.x == 0) {
-    abort_flag = 0;
+    abort_flag = 0; late_flag = 0; fills = 0;
     for (int i = 0; i < stages; ++i) { ptx::mbar_init(&bar_full[i], 1); ptx::mbar_init(&bar_empty[i], 1); }
     for (int i = 0; i < 2; ++i) { ptx::mbar_init(&acc_full[i], 1); ptx::mbar_init(&acc_empty[i], 128); }
     ptx::fence_barrier_init();
@@ -86,7 +87,7 @@ k_lmhead_tc(const __grid_constant__ CUtensorMap map_h, const __grid_constant__ C
       const uint32_t ring0 = ptx::smem_u32(smem);
       const uint32_t full0 = ptx::smem_u32(&bar_full[0]), empty0 = ptx::smem_u32(&bar_empty[0]);
       const uint64_t pol_w = ptx::l2_policy_evict_first();
-      uint32_t s = 0, ph = 0, slot = ring0;
+      uint32_t s = 0, ph = 0, slot = ring0, filled = 0;
       bool ok = true;
       for (int q = 0; q < my_pairs && ok && !p.stall; ++q) {
         // second tile of the pair may lie beyond the vocabulary: the load is zero-filled there
@@ -102,9 +103,11 @@ k_lmhead_tc(const __grid_constant__ CUtensorMap map_h, const __grid_constant__ C
           ptx::tma_load_2d_a(slot, &map_h, bar, kb * 64, grp * nv * G);
           ptx::tma_load_2d_hint_a(slot + 128 * 64 * 2, &map_w, bar, kb * 64, vrow0, pol_w);
           if (two) ptx::tma_load_2d_hint_a(slot + 2 * 128 * 64 * 2, &map_w, bar, kb * 64, vrow1, pol_w);
+          ++filled;
           if (++s == (uint32_t)stages) { s = 0; ph ^= 1u; slot = ring0; } else slot += (uint32_t)kLmStageBytes;
         }
       }
+      fills = filled;
     }
   } else if (warp == 1) {
     if (lane == 0) {
@@ -226,6 +229,12 @@ k_lmhead_tc(const __grid_constant__ CUtensorMap map_h, const __grid_constant__ C
   }
   ptx::tc_fence_before();
   __syncthreads();
+  if (threadIdx.x == 0 && abort_flag != 0) {
+    // given up, whichever role it was: what is still on its way lands before this shared memory goes to another CTA,
+    // with a limit of its own
+    for (uint32_t n = fills > (uint32_t)stages ? fills - stages : 0; n < fills; ++n)
+      ptx::mbar_wait(&bar_full[n % stages], (n / stages) & 1u, &late_flag);
+  }
   if (warp == 1) {
     ptx::tc_fence_after();
     ptx::tmem_dealloc(tmem_base, 512);

@@ -79,7 +79,7 @@ def test_warps_that_meet_in_an_epilogue_give_up_together(name, first, last, meet
 
 
 @pytest.mark.parametrize("name,kernel", [("tc_gemm.cuh", "k_gemm_tc"), ("tc_attn_few.cuh", "k_attn_few"), ("tc_chain.cuh", "k_dense_chain"),
-                                         ("tc_attn.cuh", "k_attn_tc")])
+                                         ("tc_attn.cuh", "k_attn_tc"), ("tc_lmhead.cuh", "k_lmhead_tc")])
 def test_what_is_on_its_way_is_waited_for_when_every_role_has_decided(name, kernel):
     """A CTA that has given up waits for its TMA writes before it leaves, with a limit of its own.  A producer may be
     through with its loop when another role gives up: the flag is looked at behind a barrier that all roles come to after
