@@ -634,8 +634,8 @@ k_dense_chain(const __grid_constant__ ChainMaps maps, const ChainParams p) {
     ptx::prefetch_tmap(&maps.wo_n);
   }
   if (c.warp == 1) {
-    ptx::tmem_alloc(&tmem_base_s, 512);
-    ptx::tmem_relinquish();
+    ptx::tmem_alloc(&tmem_base_s, 512, true);
+    ptx::tmem_relinquish(true);
   }
   ptx::tc_fence_before();
   __syncthreads();
@@ -719,7 +719,7 @@ k_dense_chain(const __grid_constant__ ChainMaps maps, const ChainParams p) {
   ptx::cluster_sync();
   if (c.warp == 1) {
     ptx::tc_fence_after();
-    ptx::tmem_dealloc(c.tmem_base, 512);
+    ptx::tmem_dealloc(c.tmem_base, 512, true);
   }
   if (threadIdx.x == 0 && abort_flag) atomicExch(p.status, DC_ERR_TIMEOUT);
 }

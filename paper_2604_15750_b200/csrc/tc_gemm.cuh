@@ -155,8 +155,8 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w0, const __grid_constant__ CU
     if (EPI == GEMM_EPI_QKV) ptx::prefetch_tmap(&map_w2);
   }
   if (warp == 1) {
-    ptx::tmem_alloc(&tmem_base_s, tmem_cols);
-    ptx::tmem_relinquish();
+    ptx::tmem_alloc(&tmem_base_s, tmem_cols, PAIR);
+    ptx::tmem_relinquish(PAIR);
   }
   ptx::tc_fence_before();
   __syncthreads();
@@ -429,7 +429,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w0, const __grid_constant__ CU
   if (PAIR) ptx::cluster_sync();
   if (warp == 1) {
     ptx::tc_fence_after();
-    ptx::tmem_dealloc(tmem_base, tmem_cols);
+    ptx::tmem_dealloc(tmem_base, tmem_cols, PAIR);
   }
   if (threadIdx.x == 0 && abort_flag && p.status) atomicExch(p.status, DC_ERR_TIMEOUT);
 }

@@ -91,3 +91,19 @@ def test_what_is_on_its_way_is_waited_for_when_every_role_has_decided(name, kern
     assert "__syncthreads();" in body[role_waits:flag]
     leave = body.find("cluster_sync()", drain)
     assert leave == -1 or "__syncthreads();" not in body[drain:leave]
+
+
+@pytest.mark.parametrize("name,kernel", [("tc_gemm.cuh", "k_gemm_tc"), ("tc_chain.cuh", "k_dense_chain"), ("tc_lmhead.cuh", "k_lmhead_tc"),
+                                         ("tc_attn.cuh", "k_attn_tc"), ("tc_attn_few.cuh", "k_attn_few")])
+def test_the_tcgen05_instructions_of_a_kernel_have_one_cta_group(name, kernel):
+    """Pair MMAs and commits go with an allocation, a relinquished permit and a release of cta_group::2, and those
+    of a CTA alone with cta_group::1; the pair's release comes behind a cluster barrier."""
+    src = re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, name)).read())
+    body = _kernel(name, kernel)
+    pair = bool(re.search(r"umma_\w*pair", src))
+    both = pair and bool(re.search(r"umma_(bf16_lo|bf16|commit|commit_a)\(", src))    # a template with both
+    want = "PAIR" if both else "true" if pair else ""
+    calls = re.findall(r"ptx::tmem_(?:alloc|relinquish|dealloc)\([^;]*?(PAIR|true|)\);", body)
+    assert calls == [want] * 3
+    if pair:
+        assert "cluster_sync()" in body[:body.index("tmem_dealloc")].rsplit("__syncthreads();", 1)[1]
