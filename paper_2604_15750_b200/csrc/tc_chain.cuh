@@ -705,6 +705,13 @@ k_dense_chain(const __grid_constant__ ChainMaps maps, const ChainParams p) {
     }
   }
 
+  if (c.warp == 0) {
+    // the commits that handed the last ring slots back arrive in both CTAs of the pair: neither leaves before they have
+    // (a lane a slot; one that was never filled is no wait)
+    const uint32_t bits = __shfl_sync(0xffffffffu, c.fill_bits, 0);
+    if (c.lane < 8 && abort_flag == 0) ptx::mbar_wait(&bar_empty[c.lane], ((bits >> c.lane) & 1u) ^ 1u, &abort_flag);
+    __syncwarp();
+  }
   ptx::tc_fence_before();
   __syncthreads();
   if (threadIdx.x == 0 && abort_flag != 0) {

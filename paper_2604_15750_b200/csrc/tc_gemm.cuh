@@ -225,6 +225,9 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w0, const __grid_constant__ CU
         if (++s == (uint32_t)stages) { s = 0; ph ^= 1u; slot = ring0; } else slot += (uint32_t)stage_bytes;
       }
     }
+    // The commits that hand the last slots back arrive in both CTAs of a pair: neither leaves before they have (a lane a slot).
+    if (ok) ok = __all_sync(0xffffffffu, lane >= min((int)filled, stages) ||
+                                             ptx::mbar_wait_a(empty0 + 8u * lane, ((filled - lane - 1u) / stages) & 1u, &abort_flag));
     if (el) fills = filled;
   } else if (warp == 1) {
     // ---------------- MMA issuer ----------------

@@ -107,3 +107,13 @@ def test_the_tcgen05_instructions_of_a_kernel_have_one_cta_group(name, kernel):
     assert calls == [want] * 3
     if pair:
         assert "cluster_sync()" in body[:body.index("tmem_dealloc")].rsplit("__syncthreads();", 1)[1]
+
+
+@pytest.mark.parametrize("name,kernel,slots", [("tc_gemm.cuh", "k_gemm_tc", "empty0"), ("tc_chain.cuh", "k_dense_chain", "bar_empty")])
+def test_no_cta_of_a_pair_leaves_before_its_ring_slots_have_been_handed_back(name, kernel, slots):
+    """The commit behind a k-block arrives on the slot's barrier in both CTAs.  Nothing else waits for the last of these
+    arrivals (the accumulator's is another one), so every slot is waited for, a lane each, before the last barriers."""
+    body = _kernel(name, kernel)
+    tail = [m.start() for m in re.finditer(r"mbar_wait(?:_a)?\(&?" + slots + r"(?: \+ 8u \* lane|\[c\.lane\])", body)]
+    assert len(tail) == 1
+    assert "cluster_sync()" in body[tail[0]:] and "__syncthreads();" in body[tail[0]:body.index("late_flag)", tail[0])]
