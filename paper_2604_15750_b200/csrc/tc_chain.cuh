@@ -99,7 +99,10 @@ constexpr int kChainTileK = 64;
 // attention runs.  Gate / up, down, QKV 4 / 8 / 8 against 4 / 4 / 4 against the same issued before the
 // epilogue: carried b1 (96 rows) 4161 / 4192 / 4252 us, denoise b1 (16 rows) 3710 / 3728 / 3766; boundary b1
 // (192 rows) 4715 / 4660 / 4696; 16 / 12 / 16: +1.5% there.
-constexpr int kPfGateUp = 4, kPfOproj = 64;
+// Nothing waits for the O projection's before the launch ends, and their tensor map is one of its parameters: at most 16 boxes,
+// all there are for LLaDA-8B and Dream-7B, queued behind the CTA's last loads and with its MMAs and epilogue (7 k
+// clocks) still to come.  (Through a map in device memory, acquired before its use: 0.4 .. 0.9% of a step slower.)
+constexpr int kPfGateUp = 4, kPfOproj = 16;
 __device__ __forceinline__ int chain_pf_deep(int BN) { return BN <= 128 ? 8 : 4; }   // down, QKV
 
 struct ChainCtx {
