@@ -41,6 +41,10 @@ __device__ unsigned long long g_simt_wait_ns = 2000000000ull;
 struct Group { int id, t, warp, lane, vid, nv; unsigned char* smem; };
 __device__ __forceinline__ void gsync(const Group& g) { asm volatile("bar.sync %0, 256;" ::"r"(g.id + 1) : "memory"); }
 
+// x, for the compiler a new value: what is derived from it is worked out again where it stands instead of being held in
+// registers over a whole phase.  (The 32 sums of a tile leave none for that: 2 to 4 spilled ones cost 1.5% of a step.)
+__device__ __forceinline__ int afresh(int x) { asm volatile("" : "+r"(x)); return x; }
+
 template <typename T> __device__ __forceinline__ void ldcg4(const T* src, float (&v)[4]);
 template <> __device__ __forceinline__ void ldcg4<float>(const float* src, float (&v)[4]) {
   const float4 t = __ldcg(reinterpret_cast<const float4*>(src));
@@ -177,11 +181,6 @@ __device__ __forceinline__ bool gemm_phase(const SimtStep<T>& p, const FuseGemm<
   const int cb = split ? gr.id * (chunks / 2) : 0, ce = split && gr.id == 0 ? chunks / 2 : chunks;
   const int vid = split ? (int)blockIdx.x : gr.vid, nv = split ? (int)gridDim.x : gr.nv;
   const int per = MT <= nv ? nv / MT : 1;   // groups (CTAs) on a row tile
-  const int pr = gr.t / PPR, pk = (gr.t % PPR) * PIECE;         // this thread's piece of a chunk: row, column
-  // A warp has 32 k of a chunk, half of it 16 of them, a lane 4 x 4 outputs: rows ty + 4 i, columns tx + 4 j.  (What a
-  // tile costs is the return path of its shared-memory loads, 4 clocks each: 32 a lane, and 48 with all 32 k in one
-  // lane and 4 x 2 outputs.)
-  const int ty = (gr.lane >> 2) & 3, tx = gr.lane & 3, ko = gr.warp * (KC / 8) + (gr.lane >> 4) * (KC / 16);
   bool waited = false;
 #pragma unroll 1
   for (int mt = MT <= nv ? vid % MT : vid; !waited || mt < MT; mt += (MT <= nv ? MT : nv)) {
@@ -192,6 +191,7 @@ __device__ __forceinline__ bool gemm_phase(const SimtStep<T>& p, const FuseGemm<
     // A thread copies one column piece of rows pr, pr + RS, .. of a chunk: of W the first eight rows and the other
     // eight are runs of their own (their partner features, or the same rows of the other matrix).
     auto issue = [&](bool with_w, bool with_a, int u, int c, int s) {
+      const int t = afresh(gr.t), pr = t / PPR, pk = (t % PPR) * PIECE;   // this thread's piece of a chunk: row, column
       const int k0 = c * KC + pk, full = max(0, min(16, (g.K - k0) * (int)sizeof(T)));
       if (with_w) {
         const T *wa = g.w0, *wb = g.w0;
@@ -252,11 +252,12 @@ __device__ __forceinline__ bool gemm_phase(const SimtStep<T>& p, const FuseGemm<
       T* dst = as + (size_t)r * apitch;
       const float* xr = nullptr;
       T *g0 = nullptr, *g1 = nullptr;
+      const int l = afresh(gr.lane & 15);
       bool norm = true;
-      if (g.src == SRC_LM) norm = lm_row<T>(p, row, dst, chunks * KC, first == 0, gr.lane & 15, xr, g0, g1);
+      if (g.src == SRC_LM) norm = lm_row<T>(p, row, dst, chunks * KC, first == 0, l, xr, g0, g1);
       else if (row < g.M) xr = p.x + (size_t)row * p.d;
       if (__any_sync(0xffffffffu, norm || g1 != nullptr))       // both halves of the warp take part
-        norm_row<T>(xr, g.gain, p.eps, p.d, norm ? dst : nullptr, chunks * KC, g0, g1, gr.lane & 15);
+        norm_row<T>(xr, g.gain, p.eps, p.d, norm ? dst : nullptr, chunks * KC, g0, g1, l);
     }
     f2 acc[4][4];
     float old = 0.f;             // residual value that the epilogue adds to
@@ -278,6 +279,10 @@ __device__ __forceinline__ bool gemm_phase(const SimtStep<T>& p, const FuseGemm<
         for (int i = 0; i < 4; ++i) acc[i][0] = acc[i][1] = acc[i][2] = acc[i][3] = 0ull;
         if (epi == EPI_ADD_F32 && m0 + er < g.M && u * NC + ec < g.N) old = __ldcg(g.C + (size_t)(m0 + er) * g.ldc + u * NC + ec);
       }
+      // A warp has 32 k of a chunk, half of it 16 of them, a lane 4 x 4 outputs: rows ty + 4 i, columns tx + 4 j.  (What a
+      // tile costs is the return path of its shared-memory loads, 4 clocks each: 32 a lane, and 48 with all 32 k in one
+      // lane and 4 x 2 outputs.)
+      const int t = afresh(gr.t), ty = (t >> 2) & 3, tx = t & 3, ko = (t >> 5) * (KC / 8) + ((t >> 4) & 1) * (KC / 16);
       const T* wp = ring_w + ((size_t)slot * NC + tx) * PITCH + ko;
       const T* ap = (stream_a ? as + (size_t)slot * 16 * PITCH : as + c * KC) + ty * apitch + ko;
 #pragma unroll 1

@@ -2,8 +2,12 @@
 takes a rare order of events."""
 import os
 import re
+import shutil
+import subprocess
 
 import pytest
+
+from paper_2604_15750_b200 import build
 
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2604_15750_b200", "csrc")
 
@@ -117,3 +121,13 @@ def test_no_cta_of_a_pair_leaves_before_its_ring_slots_have_been_handed_back(nam
     tail = [m.start() for m in re.finditer(r"mbar_wait(?:_a)?\(&?" + slots + r"(?: \+ 8u \* lane|\[c\.lane\])", body)]
     assert len(tail) == 1
     assert "cluster_sync()" in body[tail[0]:] and "__syncthreads();" in body[tail[0]:body.index("late_flag)", tail[0])]
+
+
+@pytest.mark.skipif(shutil.which(build._nvcc()) is None, reason="no nvcc")
+def test_the_fused_cuda_core_step_keeps_its_sums_in_registers(tmp_path):
+    """512 threads of 128 registers and 32 sums a thread: nothing is left over, and a spill is 1.5% of a step."""
+    r = subprocess.run([build._nvcc(), *build.NVCC_FLAGS, "-Xptxas", "-v", "-c", os.path.join(CSRC, "simt_step.cu"), "-o",
+                        str(tmp_path / "x.o")], stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)
+    assert r.returncode == 0, r.stdout
+    of_step = re.findall(r"Function properties for \S*k_simt_step\S*\n.*?(\d+) bytes spill stores, (\d+) bytes spill loads", r.stdout)
+    assert of_step == [("0", "0")] * 2, r.stdout
