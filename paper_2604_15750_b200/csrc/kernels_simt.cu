@@ -87,6 +87,8 @@ __global__ void __launch_bounds__(128) k_step_begin(const T* __restrict__ embed,
   cos_sin[(size_t)br * hd + half + i] = (float)sn;
 }
 
+// (An ordinary launch: what comes before the step in the stream has completed when it starts.  The GEMMs' early weight
+// loads rely on that: pdl.cuh.)
 template <typename T>
 void launch_step_begin(const T* embed, const int32_t* last_ids, const int32_t* win_ids, int max_last, int max_window,
                        int mask_id, int vocab, int d, const SeqMeta& m, float* x, int32_t* status, int head_dim,

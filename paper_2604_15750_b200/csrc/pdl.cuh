@@ -2,7 +2,9 @@
 // start while the one before it in the stream still runs: its blocks take the SMs that become free, set
 // up barriers, TMEM and tensor maps, and wait in pdl_wait() until everything before has completed and is
 // visible.  Every kernel launched this way calls pdl_wait() in all of its blocks before it touches global
-// memory (so that completion is transitive).  pdl_trigger() only allows the next kernel's blocks to be scheduled,
+// memory that a kernel of the step writes (so that completion is transitive).  k_gemm_tc loads weights before: no kernel of a
+// sequence writes them, and a sequence starts with k_step_begin, a launch without the attribute, which runs after all that
+// was in the stream before it (weights written there included).  pdl_trigger() only allows the next kernel's blocks to be scheduled,
 // once every block has called it or ended; a kernel without it counts as triggered when it ends.  A kernel that
 // allocates TMEM triggers behind the allocation: a block of the next kernel that fitted beside one of these
 // would take the columns first and hold them in pdl_wait(), whose end is behind the allocation that waits for

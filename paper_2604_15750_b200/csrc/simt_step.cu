@@ -4,8 +4,8 @@
 // third of that launch, ramp and drain, and the host needs 4 us for every launch.  Here the phases of
 // all layers, the LM head, the signals, the cross log-probs and the boundary rule run in one kernel
 // of one CTA per SM, with a counting grid barrier between phases.  Two-layer fp32 model (d 256, 96 rows,
-// vocab 4096): 22 launches and 157 us per step -> 3 launches and 102 us; a generation step 183 -> 103 us.
-// What is left (clocks of a step's 175 k): 13 barriers, 4100 .. 5300 from the arrival to the first use where the weights
+// vocab 4096): 22 launches and 157 us per step -> 3 launches and 100 us; a generation step 183 -> 103 us.
+// What is left (clocks of a step's 175 k): 12 barriers, 4100 .. 5300 from the arrival to the first use where the weights
 // of two chunks are started in between (4490 of it, the poll behind it 700) and 2500 where nothing is; the norm
 // of 16 rows 3700; a tile 3200, with its epilogue 4500.  The first context of a process on a
 // device loads the kernel when it is made (dc_create 7..16 ms instead of 0.9).

@@ -102,7 +102,7 @@ struct TcState {
   int M_max = 0;
   std::vector<LayerMaps> layers;
   std::vector<const void*> bq, bk, bv;   // per-layer q / k / v projection biases (empty: none)
-  std::map<int, ActMaps> act_maps;  // keyed by BN
+  std::map<int, ActMaps> act_maps;  // keyed by the rows of a box
   std::vector<void*> allocs;
   __nv_bfloat16 *a_buf = nullptr;  // borrowed: the normed activations of the scheduler
   __nv_bfloat16 *q = nullptr, *k = nullptr, *v = nullptr, *o = nullptr, *act = nullptr;
@@ -298,19 +298,20 @@ int tc_create(const dc_config& g, cudaStream_t s, int M_max, int Mlm_max,
   return DC_OK;
 }
 
-static int get_act_maps(TcState* t, const __nv_bfloat16* a, int BN, ActMaps** out) {
-  auto it = t->act_maps.find(BN);
+// The activation operands with a box of `rows` rows
+static int get_act_maps(TcState* t, const __nv_bfloat16* a, int rows, ActMaps** out) {
+  auto it = t->act_maps.find(rows);
   if (it == t->act_maps.end() || t->a_buf != a) {
     const dc_config& g = t->g;
     ActMaps am;
     const uint64_t hq = (uint64_t)g.n_q_heads * g.head_dim;
-    bool ok = make_map_2d(&am.a, a, t->M_max, g.d_model, BN) &&
-              make_map_2d(&am.o, t->o, t->M_max, hq, BN) &&
-              make_map_2d(&am.act, t->act, t->M_max, g.d_ff, BN);
+    bool ok = make_map_2d(&am.a, a, t->M_max, g.d_model, rows) &&
+              make_map_2d(&am.o, t->o, t->M_max, hq, rows) &&
+              make_map_2d(&am.act, t->act, t->M_max, g.d_ff, rows);
     if (!ok) return tfail(t, DC_ERR_CUDA, "activation tensor map encoding failed");
     if (t->a_buf != a) t->act_maps.clear();
     t->a_buf = const_cast<__nv_bfloat16*>(a);
-    it = t->act_maps.insert_or_assign(BN, am).first;
+    it = t->act_maps.insert_or_assign(rows, am).first;
   }
   *out = &it->second;
   return DC_OK;
@@ -365,9 +366,9 @@ static int launch_gemm(TcState* t, const CUtensorMap& w0, const CUtensorMap& w1,
   return DC_OK;
 }
 
+// K splits of the dense chain's projections back to d: enough CTAs to cover the SMs, at least 8 k-blocks each; `tiles`
+// counts the CTAs of one split
 static int pick_split(int tiles, int KB, int max_split) {
-  // enough CTAs to cover the SMs, at least 8 k-blocks each; `tiles` counts every CTA of one
-  // split (weight tiles x activation column blocks)
   int s = 148 / tiles;
   if (s < 1) s = 1;
   if (s > max_split) s = max_split;

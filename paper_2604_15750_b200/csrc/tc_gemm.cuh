@@ -30,7 +30,7 @@
 // together and elect a lane); the rotation through shared memory by four warps took 27 us a unit against 25 of
 // MMAs (shuffles take 3.5: the weight rows arrive in an order that puts the two features of a pair into one warp); gate /
 // up stood still for 11 us of every 51 while four warps drained the accumulators (sixteen take 3).  QKV 83 -> 71
-// us, gate / up 153 -> 133; the whole prefill 15.13 -> 14.01 ms, eight boundary steps 37.4 -> 34.2, 2 x 160 rows 22% less.
+// us, gate / up 153 -> 133; the whole prefill 15.13 -> 14.01 ms, eight boundary steps 37.4 -> 34.2.
 #pragma once
 #include "kernels.h"
 #include "pdl.cuh"
