@@ -166,11 +166,12 @@ def test_fused_chain_at_its_row_limits(last, win, influence, rows):
     eng.close()
 
 
-@pytest.mark.parametrize("n_q,n_kv", [(40, 20), (28, 4), (6, 2)])
-def test_fused_chain_qkv_helper_layouts(n_q, n_kv):
-    """The balanced QKV phase with 80 tiles (34 helper pairs, six of which serve two tile pairs),
-    36 tiles (Dream's head counts: one tile pair per helper, helpers left over) and 10 tiles."""
-    wl = _wl(1, n_q=n_q, n_kv=n_kv, d=512, ff=1024, vocab=2048, layers=2)
+@pytest.mark.parametrize("n_q,n_kv,d", [(40, 20, 512), (28, 4, 512), (6, 2, 512), (40, 20, 2560), (28, 4, 1280)])
+def test_fused_chain_qkv_helper_layouts(n_q, n_kv, d):
+    """The QKV phase with 80, 36 (Dream's head counts) and 10 tiles.  Helper CTA pairs hand their sums over in the
+    workspace of the K splits, which has room for that from d = 32 * tiles on: at d 512 only the 10 tiles have helpers; at
+    d 2560 80 tiles have 34 helper pairs, six of which serve two tile pairs, at d 1280 36 have one each and some left over."""
+    wl = _wl(1, n_q=n_q, n_kv=n_kv, d=d, ff=1024, vocab=2048, layers=2)
     case = Case(wl)
     eng = case.make_engine()
     gpu, ora = case.run_gpu(eng), case.run_oracle()
