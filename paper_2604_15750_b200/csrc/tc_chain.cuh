@@ -369,6 +369,7 @@ __device__ __forceinline__ void chain_gemm(ChainCtx& c, const ChainParams& p, co
       const uint32_t mfull0 = ptx::smem_u32(&c.full[0]), mempty0 = ptx::smem_u32(&c.empty[0]);
       const uint32_t desc_hi = ptx::smem_desc_hi32(), lo0 = ptx::smem_desc_lo(ptx::smem_u32(c.ring));
       const uint32_t up = (uint32_t)tile_bytes >> 4, act = (uint32_t)(nw * tile_bytes) >> 4, step = (uint32_t)slot_bytes >> 4;
+      const int refills = w.kb1 - stages;   // (QKV, which ends a launch) the k-blocks before it
       uint32_t ms = 0, lo = lo0;
       if (c.mma_units > 0) {  // the epilogue has drained both accumulators of the last unit
         ok = __all_sync(0xffffffffu, ptx::mbar_wait(c.acc_empty, (c.mma_units - 1) & 1u, c.abort_flag));   // (the lanes go on together)
@@ -392,7 +393,9 @@ __device__ __forceinline__ void chain_gemm(ChainCtx& c, const ChainParams& p, co
             for (int kk = 0; kk < kChainTileK / 16; ++kk)
               ptx::umma_bf16_pair_lo(c.tmem_base + (kk & 1) * 256, lo + 2 * kk, lo + act + 2 * kk, desc_hi, idesc, kk > 1 ? 1u : more);
           }
-          ptx::umma_commit_pair_a(mempty0 + 8u * ms);   // frees the slot in both CTAs
+          // Frees the slot in both CTAs, if it is filled once more: an arrival that nobody waits for could come when the
+          // partner has left.
+          if (EPI != CEPI_QKV || kb < refills) ptx::umma_commit_pair_a(mempty0 + 8u * ms);
         }
         if (++ms == (uint32_t)stages) { ms = 0; lo = lo0; } else lo += step;
       }
@@ -708,9 +711,8 @@ k_dense_chain(const __grid_constant__ ChainMaps maps, const ChainParams p) {
     }
   }
 
-  if (c.warp == 0) {
-    // the commits that handed the last ring slots back arrive in both CTAs of the pair: neither leaves before they have
-    // (a lane a slot; one that was never filled is no wait)
+  if (!has_qkv && c.warp == 0) {
+    // (the step's last launch, which ends with a projection: there these arrivals are waited for, a lane a slot)
     const uint32_t bits = __shfl_sync(0xffffffffu, c.fill_bits, 0);
     if (c.lane < 8 && abort_flag == 0) ptx::mbar_wait(&bar_empty[c.lane], ((bits >> c.lane) & 1u) ^ 1u, &abort_flag);
     __syncwarp();

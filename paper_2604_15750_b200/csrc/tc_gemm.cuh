@@ -225,9 +225,6 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w0, const __grid_constant__ CU
         if (++s == (uint32_t)stages) { s = 0; ph ^= 1u; slot = ring0; } else slot += (uint32_t)stage_bytes;
       }
     }
-    // The commits that hand the last slots back arrive in both CTAs of a pair: neither leaves before they have (a lane a slot).
-    if (ok) ok = __all_sync(0xffffffffu, lane >= min((int)filled, stages) ||
-                                             ptx::mbar_wait_a(empty0 + 8u * lane, ((filled - lane - 1u) / stages) & 1u, &abort_flag));
     if (el) fills = filled;
   } else if (warp == 1) {
     // ---------------- MMA issuer ----------------
@@ -240,6 +237,8 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w0, const __grid_constant__ CU
       uint32_t s = 0, ph = 0, lo = lo0;
       bool ok = true;
       const uint32_t odd = EPI == GEMM_EPI_QKV && p.dual ? 256u : 0u;   // the odd k-steps' accumulator
+      int left = 0;   // k-blocks still to come
+      for (int u = cta; u < n_units; u += n_cta) left += unit_of(u).nkb;
       int j = 0;   // accumulators of this CTA so far
       for (int u = cta; u < n_units && ok; u += n_cta) {
         const Unit w = unit_of(u);
@@ -257,6 +256,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w0, const __grid_constant__ CU
             ok = __all_sync(0xffffffffu, ptx::mbar_wait_a(full0 + 8u * s, ph, &abort_flag));
             if (!ok) break;
             const uint32_t more = i > i0 ? 1u : 0u;   // the first MMA of an accumulator overwrites it
+            --left;
             if (el) {
               const uint32_t da = lo + (NW * W_BYTES >> 4);
 #pragma unroll
@@ -270,8 +270,12 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w0, const __grid_constant__ CU
                   if (NW == 2) ptx::umma_bf16_lo(acc + 256u, lo + (W_BYTES >> 4) + 2 * kk, da + 2 * kk, hi, idesc, on);
                 }
               }
-              if (PAIR) ptx::umma_commit_pair_a(empty0 + 8u * s);   // frees the slot in both CTAs
-              else ptx::umma_commit_a(empty0 + 8u * s);
+              // Frees the slot in both CTAs, if it is filled once more: an arrival that nobody waits for could come when
+              // the partner has left.
+              if (left >= stages) {
+                if (PAIR) ptx::umma_commit_pair_a(empty0 + 8u * s);
+                else ptx::umma_commit_a(empty0 + 8u * s);
+              }
             }
             if (++s == (uint32_t)stages) { s = 0; ph ^= 1u; lo = lo0; } else lo += step;
           }
