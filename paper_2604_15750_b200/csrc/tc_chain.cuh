@@ -712,7 +712,8 @@ k_dense_chain(const __grid_constant__ ChainMaps maps, const ChainParams p) {
   }
 
   if (!has_qkv && c.warp == 0) {
-    // (the step's last launch, which ends with a projection: there these arrivals are waited for, a lane a slot)
+    // a launch that ends with a projection (the step's last): the arrivals that hand its last ring slots back come in both
+    // CTAs of the pair, and neither leaves before they have (a lane a slot; one never filled is no wait)
     const uint32_t bits = __shfl_sync(0xffffffffu, c.fill_bits, 0);
     if (c.lane < 8 && abort_flag == 0) ptx::mbar_wait(&bar_empty[c.lane], ((bits >> c.lane) & 1u) ^ 1u, &abort_flag);
     __syncwarp();
