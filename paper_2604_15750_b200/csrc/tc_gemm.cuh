@@ -23,14 +23,15 @@
 // unit, which the epilogue warps add up in registers (0.3 .. 1 us a GEMM against one), and QKV sends even k-steps to the
 // one set and odd ones to the other where a CTA has no second unit.
 //
-// What bounds it: an SM takes in 64 bytes a clock from L2, and a k-block of 256 columns needs 32 KB for 512 clocks
-// of MMAs, so the main loops run at 300..320 ns a k-block (108 GB/s an SM) where the MMAs alone would take 270; batches
-// of 2000 rows and more reach the power cap.  Device timestamps with 1024 rows of LLaDA-8B showed three other
-// things before: a lane in a branch of its own issued a k-block in 390 ns (the issuing warps now run their loops
+// What bounds it: the tensor pipe.  It is busy in 81 .. 87% of an SM's active cycles with 1024 rows of LLaDA-8B and in
+// 89 .. 92 with 2560 (O, whose units are short: 65 and 77); the SMs themselves are idle for a fifth to a quarter of a
+// launch in last rounds that are not whole, and batches of 2000 rows and more reach the power cap.  Device timestamps with
+// 1024 rows showed three other things before: a lane in a branch of its own issued a k-block in 390 ns (the issuing warps now run their loops
 // together and elect a lane); the rotation through shared memory by four warps took 27 us a unit against 25 of
 // MMAs (shuffles take 3.5: the weight rows arrive in an order that puts the two features of a pair into one warp); gate /
 // up stood still for 11 us of every 51 while four warps drained the accumulators (sixteen take 3).  QKV 83 -> 71
-// us, gate / up 153 -> 133; the whole prefill 15.13 -> 14.01 ms, eight boundary steps 37.4 -> 34.2.
+// us, gate / up 153 -> 133; the whole prefill 15.1 -> 13.6 ms, eight boundary steps 37.1 -> 33.4.  The four accumulators
+// a unit are 0.4% of that prefill, 1.5% of one of 300 rows.
 #pragma once
 #include "kernels.h"
 #include "pdl.cuh"
